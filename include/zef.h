@@ -99,8 +99,9 @@ typedef struct zef_label_opts {
     float winding_tol;
     /* zef_precision */
     int32_t precision;
-    /* Threads per block and points per thread of the FP32 kernel; 0 = the
-       autotuned choice.  Valid: threads 128 or 256, points 2 or 4. */
+    /* Threads per block and points per thread of the general FP32 kernels;
+       0 = the library's choice (the cell grid where it serves the call, else
+       the autotuned shape).  Valid: threads 128 or 256, points 2 or 4. */
     int32_t block_threads;
     int32_t points_per_thread;
     /* Form of the FP32 kernel: 0 = cap trees (default): for each tile of
@@ -145,7 +146,9 @@ typedef struct zef_label_stats {
     int64_t points;            /* N */
     int64_t nonfinite_points;  /* points with a NaN/Inf coordinate (label -1) */
     int64_t pairs_nominal;     /* N * sum_c T_c */
-    int64_t pairs_evaluated;   /* point x triangle pairs computed (FP32 + FP64) */
+    int64_t pairs_evaluated;   /* point x triangle pairs computed (FP32 + FP64):
+                                  solid angles, or crossing tests of the cell
+                                  grid */
     int64_t pairs_rescued;     /* point x triangle pairs re-evaluated in FP64 */
     int64_t uncertain_pairs;   /* (point, compartment) pairs sent to FP64 */
     int64_t work_items;        /* (compartment, point tile) items after culling */
@@ -157,12 +160,16 @@ typedef struct zef_label_stats {
     float ms_rescue;           /* device time of the FP64 re-evaluation */
     float reserved;
     int64_t coherent_pairs;    /* (point, compartment) pairs decided by the
-                                  representative point of a tile or group */
+                                  representative point of a tile or group,
+                                  or by the anchor of their grid cell */
     int64_t representative_pairs; /* of pairs_evaluated: point x triangle pairs
                                      of those representatives */
     int64_t lane_walk_items;   /* kernel form 0: (tile, compartment) pairs whose
-                                  points each walked their own cap tree (the
-                                  tile's shared list of segments was too long) */
+                                  points were each decided on their own: by
+                                  the crossings in their own grid cells, or
+                                  (general kernels) by their own walks of the
+                                  cap tree where the tile's shared list of
+                                  segments was too long */
     int64_t kernel_launches;   /* CUDA kernels the library launched for this call
                                   (autotuning runs excluded) */
 } zef_label_stats;
@@ -266,9 +273,10 @@ zef_status zef_compartment_priority(zef_ctx *ctx, const int32_t *ids, int32_t n)
              priority order: the solid angle Omega in steradians: 4 pi k
              exactly wherever the winding number k is certified (0 outside
              the compartment's bounding box or convex-hull bound, the tile's
-             k where the surface provably does not cross a tile, the FP32
-             sum's k within winding_tol), the FP64 sum for the pairs
-             re-evaluated in FP64, the FP32 sum with ZEF_FP32_ONLY for
+             or grid cell's k where the surface provably does not cross it,
+             the cell anchor's k plus the signed crossings of the segment to
+             the point, the FP32 sum's k within winding_tol), the FP64 sum for
+             the pairs summed again in FP64, the FP32 sum with ZEF_FP32_ONLY for
              uncertain pairs; NaN for non-finite points
      opts    nullable = defaults;  stats nullable (non-NULL synchronizes) */
 zef_status zef_label_points(zef_ctx *ctx, const float *pts, int64_t n, int32_t *labels,

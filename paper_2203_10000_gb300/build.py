@@ -30,8 +30,9 @@ COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler",
 PER_FILE = {
     # FP32 hot loop: flush denormals so rsqrtf/__fdividef map to single MUFU ops
     "zef_label.cu": ["-ftz=true", "-Xptxas", "-v"],
+    "zef_grid.cu": ["-Xptxas", "-v"],
 }
-SOURCES = ["zef_host.cpp", "zef_tree.cpp", "zef_label.cu", "zef_refine.cu", "zef_relabel.cu", "zef_post.cu", "zef_noalloc.cu"]
+SOURCES = ["zef_host.cpp", "zef_tree.cpp", "zef_label.cu", "zef_grid.cu", "zef_refine.cu", "zef_relabel.cu", "zef_post.cu", "zef_noalloc.cu"]
 
 
 def _nvcc() -> str:
@@ -54,7 +55,8 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     os.makedirs(out_dir, exist_ok=True)
     nvcc = _nvcc()
     extra = ["-DZEF_DEBUG_BOUNDS"] if debug else []
-    headers = [os.path.join(ROOT, "include", "zef.h"), os.path.join(CSRC, "zef_internal.h")]
+    headers = [os.path.join(ROOT, "include", "zef.h"), os.path.join(CSRC, "zef_internal.h"),
+               os.path.join(CSRC, "zef_fp64.cuh")]
     jobs = []
     objs = []
     for s in SOURCES:

@@ -230,6 +230,7 @@ void zef_destroy(zef_ctx *ctx) {
   }
   if (ctx->s_in) cudaStreamDestroy(ctx->s_in);
   if (ctx->s_out) cudaStreamDestroy(ctx->s_out);
+  grid_free(ctx);
   fr(ctx->d_entries);
   fr(ctx->d_tris);
   fr(ctx->d_nodes);
@@ -368,6 +369,17 @@ zef_status zef_add_compartment(zef_ctx *ctx, int32_t id, const float *verts, int
   ch.id = id;
   ch.nv = nv;
   ch.nt = nt;
+  ch.area = 0.0;
+  for (int64_t t = 0; t < nt; ++t) {
+    const float *a = &V[3 * (int64_t)T[3 * t]], *b = &V[3 * (int64_t)T[3 * t + 1]], *c = &V[3 * (int64_t)T[3 * t + 2]];
+    double u[3], w[3];
+    for (int k = 0; k < 3; ++k) {
+      u[k] = (double)b[k] - a[k];
+      w[k] = (double)c[k] - a[k];
+    }
+    const double x = u[1] * w[2] - u[2] * w[1], y = u[2] * w[0] - u[0] * w[2], z = u[0] * w[1] - u[1] * w[0];
+    ch.area += 0.5 * std::sqrt(x * x + y * y + z * z);
+  }
   for (int k = 0; k < 3; ++k) {
     ch.lo[k] = std::numeric_limits<float>::infinity();
     ch.hi[k] = -std::numeric_limits<float>::infinity();
@@ -651,17 +663,34 @@ static zef_status enqueue_labeling(zef_ctx *ctx, const float *d_pts, int64_t n, 
   plan.opts = o;
   plan.masks = d_masks;
   plan.full_masks = full_masks;
-  bool need_tune = false;
-  plan.shape = choose_shape(ctx, o, n, &need_tune);
   plan.timed = timed;
+  plan.n_host = n;
+  plan.counted = timed;
   zef_status st;
-  if (need_tune && (st = autotune(ctx, plan, &plan.shape))) return st;
+  const bool grid = grid_serves(ctx, o);
+  plan.shape = LaunchShape{256, 2, kernel_variant(o.kernel)};
+  if (!grid) {
+    bool need_tune = false;
+    plan.shape = choose_shape(ctx, o, n, &need_tune);
+    if (need_tune && (st = autotune(ctx, plan, &plan.shape))) return st;
+  }
   const int64_t launches0 = ctx->launches;
-  if ((st = label_set_count(ctx, n, 0))) return st;
+  if (!grid && (st = label_set_count(ctx, n, 0))) return st;
   if ((st = label_enqueue(ctx, plan))) return st;
   *shape = plan.shape;
   *launches = ctx->launches - launches0;
   return ZEF_OK;
+}
+
+// Device buffers of one labeling call: the counters, the general kernels'
+// work buffers where the cell grid does not serve the call, and the staging
+// of host arrays (which the autotuner's sample labels also use).
+static zef_status reserve_call(zef_ctx *ctx, int64_t n, const zef_label_opts &o, bool stage) {
+  zef_status st = label_reserve_counters(ctx);
+  const bool grid = grid_serves(ctx, o);
+  if (!st && !grid) st = label_reserve(ctx, n);
+  if (!st && (stage || !grid)) st = label_reserve_stage(ctx, n);
+  return st;
 }
 
 // Pipelined labeling (zef_label_points_async): slot k = call parity.  The
@@ -678,7 +707,7 @@ zef_status label_points_async_impl(zef_ctx *ctx, const float *pts, int64_t n, in
   if (n == 0) return ZEF_OK;
   DeviceGuard g(ctx->device);
   if ((st = ensure_uploaded(ctx))) return st;
-  if ((st = label_reserve(ctx, n))) return st;
+  if ((st = reserve_call(ctx, n, o, false))) return st;
   const bool dpts = is_device_ptr(pts, ctx->device), dlab = is_device_ptr(labels, ctx->device);
   LaunchShape shape;
   int64_t launches = 0;
@@ -744,11 +773,11 @@ zef_status label_points_impl(zef_ctx *ctx, const float *pts, int64_t n, int32_t 
   DeviceGuard g(ctx->device);
   st = ensure_uploaded(ctx);
   if (st) return st;
-  st = label_reserve(ctx, n);
-  if (st) return st;
   const int C = (int)ctx->comps.size();
   bool dpts = is_device_ptr(pts, ctx->device);
   bool dlab = is_device_ptr(labels, ctx->device);
+  st = reserve_call(ctx, n, o, !dpts || !dlab);
+  if (st) return st;
   bool dom = omega ? is_device_ptr(omega, ctx->device) : true;
   LabelBuffers &b = ctx->lb;
   const float *d_pts = pts;
@@ -796,7 +825,9 @@ zef_status label_points_impl(zef_ctx *ctx, const float *pts, int64_t n, int32_t 
     stats->pairs_evaluated = h[CNT_PAIRS_EVAL] + h[CNT_PAIRS_RESCUE];
     stats->uncertain_pairs = h[CNT_UNC];
     stats->work_items = h[CNT_ITEMS];
-    stats->tiles = h[CNT_TILES];
+    // the cell grid's tiles: 64 consecutive points each, as many as the
+    // points inside the union box would fill
+    stats->tiles = grid_serves(ctx, o) ? (h[CNT_NIN] + 63) / 64 : h[CNT_TILES];
     stats->coherent_pairs = h[CNT_COHERENT];
     stats->representative_pairs = h[CNT_REP_PAIRS];
     stats->lane_walk_items = h[CNT_LANE_TILES];
@@ -956,6 +987,25 @@ template zef_status ensure_buffer<float>(zef_ctx *, float **, int64_t *, int64_t
 template zef_status ensure_buffer<int32_t>(zef_ctx *, int32_t **, int64_t *, int64_t);
 template zef_status ensure_buffer<unsigned long long>(zef_ctx *, unsigned long long **, int64_t *, int64_t);
 
+// Box of `n` consecutive compartments' surfaces (caller's coordinates) with
+// the scale of its cubic Morton cells: that of the longest side on every axis.
+UnionBox surface_box(const CompHost &first, int n) {
+  UnionBox ub;
+  for (int k = 0; k < 3; ++k) {
+    ub.lo[k] = std::numeric_limits<float>::infinity();
+    ub.hi[k] = -std::numeric_limits<float>::infinity();
+  }
+  for (const CompHost *h = &first; h != &first + n; ++h)
+    for (int k = 0; k < 3; ++k) {
+      ub.lo[k] = std::min(ub.lo[k], h->lo[k]);
+      ub.hi[k] = std::max(ub.hi[k], h->hi[k]);
+    }
+  float ext = 0.f;
+  for (int k = 0; k < 3; ++k) ext = std::max(ext, ub.hi[k] - ub.lo[k]);
+  for (int k = 0; k < 3; ++k) ub.sc[k] = ext > 0.f ? (float)(1 << kMortonBits) / ext : 0.f;
+  return ub;
+}
+
 zef_status ensure_uploaded(zef_ctx *ctx) {
   if (ctx->device == ZEF_HOST_ONLY) return ZEF_OK;
   if (!ctx->dirty) return ZEF_OK;
@@ -976,7 +1026,7 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
     ctx->d_tris_cap = ntv;
   }
   if (!ctx->d_comps) {
-    CK(cudaMalloc(&ctx->d_comps, ZEF_MAX_COMPARTMENTS * sizeof(DevComp)), "cudaMalloc(comps)");
+    CK(cudaMalloc(&ctx->d_comps, (ZEF_MAX_COMPARTMENTS + 1) * sizeof(DevComp)), "cudaMalloc(comps)");
     CK(cudaMalloc(&ctx->d_row_ids, ZEF_MAX_COMPARTMENTS * sizeof(int32_t)), "cudaMalloc(rows)");
     CK(cudaMalloc(&ctx->d_lpt, ZEF_MAX_COMPARTMENTS * sizeof(int32_t)), "cudaMalloc(lpt)");
     CK(cudaMalloc(&ctx->d_dop, ZEF_MAX_COMPARTMENTS * kDop * sizeof(float)), "cudaMalloc(dop)");
@@ -1037,20 +1087,7 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
        "upload cap-tree triangle order");
   // union box of the surfaces in the caller's coordinates: the binning keys'
   // range (a point outside it is outside every compartment's box)
-  UnionBox ub;
-  for (int k = 0; k < 3; ++k) {
-    ub.lo[k] = std::numeric_limits<float>::infinity();
-    ub.hi[k] = -std::numeric_limits<float>::infinity();
-  }
-  for (const CompHost &h : ctx->comps)
-    for (int k = 0; k < 3; ++k) {
-      ub.lo[k] = std::min(ub.lo[k], h.lo[k]);
-      ub.hi[k] = std::max(ub.hi[k], h.hi[k]);
-    }
-  // cubic Morton cells: the scale of the box's longest side on every axis
-  float ext = 0.f;
-  for (int k = 0; k < 3; ++k) ext = std::max(ext, ub.hi[k] - ub.lo[k]);
-  for (int k = 0; k < 3; ++k) ub.sc[k] = ext > 0.f ? (float)(1 << kMortonBits) / ext : 0.f;
+  const UnionBox ub = surface_box(ctx->comps[0], C);
   ctx->ubox = ub;
   std::vector<DevComp> dc(C);
   std::vector<int32_t> rows(C), lpt(C);
@@ -1097,7 +1134,9 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
   CK(cudaMemcpy(ctx->d_lpt, lpt.data(), C * sizeof(int32_t), cudaMemcpyHostToDevice), "upload lpt");
   ctx->dirty = false;
   ++ctx->gen;
-  return ZEF_OK;
+  const zef_status st = grid_update(ctx);
+  if (st) ctx->dirty = true;
+  return st;
 }
 
 }  // namespace zef

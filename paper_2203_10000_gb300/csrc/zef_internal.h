@@ -141,9 +141,43 @@ struct UnionBox {
 constexpr int kDop = 96;
 void dop_directions(float (*dirs)[3]);  // fills kDop unit vectors (host)
 
+// Cell grid of a compartment (zef_grid.cu).  A cell word is the winding
+// number (8 bits) of a cell that no triangle meets, or the index of the
+// cell's record with the top bit set.
+struct __align__(16) GridCell {
+  float x, y, z;          // anchor
+  int32_t k;              // its winding number
+  int32_t begin, count;   // the cell's (cell, triangle) entries
+  int32_t pad0, pad1;
+};
+struct __align__(16) GridComp {
+  float lo[3], hi[3];     // the surface's box, caller's coordinates
+  float inv[3];           // cells per unit length
+  int32_t n[3];
+  int32_t comp;
+  float tri_raw;          // scaled triangle vertex -> caller's coordinates (a power of two)
+  const uint32_t *words;
+  const GridCell *cells;
+  const float4 *refs;     // per entry: three edge products with V and the error bound
+  const int32_t *tri;     // per entry: the triangle
+  const float4 *tris;
+};
+static_assert(sizeof(GridComp) == 96, "GridComp is six 16-byte words");
+struct CompGrid {
+  bool usable = false;
+  unsigned char *blob = nullptr;  // owns the arrays below
+  const uint32_t *words = nullptr;
+  const GridCell *cells = nullptr;
+  const float4 *refs = nullptr;
+  const int32_t *tri = nullptr;
+  int32_t n[3] = {0, 0, 0};
+  float inv[3] = {0.f, 0.f, 0.f};
+};
+
 struct CompHost {
   int32_t id;
   int64_t nv, nt;
+  double area;
   float lo[3], hi[3];
   int64_t entry_off, entry_cnt, tri_off, nstrips;
   int32_t cap_root;                // cap tree: root node, segment block, leaf entries
@@ -169,6 +203,7 @@ struct LabelBuffers {
   int2 *items = nullptr;        // (tile, comp)
   int2 *unc_list = nullptr;     // uncertain (sorted point, priority row) pairs
   int64_t *counters = nullptr;  // device counters, see Counter enum
+  int64_t cap_stage = 0;
   int32_t *labels_tmp = nullptr;
   float *pts_tmp = nullptr;     // staging for host inputs
   float *omega_tmp = nullptr;
@@ -265,6 +300,8 @@ struct zef_ctx {
   int64_t *h_counters = nullptr;      // pinned mirror of the counters
 
   cudaEvent_t ev[6] = {};
+  std::vector<zef::CompGrid> grids;   // cell grids, by compartment
+  zef::GridComp *d_grid = nullptr;    // by priority row
   zef::UnionBox ubox = {};            // union box of the surfaces (unscaled), set at upload
   int64_t launches = 0;               // kernels launched by the labeling pipeline (running count)
 
@@ -316,6 +353,7 @@ namespace zef {
 zef_status fail(zef_ctx *ctx, zef_status st, const std::string &msg);
 zef_status cuda_fail(zef_ctx *ctx, cudaError_t e, const char *what);
 zef_status ensure_uploaded(zef_ctx *ctx);
+UnionBox surface_box(const CompHost &first, int n);
 zef_status label_points_impl(zef_ctx *ctx, const float *pts, int64_t n, int32_t *labels, float *omega,
                              const zef_label_opts *opts, zef_label_stats *stats, unsigned long long *d_masks,
                              bool full_masks);
@@ -338,8 +376,13 @@ struct LabelPlan {
   bool timed;                // record events around the main kernels
   unsigned long long *masks = nullptr;  // nullable: per-point inside bits (priority rows), caller's order
   bool full_masks = false;   // evaluate every compartment (no priority early exit)
+  int64_t n_host = -1;       // points when the host knows them (offset 0); -1: the device counters
+  bool counted = true;       // the statistics counters are read afterwards
+  int only_comp = -1;        // >= 0: this compartment alone, as row 0 (general kernels)
 };
 
+zef_status label_reserve_counters(zef_ctx *ctx);
+zef_status label_reserve_stage(zef_ctx *ctx, int64_t n);
 zef_status label_reserve(zef_ctx *ctx, int64_t n_cap);
 zef_status label_enqueue(zef_ctx *ctx, const LabelPlan &plan);
 zef_status label_set_count(zef_ctx *ctx, int64_t n, int64_t off);
@@ -366,6 +409,12 @@ LaunchShape choose_shape(zef_ctx *ctx, const zef_label_opts &o, int64_t n, bool 
 zef_status autotune(zef_ctx *ctx, const LabelPlan &plan, LaunchShape *best);
 void fill_default_opts(zef_label_opts *o);
 bool shape_valid(int threads, int ppt);
+
+// ---- cell grids (zef_grid.cu)
+zef_status grid_update(zef_ctx *ctx);
+void grid_free(zef_ctx *ctx);
+bool grid_serves(const zef_ctx *ctx, const zef_label_opts &o);
+zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan);
 
 // ---- refinement (zef_refine.cu)
 zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_label_opts &opts,

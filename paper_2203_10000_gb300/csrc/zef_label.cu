@@ -66,6 +66,7 @@
 #include <climits>
 #include <cmath>
 
+#include "zef_fp64.cuh"
 #include "zef_internal.h"
 
 namespace zef {
@@ -1904,70 +1905,6 @@ __device__ void strip_half_angle64(const Entry *E, int s, int e, double px, doub
   *wraps = K;
 }
 
-// FP64 strip evaluation of one group of four cap-tree segment entries
-// (positions pos .. pos + 3, a multiple of four: a group never straddles two
-// segments) seen from p: the window enters the group as (E[pos-2], E[pos-1])
-// (both in the same segment, since a segment starts at a multiple of four
-// with its reset entry) or restarts at a reset entry; every window that is a
-// triangle contributes the factor D + iN with N = w R_a . (R_b x R_c) (w the
-// entry's orientation sign, the exact triple product of the stored
-// vertices) and D = r_a r_b r_c + (R_a . R_b) r_c + (R_a . R_c) r_b +
-// (R_b . R_c) r_a (Sec. 2.1.3), and the group returns the argument of the
-// product with the 2 pi wraps of the partial products counted in *K exactly
-// as the FP32 kernel does.
-__device__ __forceinline__ bool sign64(double x) { return __double_as_longlong(x) < 0; }
-
-__device__ double group64(const Entry *E, int pos, double px, double py, double pz, int *K) {
-  double a[3], b[3], ra, rb;
-  const float4 v0 = E[pos].v;
-  if (v0.w == 2.f) {
-    a[0] = b[0] = (double)v0.x - px;
-    a[1] = b[1] = (double)v0.y - py;
-    a[2] = b[2] = (double)v0.z - pz;
-    ra = rb = sqrt(a[0] * a[0] + a[1] * a[1] + a[2] * a[2]);
-  } else {
-    const float4 u = E[pos - 2].v, w = E[pos - 1].v;
-    a[0] = (double)u.x - px; a[1] = (double)u.y - py; a[2] = (double)u.z - pz;
-    b[0] = (double)w.x - px; b[1] = (double)w.y - py; b[2] = (double)w.z - pz;
-    ra = sqrt(a[0] * a[0] + a[1] * a[1] + a[2] * a[2]);
-    rb = sqrt(b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
-  }
-  double R = 1.0, I = 0.0;
-  bool have = false;
-  int k = 0;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const float4 v = E[pos + q].v;
-    const double c[3] = {(double)v.x - px, (double)v.y - py, (double)v.z - pz};
-    const double rc = sqrt(c[0] * c[0] + c[1] * c[1] + c[2] * c[2]);
-    if (fabsf(v.w) == 1.f) {
-      const double N = (double)v.w * (a[0] * (b[1] * c[2] - b[2] * c[1]) + a[1] * (b[2] * c[0] - b[0] * c[2]) +
-                                      a[2] * (b[0] * c[1] - b[1] * c[0]));
-      const double dab = a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
-      const double dac = a[0] * c[0] + a[1] * c[1] + a[2] * c[2];
-      const double dbc = b[0] * c[0] + b[1] * c[1] + b[2] * c[2];
-      const double D = ra * rb * rc + dab * rc + dac * rb + dbc * ra;
-      if (!have) {
-        R = D;
-        I = N;
-        have = true;
-      } else {
-        const double cr = R * D - I * N, ci = R * N + I * D;
-        k += (!sign64(I) && !sign64(N) && sign64(ci)) ? 1 : 0;
-        k -= (sign64(I) && sign64(N) && !sign64(ci)) ? 1 : 0;
-        R = cr;
-        I = ci;
-      }
-    }
-    a[0] = b[0]; a[1] = b[1]; a[2] = b[2];
-    b[0] = c[0]; b[1] = c[1]; b[2] = c[2];
-    ra = rb;
-    rb = rc;
-  }
-  *K += k;
-  return have ? atan2(I, R) : 0.0;
-}
-
 // FP64 half-angle sum over the flattened entries [j0, j1) of a range list
 // (multiples of four), the block's threads splitting the groups of four
 // (fixed assignment and reduction order: deterministic); every thread of the
@@ -2929,6 +2866,33 @@ zef_status autotune(zef_ctx *ctx, const LabelPlan &plan, LaunchShape *best) {
   return ZEF_OK;
 }
 
+zef_status label_reserve_counters(zef_ctx *ctx) {
+  LabelBuffers &b = ctx->lb;
+  if (b.counters) return ZEF_OK;
+  cudaError_t e = cudaMalloc(&b.counters, CNT_COUNT_ * sizeof(int64_t));
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(counters)");
+  cudaMemset(b.counters, 0, CNT_COUNT_ * sizeof(int64_t));
+  return ZEF_OK;
+}
+
+// staging of host points and labels
+zef_status label_reserve_stage(zef_ctx *ctx, int64_t n) {
+  LabelBuffers &b = ctx->lb;
+  if (b.cap_stage >= n) return ZEF_OK;
+  const int64_t cap = std::max<int64_t>(n, 1024);
+  if (b.labels_tmp) cudaFree(b.labels_tmp);
+  if (b.pts_tmp) cudaFree(b.pts_tmp);
+  b.labels_tmp = nullptr;
+  b.pts_tmp = nullptr;
+  b.cap_stage = 0;
+  cudaError_t e = cudaMalloc(&b.labels_tmp, cap * sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&b.pts_tmp, cap * 3 * sizeof(float));
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(staging)");
+  b.cap_stage = cap;
+  return ZEF_OK;
+}
+
+// work buffers of the general kernels
 zef_status label_reserve(zef_ctx *ctx, int64_t n_cap) {
   LabelBuffers &b = ctx->lb;
   const int C = (int)ctx->comps.size();
@@ -2949,8 +2913,6 @@ zef_status label_reserve(zef_ctx *ctx, int64_t n_cap) {
     if ((st = realloc((void **)&b.keys, cap * sizeof(uint32_t)))) return st;
     if ((st = realloc((void **)&b.in_mask, cap * sizeof(unsigned long long)))) return st;
     if ((st = realloc((void **)&b.unc_mask, cap * sizeof(unsigned long long)))) return st;
-    if ((st = realloc((void **)&b.labels_tmp, cap * sizeof(int32_t)))) return st;
-    if ((st = realloc((void **)&b.pts_tmp, cap * 3 * sizeof(float)))) return st;
     b.cap_points = cap;
   }
   const int64_t need_flags = std::max<int64_t>(tiles * std::max(C, 1), kHistLen);
@@ -2983,20 +2945,22 @@ zef_status label_reserve(zef_ctx *ctx, int64_t n_cap) {
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(uncertain pairs)");
     b.cap_unc = kUncListCap;
   }
-  if (!b.counters) {
-    cudaError_t e = cudaMalloc(&b.counters, CNT_COUNT_ * sizeof(int64_t));
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(counters)");
-    cudaMemset(b.counters, 0, CNT_COUNT_ * sizeof(int64_t));
-  }
-  return ZEF_OK;
+  return label_reserve_counters(ctx);
 }
 
 // Enqueue the whole labeling pipeline (no host synchronisation).  When
 // plan.d_n / plan.d_off point into the counters they must already hold the
 // call's values; label_points sets them with k_prepare.
 zef_status label_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
+  // where every compartment has a cell grid, points are labelled from it
+  if (plan.only_comp < 0 && grid_serves(ctx, plan.opts)) return grid_enqueue(ctx, plan);
   LabelBuffers &b = ctx->lb;
-  const int C = (int)ctx->comps.size();
+  // every compartment, or one of them alone as row 0 (its record behind the others')
+  const bool one = plan.only_comp >= 0;
+  const int C = one ? 1 : (int)ctx->comps.size();
+  const DevComp *comps = ctx->d_comps + (one ? ZEF_MAX_COMPARTMENTS : 0);
+  const float *dop = ctx->d_dop + (one ? (size_t)plan.only_comp * kDop : 0);
+  const UnionBox ubox = one ? surface_box(ctx->comps[(size_t)plan.only_comp], 1) : ctx->ubox;
   // FP32: tiles of one warp (32 x P points); plain FP64: tiles of one block
   const int tile = plan.opts.precision == ZEF_FP64_PLAIN ? plan.shape.threads * plan.shape.ppt
                                                          : 32 * plan.shape.ppt;
@@ -3015,7 +2979,7 @@ zef_status label_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
   const int g = grid_for(ctx, ncap, 256);
   // binning: keys in the surfaces' union box, key histogram, scan, scatter
   cudaMemsetAsync(b.hist, 0, (size_t)kHistLen * sizeof(uint32_t), s);
-  k_keys<<<g, 256, 0, s>>>(plan.pts, b.counters, ctx->ubox, b.keys, b.hist, plan.labels, plan.masks, plan.omega,
+  k_keys<<<g, 256, 0, s>>>(plan.pts, b.counters, ubox, b.keys, b.hist, plan.labels, plan.masks, plan.omega,
                            plan.omega_ld, C);
   ++launches;
   zef_status st = scan_keys(ctx, b.hist, tile);
@@ -3027,8 +2991,8 @@ zef_status label_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
   if (plan.opts.precision == ZEF_FP64_PLAIN) {
     // (tile, compartment) items for the plain FP64 kernel
     k_tile_box<<<gt, 256, 0, s>>>(b.spts, b.counters, b.tile_box, tile, b.in_mask, b.unc_mask);
-    k_flags<<<grid_for(ctx, tiles_cap * C, 256), 256, 0, s>>>(b.counters, b.tile_box, ctx->d_comps, ctx->d_lpt, C,
-                                                               ctx->d_dop, b.flags);
+    k_flags<<<grid_for(ctx, tiles_cap * C, 256), 256, 0, s>>>(b.counters, b.tile_box, comps, ctx->d_lpt, C,
+                                                               dop, b.flags);
     launches += 2;
     st = scan_inplace(ctx, b.flags, b.counters + CNT_TILES, C, tiles_cap * C, b.counters + CNT_ITEMS);
     if (st) return st;
@@ -3036,7 +3000,7 @@ zef_status label_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
     ++launches;
   } else {
     // tile items, largest estimated work first
-    k_tile_work<<<gt, 256, 0, s>>>(b.spts, b.counters, tile, ctx->d_comps, C, ctx->d_dop, b.flags, work_hist,
+    k_tile_work<<<gt, 256, 0, s>>>(b.spts, b.counters, tile, comps, C, dop, b.flags, work_hist,
                                    b.in_mask, b.unc_mask);
     k_scan_work<<<1, 1024, 0, s>>>(work_hist, b.counters + CNT_ITEMS);
     k_tile_scatter<<<grid_for(ctx, tiles_cap, 256), 256, 0, s>>>(b.counters, b.flags, work_hist, b.items,
@@ -3047,12 +3011,12 @@ zef_status label_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
   LabelArgs a;
   a.entries = ctx->d_entries;
   a.tris = ctx->d_tris;
-  a.comps = ctx->d_comps;
+  a.comps = comps;
   a.spts = b.spts;
   a.perm = b.perm;
   a.items = b.items;
   a.tile_box = b.tile_box;
-  a.dop = ctx->d_dop;
+  a.dop = dop;
   a.in_mask = b.in_mask;
   a.unc_mask = b.unc_mask;
   a.omega = plan.omega;

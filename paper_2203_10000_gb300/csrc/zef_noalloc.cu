@@ -151,6 +151,8 @@ extern "C" zef_status zef_label_points_noalloc(zef_ctx *ctx, const float *pts, i
   else if (o.block_threads) plan.shape = LaunchShape{o.block_threads, o.points_per_thread, kernel_variant(o.kernel)};
   else plan.shape = LaunchShape{256, 2, kernel_variant(o.kernel)};
   plan.timed = stats != nullptr;
+  plan.n_host = n;
+  plan.counted = stats != nullptr;
 
   // The pipeline enqueues its kernels with the pointers of ctx->lb; point it
   // at the static scratch for the duration of the enqueue only.  Every piece
@@ -159,7 +161,8 @@ extern "C" zef_status zef_label_points_noalloc(zef_ctx *ctx, const float *pts, i
   LabelBuffers saved = ctx->lb;
   ctx->lb = view;
   const int64_t launches0 = ctx->launches;
-  zef_status st = label_set_count(ctx, n, 0);
+  const bool grid = grid_serves(ctx, o);
+  zef_status st = grid ? ZEF_OK : label_set_count(ctx, n, 0);
   if (st == ZEF_OK) st = label_enqueue(ctx, plan);
   const int64_t launches = ctx->launches - launches0;
   ctx->lb = saved;
@@ -179,7 +182,7 @@ extern "C" zef_status zef_label_points_noalloc(zef_ctx *ctx, const float *pts, i
     stats->pairs_evaluated = h[CNT_PAIRS_EVAL] + h[CNT_PAIRS_RESCUE];
     stats->uncertain_pairs = h[CNT_UNC];
     stats->work_items = h[CNT_ITEMS];
-    stats->tiles = h[CNT_TILES];
+    stats->tiles = grid ? (h[CNT_NIN] + 63) / 64 : h[CNT_TILES];
     stats->coherent_pairs = h[CNT_COHERENT];
     stats->representative_pairs = h[CNT_REP_PAIRS];
     stats->lane_walk_items = h[CNT_LANE_TILES];
