@@ -288,7 +288,7 @@ def grid_roofline(n_points, surface_bytes, ms_label):
 
 
 def label_roofline(args_kernel, args_shape, st, w, n_points, ms_label, peak, sms, clocks=None, traffic=None):
-    if args_kernel == 0 and not args_shape and st["kernel_launches"] <= 2:   # the cell grids served the call
+    if args_kernel == 0 and not args_shape and st["kernel_launches"] <= 3:   # the cell grids served the call
         return grid_roofline(n_points, sum(12 * len(s.verts) + 12 * s.ntris for s in w.surfaces), ms_label)
     return roofline(st, ms_label, peak, sms, clocks, traffic)
 

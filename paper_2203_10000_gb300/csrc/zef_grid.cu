@@ -35,7 +35,13 @@
 // every point near a surface (FP32 ALUs, 54 of the 58 ms of 56.2 M points in
 // 24 compartments); here such a point costs about a dozen crossing tests held
 // by the lanes of one warp, and every other point one word per compartment.
-// No sort of the points, no work list and no work buffers: one launch.
+// No sort of the points and no work list: one launch, two for large calls.
+// 56.2 M points in 24 compartments take 0.63 ms (58 ms with the tile kernels,
+// 2.4 ms when every compartment met by a warp was looked up and its cells
+// taken one after the other), 20.5 M in 20 small structures 0.10 ms (2.8),
+// 36,864 with solid angles 9.5 us (259).  What bounds them now: the streaming
+// kernel is near half the copy bandwidth (12 + 4 bytes a point), the open
+// points' kernel waits on its two dependent L2 reads per point.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -58,9 +64,22 @@ namespace zef {
 namespace {
 
 constexpr float kFourPi = 12.5663706143591729539f;
-constexpr uint32_t kMixed = 0x80000000u;    // cell word: index of the cell's record, else its winding number
-constexpr uint32_t kUnknown = 0x40000000u;  // cell word: anchor's winding number unknown
-constexpr int kNoK = INT32_MIN;             // record: anchor's winding number unknown
+// Cell word of a cell that triangles meet: the top bit, the chunks of its
+// block in two bits (0: more than three, see the block's header), and the
+// block's offset in 16-byte words.  Otherwise the winding number (8 bits), or
+// kUnknown.
+constexpr uint32_t kMixed = 0x80000000u;
+constexpr uint32_t kUnknown = 0x40000000u;
+constexpr int kChunkShift = 29;
+constexpr uint32_t kOffsetMask = (1u << kChunkShift) - 1u;
+constexpr int kNoK = -128;  // block header: the anchor's winding number is unknown
+// A block: a header (anchor x, y, z; k in the low 8 bits of w and the number
+// of chunks above), then chunks of kSub entries: kSub first words (a x b, V),
+// kSub second (b x c, error bound), kSub third (c x a, triangle index), so
+// that kSub lanes read 128 bytes at a time.  The last chunk is filled up with
+// entries that the test calls a miss.
+constexpr int kSub = 8;
+constexpr int kChunkWords = 3 * kSub;
 // Every cell is treated as grown by kGrow of its width on each side: a point
 // whose cell index is off by the rounding of (x - lo) * n / extent (at most a
 // few 2^-24 n of a cell, n <= 512) still lies in the grown cell.
@@ -68,6 +87,11 @@ constexpr double kGrow = 2e-3;
 constexpr float kGrowF = 2e-3f;
 constexpr int64_t kMaxCells = 1 << 23;
 constexpr int kMaxAxis = 512;
+// Cells of the label field: 32 MB (64 with more than 32 compartments), which
+// the L2 holds beside the blocks in use.  56.2 M points: 657 us with 2^21
+// cells, 630 with 2^22, 607 with 2^23; 20.5 M points in 20 small structures:
+// 108, 109 and 111.
+constexpr int64_t kMaxField = 1 << 22;
 constexpr int kMaxList = 1024;  // longest triangle list of a usable grid
 
 struct Geom {
@@ -123,15 +147,17 @@ __global__ void __launch_bounds__(256) k_gr_refs(const float4 *tris, float to_ra
   }
 }
 
-// non-empty cells (to be scanned into record numbers) and the longest list
-__global__ void __launch_bounds__(256) k_gr_flags(const uint32_t *cnt, int64_t cells, uint32_t *flag,
+// words of every cell's block (to be scanned into offsets) and the longest list
+__global__ void __launch_bounds__(256) k_gr_sizes(const uint32_t *cnt, int64_t cells, uint32_t *size,
                                                   unsigned long long *longest) {
   uint32_t mx = 0;
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < cells; c += (int64_t)gridDim.x * blockDim.x) {
-    flag[c] = cnt[c] ? 1u : 0u;
-    mx = max(mx, cnt[c]);
+    const uint32_t v = cnt[c];
+    size[c] = v ? 1u + kChunkWords * ((v + kSub - 1) / kSub) : 0u;
+    mx = max(mx, v);
   }
-  mx = __reduce_max_sync(0xffffffffu, mx);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0 && mx) atomicMax(longest, (unsigned long long)mx);
 }
 
@@ -186,15 +212,14 @@ __global__ void __launch_bounds__(256) k_gr_anchor(const float4 *tris, float to_
   }
 }
 
-// Words and records of the cells and the stored products of every (cell,
-// triangle) pair, from the anchors' solid angles.  Vertices relative to the
-// anchor are exact in FP64 up to its rounding; s (a power of two) brings them
-// to about [-64, 64]; the stored cross products carry one factor s more, for
-// the unscaled d = p - q of the kernel.
+// Words and blocks of the cells, from the anchors' solid angles.  Vertices
+// relative to the anchor are exact in FP64 up to its rounding; s (a power of
+// two) brings them to about [-64, 64]; the stored cross products carry one
+// factor s more, for the unscaled d = p - q of the kernel.
 __global__ void __launch_bounds__(256) k_gr_finish(const float4 *tris, float to_raw, double s, Geom g, int64_t cells,
-                                                   const uint32_t *last, const uint32_t *rank, const int32_t *list,
+                                                   const uint32_t *last, const uint32_t *off, const int32_t *list,
                                                    const float *anchor, const float *omega, uint32_t *words,
-                                                   GridCell *recs, float4 *refs) {
+                                                   float4 *blocks) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c < cells; c += nw) {
@@ -207,19 +232,20 @@ __global__ void __launch_bounds__(256) k_gr_finish(const float4 *tris, float to_
       continue;
     }
     const float qx = anchor[3 * c], qy = anchor[3 * c + 1], qz = anchor[3 * c + 2];
+    const uint32_t chunks = (e - b + kSub - 1) / kSub;
+    float4 *block = blocks + off[c];
     if (lane == 0) {
-      words[c] = kMixed | rank[c];
-      GridCell r;
-      r.x = qx;
-      r.y = qy;
-      r.z = qz;
-      r.k = known ? (int)kf : kNoK;
-      r.begin = (int)b;
-      r.count = (int)(e - b);
-      r.pad0 = r.pad1 = 0;
-      recs[rank[c]] = r;
+      words[c] = kMixed | (chunks <= 3 ? chunks << kChunkShift : 0u) | off[c];
+      block[0] = make_float4(qx, qy, qz, __uint_as_float((chunks << 8) | ((uint32_t)(known ? (int)kf : kNoK) & 0xffu)));
     }
-    for (uint32_t j = b + lane; j < e; j += 32) {
+    for (uint32_t j = b + lane; j < b + chunks * kSub; j += 32) {
+      float4 *o = block + 1 + (j - b) / kSub * kChunkWords + (j - b) % kSub;
+      if (j >= e) {  // V > E > 0 and W = -V < -8 E: the segment ends before the plane
+        o[0] = make_float4(0.f, 0.f, 0.f, 1.f);
+        o[kSub] = make_float4(0.f, 0.f, 0.f, 0.01f);
+        o[2 * kSub] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+        continue;
+      }
       const int64_t t = list[j];
       double v[3][3];
 #pragma unroll
@@ -250,10 +276,9 @@ __global__ void __launch_bounds__(256) k_gr_finish(const float4 *tris, float to_
       // products and two sums (5 2^-24 of the sum of the |terms|, which is at
       // most M), plus the FP64 error of N and V
       const double E = 6.2 * 5.9604644775390625e-08 * M + 3.6e-15 * P + 1e-36;
-      float4 *o = refs + 3 * (int64_t)j;
       o[0] = make_float4((float)(N[0][0] * s), (float)(N[0][1] * s), (float)(N[0][2] * s), (float)V);
-      o[1] = make_float4((float)(N[1][0] * s), (float)(N[1][1] * s), (float)(N[1][2] * s), __double2float_ru(E));
-      o[2] = make_float4((float)(N[2][0] * s), (float)(N[2][1] * s), (float)(N[2][2] * s), 0.f);
+      o[kSub] = make_float4((float)(N[1][0] * s), (float)(N[1][1] * s), (float)(N[1][2] * s), __double2float_ru(E));
+      o[2 * kSub] = make_float4((float)(N[2][0] * s), (float)(N[2][1] * s), (float)(N[2][2] * s), __int_as_float((int)t));
     }
   }
 }
@@ -272,7 +297,10 @@ struct GridArgs {
   int ncomp;
   int early;                  // a point certainly inside needs no later compartment
   int stats;
+  int iters;                  // streaming kernel: consecutive tiles of a warp
+  int32_t *pending;           // streaming kernel: indices of the points the field leaves open
   UnionBox ub;
+  LabelField field;
   uint32_t *status;
   const DevComp *comps;       // FP64 solid angles: cap trees (scaled coordinates)
   const CapNode *nodes;
@@ -295,13 +323,17 @@ enum GridStat { GS_EVAL = 0, GS_COHERENT, GS_OWN, GS_ITEMS, GS_NONFINITE, GS_NIN
 __device__ __noinline__ bool resolve64(const GridArgs &a, const GridComp &g, uint32_t word, float x, float y, float z,
                                        int lane, float *omega) {
   if (word & kMixed) {
-    const GridCell r = g.cells[word & ~kMixed];
-    int net = 0;
-    bool open = r.k == kNoK;
+    const float4 *block = g.blocks + (word & kOffsetMask);
+    const float4 r = block[0];
+    const int k0 = (int)(signed char)(__float_as_uint(r.w) & 0xffu), count = (int)(__float_as_uint(r.w) >> 8) * kSub;
+    int net = 0, tested = 0;
+    bool open = k0 == kNoK;
     if (!open) {
       const double dx = (double)x - r.x, dy = (double)y - r.y, dz = (double)z - r.z;
-      for (int j = lane; j < r.count; j += 32) {
-        const int64_t t = g.tri[r.begin + j];
+      for (int j = lane; j < count; j += 32) {
+        const int64_t t = __float_as_int(block[1 + j / kSub * kChunkWords + 2 * kSub + j % kSub].w);
+        if (t < 0) continue;
+        ++tested;
         double v[3][3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -339,12 +371,13 @@ __device__ __noinline__ bool resolve64(const GridArgs &a, const GridComp &g, uin
     }
     if (!__any_sync(0xffffffffu, open)) {
       net = __reduce_add_sync(0xffffffffu, net);
+      tested = __reduce_add_sync(0xffffffffu, tested);
       if (lane == 0 && a.stats) {
         count_add(a, CNT_UNC, 1);
-        count_add(a, CNT_PAIRS_RESCUE, (unsigned long long)r.count);
+        count_add(a, CNT_PAIRS_RESCUE, (unsigned long long)tested);
       }
-      *omega = kFourPi * (float)(r.k + net);
-      return r.k + net >= 1;
+      *omega = kFourPi * (float)(k0 + net);
+      return k0 + net >= 1;
     }
   }
   // FP64 solid angle: the caps of the nodes whose box misses the point, the
@@ -400,275 +433,463 @@ __device__ __noinline__ bool resolve64(const GridArgs &a, const GridComp &g, uin
   return om > 6.283185307179586476925;
 }
 
-// order-preserving int of a float, and back
-__device__ __forceinline__ int ord(float f) {
-  const int b = __float_as_int(f);
-  return b ^ ((b >> 31) & 0x7fffffff);
+// ---- the label field: one cell grid over the union box of all surfaces.  A
+// cell holds, per priority row, whether its points have winding number 1
+// (`ins`) or need the compartment's own grid (`mix`: its cells there are not
+// all empty of triangles with one winding number of 0 or 1); neither bit: 0.
+template <bool WIDE>
+struct FieldCell;
+template <>
+struct FieldCell<false> {
+  using T = uint2;
+  using M = uint32_t;
+};
+template <>
+struct FieldCell<true> {
+  using T = ulonglong2;
+  using M = unsigned long long;
+};
+
+// Index of x on an axis of n cells; monotone in x, so the indices of a box's
+// ends bound those of its points.
+__device__ __forceinline__ int axis_cell(float x, float lo, float inv, int n) {
+  return min(max((int)((x - lo) * inv), 0), n - 1);
 }
-__device__ __forceinline__ float unord(int b) { return __int_as_float(b ^ ((b >> 31) & 0x7fffffff)); }
+
+template <bool WIDE>
+__global__ void __launch_bounds__(256) k_gr_field(LabelField f, const GridComp *grid, int ncomp) {
+  using M = typename FieldCell<WIDE>::M;
+  __shared__ GridComp s_g[ZEF_MAX_COMPARTMENTS];
+  for (int j = threadIdx.x; j < ncomp * (int)(sizeof(GridComp) / 16); j += blockDim.x)
+    reinterpret_cast<uint4 *>(s_g)[j] = reinterpret_cast<const uint4 *>(grid)[j];
+  __syncthreads();
+  const int64_t cells = (int64_t)f.n[0] * f.n[1] * f.n[2];
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < cells; c += (int64_t)gridDim.x * blockDim.x) {
+    const int xyz[3] = {(int)(c % f.n[0]), (int)(c / f.n[0] % f.n[1]), (int)(c / f.n[0] / f.n[1])};
+    float lo[3], hi[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {  // the cell grown by kGrow: it holds every point that k_grid_label puts in it
+      lo[k] = __double2float_rd(f.lo[k] + (xyz[k] - kGrow) * f.h[k]);
+      hi[k] = __double2float_ru(f.lo[k] + (xyz[k] + 1 + kGrow) * f.h[k]);
+    }
+    M ins = 0, mix = 0;
+    for (int r = 0; r < ncomp; ++r) {
+      const GridComp &g = s_g[r];
+      bool out = false, part = false;  // the cell misses the surface's box / reaches out of it
+      int i0[3], i1[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        out |= hi[k] < g.lo[k] || lo[k] > g.hi[k];
+        part |= lo[k] < g.lo[k] || hi[k] > g.hi[k];
+        i0[k] = axis_cell(fmaxf(lo[k], g.lo[k]), g.lo[k], g.inv[k], g.n[k]);
+        i1[k] = axis_cell(fminf(hi[k], g.hi[k]), g.lo[k], g.inv[k], g.n[k]);
+      }
+      if (out) continue;
+      uint32_t w = part ? 0u : 0xffffffffu;  // the winding number so far (none yet: all ones)
+      bool same = true;
+      for (int z = i0[2]; z <= i1[2] && same; ++z)
+        for (int y = i0[1]; y <= i1[1] && same; ++y)
+          for (int x = i0[0]; x <= i1[0] && same; ++x) {
+            const uint32_t v = g.words[((int64_t)z * g.n[1] + y) * g.n[0] + x];
+            if (v > 1u) same = false;  // triangles, unknown, or a winding number other than 0 and 1
+            else if (w == 0xffffffffu) w = v;
+            else if (w != v) same = false;
+          }
+      if (!same) mix |= (M)1 << r;
+      else if (w == 1u) ins |= (M)1 << r;
+    }
+    typename FieldCell<WIDE>::T o;
+    o.x = ins;
+    o.y = mix;
+    reinterpret_cast<typename FieldCell<WIDE>::T *>(f.cells)[c] = o;
+  }
+}
 
 constexpr int kGlThreads = 256;
-constexpr int kGlP = 2;               // points per lane
-constexpr int kGlTile = 32 * kGlP;    // points of a warp's tile
+constexpr int kGlWarps = kGlThreads / 32;
+constexpr int kGlP = 2;               // fused kernel: points per lane and step
+constexpr int kGlTile = 32 * kGlP;
+constexpr int kGlQueue = 32 + kGlTile;  // fewer than 32 left over, one tile's more
+constexpr int kGsP = 4;               // streaming kernel
+constexpr int kGsTile = 32 * kGsP;
+constexpr int kGsQueue = 64 + kGsTile;
+constexpr int kGlMaxIters = 32;       // consecutive tiles of a warp
+constexpr int kLanes = 4;             // lanes per point of the crossing tests
 
-// One warp per tile of 64 consecutive points.  The tile's box selects the
-// compartments (one per lane); for each of them every lane looks its points'
-// cells up; points in cells with triangles are taken cell by cell: the lanes
-// hold 32 of the cell's triangles (stored products, 48 bytes each, read
-// once per tile and cell) and the points of the cell are broadcast one after
-// the other, so the work of a point does not depend on its neighbours' lists.
-__global__ void __launch_bounds__(kGlThreads) k_grid_label(GridArgs a) {
-  __shared__ GridComp s_g[ZEF_MAX_COMPARTMENTS];
+__device__ __forceinline__ int first_row(uint32_t m) { return __ffs((int)m) - 1; }
+__device__ __forceinline__ int first_row(unsigned long long m) { return __ffsll((long long)m) - 1; }
+// rows that can still matter: with the priority early exit those before the
+// first row the point is known to be inside of
+template <class M>
+__device__ __forceinline__ M open_rows(M ins, M mix, int early) {
+  return early ? mix & ((ins & (M)(0 - ins)) - 1) : mix;
+}
+
+// A point whose label the field leaves open.
+template <bool WIDE>
+struct __align__(16) Pending {
+  float x, y, z;
+  int32_t i;
+  typename FieldCell<WIDE>::M ins, mix;
+};
+
+// Shared memory of the batches of one block.
+struct Batch {
+  float4 p[kGlWarps][32];             // x, y, z, word of the batch's points in cells with triangles
+  const float4 *blocks[kGlWarps][32];  // their compartments' blocks
+};
+
+// Decides a batch of up to 32 points (one per lane, `have`): every lane looks
+// its point's cell up in the grid of the first row the point still needs;
+// points in cells with triangles are then taken eight at a time, four lanes
+// each over the entries of the point's own cell (two dependent reads per
+// point -- word, block -- whatever cells and compartments the batch lies in).
+template <bool WIDE>
+__device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, const int32_t *s_id, Batch &sb, int wid,
+                                       int lane, int64_t off, float x, float y, float z, int32_t i, bool have,
+                                       typename FieldCell<WIDE>::M mask, typename FieldCell<WIDE>::M mix,
+                                       uint32_t &st_eval, uint32_t &st_own) {
+  using M = typename FieldCell<WIDE>::M;
+  const int sub = lane / kLanes, ti = lane % kLanes;
+  M pend = have ? open_rows<M>(mask, mix, a.early) : 0;
+  while (__any_sync(0xffffffffu, pend != 0)) {
+    const bool mine = pend != 0;
+    const int r = mine ? first_row(pend) : 0;
+    pend &= pend - 1;
+    const GridComp &g = s_g[r];
+    const bool in = mine && x >= g.lo[0] && x <= g.hi[0] && y >= g.lo[1] && y <= g.hi[1] && z >= g.lo[2] && z <= g.hi[2];
+    uint32_t word = 0u;
+    if (in) {
+      const int cx = axis_cell(x, g.lo[0], g.inv[0], g.n[0]), cy = axis_cell(y, g.lo[1], g.inv[1], g.n[1]),
+                cz = axis_cell(z, g.lo[2], g.inv[2], g.n[2]);
+      const int c = (cz * g.n[1] + cy) * g.n[0] + cx;  // at most kMaxCells
+      if (ZEF_BOUNDS_OK(c >= 0 && c < g.n[0] * g.n[1] * g.n[2], a.status, 30)) word = __ldg(g.words + c);
+    }
+    const bool mixed = (word & kMixed) != 0u;
+    bool unc = (word & (kMixed | kUnknown)) == kUnknown;
+    int k = (int)(signed char)(word & 0xffu);
+    const uint32_t m = __ballot_sync(0xffffffffu, mixed);
+    if (m) {
+      const int np = __popc(m), rank = __popc(m & ((1u << lane) - 1u));
+      if (mixed) {
+        sb.p[wid][rank] = make_float4(x, y, z, __uint_as_float(word));
+        sb.blocks[wid][rank] = g.blocks;
+      }
+      __syncwarp();
+      for (int j0 = 0; j0 < np; j0 += 32 / kLanes) {
+        const int j = min(j0 + sub, np - 1);  // a step short of points repeats the last one
+        const float4 q = sb.p[wid][j];
+        const uint32_t w = __float_as_uint(q.w);
+        const float4 *block = sb.blocks[wid][j] + (w & kOffsetMask);
+        const float4 h = __ldg(block);
+        const float4 *t = block + 1 + ti;
+        int chunks = (int)((w & ~kMixed) >> kChunkShift);
+        if (!chunks) chunks = (int)(__float_as_uint(h.w) >> 8);
+        const int k0 = (int)(signed char)(__float_as_uint(h.w) & 0xffu);
+        const float dx = q.x - h.x, dy = q.y - h.y, dz = q.z - h.z;
+        bool open = k0 == kNoK;
+        int net = 0;
+        for (int b = 0; b < chunks; ++b, t += kChunkWords) {
+          float4 e[kSub / kLanes][3];
+#pragma unroll
+          for (int u = 0; u < kSub / kLanes; ++u)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) e[u][d] = __ldg(t + u * kLanes + d * kSub);
+#pragma unroll
+          for (int u = 0; u < kSub / kLanes; ++u) {
+            const float4 n0 = e[u][0], n1 = e[u][1], n2 = e[u][2];
+            const float v0 = fmaf(n0.x, dx, fmaf(n0.y, dy, n0.z * dz));
+            const float v1 = fmaf(n1.x, dx, fmaf(n1.y, dy, n1.z * dz));
+            const float v2 = fmaf(n2.x, dx, fmaf(n2.y, dy, n2.z * dz));
+            const float V = n0.w, E = n1.w, EW = 8.f * n1.w, W = (v0 + v1 + v2) - V;
+            const float mn = fminf(v0, fminf(v1, v2)), mx = fmaxf(v0, fmaxf(v1, v2));
+            const bool vp = V > E, vn = V < -E, wp = W > EW, wn = W < -EW;
+            const bool cross_out = vp && wp && mn > E, cross_in = vn && wn && mx < -E;
+            const bool none = (mn < -E && mx > E) || (vn && wp) || (vp && wn);
+            net += cross_in ? 1 : cross_out ? -1 : 0;
+            open |= !(none || cross_out || cross_in);
+          }
+        }
+        // over the point's lanes, then back to the lane that owns the point
+#pragma unroll
+        for (int o = kLanes / 2; o > 0; o >>= 1) net += __shfl_xor_sync(0xffffffffu, net, o);
+        const uint32_t bu = __ballot_sync(0xffffffffu, open);
+        const int kn = __shfl_sync(0xffffffffu, k0 + net, (rank - j0) * kLanes & 31);
+        if (mixed && rank >= j0 && rank < j0 + 32 / kLanes) {
+          k = kn;
+          unc = ((bu >> ((rank - j0) * kLanes)) & ((1u << kLanes) - 1u)) != 0u;
+        }
+        if (a.stats && j0 + sub < np && ti == 0) st_eval += (uint32_t)chunks * kSub;
+      }
+      __syncwarp();
+      ++st_own;
+    }
+    float om = kFourPi * (float)k;
+    bool inside = in && !unc && k >= 1;
+    uint32_t um = __ballot_sync(0xffffffffu, unc);
+    while (um) {
+      const int src = __ffs(um) - 1;
+      um &= um - 1;
+      float o64;
+      const bool i64 = resolve64(a, s_g[__shfl_sync(0xffffffffu, r, src)], __shfl_sync(0xffffffffu, word, src),
+                                 __shfl_sync(0xffffffffu, x, src), __shfl_sync(0xffffffffu, y, src),
+                                 __shfl_sync(0xffffffffu, z, src), lane, &o64);
+      if (lane == src) {
+        inside = i64;
+        om = o64;
+      }
+    }
+    if (inside) {
+      mask |= (M)1 << r;
+      if (a.early) pend = 0;
+    }
+    if (a.omega && mine) a.omega[(int64_t)r * a.omega_ld + i] = in ? om : 0.f;
+  }
+  if (have) {
+    a.labels[off + i] = mask ? s_id[first_row(mask)] : 0;
+    if (a.masks) a.masks[off + i] = mask;
+  }
+}
+
+// Field cell of a point: zero outside the union box and for a non-finite
+// point (whose comparisons fail).
+template <bool WIDE>
+__device__ __forceinline__ typename FieldCell<WIDE>::T field_cell(const GridArgs &a, float x, float y, float z,
+                                                                  bool *in_box) {
+  typename FieldCell<WIDE>::T c;
+  c.x = 0;
+  c.y = 0;
+  *in_box = x >= a.ub.lo[0] && x <= a.ub.hi[0] && y >= a.ub.lo[1] && y <= a.ub.hi[1] && z >= a.ub.lo[2] && z <= a.ub.hi[2];
+  if (*in_box) {
+    const int cx = axis_cell(x, a.field.lo[0], a.field.inv[0], a.field.n[0]),
+              cy = axis_cell(y, a.field.lo[1], a.field.inv[1], a.field.n[1]),
+              cz = axis_cell(z, a.field.lo[2], a.field.inv[2], a.field.n[2]);
+    c = __ldg(reinterpret_cast<const typename FieldCell<WIDE>::T *>(a.field.cells) +
+              ((cz * a.field.n[1] + cy) * a.field.n[0] + cx));
+  }
+  return c;
+}
+
+struct LaneStats {
+  uint32_t coh = 0, nonfin = 0, nin = 0, eval = 0, own = 0;
+};
+
+__device__ void flush_stats(const GridArgs &a, const LaneStats &st, unsigned long long (*s_stat)[GS_COUNT], int wid,
+                            int lane) {
+  uint32_t v[GS_COUNT];
+  v[GS_EVAL] = st.eval;
+  v[GS_COHERENT] = st.coh;
+  v[GS_OWN] = lane == 0 ? st.own : 0u;  // counted by the whole warp
+  v[GS_ITEMS] = 0u;
+  v[GS_NONFINITE] = st.nonfin;
+  v[GS_NIN] = st.nin;
+#pragma unroll
+  for (int q = 0; q < GS_COUNT; ++q) v[q] = __reduce_add_sync(0xffffffffu, v[q]);
+  v[GS_ITEMS] = (v[GS_NIN] + 63) / 64;
+  if (lane == 0)
+#pragma unroll
+    for (int q = 0; q < GS_COUNT; ++q) s_stat[wid][q] = v[q];
+  __syncthreads();
+  if (threadIdx.x < GS_COUNT) {
+    unsigned long long t = 0ull;
+    for (int w = 0; w < kGlWarps; ++w) t += s_stat[w][threadIdx.x];
+    constexpr int kCnt[GS_COUNT] = {CNT_PAIRS_EVAL, CNT_COHERENT, CNT_LANE_TILES, CNT_ITEMS, CNT_NONFINITE, CNT_NIN};
+    if (t) count_add(a, kCnt[threadIdx.x], t);
+  }
+}
+
+__device__ __forceinline__ void load_grids(const GridArgs &a, GridComp *s_g, int32_t *s_id) {
   for (int j = threadIdx.x; j < a.ncomp * (int)(sizeof(GridComp) / 16); j += kGlThreads)
     reinterpret_cast<uint4 *>(s_g)[j] = reinterpret_cast<const uint4 *>(a.grid)[j];
-  __shared__ unsigned long long s_stat[kGlThreads / 32][GS_COUNT];
+  for (int j = threadIdx.x; j < a.ncomp; j += kGlThreads) s_id[j] = a.row_ids[j];
+}
+
+// Label, inside bits and Omega rows that the field decides of point i.
+template <bool WIDE>
+__device__ __forceinline__ void field_store(const GridArgs &a, const int32_t *s_id, int64_t off, int64_t i,
+                                            typename FieldCell<WIDE>::M ins, typename FieldCell<WIDE>::M mix, bool fin,
+                                            bool open) {
+  if (!open) {
+    a.labels[off + i] = !fin ? -1 : ins ? s_id[first_row(ins)] : 0;
+    if (a.masks) a.masks[off + i] = ins;
+  }
+  if (a.omega)
+    for (int r = 0; r < a.ncomp; ++r)
+      if (!((mix >> r) & 1))
+        a.omega[(int64_t)r * a.omega_ld + i] = !fin ? __int_as_float(0x7fc00000) : (ins >> r) & 1 ? kFourPi : 0.f;
+}
+
+// One launch (small calls): a warp reads 64 consecutive points, looks their
+// field cells up and writes the labels of the points that the field decides;
+// the others go to the warp's queue in shared memory, and whenever it holds
+// 32 they are decided together.
+template <bool WIDE>
+__global__ void __launch_bounds__(kGlThreads, 4) k_grid_label(GridArgs a) {
+  using M = typename FieldCell<WIDE>::M;
+  __shared__ GridComp s_g[ZEF_MAX_COMPARTMENTS];
+  __shared__ int32_t s_id[ZEF_MAX_COMPARTMENTS];
+  __shared__ Pending<WIDE> s_q[kGlWarps][kGlQueue];
+  __shared__ Batch sb;
+  __shared__ unsigned long long s_stat[kGlWarps][GS_COUNT];
+  load_grids(a, s_g, s_id);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane < GS_COUNT) s_stat[wid][lane] = 0ull;
   __syncthreads();
   const int64_t n = a.n_host >= 0 ? a.n_host : a.counters[CNT_N];
   const int64_t off = a.n_host >= 0 ? 0 : a.counters[CNT_OFF];
-  const int64_t step = (int64_t)gridDim.x * (kGlThreads / 32) * kGlTile;
-  for (int64_t base = ((int64_t)blockIdx.x * (kGlThreads / 32) + wid) * kGlTile; base < n; base += step) {
-    float x[kGlP], y[kGlP], z[kGlP];
-    bool fin[kGlP], done[kGlP];
-    unsigned long long mask[kGlP];
-    int lo[3] = {INT32_MAX, INT32_MAX, INT32_MAX}, hi[3] = {INT32_MIN, INT32_MIN, INT32_MIN};
+  const float *pts = a.pts + 3 * off;
+  int queued = 0;
+  LaneStats st;
+  const int64_t step = (int64_t)gridDim.x * kGlWarps * kGlTile;
+  for (int64_t base = ((int64_t)blockIdx.x * kGlWarps + wid) * kGlTile;; base += step) {
+    const bool last = base >= n;  // warp-uniform: no points left, only the queue
 #pragma unroll
     for (int u = 0; u < kGlP; ++u) {
       const int64_t i = base + 32 * u + lane;
-      x[u] = y[u] = z[u] = 0.f;
+      float x = __int_as_float(0x7fc00000), y = x, z = x;
       if (i < n) {
-        const float *p = a.pts + 3 * (off + i);
-        x[u] = p[0];
-        y[u] = p[1];
-        z[u] = p[2];
+        x = pts[3 * i];
+        y = pts[3 * i + 1];
+        z = pts[3 * i + 2];
       }
-      fin[u] = i < n && isfinite(x[u]) && isfinite(y[u]) && isfinite(z[u]);
-      done[u] = !fin[u];
-      mask[u] = 0ull;
-      if (fin[u]) {
-        lo[0] = min(lo[0], ord(x[u])); hi[0] = max(hi[0], ord(x[u]));
-        lo[1] = min(lo[1], ord(y[u])); hi[1] = max(hi[1], ord(y[u]));
-        lo[2] = min(lo[2], ord(z[u])); hi[2] = max(hi[2], ord(z[u]));
-      }
-    }
-    float wlo[3], whi[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      wlo[k] = unord(__reduce_min_sync(0xffffffffu, lo[k]));
-      whi[k] = unord(__reduce_max_sync(0xffffffffu, hi[k]));
-    }
-    unsigned long long met = 0ull;
-    for (int c0 = 0; c0 < a.ncomp; c0 += 32) {
-      const int c = c0 + lane;
-      bool ov = false;
-      if (c < a.ncomp) {
-        const GridComp &g = s_g[c];
-        ov = wlo[0] <= g.hi[0] && whi[0] >= g.lo[0] && wlo[1] <= g.hi[1] && whi[1] >= g.lo[1] && wlo[2] <= g.hi[2] &&
-             whi[2] >= g.lo[2];
-      }
-      met |= (unsigned long long)__ballot_sync(0xffffffffu, ov) << c0;
-    }
-    uint32_t ev = 0, coh = 0;  // crossing tests, points decided by their cell alone (whole warp)
-    uint32_t own = 0;          // compartments with points decided by their own crossings
-    unsigned long long todo = met;
-    int r_done = 0;            // rows below r_done have their Omega written
-    while (todo) {
-      const int r = __ffsll((long long)todo) - 1;
-      todo &= todo - 1;
-      const GridComp &g = s_g[r];
-      bool in[kGlP], mixed[kGlP], unc[kGlP], inside[kGlP];
-      uint32_t word[kGlP], m[kGlP];
-      int k[kGlP];
-#pragma unroll
-      for (int u = 0; u < kGlP; ++u) {
-        in[u] = !done[u] && x[u] >= g.lo[0] && x[u] <= g.hi[0] && y[u] >= g.lo[1] && y[u] <= g.hi[1] &&
-                z[u] >= g.lo[2] && z[u] <= g.hi[2];
-        word[u] = 0u;
-        if (in[u]) {
-          const int cx = min((int)((x[u] - g.lo[0]) * g.inv[0]), g.n[0] - 1);
-          const int cy = min((int)((y[u] - g.lo[1]) * g.inv[1]), g.n[1] - 1);
-          const int cz = min((int)((z[u] - g.lo[2]) * g.inv[2]), g.n[2] - 1);
-          const int64_t c = ((int64_t)cz * g.n[1] + cy) * g.n[0] + cx;
-          if (ZEF_BOUNDS_OK(cx >= 0 && cy >= 0 && cz >= 0 && c < (int64_t)g.n[0] * g.n[1] * g.n[2], a.status, 30))
-            word[u] = __ldg(g.words + c);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kGlP; ++u) {
-        mixed[u] = (word[u] & kMixed) != 0u;
-        unc[u] = (word[u] & (kMixed | kUnknown)) == kUnknown;
-        k[u] = (int)(signed char)(word[u] & 0xffu);
-        m[u] = __ballot_sync(0xffffffffu, mixed[u]);
-      }
+      bool in_box;
+      const auto c = field_cell<WIDE>(a, x, y, z, &in_box);
+      const M ins = c.x, mix = c.y;
+      const bool fin = isfinite(x) && isfinite(y) && isfinite(z), open = open_rows<M>(ins, mix, a.early) != 0;
       if (a.stats) {
-        bool any_in = false;
-#pragma unroll
-        for (int u = 0; u < kGlP; ++u) {
-          coh += __popc(__ballot_sync(0xffffffffu, in[u] && !mixed[u]));
-          any_in |= m[u] != 0u;
-        }
-        own += any_in ? 1u : 0u;
+        st.coh += sizeof(M) == 8 ? __popcll(ins) : __popc((uint32_t)ins);
+        st.nin += in_box ? 1 : 0;
+        st.nonfin += i < n && !fin ? 1 : 0;
       }
-      for (;;) {
-        // next cell: that of the first point left
-        uint32_t w0;
-        if (m[0]) w0 = __shfl_sync(0xffffffffu, word[0], __ffs(m[0]) - 1);
-        else if (m[kGlP - 1]) w0 = __shfl_sync(0xffffffffu, word[kGlP - 1], __ffs(m[kGlP - 1]) - 1);
-        else break;
-        const GridCell *rec = g.cells + (w0 & ~kMixed);
-        const float4 q = __ldg(reinterpret_cast<const float4 *>(rec));      // x, y, z, k
-        const int4 l = __ldg(reinterpret_cast<const int4 *>(rec) + 1);      // begin, count
-        const int k0 = __float_as_int(q.w);
-        uint32_t peers[kGlP];
-        float dx[kGlP], dy[kGlP], dz[kGlP];
-        int net[kGlP];
-        bool open[kGlP];
-#pragma unroll
-        for (int u = 0; u < kGlP; ++u) {
-          peers[u] = __ballot_sync(0xffffffffu, mixed[u] && word[u] == w0);
-          m[u] &= ~peers[u];
-          dx[u] = x[u] - q.x;
-          dy[u] = y[u] - q.y;
-          dz[u] = z[u] - q.z;
-          net[u] = 0;
-          open[u] = k0 == kNoK;
-        }
-        for (int b = 0; b < l.y; b += 32) {
-          const bool act = b + lane < l.y;
-          float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0;
-          if (act) {
-            const float4 *t = g.refs + 3 * (int64_t)(l.x + b + lane);
-            n0 = __ldg(t);
-            n1 = __ldg(t + 1);
-            n2 = __ldg(t + 2);
-          }
-          const float V = n0.w, E = n1.w, EW = 8.f * n1.w;
-          const bool vp = act && V > E, vn = act && V < -E;
-#pragma unroll
-          for (int u = 0; u < kGlP; ++u) {
-            uint32_t pp = peers[u];
-            while (pp) {
-              const int src = __ffs(pp) - 1;
-              pp &= pp - 1;
-              const float ex = __shfl_sync(0xffffffffu, dx[u], src), ey = __shfl_sync(0xffffffffu, dy[u], src),
-                          ez = __shfl_sync(0xffffffffu, dz[u], src);
-              const float v0 = fmaf(n0.x, ex, fmaf(n0.y, ey, n0.z * ez));
-              const float v1 = fmaf(n1.x, ex, fmaf(n1.y, ey, n1.z * ez));
-              const float v2 = fmaf(n2.x, ex, fmaf(n2.y, ey, n2.z * ez));
-              const float W = (v0 + v1 + v2) - V;
-              const float mn = fminf(v0, fminf(v1, v2)), mx = fmaxf(v0, fmaxf(v1, v2));
-              const bool wp = W > EW, wn = W < -EW;
-              const bool cross_out = vp && wp && mn > E, cross_in = vn && wn && mx < -E;
-              const bool none = (mn < -E && mx > E) || (vn && wp) || (vp && wn) || !act;
-              const uint32_t bo = __ballot_sync(0xffffffffu, cross_out), bi = __ballot_sync(0xffffffffu, cross_in);
-              const uint32_t bu = __ballot_sync(0xffffffffu, !(none || cross_out || cross_in));
-              if (lane == src) {
-                net[u] += __popc(bi) - __popc(bo);
-                open[u] |= bu != 0u;
-              }
-            }
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < kGlP; ++u) {
-          if (mixed[u] && word[u] == w0) {
-            k[u] = k0 + net[u];
-            unc[u] = open[u];
-          }
-          if (a.stats) ev += (uint32_t)__popc(peers[u]) * (uint32_t)l.y;
-        }
+      if (i < n) field_store<WIDE>(a, s_id, off, i, ins, mix, fin, open);
+      const uint32_t ob = __ballot_sync(0xffffffffu, open);
+      if (open) {
+        Pending<WIDE> p;
+        p.x = x;
+        p.y = y;
+        p.z = z;
+        p.i = (int32_t)i;
+        p.ins = ins;
+        p.mix = mix;
+        s_q[wid][queued + __popc(ob & ((1u << lane) - 1u))] = p;
       }
-#pragma unroll
-      for (int u = 0; u < kGlP; ++u) {
-        float om = kFourPi * (float)k[u];
-        inside[u] = in[u] && !unc[u] && k[u] >= 1;
-        uint32_t um = __ballot_sync(0xffffffffu, unc[u]);
-        while (um) {
-          const int src = __ffs(um) - 1;
-          um &= um - 1;
-          float o64;
-          const bool i64 = resolve64(a, g, __shfl_sync(0xffffffffu, word[u], src), __shfl_sync(0xffffffffu, x[u], src),
-                                     __shfl_sync(0xffffffffu, y[u], src), __shfl_sync(0xffffffffu, z[u], src), lane,
-                                     &o64);
-          if (lane == src) {
-            inside[u] = i64;
-            om = o64;
-          }
-        }
-        if (inside[u]) mask[u] |= 1ull << r;
-        if (a.omega) {
-          const int64_t i = base + 32 * u + lane;
-          if (i < n)
-            a.omega[(int64_t)r * a.omega_ld + i] = !fin[u] ? __int_as_float(0x7fc00000) : in[u] ? om : 0.f;
-        }
-        done[u] = done[u] || (a.early && inside[u]);
-      }
-      if (a.omega) {  // rows of compartments the tile does not meet
-        for (int q = r_done; q < r; ++q)
-#pragma unroll
-          for (int u = 0; u < kGlP; ++u) {
-            const int64_t i = base + 32 * u + lane;
-            if (i < n) a.omega[(int64_t)q * a.omega_ld + i] = fin[u] ? 0.f : __int_as_float(0x7fc00000);
-          }
-        r_done = r + 1;
-      }
-      if (a.early) {
-        bool all = true;
-#pragma unroll
-        for (int u = 0; u < kGlP; ++u) all = all && done[u];
-        if (__all_sync(0xffffffffu, all)) break;
-      }
+      queued += __popc(ob);
     }
-    if (a.omega)
-      for (int q = r_done; q < a.ncomp; ++q)
+    __syncwarp();
+    while (queued >= 32 || (last && queued > 0)) {
+      const Pending<WIDE> p = s_q[wid][lane];
+      const int cnt = min(queued, 32);
+      decide<WIDE>(a, s_g, s_id, sb, wid, lane, off, p.x, p.y, p.z, p.i, lane < cnt, p.ins, p.mix, st.eval, st.own);
+      for (int j = lane; j + 32 < queued; j += 32) {
+        const Pending<WIDE> t = s_q[wid][j + 32];
+        s_q[wid][j] = t;
+      }
+      queued -= cnt;
+      __syncwarp();
+    }
+    if (last) break;
+  }
+  if (a.stats) flush_stats(a, st, s_stat, wid, lane);
+}
+
+// Two launches (large calls).  Streaming: labels of the points that the field
+// decides (12 bytes in, 4 out per point, the field from L2; few registers, so
+// many loads in flight); the indices of the others are listed, a warp's
+// consecutive points in runs of at least 64.
+template <bool WIDE>
+__global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
+  using M = typename FieldCell<WIDE>::M;
+  __shared__ int32_t s_id[ZEF_MAX_COMPARTMENTS];
+  __shared__ int32_t s_q[kGlWarps][kGsQueue];
+  __shared__ unsigned long long s_stat[kGlWarps][GS_COUNT];
+  for (int j = threadIdx.x; j < a.ncomp; j += kGlThreads) s_id[j] = a.row_ids[j];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __syncthreads();
+  const int64_t n = a.n_host >= 0 ? a.n_host : a.counters[CNT_N];
+  const int64_t off = a.n_host >= 0 ? 0 : a.counters[CNT_OFF];
+  const float *pts = a.pts + 3 * off;
+  int queued = 0;
+  LaneStats st;
+  const int64_t first = ((int64_t)blockIdx.x * kGlWarps + wid) * a.iters * kGsTile;
+  const int64_t end = min(n, first + (int64_t)a.iters * kGsTile);
+  for (int64_t base = first; base < end; base += kGsTile) {
+    float x[kGsP], y[kGsP], z[kGsP];
+    bool in_box[kGsP];
+    typename FieldCell<WIDE>::T c[kGsP];
 #pragma unroll
-        for (int u = 0; u < kGlP; ++u) {
-          const int64_t i = base + 32 * u + lane;
-          if (i < n) a.omega[(int64_t)q * a.omega_ld + i] = fin[u] ? 0.f : __int_as_float(0x7fc00000);
-        }
-#pragma unroll
-    for (int u = 0; u < kGlP; ++u) {
+    for (int u = 0; u < kGsP; ++u) {
       const int64_t i = base + 32 * u + lane;
-      if (i < n) {
-        a.labels[off + i] = !fin[u] ? -1 : mask[u] ? __ldg(a.row_ids + (__ffsll((long long)mask[u]) - 1)) : 0;
-        if (a.masks) a.masks[off + i] = mask[u];
+      x[u] = y[u] = z[u] = __int_as_float(0x7fc00000);
+      if (i < end) {
+        x[u] = __ldcs(pts + 3 * i);
+        y[u] = __ldcs(pts + 3 * i + 1);
+        z[u] = __ldcs(pts + 3 * i + 2);
       }
     }
-    if (a.stats) {
-      uint32_t nonfin = 0, nin = 0;
 #pragma unroll
-      for (int u = 0; u < kGlP; ++u) {
-        const int64_t i = base + 32 * u + lane;
-        nonfin += __popc(__ballot_sync(0xffffffffu, i < n && !fin[u]));
-        nin += __popc(__ballot_sync(0xffffffffu, fin[u] && x[u] >= a.ub.lo[0] && x[u] <= a.ub.hi[0] &&
-                                                     y[u] >= a.ub.lo[1] && y[u] <= a.ub.hi[1] &&
-                                                     z[u] >= a.ub.lo[2] && z[u] <= a.ub.hi[2]));
+    for (int u = 0; u < kGsP; ++u) c[u] = field_cell<WIDE>(a, x[u], y[u], z[u], &in_box[u]);
+#pragma unroll
+    for (int u = 0; u < kGsP; ++u) {
+      const int64_t i = base + 32 * u + lane;
+      const M ins = c[u].x, mix = c[u].y;
+      const bool fin = isfinite(x[u]) && isfinite(y[u]) && isfinite(z[u]);
+      const bool open = open_rows<M>(ins, mix, a.early) != 0;
+      if (a.stats) {
+        st.coh += sizeof(M) == 8 ? __popcll(ins) : __popc((uint32_t)ins);
+        st.nin += in_box[u] ? 1 : 0;
+        st.nonfin += i < end && !fin ? 1 : 0;
       }
-      if (lane == 0) {
-        s_stat[wid][GS_EVAL] += ev;
-        s_stat[wid][GS_COHERENT] += coh;
-        s_stat[wid][GS_OWN] += own;
-        s_stat[wid][GS_ITEMS] += met ? 1 : 0;
-        s_stat[wid][GS_NONFINITE] += nonfin;
-        s_stat[wid][GS_NIN] += nin;
-      }
+      if (i < end) field_store<WIDE>(a, s_id, off, i, ins, mix, fin, open);
+      const uint32_t ob = __ballot_sync(0xffffffffu, open);
+      if (open) s_q[wid][queued + __popc(ob & ((1u << lane) - 1u))] = (int32_t)i;
+      queued += __popc(ob);
+    }
+    if (queued >= 64 || (base + kGsTile >= end && queued > 0)) {
+      __syncwarp();
+      unsigned long long at = 0;
+      if (lane == 0) at = atomicAdd((unsigned long long *)(a.counters + CNT_PEND), (unsigned long long)queued);
+      at = __shfl_sync(0xffffffffu, at, 0);
+      for (int j = lane; j < queued; j += 32) a.pending[at + j] = s_q[wid][j];
+      queued = 0;
+      __syncwarp();
     }
   }
-  if (a.stats) {
-    __syncthreads();
-    if (threadIdx.x < GS_COUNT) {
-      unsigned long long v = 0ull;
-      for (int w = 0; w < kGlThreads / 32; ++w) v += s_stat[w][threadIdx.x];
-      constexpr int kCnt[GS_COUNT] = {CNT_PAIRS_EVAL, CNT_COHERENT, CNT_LANE_TILES, CNT_ITEMS, CNT_NONFINITE, CNT_NIN};
-      if (v) count_add(a, kCnt[threadIdx.x], v);
+  if (a.stats) flush_stats(a, st, s_stat, wid, lane);
+}
+
+// The listed points, 32 at a time.
+template <bool WIDE>
+__global__ void __launch_bounds__(kGlThreads, 4) k_grid_pending(GridArgs a) {
+  __shared__ GridComp s_g[ZEF_MAX_COMPARTMENTS];
+  __shared__ int32_t s_id[ZEF_MAX_COMPARTMENTS];
+  __shared__ Batch sb;
+  __shared__ unsigned long long s_stat[kGlWarps][GS_COUNT];
+  const int64_t m = a.counters[CNT_PEND];
+  if ((int64_t)blockIdx.x * kGlThreads >= m) return;
+  load_grids(a, s_g, s_id);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __syncthreads();
+  const int64_t off = a.n_host >= 0 ? 0 : a.counters[CNT_OFF];
+  const float *pts = a.pts + 3 * off;
+  LaneStats st;
+  for (int64_t j0 = (int64_t)blockIdx.x * kGlThreads + 32 * wid; j0 < m; j0 += (int64_t)gridDim.x * kGlThreads) {
+    const bool have = j0 + lane < m;
+    const int32_t i = have ? a.pending[j0 + lane] : 0;
+    float x = __int_as_float(0x7fc00000), y = x, z = x;
+    if (have) {
+      x = pts[3 * (int64_t)i];
+      y = pts[3 * (int64_t)i + 1];
+      z = pts[3 * (int64_t)i + 2];
     }
+    bool in_box;
+    const auto c = field_cell<WIDE>(a, x, y, z, &in_box);
+    decide<WIDE>(a, s_g, s_id, sb, wid, lane, off, x, y, z, i, have, c.x, c.y, st.eval, st.own);
   }
+  if (a.stats) flush_stats(a, st, s_stat, wid, lane);
 }
 
 __global__ void k_grid_reset(int64_t *cnt) {
   constexpr int c[] = {CNT_ITEMS, CNT_UNC,      CNT_NONFINITE, CNT_PAIRS_EVAL, CNT_PAIRS_RESCUE,
-                       CNT_COHERENT, CNT_REP_PAIRS, CNT_LANE_TILES, CNT_NIN,     CNT_TILES};
+                       CNT_COHERENT, CNT_REP_PAIRS, CNT_LANE_TILES, CNT_NIN,     CNT_TILES, CNT_PEND};
   if (threadIdx.x < sizeof(c) / sizeof(c[0])) cnt[c[threadIdx.x]] = 0;
 }
 
@@ -686,10 +907,32 @@ bool grid_opts(const zef_label_opts &o) {
 // forms, raw FP32 sums, FP32 or FP64 alone, every point evaluated for
 // itself, or a margin that covers the certified values.
 bool grid_serves(const zef_ctx *ctx, const zef_label_opts &o) {
-  if (!grid_opts(o) || ctx->grids.size() != ctx->comps.size()) return false;
+  if (!grid_opts(o) || ctx->grids.size() != ctx->comps.size() || !ctx->field.cells) return false;
   for (const CompGrid &g : ctx->grids)
     if (!g.usable) return false;
   return true;
+}
+
+// Calls of at least kListedMin points list the points that the field leaves
+// open and decide them in a second kernel: the streaming part alone needs 40
+// registers instead of 64 and the lists fill every batch (56.2 M points: 958
+// us in one kernel, 657 in two; 5 M: 151 and 97).  Below that the second
+// launch costs more than it saves (scratch: 4 bytes per point, which the allocation-free entry point,
+// at most 65,536 points, never needs).
+constexpr int64_t kListedMin = 1 << 18;
+static_assert(kListedMin > ZEF_NOALLOC_MAX_POINTS, "the allocation-free entry point has no list");
+static bool grid_listed(const zef_ctx *ctx, int64_t n_cap) { return n_cap >= kListedMin && ctx->lb.cap_pending >= n_cap; }
+
+zef_status grid_reserve(zef_ctx *ctx, int64_t n_cap) {
+  LabelBuffers &b = ctx->lb;
+  if (n_cap < kListedMin || b.cap_pending >= n_cap) return ZEF_OK;
+  if (b.pending) cudaFree(b.pending);
+  b.pending = nullptr;
+  b.cap_pending = 0;
+  cudaError_t e = cudaMalloc(&b.pending, (size_t)n_cap * sizeof(int32_t));
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(open points)");
+  b.cap_pending = n_cap;
+  return ZEF_OK;
 }
 
 zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
@@ -708,22 +951,44 @@ zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
   a.early = plan.omega == nullptr && !plan.full_masks;
   a.stats = plan.counted;
   a.ub = ctx->ubox;
+  a.field = ctx->field;
   a.status = ctx->d_status;
   a.comps = ctx->d_comps;
   a.nodes = ctx->d_nodes;
   a.cseg = ctx->d_cseg;
   a.scale = ctx->scale;
+  // The list serves calls that fill the GPU; below that one launch is shorter.
+  const bool listed = grid_listed(ctx, plan.n_cap);
+  a.pending = ctx->lb.pending;
   if (plan.timed) cudaEventRecord(ctx->ev[0], s);
-  if (a.stats) {
+  if (a.stats || listed) {
     k_grid_reset<<<1, 32, 0, s>>>(ctx->lb.counters);
     ++ctx->launches;
   }
   NvtxRange nvtx_stage("zef.label_kernel");
   if (plan.timed) cudaEventRecord(ctx->ev[1], s);
-  const int per_block = kGlThreads / 32 * kGlTile;
-  const int64_t blocks = std::min<int64_t>((plan.n_cap + per_block - 1) / per_block, (int64_t)ctx->num_sms * 32);
-  k_grid_label<<<(unsigned)std::max<int64_t>(blocks, 1), kGlThreads, 0, s>>>(a);
-  ++ctx->launches;
+  const bool wide = a.ncomp > 32;
+  if (listed) {
+    const int64_t tiles = (plan.n_cap + kGsTile - 1) / kGsTile;
+    // a warp's consecutive tiles list neighbouring points together
+    a.iters = (int)std::min<int64_t>(kGlMaxIters, std::max<int64_t>(1, tiles / ((int64_t)ctx->num_sms * 16 * kGlWarps)));
+    const unsigned blocks = (unsigned)((tiles + (int64_t)a.iters * kGlWarps - 1) / ((int64_t)a.iters * kGlWarps));
+    const unsigned pblocks = (unsigned)std::min<int64_t>((plan.n_cap + kGlThreads - 1) / kGlThreads, (int64_t)ctx->num_sms * 16);
+    if (wide) {
+      k_grid_stream<true><<<blocks, kGlThreads, 0, s>>>(a);
+      k_grid_pending<true><<<pblocks, kGlThreads, 0, s>>>(a);
+    } else {
+      k_grid_stream<false><<<blocks, kGlThreads, 0, s>>>(a);
+      k_grid_pending<false><<<pblocks, kGlThreads, 0, s>>>(a);
+    }
+    ctx->launches += 2;
+  } else {
+    a.iters = 1;
+    const unsigned blocks = (unsigned)std::max<int64_t>(1, (plan.n_cap + kGlWarps * kGlTile - 1) / (kGlWarps * kGlTile));
+    if (wide) k_grid_label<true><<<blocks, kGlThreads, 0, s>>>(a);
+    else k_grid_label<false><<<blocks, kGlThreads, 0, s>>>(a);
+    ++ctx->launches;
+  }
   if (plan.timed) {
     cudaEventRecord(ctx->ev[2], s);
     cudaEventRecord(ctx->ev[3], s);
@@ -740,13 +1005,16 @@ void grid_free(zef_ctx *ctx) {
     if (g.blob) cudaFree(g.blob);
   ctx->grids.clear();
   if (ctx->d_grid) cudaFree(ctx->d_grid);
+  if (ctx->field.cells) cudaFree(ctx->field.cells);
   ctx->d_grid = nullptr;
+  ctx->field.cells = nullptr;
 }
 
-// Cell grid of compartment c (uploaded, with its cap tree).  Cells are two
-// mean triangle edges wide (a cell then lists about a dozen triangles, which
-// one warp holds at once, and about 1.5 cells per crossed cell face area are
-// mixed), at least eight along the longest side, at most kMaxCells in all.
+// Cell grid of compartment c (uploaded, with its cap tree).  Cells are one
+// mean triangle edge wide (a cell with triangles then lists about seven of
+// them, one chunk; 56.2 M points in 24 compartments: 650 us at 0.8 edges, 657
+// at 1.0, 729 at 1.3, and the memory grows with the inverse square), at least
+// eight along the longest side, at most kMaxCells in all.
 // A surface whose grid would not pay -- a list longer than kMaxList (all its
 // triangles in a few cells), coordinates whose cubes leave FP32's range, no
 // memory -- is left without: calls then take the general kernels.
@@ -761,7 +1029,7 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   }
   *out = gr;
   if (!(big > 1e-12f && big < 1e12f && longest > 1e-6f * big)) return ZEF_OK;
-  double w = 2.0 * std::sqrt(h.area / (0.43 * (double)h.nt));
+  double w = 1.0 * std::sqrt(h.area / (0.43 * (double)h.nt));
   w = std::min(w, (double)longest / 8.0);
   w = std::max(w, (double)longest / kMaxAxis);
   Geom g;
@@ -787,7 +1055,7 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   const int nt = (int)h.nt;
   cudaStream_t st = ctx->stream;
 
-  // scratch: counts / list ends, record numbers, block sums, two totals, anchors, their Omega
+  // scratch: counts / list ends, block sizes / offsets, scan sums, totals, anchors, their Omega
   const int64_t bs = cells / 2048 + 2;
   const size_t o_flag = (size_t)cells * 4, o_sum = o_flag + (size_t)cells * 4, o_tot = (o_sum + (size_t)bs * 4 + 15) & ~(size_t)15,
                o_anch = o_tot + 32, o_om = o_anch + (size_t)cells * 12, bytes = o_om + (size_t)cells * 4;
@@ -807,7 +1075,7 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   const int g_t = grid_blocks(ctx, (int64_t)nt * 32, 256), g_c = grid_blocks(ctx, cells, 256),
             g_w = grid_blocks(ctx, cells * 32, 256);
   k_gr_refs<<<g_t, 256, 0, st>>>(tris, to_raw, nt, g, cnt, nullptr);
-  k_gr_flags<<<g_c, 256, 0, st>>>(cnt, cells, flag, (unsigned long long *)(tot + 2));
+  k_gr_sizes<<<g_c, 256, 0, st>>>(cnt, cells, flag, (unsigned long long *)(tot + 2));
   zef_status zs = scan_exclusive(ctx, cnt, nullptr, 1, cells, tot, bsum);
   if (!zs) zs = scan_exclusive(ctx, flag, nullptr, 1, cells, tot + 1, bsum);
   int64_t totals[3] = {0, 0, 0};
@@ -820,18 +1088,21 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
     cudaFree(tmp);
     return zs;
   }
-  const int64_t refs = totals[0], mixed = totals[1];
-  if (totals[2] > kMaxList || refs > 64 * (int64_t)nt + 65536) {
+  const int64_t refs = totals[0], words16 = totals[1];
+  if (totals[2] > kMaxList || refs > 64 * (int64_t)nt + 65536 || words16 > (int64_t)kOffsetMask) {
     cudaFree(tmp);
     return ZEF_OK;
   }
-  // stored products, records, words, triangle indices
-  const size_t p_cell = (size_t)refs * 48, p_word = p_cell + (size_t)mixed * sizeof(GridCell),
-               p_tri = p_word + (size_t)cells * 4, p_end = p_tri + (size_t)refs * 4;
+  // blocks and words; the triangle lists are scratch
+  const size_t p_word = (size_t)words16 * 16, p_end = p_word + (size_t)cells * 4;
   unsigned char *blob = nullptr;
-  e = cudaMalloc(&blob, p_end);
-  if (e != cudaSuccess) return no_memory(e);
-  int32_t *list = (int32_t *)(blob + p_tri);
+  int32_t *list = nullptr;
+  e = cudaMalloc(&list, std::max<size_t>((size_t)refs * 4, 16));
+  if (e == cudaSuccess) e = cudaMalloc(&blob, p_end);
+  if (e != cudaSuccess) {
+    if (list) cudaFree(list);
+    return no_memory(e);
+  }
   k_gr_refs<<<g_t, 256, 0, st>>>(tris, to_raw, nt, g, cnt, list);  // cnt: list starts -> ends
   k_gr_anchor<<<g_w, 256, 0, st>>>(tris, to_raw, g, cells, cnt, list, anchor);
   // the anchors' solid angles of this compartment alone
@@ -861,16 +1132,18 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   if (zs) {
     cudaStreamSynchronize(st);
     cudaFree(blob);
+    cudaFree(list);
     cudaFree(tmp);
     if (zs != ZEF_ERR_OOM) return zs;
     cudaGetLastError();
     return ZEF_OK;
   }
   k_gr_finish<<<g_w, 256, 0, st>>>(tris, to_raw, s, g, cells, cnt, flag, list, anchor, omega, (uint32_t *)(blob + p_word),
-                                   (GridCell *)(blob + p_cell), (float4 *)blob);
+                                   (float4 *)blob);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(tmp);
+  cudaFree(list);
   if (e != cudaSuccess) {
     cudaFree(blob);
     return cuda_fail(ctx, e, "cell grid");
@@ -878,9 +1151,7 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   gr.blob = blob;
   gr.usable = true;
   gr.words = (const uint32_t *)(blob + p_word);
-  gr.cells = (const GridCell *)(blob + p_cell);
-  gr.refs = (const float4 *)blob;
-  gr.tri = list;
+  gr.blocks = (const float4 *)blob;
   for (int k = 0; k < 3; ++k) {
     gr.n[k] = g.n[k];
     gr.inv[k] = g.inv[k];
@@ -916,12 +1187,53 @@ zef_status grid_update(zef_ctx *ctx) {
     r.comp = (int32_t)c;
     r.tri_raw = 1.f / ctx->scale;
     r.words = g.words;
-    r.cells = g.cells;
-    r.refs = g.refs;
-    r.tri = g.tri;
+    r.blocks = g.blocks;
     r.tris = ctx->d_tris + h.tri_off * 3;
   }
   CK(cudaMemcpy(ctx->d_grid, d.data(), C * sizeof(GridComp), cudaMemcpyHostToDevice), "upload cell grids");
+
+  // the label field: cells as wide as the finest compartment grid's, at most
+  // kMaxField of them (one or two 64-bit words each: it stays in L2)
+  if (ctx->field.cells) cudaFree(ctx->field.cells);
+  ctx->field.cells = nullptr;
+  LabelField f = {};
+  float ext[3], longest = 0.f;
+  for (int k = 0; k < 3; ++k) {
+    ext[k] = ctx->ubox.hi[k] - ctx->ubox.lo[k];
+    longest = std::max(longest, ext[k]);
+  }
+  double w = longest;
+  for (size_t c = 0; c < C; ++c) {
+    if (!ctx->grids[c].usable) return ZEF_OK;
+    for (int k = 0; k < 3; ++k)
+      if (ctx->grids[c].n[k] > 1) w = std::min(w, (double)(ctx->comps[c].hi[k] - ctx->comps[c].lo[k]) / ctx->grids[c].n[k]);
+  }
+  int64_t cells = 0;
+  for (;; w *= 1.05) {
+    cells = 1;
+    for (int k = 0; k < 3; ++k) {
+      f.n[k] = (int)std::min<double>(kMaxAxis, std::max(1.0, std::ceil(ext[k] / w)));
+      cells *= f.n[k];
+    }
+    if (cells <= kMaxField) break;
+  }
+  for (int k = 0; k < 3; ++k) {
+    f.lo[k] = ctx->ubox.lo[k];
+    f.h[k] = (double)ext[k] / f.n[k];
+    f.inv[k] = ext[k] > 0.f ? (float)(f.n[k] / (double)ext[k]) : 0.f;
+  }
+  const bool wide = C > 32;
+  cudaError_t e = cudaMalloc(&f.cells, (size_t)cells * (wide ? sizeof(ulonglong2) : sizeof(uint2)));
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return ZEF_OK;  // no field: the general kernels
+  }
+  CK(e, "cudaMalloc(label field)");
+  ctx->field = f;
+  const int g_f = grid_blocks(ctx, cells, 256);
+  if (wide) k_gr_field<true><<<g_f, 256, 0, ctx->stream>>>(f, ctx->d_grid, (int)C);
+  else k_gr_field<false><<<g_f, 256, 0, ctx->stream>>>(f, ctx->d_grid, (int)C);
+  CK(cudaGetLastError(), "label field");
   return ZEF_OK;
 }
 

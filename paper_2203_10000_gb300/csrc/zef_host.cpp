@@ -244,7 +244,7 @@ void zef_destroy(zef_ctx *ctx) {
   LabelBuffers &b = ctx->lb;
   fr(b.spts); fr(b.perm); fr(b.keys); fr(b.in_mask); fr(b.unc_mask); fr(b.tile_box);
   fr(b.hist); fr(b.flags); fr(b.block_sums); fr(b.items); fr(b.unc_list); fr(b.counters);
-  fr(b.labels_tmp); fr(b.pts_tmp); fr(b.omega_tmp); fr(b.tune_pts);
+  fr(b.pending); fr(b.labels_tmp); fr(b.pts_tmp); fr(b.omega_tmp); fr(b.tune_pts);
   fr(ctx->el_node_labels); fr(ctx->el_masks); fr(ctx->el_tets); fr(ctx->el_labels);
   for (auto &p : ctx->rf_buf) fr(p);
   for (auto &p : ctx->rb_buf) fr(p);
@@ -688,7 +688,7 @@ static zef_status enqueue_labeling(zef_ctx *ctx, const float *d_pts, int64_t n, 
 static zef_status reserve_call(zef_ctx *ctx, int64_t n, const zef_label_opts &o, bool stage) {
   zef_status st = label_reserve_counters(ctx);
   const bool grid = grid_serves(ctx, o);
-  if (!st && !grid) st = label_reserve(ctx, n);
+  if (!st) st = grid ? grid_reserve(ctx, n) : label_reserve(ctx, n);
   if (!st && (stage || !grid)) st = label_reserve_stage(ctx, n);
   return st;
 }

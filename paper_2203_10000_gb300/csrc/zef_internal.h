@@ -141,15 +141,7 @@ struct UnionBox {
 constexpr int kDop = 96;
 void dop_directions(float (*dirs)[3]);  // fills kDop unit vectors (host)
 
-// Cell grid of a compartment (zef_grid.cu).  A cell word is the winding
-// number (8 bits) of a cell that no triangle meets, or the index of the
-// cell's record with the top bit set.
-struct __align__(16) GridCell {
-  float x, y, z;          // anchor
-  int32_t k;              // its winding number
-  int32_t begin, count;   // the cell's (cell, triangle) entries
-  int32_t pad0, pad1;
-};
+// Cell grid of a compartment (zef_grid.cu).
 struct __align__(16) GridComp {
   float lo[3], hi[3];     // the surface's box, caller's coordinates
   float inv[3];           // cells per unit length
@@ -157,19 +149,24 @@ struct __align__(16) GridComp {
   int32_t comp;
   float tri_raw;          // scaled triangle vertex -> caller's coordinates (a power of two)
   const uint32_t *words;
-  const GridCell *cells;
-  const float4 *refs;     // per entry: three edge products with V and the error bound
-  const int32_t *tri;     // per entry: the triangle
+  const float4 *blocks;   // per cell with triangles: anchor and entries
   const float4 *tris;
 };
-static_assert(sizeof(GridComp) == 96, "GridComp is six 16-byte words");
+static_assert(sizeof(GridComp) == 80, "GridComp is five 16-byte words");
+// Cell grid over the union box of the surfaces: per cell the rows whose
+// winding number is 1 in all of it and the rows that need their own grid
+// (uint2, or ulonglong2 with more than 32 compartments).
+struct LabelField {
+  float lo[3], inv[3];
+  int32_t n[3];
+  double h[3];
+  void *cells;
+};
 struct CompGrid {
   bool usable = false;
   unsigned char *blob = nullptr;  // owns the arrays below
   const uint32_t *words = nullptr;
-  const GridCell *cells = nullptr;
-  const float4 *refs = nullptr;
-  const int32_t *tri = nullptr;
+  const float4 *blocks = nullptr;
   int32_t n[3] = {0, 0, 0};
   float inv[3] = {0.f, 0.f, 0.f};
 };
@@ -203,6 +200,8 @@ struct LabelBuffers {
   int2 *items = nullptr;        // (tile, comp)
   int2 *unc_list = nullptr;     // uncertain (sorted point, priority row) pairs
   int64_t *counters = nullptr;  // device counters, see Counter enum
+  int32_t *pending = nullptr;   // cell grid: points whose label the field leaves open
+  int64_t cap_pending = 0;
   int64_t cap_stage = 0;
   int32_t *labels_tmp = nullptr;
   float *pts_tmp = nullptr;     // staging for host inputs
@@ -245,6 +244,7 @@ enum Counter {
   CNT_CL_GREEN,       // tets split along one to three edges
   CNT_CL_GEXTRA,      // children those splits add
   CNT_LANE_TILES,     // cap trees: (tile, compartment) pairs evaluated by per-lane walks
+  CNT_PEND,           // cell grid: points whose label the field leaves open
   CNT_UNC_LIST,       // uncertain pairs appended to the pair list (may exceed its capacity)
   CNT_COUNT_ = 32
 };
@@ -302,6 +302,7 @@ struct zef_ctx {
   cudaEvent_t ev[6] = {};
   std::vector<zef::CompGrid> grids;   // cell grids, by compartment
   zef::GridComp *d_grid = nullptr;    // by priority row
+  zef::LabelField field = {};
   zef::UnionBox ubox = {};            // union box of the surfaces (unscaled), set at upload
   int64_t launches = 0;               // kernels launched by the labeling pipeline (running count)
 
@@ -413,6 +414,7 @@ bool shape_valid(int threads, int ppt);
 // ---- cell grids (zef_grid.cu)
 zef_status grid_update(zef_ctx *ctx);
 void grid_free(zef_ctx *ctx);
+zef_status grid_reserve(zef_ctx *ctx, int64_t n_cap);
 bool grid_serves(const zef_ctx *ctx, const zef_label_opts &o);
 zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan);
 

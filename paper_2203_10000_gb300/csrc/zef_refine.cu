@@ -636,7 +636,8 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
   const int64_t new_cap = std::max<int64_t>(1, std::min<int64_t>(6 * fmax, ncap - N0));
   if ((st = label_reserve_counters(ctx))) return st;
   const bool grid = grid_serves(ctx, opts);  // labels from the cell grids: no work buffers
-  if (!grid && (st = label_reserve(ctx, std::max<int64_t>(new_cap, mesh->labels_valid ? 1 : N0)))) return st;
+  const int64_t n_lab = std::max<int64_t>(new_cap, mesh->labels_valid ? 1 : N0);
+  if ((st = grid ? grid_reserve(ctx, n_lab) : label_reserve(ctx, n_lab))) return st;
   LabelBuffers &b = ctx->lb;
 
   LaunchShape shape{256, 2, kernel_variant(opts.kernel)};
@@ -692,7 +693,8 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
                        (uint64_t)(uintptr_t)b.spts, (uint64_t)(uintptr_t)b.flags, (uint64_t)(uintptr_t)b.hist,
                        (uint64_t)(uintptr_t)b.counters, (uint64_t)b.cap_points, (uint64_t)shape.threads,
                        (uint64_t)shape.ppt, (uint64_t)shape.variant, (uint64_t)opts.precision, fbits(opts.margin),
-                       fbits(opts.winding_tol), (uint64_t)opts.flags, (uint64_t)grid, (uint64_t)(uintptr_t)ctx->d_entries, (uint64_t)conforming, ctx->gen,
+                       fbits(opts.winding_tol), (uint64_t)opts.flags, (uint64_t)grid, (uint64_t)(uintptr_t)b.pending,
+                       (uint64_t)b.cap_pending, (uint64_t)(uintptr_t)ctx->d_entries, (uint64_t)conforming, ctx->gen,
                        (uint64_t)(uintptr_t)r.state, (uint64_t)(uintptr_t)r.gx})
       key = hash_mix(key, v);
     if (!ctx->rf_exec || ctx->rf_key != key) {

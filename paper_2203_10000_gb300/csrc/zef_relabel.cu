@@ -208,7 +208,7 @@ zef_status relabel_run(zef_ctx *ctx, const float *nodes_in, int64_t n, const int
   }
   if ((st = label_reserve_counters(ctx))) return st;
   const bool grid = grid_serves(ctx, opts);  // labels from the cell grids: no work buffers
-  if (!grid && (st = label_reserve(ctx, n))) return st;
+  if ((st = grid ? grid_reserve(ctx, n) : label_reserve(ctx, n))) return st;
   LabelBuffers &b = ctx->lb;
 
   LaunchShape shape{256, 2, kernel_variant(opts.kernel)};
@@ -241,7 +241,8 @@ zef_status relabel_run(zef_ctx *ctx, const float *nodes_in, int64_t n, const int
                      (uint64_t)(uintptr_t)b.spts, (uint64_t)(uintptr_t)b.flags, (uint64_t)(uintptr_t)b.hist,
                      (uint64_t)(uintptr_t)b.counters, (uint64_t)b.cap_points, (uint64_t)shape.threads,
                      (uint64_t)shape.ppt, (uint64_t)shape.variant, (uint64_t)opts.precision, bits(opts.margin),
-                     bits(opts.winding_tol), (uint64_t)opts.flags, (uint64_t)grid, (uint64_t)(uintptr_t)ctx->d_entries, ctx->gen})
+                     bits(opts.winding_tol), (uint64_t)opts.flags, (uint64_t)grid,
+                     (uint64_t)(uintptr_t)b.pending, (uint64_t)b.cap_pending, (uint64_t)(uintptr_t)ctx->d_entries, ctx->gen})
     key = mix(key, v);
   if (!ctx->rb_exec || ctx->rb_key != key) {
     if (ctx->rb_exec) {
