@@ -397,8 +397,8 @@ typedef struct zef_smooth_opts {
    tet edge).  One iteration: x' = x + lambda L(x), then x'' = x' - mu L(x'),
    with L(x)_i = sum over j in N_i of (x_j - x_i) / |N_i|, summed in
    ascending neighbour order in float32 (deterministic); nodes with
-   fixed[i] != 0 (nullable array) do not move.  The iteration loop runs on
-   the device as one CUDA graph with a conditional while-node.
+   fixed[i] != 0 (nullable array) do not move.  The iterations are enqueued
+   in batches that stop on the device.
      nodes      [n_nodes][3] float32, in/out
      tets       [n_tets][4] int32 node indices
      fixed      nullable; [n_nodes] uint8
