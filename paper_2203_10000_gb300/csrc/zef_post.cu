@@ -2,14 +2,12 @@
 // smoothing (Sec. 2.2.1) and inflation towards a compartment surface
 // (Sec. 2.2.2).
 //
-// Both work on the mesh's unique edges, gathered once per call into a CSR
-// adjacency: every tet inserts its six edges into an open-addressing table
-// (an edge's probe starts in the run of slots of its lower node, so the
-// edges of nearby tets, which share nodes with nearby numbers, land in nearby
-// slots), the first insertion of a key counts the edge at both nodes, the degrees are
-// scanned into row offsets, the table's keys are scattered into the rows and
-// each row is sorted, so that every sum over a node's neighbours runs in
-// ascending neighbour order (deterministic results).
+// Both work on the mesh's unique edges, gathered once per call into rows of
+// neighbours per node: blocks take runs of tets, find the unique edges of
+// their run in shared memory and add them to the rows (counted first, then
+// written), and each row is sorted and its repeats dropped, so that every sum
+// over a node's neighbours runs in ascending neighbour order (deterministic
+// results).
 //
 // Smoothing: one iteration is the forward step x' = x + lambda L(x) with a
 // fixed-order reduction of ||x' - x||^2, the backward step x'' = x' - mu L(x'),
@@ -67,9 +65,9 @@ struct Adj {
   unsigned long long *keys;  // open-addressing table of edge keys (lo << 32 | hi)
   unsigned long long mask;   // table size - 1
   int shift;                 // log2 of the slots per node (table size >= n << shift)
-  uint32_t *deg;             // [n + 1] degrees, scanned into row offsets
-  uint32_t *fill;            // [n] scatter cursors
-  int32_t *nbr;              // [2 E] neighbours, rows sorted ascending
+  uint32_t *deg;             // [n + 1] entries counted per node, scanned into row offsets
+  uint32_t *fill;            // [n] scatter cursors, then neighbours per row
+  int32_t *nbr;              // row i: nbr[deg[i]], fill[i] neighbours, ascending
   int64_t n;
   int64_t *words;            // PpWord
 };
@@ -115,6 +113,118 @@ __global__ void __launch_bounds__(256) k_pp_edges(Adj g, const int32_t *tets, in
     }
   }
 }
+
+// ---- edges of runs of tets, each edge once per run
+// A block takes kRunTets consecutive tets.  Their nodes go into a table in
+// shared memory, their edges (pairs of node slots) into another, so that an
+// edge shared inside the run -- most are: refinement appends the children of
+// neighbouring tets together -- is counted or written once, and each node's
+// global counter is incremented once by all of the run's edges at it.  FILL =
+// false counts the entries of every row; FILL = true, on the scanned counts,
+// takes each node's share of its row and writes the neighbours.  A row then
+// holds an edge once per run that has it (k_pp_sort_rows drops the repeats;
+// 14.7 M tets of a refined head: 68 M entries for 44 M neighbours, 10 M
+// (node, run) pairs for 59 M tet corners).  There the passes take 0.58 and
+// 1.24 ms and the rows 0.84; one table of all edges in global memory took
+// 0.35 (clearing 2.1 GB) + 2.25 (93 M compare-and-swaps) + 1.04 (scanning it)
+// + 0.79.
+constexpr int kRunTets = 512;
+constexpr int kRunNodes = 4096;   // node slots: at most 2048 nodes
+constexpr int kRunEdges = 8192;   // edge slots: at most 3072 edges
+constexpr size_t kRunShared = (size_t)(2 * kRunNodes + kRunEdges) * sizeof(uint32_t);
+constexpr uint32_t kNoSlot = 0xffffffffu;
+
+template <bool FILL>
+__global__ void __launch_bounds__(256) k_pp_runs(Adj g, const int32_t *tets, int64_t m, uint32_t *status) {
+  extern __shared__ uint32_t sm[];
+  uint32_t *nkey = sm, *ncnt = sm + kRunNodes, *ekey = sm + 2 * kRunNodes;
+  if (FILL && g.words[PP_BAD]) return;
+  for (int64_t t0 = (int64_t)blockIdx.x * kRunTets; t0 < m; t0 += (int64_t)gridDim.x * kRunTets) {
+    for (int j = threadIdx.x; j < kRunNodes; j += 256) {
+      nkey[j] = kNoSlot;
+      ncnt[j] = 0u;
+    }
+    for (int j = threadIdx.x; j < kRunEdges; j += 256) ekey[j] = kNoSlot;
+    __syncthreads();
+    uint32_t slot[kRunTets / 256][4];
+    bool ok[kRunTets / 256];
+#pragma unroll
+    for (int q = 0; q < kRunTets / 256; ++q) {
+      const int64_t t = t0 + q * 256 + threadIdx.x;
+      ok[q] = t < m;
+      int32_t v[4] = {0, 0, 0, 0};
+      if (ok[q]) {
+        bool bad = false;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          v[k] = tets[4 * t + k];
+          bad |= v[k] < 0 || v[k] >= g.n;
+        }
+        if (bad) {
+          ok[q] = false;
+          atomicOr(status, ST_INVALID);
+          atomicExch((unsigned long long *)(g.words + PP_BAD), 1ull);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        slot[q][k] = 0u;
+        if (!ok[q]) continue;
+        const uint32_t key = (uint32_t)v[k];
+        uint32_t h = (key * 2654435761u) >> 20;
+        for (;;) {  // ends: at most 2048 of the 4096 slots are taken
+          const uint32_t prev = atomicCAS(nkey + h, kNoSlot, key);
+          if (prev == kNoSlot || prev == key) break;
+          h = (h + 1) & (kRunNodes - 1);
+        }
+        slot[q][k] = h;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kRunTets / 256; ++q) {
+      if (!ok[q]) continue;
+#pragma unroll
+      for (int e = 0; e < 6; ++e) {
+        constexpr int kA[6] = {0, 0, 0, 1, 1, 2}, kB[6] = {1, 2, 3, 2, 3, 3};
+        const uint32_t x = slot[q][kA[e]], y = slot[q][kB[e]];
+        if (x == y) continue;  // a repeated node
+        const uint32_t key = (min(x, y) << 12) | max(x, y);
+        uint32_t h = (key * 2654435761u) >> 19;
+        for (;;) {  // ends: at most 3072 of the 8192 slots are taken
+          const uint32_t prev = atomicCAS(ekey + h, kNoSlot, key);
+          if (prev == kNoSlot) {
+            atomicAdd(ncnt + x, 1u);
+            atomicAdd(ncnt + y, 1u);
+            break;
+          }
+          if (prev == key) break;
+          h = (h + 1) & (kRunEdges - 1);
+        }
+      }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < kRunNodes; j += 256) {
+      const uint32_t c = ncnt[j];
+      if (!c) continue;
+      const uint32_t v = nkey[j];
+      if (FILL) ncnt[j] = g.deg[v] + atomicAdd(g.fill + v, c);
+      else atomicAdd(g.deg + v, c);
+    }
+    __syncthreads();
+    if (FILL) {
+      for (int j = threadIdx.x; j < kRunEdges; j += 256) {
+        const uint32_t key = ekey[j];
+        if (key == kNoSlot) continue;
+        const uint32_t x = key >> 12, y = key & (kRunNodes - 1);
+        g.nbr[atomicAdd(ncnt + x, 1u)] = (int32_t)nkey[y];
+        g.nbr[atomicAdd(ncnt + y, 1u)] = (int32_t)nkey[x];
+      }
+      __syncthreads();
+    }
+  }
+}
+static_assert(kRunNodes == 1 << 12 && kRunEdges == 1 << 13, "slot numbers and hash shifts");
 
 // one undirected edge into the table (first insertion counts it at both ends)
 __device__ __forceinline__ void insert_edge(const Adj &g, uint32_t a, uint32_t b) {
@@ -234,22 +344,109 @@ __global__ void __launch_bounds__(256) k_pp_scatter(Adj g) {
   }
 }
 
-// ascending order inside every row (insertion sort; rows hold a few dozen)
-__global__ void __launch_bounds__(256) k_pp_sort_rows(Adj g) {
-  if (g.words[PP_BAD]) return;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-    int32_t *r = g.nbr + g.deg[i];
-    const int cnt = (int)(g.deg[i + 1] - g.deg[i]);
-    for (int k = 1; k < cnt; ++k) {
-      const int32_t v = r[k];
-      int j = k - 1;
-      while (j >= 0 && r[j] > v) {
-        r[j + 1] = r[j];
-        --j;
+// Every row ascending and without repeats; fill[i] becomes its length.  A warp
+// takes 32 consecutive rows, which lie together in memory: they are staged in
+// shared memory (coalesced), one thread per row inserts its entries into the
+// row's sorted, repeat-free prefix there, and the rows go back.  Rows longer
+// than kRowThread, and the rows of a warp that do not fit the stage, are
+// sorted one after the other by the whole warp (places by counting); a row of
+// more than kRowStage / 2 entries by one lane where it is.
+constexpr int kRowThread = 48;
+constexpr int kRowStage = 1536;         // entries per warp
+constexpr int32_t kRepeat = INT32_MAX;  // above every node index (below 2^31 - 1)
+
+__device__ int sort_row_warp(int32_t *r, int cnt, int32_t *buf, int lane) {
+  if (cnt > kRowStage / 2) {
+    int out = 1;
+    if (lane == 0) {
+      for (int k = 1; k < cnt; ++k) {
+        const int32_t v = r[k];
+        int j = k - 1;
+        while (j >= 0 && r[j] > v) {
+          r[j + 1] = r[j];
+          --j;
+        }
+        r[j + 1] = v;
       }
-      r[j + 1] = v;
+      for (int k = 1; k < cnt; ++k)
+        if (r[k] != r[out - 1]) r[out++] = r[k];
+    }
+    return __shfl_sync(0xffffffffu, out, 0);
+  }
+  int32_t *u = buf + kRowStage / 2;
+  for (int j = lane; j < cnt; j += 32) buf[j] = r[j];
+  __syncwarp();
+  int out = 0;
+  for (int j = lane; j < cnt; j += 32) {
+    const int32_t v = buf[j];
+    bool rep = false;
+    for (int q = 0; q < j; ++q) rep |= buf[q] == v;
+    u[j] = rep ? kRepeat : v;
+    out += rep ? 0 : 1;
+  }
+  __syncwarp();
+  for (int j = lane; j < cnt; j += 32) {
+    const int32_t v = u[j];
+    if (v == kRepeat) continue;
+    int place = 0;
+    for (int q = 0; q < cnt; ++q) place += u[q] < v ? 1 : 0;
+    r[place] = v;
+  }
+  __syncwarp();
+  return (int)__reduce_add_sync(0xffffffffu, (uint32_t)out);
+}
+
+__global__ void __launch_bounds__(256) k_pp_sort_rows(Adj g) {
+  extern __shared__ int32_t s_rows[];
+  if (g.words[PP_BAD]) return;
+  const int lane = threadIdx.x & 31;
+  int32_t *buf = s_rows + (threadIdx.x >> 5) * kRowStage;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); i0 < g.n; i0 += step) {
+    const int64_t i = i0 + lane;
+    const uint32_t b0 = g.deg[i0], e0 = g.deg[min(i0 + 32, g.n)];
+    const uint32_t b = i < g.n ? g.deg[i] : e0, e = i < g.n ? g.deg[i + 1] : e0;
+    const int cnt = (int)(e - b), total = (int)(e0 - b0);
+    const bool staged = e0 - b0 <= (uint32_t)kRowStage;
+    const bool mine = staged && cnt <= kRowThread;
+    if (staged) {
+      for (int j = lane; j < total; j += 32) buf[j] = g.nbr[b0 + j];
+      __syncwarp();
+      if (mine) {
+        int32_t *a = buf + (b - b0);
+        int out = 0;
+        for (int k = 0; k < cnt; ++k) {
+          const int32_t v = a[k];
+          int j = out - 1;
+          while (j >= 0 && a[j] > v) --j;
+          if (j >= 0 && a[j] == v) continue;
+          for (int q = out; q > j + 1; --q) a[q] = a[q - 1];
+          a[j + 1] = v;
+          ++out;
+        }
+        if (i < g.n) g.fill[i] = (uint32_t)out;
+      }
+      __syncwarp();
+      for (int j = lane; j < total; j += 32) g.nbr[b0 + j] = buf[j];
+      __syncwarp();
+    }
+    uint32_t rest = __ballot_sync(0xffffffffu, !mine && i < g.n);
+    while (rest) {
+      const int src = __ffs(rest) - 1;
+      rest &= rest - 1;
+      const uint32_t rb = __shfl_sync(0xffffffffu, b, src);
+      const int out = sort_row_warp(g.nbr + rb, __shfl_sync(0xffffffffu, cnt, src), buf, lane);
+      if (lane == src) g.fill[i] = (uint32_t)out;
     }
   }
+}
+
+// rows sorted (one launch)
+zef_status sort_rows(zef_ctx *ctx, const Adj &g) {
+  constexpr size_t smem = (size_t)8 * kRowStage * sizeof(int32_t);
+  CK(cudaFuncSetAttribute(k_pp_sort_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "shared memory");
+  k_pp_sort_rows<<<grid_blocks(ctx, g.n, 256), 256, smem, ctx->stream>>>(g);
+  return ZEF_OK;
 }
 
 // ---- smoothing
@@ -284,7 +481,7 @@ __device__ __forceinline__ double block_sum(double v) {
 
 // p + w sum_j (p_j - p), j the neighbours of node i in ascending order
 __device__ __forceinline__ float4 lap_step(const Adj &g, const float4 *p, int64_t i, float4 c, float weight) {
-  const uint32_t b = g.deg[i], e = g.deg[i + 1];
+  const uint32_t b = g.deg[i], e = b + g.fill[i];
   float a0 = 0.f, a1 = 0.f, a2 = 0.f;
   for (uint32_t k = b; k < e; ++k) {
     const float4 q = p[g.nbr[k]];
@@ -296,19 +493,27 @@ __device__ __forceinline__ float4 lap_step(const Adj &g, const float4 *p, int64_
   return make_float4(fmaf(w, a0, c.x), fmaf(w, a1, c.y), fmaf(w, a2, c.z), 0.f);
 }
 
-// y = x + lambda L(x) (fixed nodes keep x); block sums of |y - x|^2 in a fixed order
+// y = x + lambda L(x) (fixed nodes keep x); block sums of |y - x|^2 in a fixed
+// order.  With xi = 0 only a sum of zero stops the loop, so NORM = false leaves
+// 1 when some node of the block moved, else 0, and does no FP64 work.
+template <bool NORM>
 __global__ void __launch_bounds__(256) k_sm_forward(Smooth s) {
   if (s.g.words[PP_STOP]) return;
   double acc = 0.0;
+  bool moved = false;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < s.g.n; i += (int64_t)gridDim.x * blockDim.x) {
     const float4 c = s.x[i];
     float4 o = c;
     if (!(s.fixed && s.fixed[i])) o = lap_step(s.g, s.x, i, c, s.lambda);
     s.y[i] = o;
-    const double d0 = (double)o.x - c.x, d1 = (double)o.y - c.y, d2 = (double)o.z - c.z;
-    acc += d0 * d0 + d1 * d1 + d2 * d2;
+    if (NORM) {
+      const double d0 = (double)o.x - c.x, d1 = (double)o.y - c.y, d2 = (double)o.z - c.z;
+      acc += d0 * d0 + d1 * d1 + d2 * d2;
+    } else {
+      moved |= o.x != c.x || o.y != c.y || o.z != c.z;  // true for NaN, whose sum is not zero either
+    }
   }
-  const double sum = block_sum(acc);
+  const double sum = NORM ? block_sum(acc) : (__syncthreads_or(moved) ? 1.0 : 0.0);
   if (threadIdx.x == 0) s.partial[blockIdx.x] = sum;
 }
 
@@ -336,16 +541,16 @@ __global__ void __launch_bounds__(256) k_sm_next(Smooth s) {
   if (small || it >= s.max_iters || s.g.words[PP_BAD]) s.g.words[PP_STOP] = 1;
 }
 
-// positions into float4 and their sum of squares (with `off`, the CSR row
-// offsets, only of the nodes that have a neighbour): block sums in a fixed
+// positions into float4 and their sum of squares (with `len`, the rows'
+// lengths, only of the nodes that have a neighbour): block sums in a fixed
 // order, then one block
-__global__ void __launch_bounds__(256) k_sm_pack(const float *x, int64_t n, const uint32_t *off, float4 *out,
+__global__ void __launch_bounds__(256) k_sm_pack(const float *x, int64_t n, const uint32_t *len, float4 *out,
                                                  double *partial) {
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float4 p = make_float4(x[3 * i], x[3 * i + 1], x[3 * i + 2], 0.f);
     out[i] = p;
-    if (!off || off[i + 1] > off[i]) acc += (double)p.x * p.x + (double)p.y * p.y + (double)p.z * p.z;
+    if (!len || len[i]) acc += (double)p.x * p.x + (double)p.y * p.y + (double)p.z * p.z;
   }
   const double sum = block_sum(acc);
   if (threadIdx.x == 0) partial[blockIdx.x] = sum;
@@ -387,7 +592,7 @@ __global__ void __launch_bounds__(256) k_in_flag(Adj g, const unsigned long long
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
     uint32_t f = 0;
     if (mask[i] & bit)
-      for (uint32_t k = g.deg[i]; k < g.deg[i + 1]; ++k)
+      for (uint32_t k = g.deg[i], e = k + g.fill[i]; k < e; ++k)
         if (!(mask[g.nbr[k]] & bit)) {
           f = 1;
           break;
@@ -425,7 +630,7 @@ __global__ void __launch_bounds__(256) k_in_move(Adj g, const float *x, float *o
     const float p0 = x[3 * (int64_t)i] * scale, p1 = x[3 * (int64_t)i + 1] * scale, p2 = x[3 * (int64_t)i + 2] * scale;
     float m0 = 0.f, m1 = 0.f, m2 = 0.f;
     int cnt = 0;
-    for (uint32_t k = g.deg[i]; k < g.deg[i + 1]; ++k) {
+    for (uint32_t k = g.deg[i], e = k + g.fill[i]; k < e; ++k) {
       const int32_t j = g.nbr[k];
       if (mask[j] & bit) continue;
       const float e0 = x[3 * (int64_t)j] - x[3 * (int64_t)i], e1 = x[3 * (int64_t)j + 1] - x[3 * (int64_t)i + 1],
@@ -526,12 +731,16 @@ int slot_shift(int64_t cap, int64_t n) {
   return sh;
 }
 
-// Unique-edge CSR of the tets (buffers 0-4 of pp_buf); synchronizes.
-zef_status build_adjacency(zef_ctx *ctx, const int32_t *tets, int64_t m, int64_t n, Adj *out, int64_t *edges) {
+// Rows of the tets' unique edges (buffers 0-5 of pp_buf); synchronizes.
+// Counting and writing by runs needs no table, but its row offsets (32 bits)
+// count an edge once per run, at most 12 m in all; meshes beyond that take
+// the table of unique edges.
+zef_status build_adjacency(zef_ctx *ctx, const int32_t *tets, int64_t m, int64_t n, Adj *out) {
+  const bool runs = 12 * m <= (int64_t)0xffffffffu;
   int64_t cap = 1024;
-  while (cap < 12 * std::max<int64_t>(m, 1)) cap <<= 1;  // 6 m edge slots, load <= 1/2
+  while (!runs && cap < 12 * std::max<int64_t>(m, 1)) cap <<= 1;  // 6 m edge slots, load <= 1/2
   zef_status st;
-  if ((st = pp_grow(ctx, 0, (size_t)cap * sizeof(unsigned long long)))) return st;
+  if (!runs && (st = pp_grow(ctx, 0, (size_t)cap * sizeof(unsigned long long)))) return st;
   if ((st = pp_grow(ctx, 1, (size_t)(n + 1) * sizeof(uint32_t)))) return st;
   if ((st = pp_grow(ctx, 2, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t)))) return st;
   if ((st = pp_grow(ctx, 4, (size_t)PP_WORDS * sizeof(int64_t)))) return st;
@@ -542,18 +751,26 @@ zef_status build_adjacency(zef_ctx *ctx, const int32_t *tets, int64_t m, int64_t
   g.shift = slot_shift(cap, n);
   g.deg = (uint32_t *)ctx->pp_buf[1];
   g.fill = (uint32_t *)ctx->pp_buf[2];
+  g.nbr = nullptr;
   g.n = n;
   g.words = (int64_t *)ctx->pp_buf[4];
   cudaStream_t s = ctx->stream;
-  CK(cudaMemsetAsync(g.keys, 0xff, (size_t)cap * sizeof(unsigned long long), s), "clear edge table");
   CK(cudaMemsetAsync(g.deg, 0, (size_t)(n + 1) * sizeof(uint32_t), s), "clear degrees");
   CK(cudaMemsetAsync(g.fill, 0, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t), s), "clear cursors");
   k_pp_words<<<1, 32, 0, s>>>(g.words);
-  if (m > 0) k_pp_edges<<<grid_blocks(ctx, m, 256), 256, 0, s>>>(g, tets, m, ctx->d_status);
+  const unsigned run_blocks = (unsigned)std::min<int64_t>((m + kRunTets - 1) / kRunTets, (int64_t)ctx->num_sms * 12);
+  if (runs) {
+    CK(cudaFuncSetAttribute(k_pp_runs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunShared), "shared memory");
+    CK(cudaFuncSetAttribute(k_pp_runs<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunShared), "shared memory");
+    if (m > 0) k_pp_runs<false><<<run_blocks, 256, kRunShared, s>>>(g, tets, m, ctx->d_status);
+  } else {
+    CK(cudaMemsetAsync(g.keys, 0xff, (size_t)cap * sizeof(unsigned long long), s), "clear edge table");
+    k_pp_edges<<<grid_blocks(ctx, m, 256), 256, 0, s>>>(g, tets, m, ctx->d_status);
+  }
   st = scan_exclusive(ctx, g.deg, nullptr, 1, n + 1, nullptr, (uint32_t *)ctx->pp_buf[5]);
   if (st) return st;
   int64_t words[PP_WORDS];
-  uint32_t deg_sum = 0;  // 2 x edges: the scanned degrees' last entry
+  uint32_t deg_sum = 0;  // entries of all rows: the scanned counts' last
   CK(cudaMemcpyAsync(words, g.words, sizeof(words), cudaMemcpyDeviceToHost, s), "read adjacency status");
   CK(cudaMemcpyAsync(&deg_sum, g.deg + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s), "read edge count");
   CK(cudaStreamSynchronize(s), "build adjacency");
@@ -561,11 +778,11 @@ zef_status build_adjacency(zef_ctx *ctx, const int32_t *tets, int64_t m, int64_t
     zef_synchronize(ctx);  // clears the recorded status
     return fail(ctx, ZEF_ERR_INVALID_ARG, "a tet references a node index outside [0, num_nodes)");
   }
-  *edges = (int64_t)deg_sum / 2;
   if ((st = pp_grow(ctx, 3, (size_t)std::max<int64_t>((int64_t)deg_sum, 1) * sizeof(int32_t)))) return st;
   g.nbr = (int32_t *)ctx->pp_buf[3];
-  k_pp_scatter<<<grid_blocks(ctx, cap, 256), 256, 0, s>>>(g);
-  k_pp_sort_rows<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g);
+  if (!runs) k_pp_scatter<<<grid_blocks(ctx, cap, 256), 256, 0, s>>>(g);
+  else if (m > 0) k_pp_runs<true><<<run_blocks, 256, kRunShared, s>>>(g, tets, m, ctx->d_status);
+  if ((st = sort_rows(ctx, g))) return st;
   CK(cudaGetLastError(), "adjacency kernels");
   *out = g;
   return ZEF_OK;
@@ -604,13 +821,14 @@ zef_status smooth_loop(zef_ctx *ctx, float *x, int64_t n, const Adj &g, const ui
   sm.max_iters = o.max_iters;
   sm.partial = partial;
   sm.nblocks = nblocks;
-  k_sm_pack<<<nblocks, threads, 0, s>>>(x, n, boundary_norm ? g.deg : nullptr, sm.x, partial);
+  k_sm_pack<<<nblocks, threads, 0, s>>>(x, n, boundary_norm ? g.fill : nullptr, sm.x, partial);
   k_sm_norm<<<1, threads, 0, s>>>(partial, nblocks, partial + nblocks);
   int batch = o.xi > 0.f ? 1 : 32;
   for (int left = o.max_iters; left > 0;) {
     const int k = std::min(batch, left);
     for (int q = 0; q < k; ++q) {
-      k_sm_forward<<<nblocks, threads, 0, s>>>(sm);
+      if (o.xi > 0.f) k_sm_forward<true><<<nblocks, threads, 0, s>>>(sm);
+      else k_sm_forward<false><<<nblocks, threads, 0, s>>>(sm);
       k_sm_backward<<<nblocks, threads, 0, s>>>(sm);
       k_sm_next<<<1, threads, 0, s>>>(sm);
     }
@@ -684,7 +902,7 @@ zef_status build_surface_adjacency(zef_ctx *ctx, const int32_t *tets, const int3
   if ((st = pp_grow(ctx, 3, (size_t)std::max<int64_t>((int64_t)deg_sum, 1) * sizeof(int32_t)))) return st;
   g.nbr = (int32_t *)ctx->pp_buf[3];
   k_pp_scatter<<<grid_blocks(ctx, cap, 256), 256, 0, s>>>(g);
-  k_pp_sort_rows<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g);
+  if ((st = sort_rows(ctx, g))) return st;
   CK(cudaGetLastError(), "boundary adjacency kernels");
   *out = g;
   return ZEF_OK;
@@ -718,8 +936,7 @@ zef_status taubin_run(zef_ctx *ctx, float *nodes, int64_t n, const int32_t *tets
     }
   }
   Adj g;
-  int64_t edges = 0;
-  if ((st = build_adjacency(ctx, tt, m, n, &g, &edges))) return st;  // synchronizes
+  if ((st = build_adjacency(ctx, tt, m, n, &g))) return st;  // synchronizes
   int64_t words[PP_WORDS] = {0};
   if ((st = smooth_loop(ctx, x, n, g, fx, o, false, words))) return st;
   if (!dn) CK(cudaMemcpy(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost), "copy nodes back");
@@ -797,13 +1014,13 @@ zef_status inflate_run(zef_ctx *ctx, float *nodes, int64_t n, const int32_t *tet
   st = label_points_impl(ctx, x, n, (int32_t *)ctx->pp_buf[12], nullptr, nullptr, nullptr, mask, true);
   if (st) return st;
   Adj g;
-  int64_t edges = 0;
-  if ((st = build_adjacency(ctx, tt, m, n, &g, &edges))) return st;
+  if ((st = build_adjacency(ctx, tt, m, n, &g))) return st;
   // nodes inside with an outside neighbour, listed in index order
   if ((st = pp_grow(ctx, 13, (size_t)(n + 1) * sizeof(uint32_t)))) return st;
   if ((st = pp_grow(ctx, 9, (size_t)n * 3 * sizeof(float)))) return st;
   uint32_t *flag = (uint32_t *)ctx->pp_buf[13];
-  uint32_t *list = (uint32_t *)ctx->pp_buf[2];  // the scatter cursors are free again
+  if ((st = pp_grow(ctx, 14, (size_t)n * sizeof(uint32_t)))) return st;
+  uint32_t *list = (uint32_t *)ctx->pp_buf[14];
   float *out = (float *)ctx->pp_buf[9];
   k_in_flag<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g, mask, row, flag);
   st = scan_exclusive(ctx, flag, nullptr, 1, n, g.words + PP_LISTED, (uint32_t *)ctx->pp_buf[5]);
