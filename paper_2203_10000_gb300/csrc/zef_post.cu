@@ -16,9 +16,10 @@
 // (node i itself belongs to its neighbourhood and adds nothing to the sum).
 //
 // Smoothing of the tissue boundaries (surface variant of Sec. 2.2.1): the
-// tets' faces go into an open-addressing table keyed by their sorted node
-// triple (128-bit compare-and-swap) with the smallest and largest element
-// label of the tets that share them; a face whose two labels differ is a
+// faces whose three nodes each touch more than one element label go into an
+// open-addressing table keyed by their sorted node triple (128-bit
+// compare-and-swap) with the smallest and largest element label of the tets
+// that share them; a face whose two labels differ is a
 // boundary face, and its three edges build the adjacency of the same
 // iteration, so that only the boundary nodes move.
 //
@@ -50,7 +51,7 @@ namespace {
 constexpr unsigned long long kNoKey = ~0ull;
 __constant__ int kEdgeLocal[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
 // words of the post-processing statistics (device)
-enum PpWord { PP_EDGES = 0, PP_BAD, PP_ITER, PP_STOP, PP_LISTED, PP_FACES, PP_FULL, PP_WORDS };
+enum PpWord { PP_CAND = 0, PP_BAD, PP_ITER, PP_STOP, PP_LISTED, PP_FACES, PP_FULL, PP_WORDS };
 
 __device__ __forceinline__ unsigned long long pp_mix(unsigned long long x) {
   x ^= x >> 33;
@@ -273,26 +274,86 @@ __global__ void __launch_bounds__(256) k_sf_clear(FaceTab f) {
   }
 }
 
-// every tet's four faces into the table with the tet's element label
-__global__ void __launch_bounds__(256) k_sf_faces(FaceTab f, const int32_t *tets, const int32_t *labels, int64_t m,
-                                                 int64_t n, int64_t *words, uint32_t *status) {
+// ---- which faces can lie on a boundary
+// A face between two labels has three nodes that both labels touch, so only
+// the faces of such (mixed) nodes go into the table.  Pass 1 leaves some tet's
+// label at every node (whichever store comes last), pass 2 marks the nodes
+// where a tet's label differs from it: exactly the nodes of more than one
+// label.  Pass 3 counts the faces with three marked nodes, for the table's
+// size.
+__device__ __forceinline__ bool load_tet(const int32_t *tets, int64_t t, int64_t n, int32_t (&v)[4]) {
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = tets[4 * t + k];
+    ok &= v[k] >= 0 && v[k] < n;
+  }
+  return ok;
+}
+
+__global__ void __launch_bounds__(256) k_sf_first(const int32_t *tets, const int32_t *labels, int64_t m, int64_t n,
+                                                 int32_t *first, int64_t *words, uint32_t *status) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
     int32_t v[4];
-    bool bad = false;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      v[k] = tets[4 * t + k];
-      bad |= v[k] < 0 || v[k] >= n;
-    }
-    if (bad) {
+    if (!load_tet(tets, t, n, v)) {
       atomicOr(status, ST_INVALID);
       atomicExch((unsigned long long *)(words + PP_BAD), 1ull);
       continue;
     }
     const int32_t lab = labels[t];
 #pragma unroll
+    for (int k = 0; k < 4; ++k)
+      asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(first + v[k]), "r"(lab) : "memory");
+  }
+}
+
+__global__ void __launch_bounds__(256) k_sf_mixed(const int32_t *tets, const int32_t *labels, int64_t m, int64_t n,
+                                                 const int32_t *first, uint8_t *mixed) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
+    int32_t v[4];
+    if (!load_tet(tets, t, n, v)) continue;
+    const int32_t lab = labels[t];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (first[v[k]] != lab) mixed[v[k]] = 1;
+  }
+}
+
+// bits of the tet's mixed nodes
+__device__ __forceinline__ uint32_t mixed_bits(const uint8_t *mixed, const int32_t (&v)[4]) {
+  uint32_t b = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) b |= mixed[v[k]] ? 1u << k : 0u;
+  return b;
+}
+
+__global__ void __launch_bounds__(256) k_sf_count(const int32_t *tets, int64_t m, int64_t n, const uint8_t *mixed,
+                                                 int64_t *words) {
+  uint32_t c = 0;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
+    int32_t v[4];
+    if (!load_tet(tets, t, n, v)) continue;
+    const int k = __popc(mixed_bits(mixed, v));
+    c += k == 4 ? 4u : k == 3 ? 1u : 0u;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long *)(words + PP_CAND), (unsigned long long)c);
+}
+
+// the faces of mixed nodes into the table with their tets' element labels
+__global__ void __launch_bounds__(256) k_sf_faces(FaceTab f, const int32_t *tets, const int32_t *labels, int64_t m,
+                                                 int64_t n, const uint8_t *mixed, int64_t *words) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
+    int32_t v[4];
+    if (!load_tet(tets, t, n, v)) continue;
+    const uint32_t mb = mixed_bits(mixed, v);
+    if (__popc(mb) < 3) continue;
+    const int32_t lab = labels[t];
+#pragma unroll
     for (int q = 0; q < 4; ++q) {
       // face q leaves out vertex 3 - q
+      if ((mb | 1u << (3 - q)) != 0xfu) continue;
       uint32_t a = (uint32_t)v[q == 3 ? 1 : 0], b = (uint32_t)v[q >= 2 ? 2 : 1], c = (uint32_t)v[q >= 1 ? 3 : 2];
       uint32_t lo = min(a, min(b, c)), hi = max(a, max(b, c));
       const uint32_t mid = a ^ b ^ c ^ lo ^ hi;
@@ -320,16 +381,21 @@ __global__ void __launch_bounds__(256) k_sf_faces(FaceTab f, const int32_t *tets
 
 // the boundary faces (two tets, different labels) and their edges
 __global__ void __launch_bounds__(256) k_sf_edges(FaceTab f, Adj g) {
+  uint32_t faces = 0;
   for (unsigned long long s = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; s <= f.mask;
        s += (unsigned long long)gridDim.x * blockDim.x) {
     const unsigned long long klo = f.keys[2 * s];
     if (klo == kNoKey || f.lo[s] == f.hi[s]) continue;
     const uint32_t a = (uint32_t)(klo & 0xffffffffu), b = (uint32_t)(klo >> 32), c = (uint32_t)f.keys[2 * s + 1];
-    atomicAdd((unsigned long long *)(g.words + PP_FACES), 1ull);
+    ++faces;
     insert_edge(g, a, b);
     insert_edge(g, a, c);
     insert_edge(g, b, c);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) faces += __shfl_xor_sync(0xffffffffu, faces, o);
+  if ((threadIdx.x & 31) == 0 && faces)
+    atomicAdd((unsigned long long *)(g.words + PP_FACES), (unsigned long long)faces);
 }
 
 __global__ void __launch_bounds__(256) k_pp_scatter(Adj g) {
@@ -846,27 +912,55 @@ zef_status smooth_loop(zef_ctx *ctx, float *x, int64_t n, const Adj &g, const ui
   return ZEF_OK;
 }
 
-// CSR adjacency of the tissue-boundary faces' edges (buffers 0-5 as
-// build_adjacency, 14-16 for the face table); synchronizes.
+// Rows of the tissue-boundary faces' edges (buffers 0-5 as build_adjacency, 14
+// for the face table, 15 and 16 for the nodes' labels and marks);
+// synchronizes.  14.7 M tets of a refined head with 1.6 M boundary faces:
+// 0.6 + 6.1 ms clearing a table for, and inserting, all 59 M faces, and 4.0 ms
+// scanning it with one counter for all faces, before the faces were chosen by
+// their nodes.
 zef_status build_surface_adjacency(zef_ctx *ctx, const int32_t *tets, const int32_t *labels, int64_t m, int64_t n,
                                    Adj *out, int64_t *faces) {
-  int64_t fcap = 1024;
-  while (fcap < 8 * std::max<int64_t>(m, 1)) fcap <<= 1;  // 4 m face slots, load <= 1/2
-  int64_t cap = 1024;
-  while (cap < 12 * std::max<int64_t>(m, 1)) cap <<= 1;   // boundary edges: far fewer than the tets' 6 m
   zef_status st;
-  if ((st = pp_grow(ctx, 14, (size_t)fcap * 2 * sizeof(unsigned long long)))) return st;
-  if ((st = pp_grow(ctx, 15, (size_t)fcap * sizeof(int32_t)))) return st;
-  if ((st = pp_grow(ctx, 16, (size_t)fcap * sizeof(int32_t)))) return st;
-  if ((st = pp_grow(ctx, 0, (size_t)cap * sizeof(unsigned long long)))) return st;
   if ((st = pp_grow(ctx, 1, (size_t)(n + 1) * sizeof(uint32_t)))) return st;
   if ((st = pp_grow(ctx, 2, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t)))) return st;
   if ((st = pp_grow(ctx, 4, (size_t)PP_WORDS * sizeof(int64_t)))) return st;
   if ((st = pp_grow(ctx, 5, (size_t)((n + 1) / 2048 + 2) * sizeof(uint32_t)))) return st;
+  if ((st = pp_grow(ctx, 15, (size_t)std::max<int64_t>(n, 1) * sizeof(int32_t)))) return st;
+  if ((st = pp_grow(ctx, 16, (size_t)std::max<int64_t>(n, 1)))) return st;
+  int32_t *first = (int32_t *)ctx->pp_buf[15];
+  uint8_t *mixed = (uint8_t *)ctx->pp_buf[16];
+  int64_t *dwords = (int64_t *)ctx->pp_buf[4];
+  cudaStream_t s = ctx->stream;
+  int64_t words[PP_WORDS] = {0};
+  k_pp_words<<<1, 32, 0, s>>>(dwords);
+  if (m > 0) {
+    const int g_t = grid_blocks(ctx, m, 256);
+    CK(cudaMemsetAsync(mixed, 0, (size_t)n, s), "clear node marks");
+    k_sf_first<<<g_t, 256, 0, s>>>(tets, labels, m, n, first, dwords, ctx->d_status);
+    k_sf_mixed<<<g_t, 256, 0, s>>>(tets, labels, m, n, first, mixed);
+    k_sf_count<<<g_t, 256, 0, s>>>(tets, m, n, mixed, dwords);
+    CK(cudaMemcpyAsync(words, dwords, sizeof(words), cudaMemcpyDeviceToHost, s), "read face count");
+    CK(cudaStreamSynchronize(s), "boundary nodes");
+    if (words[PP_BAD]) {
+      zef_synchronize(ctx);  // clears the recorded status
+      return fail(ctx, ZEF_ERR_INVALID_ARG, "a tet references a node index outside [0, num_nodes)");
+    }
+  }
+  const int64_t cand = words[PP_CAND];
+  if (cand == 0) {
+    *faces = 0;
+    return ZEF_OK;
+  }
+  int64_t fcap = 1024;
+  while (fcap < 2 * cand) fcap <<= 1;     // load <= 1/2
+  int64_t cap = 1024;
+  while (cap < 3 * cand) cap <<= 1;       // a boundary face was counted twice: at most 3/2 cand edges, load <= 1/2
+  if ((st = pp_grow(ctx, 14, (size_t)fcap * (2 * sizeof(unsigned long long) + 2 * sizeof(int32_t))))) return st;
+  if ((st = pp_grow(ctx, 0, (size_t)cap * sizeof(unsigned long long)))) return st;
   FaceTab f;
   f.keys = (unsigned long long *)ctx->pp_buf[14];
-  f.lo = (int32_t *)ctx->pp_buf[15];
-  f.hi = (int32_t *)ctx->pp_buf[16];
+  f.lo = (int32_t *)(f.keys + 2 * fcap);
+  f.hi = f.lo + fcap;
   f.mask = (unsigned long long)(fcap - 1);
   Adj g;
   g.keys = (unsigned long long *)ctx->pp_buf[0];
@@ -874,29 +968,21 @@ zef_status build_surface_adjacency(zef_ctx *ctx, const int32_t *tets, const int3
   g.shift = slot_shift(cap, n);
   g.deg = (uint32_t *)ctx->pp_buf[1];
   g.fill = (uint32_t *)ctx->pp_buf[2];
+  g.nbr = nullptr;
   g.n = n;
-  g.words = (int64_t *)ctx->pp_buf[4];
-  cudaStream_t s = ctx->stream;
+  g.words = dwords;
   k_sf_clear<<<grid_blocks(ctx, fcap, 256), 256, 0, s>>>(f);
   CK(cudaMemsetAsync(g.keys, 0xff, (size_t)cap * sizeof(unsigned long long), s), "clear edge table");
   CK(cudaMemsetAsync(g.deg, 0, (size_t)(n + 1) * sizeof(uint32_t), s), "clear degrees");
   CK(cudaMemsetAsync(g.fill, 0, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t), s), "clear cursors");
-  k_pp_words<<<1, 32, 0, s>>>(g.words);
-  if (m > 0) {
-    k_sf_faces<<<grid_blocks(ctx, m, 256), 256, 0, s>>>(f, tets, labels, m, n, g.words, ctx->d_status);
-    k_sf_edges<<<grid_blocks(ctx, fcap, 256), 256, 0, s>>>(f, g);
-  }
+  k_sf_faces<<<grid_blocks(ctx, m, 256), 256, 0, s>>>(f, tets, labels, m, n, mixed, dwords);
+  k_sf_edges<<<grid_blocks(ctx, fcap, 256), 256, 0, s>>>(f, g);
   st = scan_exclusive(ctx, g.deg, nullptr, 1, n + 1, nullptr, (uint32_t *)ctx->pp_buf[5]);
   if (st) return st;
-  int64_t words[PP_WORDS];
   uint32_t deg_sum = 0;
   CK(cudaMemcpyAsync(words, g.words, sizeof(words), cudaMemcpyDeviceToHost, s), "read adjacency status");
   CK(cudaMemcpyAsync(&deg_sum, g.deg + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s), "read edge count");
   CK(cudaStreamSynchronize(s), "build boundary adjacency");
-  if (words[PP_BAD]) {
-    zef_synchronize(ctx);  // clears the recorded status
-    return fail(ctx, ZEF_ERR_INVALID_ARG, "a tet references a node index outside [0, num_nodes)");
-  }
   if (words[PP_FULL]) return fail(ctx, ZEF_ERR_CUDA, "internal: face or edge table full");
   *faces = words[PP_FACES];
   if ((st = pp_grow(ctx, 3, (size_t)std::max<int64_t>((int64_t)deg_sum, 1) * sizeof(int32_t)))) return st;

@@ -1,8 +1,10 @@
-"""Neighbour rows of the post-processing on meshes whose tets are in random
+"""Neighbour rows of the post-processing, and the boundary faces of its
+surface variant, on meshes whose tets are in random
 order (an edge in many runs of tets), in runs of every remainder, with a node
 of several hundred neighbours (rows longer than the staged ones) and with
 repeated nodes: one smoothing step against the FP64 oracle, which builds its
-neighbourhoods from sets."""
+neighbourhoods from sets; boundary smoothing of labelings that make every
+node, or hardly any, a boundary node."""
 import numpy as np
 import pytest
 
@@ -54,3 +56,26 @@ def test_rows_by_one_smoothing_step(zef, name, nodes, tets):
     # a row of d float32 differences summed in order: d 2^-24 of their size each way
     d = max(len(s) for s in nbr)
     assert np.abs(got.cpu().numpy() - p).max() <= 2 * (d + 8) * 2.0 ** -24 * 2 * np.abs(x).max()
+
+
+@pytest.mark.parametrize("kind", ["random", "extremes", "one tet", "halves", "one label"])
+def test_boundary_faces_and_rows(zef, kind):
+    from oracle import postprocess as pp
+    nodes, tets = zs.lattice_5tet(7, 1.0, (0.0, 0.0, 0.0))
+    rng = np.random.default_rng(3)
+    tets = tets[rng.permutation(len(tets))]
+    lab = {"random": rng.integers(-1, 4, len(tets)),
+           "extremes": rng.choice([-2 ** 31, 2 ** 31 - 1], len(tets)),
+           "one tet": (np.arange(len(tets)) == 77) * 5,
+           "halves": (nodes[tets].mean(1)[:, 0] > 3.3) * 9 - 4,
+           "one label": np.full(len(tets), 6)}[kind].astype(np.int32)
+    x = (nodes + 0.1 * rng.standard_normal(nodes.shape)).astype(np.float32)
+    ctx = zef.Context(0)
+    got = torch.from_numpy(x.copy()).cuda()
+    it, faces = ctx.taubin_smooth_surface(got, torch.from_numpy(np.ascontiguousarray(tets)).cuda(),
+                                          torch.from_numpy(lab).cuda(), 0.4, 0.4, 0.0, 3)
+    ctx.close()
+    want, oit, ofaces = pp.taubin_smooth_surface(x, tets, lab, 0.4, 0.4, 0.0, 3)
+    assert (it, faces) == (oit, ofaces)
+    # 2 k half-steps of about 2^-20 of the largest coordinate each
+    assert np.abs(got.cpu().numpy() - want).max() <= 2 * 3 * 2.0 ** -20 * np.abs(x).max()
