@@ -68,18 +68,16 @@ constexpr float kFourPi = 12.5663706143591729539f;
 // block in two bits (0: more than three, see the block's header), and the
 // block's offset in 16-byte words.  Otherwise the winding number (8 bits), or
 // kUnknown.
-constexpr uint32_t kMixed = 0x80000000u;
+constexpr uint32_t kMixed = kCellMixed;
 constexpr uint32_t kUnknown = 0x40000000u;
-constexpr int kChunkShift = 29;
-constexpr uint32_t kOffsetMask = (1u << kChunkShift) - 1u;
+constexpr int kChunkShift = kCellChunkShift;
+constexpr uint32_t kOffsetMask = kCellOffset;
 constexpr int kNoK = -128;  // block header: the anchor's winding number is unknown
 // A block: a header (anchor x, y, z; k in the low 8 bits of w and the number
 // of chunks above), then chunks of kSub entries: kSub first words (a x b, V),
 // kSub second (b x c, error bound), kSub third (c x a, triangle index), so
 // that kSub lanes read 128 bytes at a time.  The last chunk is filled up with
 // entries that the test calls a miss.
-constexpr int kSub = 8;
-constexpr int kChunkWords = 3 * kSub;
 // Every cell is treated as grown by kGrow of its width on each side: a point
 // whose cell index is off by the rounding of (x - lo) * n / extent (at most a
 // few 2^-24 n of a cell, n <= 512) still lies in the grown cell.

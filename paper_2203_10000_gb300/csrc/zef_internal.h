@@ -153,6 +153,14 @@ struct __align__(16) GridComp {
   const float4 *tris;
 };
 static_assert(sizeof(GridComp) == 80, "GridComp is five 16-byte words");
+// Layout of a cell's block (zef_grid.cu): a header word, then chunks of kSub
+// entries of three words each.
+constexpr uint32_t kCellMixed = 0x80000000u;
+constexpr int kCellChunkShift = 29;
+constexpr uint32_t kCellOffset = (1u << kCellChunkShift) - 1u;
+constexpr int kSub = 8;
+constexpr int kChunkWords = 3 * kSub;
+
 // Cell grid over the union box of the surfaces: per cell the rows whose
 // winding number is 1 in all of it and the rows that need their own grid
 // (uint2, or ulonglong2 with more than 32 compartments).

@@ -4,10 +4,10 @@
 //
 // Both work on the mesh's unique edges, gathered once per call into rows of
 // neighbours per node: blocks take runs of tets, find the unique edges of
-// their run in shared memory and add them to the rows (counted first, then
-// written), and each row is sorted and its repeats dropped, so that every sum
-// over a node's neighbours runs in ascending neighbour order (deterministic
-// results).
+// their run in shared memory and leave each node's neighbours in the run as a
+// piece linked to the node; a node's row is its pieces merged, ascending and
+// without repeats, so that every sum over a node's neighbours runs in
+// ascending neighbour order (deterministic results).
 //
 // Smoothing: one iteration is the forward step x' = x + lambda L(x) with a
 // fixed-order reduction of ||x' - x||^2, the backward step x'' = x' - mu L(x'),
@@ -23,11 +23,10 @@
 // boundary face, and its three edges build the adjacency of the same
 // iteration, so that only the boundary nodes move.
 //
-// Inflation: the nodes are labeled (inside bits of every compartment); every
-// node inside compartment c with an outside neighbour is listed, and one warp
-// per listed node intersects each of its crossing edges with c's triangles
-// (lanes split the triangles, a warp minimum keeps the intersection nearest
-// to the inside node); the node moves by zeta t (x_j - x_i) averaged over its
+// Inflation: the nodes are labeled (inside bits of every compartment); the
+// edges from a node inside compartment c to a neighbour outside are listed,
+// eight lanes per edge find its intersection with c's triangles nearest to the
+// inside node, and the node moves by zeta t (x_j - x_i) averaged over its
 // crossing edges, t the edge parameter of that intersection.
 #include <cuda_runtime.h>
 
@@ -51,7 +50,7 @@ namespace {
 constexpr unsigned long long kNoKey = ~0ull;
 __constant__ int kEdgeLocal[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
 // words of the post-processing statistics (device)
-enum PpWord { PP_CAND = 0, PP_BAD, PP_ITER, PP_STOP, PP_LISTED, PP_FACES, PP_FULL, PP_WORDS };
+enum PpWord { PP_CAND = 0, PP_BAD, PP_ITER, PP_STOP, PP_LISTED, PP_FACES, PP_FULL, PP_POOL, PP_ROWS, PP_WORDS };
 
 __device__ __forceinline__ unsigned long long pp_mix(unsigned long long x) {
   x ^= x >> 33;
@@ -66,8 +65,8 @@ struct Adj {
   unsigned long long *keys;  // open-addressing table of edge keys (lo << 32 | hi)
   unsigned long long mask;   // table size - 1
   int shift;                 // log2 of the slots per node (table size >= n << shift)
-  uint32_t *deg;             // [n + 1] entries counted per node, scanned into row offsets
-  uint32_t *fill;            // [n] scatter cursors, then neighbours per row
+  uint32_t *deg;             // [n + 1] row starts (the table's: degrees, scanned)
+  uint32_t *fill;            // [n] neighbours per row (the table's: scatter cursors before)
   int32_t *nbr;              // row i: nbr[deg[i]], fill[i] neighbours, ascending
   int64_t n;
   int64_t *words;            // PpWord
@@ -119,33 +118,35 @@ __global__ void __launch_bounds__(256) k_pp_edges(Adj g, const int32_t *tets, in
 // A block takes kRunTets consecutive tets.  Their nodes go into a table in
 // shared memory, their edges (pairs of node slots) into another, so that an
 // edge shared inside the run -- most are: refinement appends the children of
-// neighbouring tets together -- is counted or written once, and each node's
-// global counter is incremented once by all of the run's edges at it.  FILL =
-// false counts the entries of every row; FILL = true, on the scanned counts,
-// takes each node's share of its row and writes the neighbours.  A row then
-// holds an edge once per run that has it (k_pp_sort_rows drops the repeats;
-// 14.7 M tets of a refined head: 68 M entries for 44 M neighbours, 10 M
-// (node, run) pairs for 59 M tet corners).  There the passes take 0.58 and
-// 1.24 ms and the rows 0.84; one table of all edges in global memory took
-// 0.35 (clearing 2.1 GB) + 2.25 (93 M compare-and-swaps) + 1.04 (scanning it)
-// + 0.79.
-constexpr int kRunTets = 512;
-constexpr int kRunNodes = 4096;   // node slots: at most 2048 nodes
-constexpr int kRunEdges = 8192;   // edge slots: at most 3072 edges
-constexpr size_t kRunShared = (size_t)(2 * kRunNodes + kRunEdges) * sizeof(uint32_t);
+// neighbouring tets together -- is kept once.  The run's neighbours, ordered by
+// node, go to the pool as one contiguous write of pieces (next piece of the
+// node, count, neighbours), each linked into its node's list.
+// 14.7 M tets of a refined head: 71 M neighbours in 11.3 M pieces, for 44 M
+// neighbours without repeats and 59 M tet corners.
+// (256 tets a run keep five blocks on an SM; 512 would leave 68 M in 10.4 M.)
+constexpr int kRunTets = 256;
+constexpr int kRunBits = 11;
+constexpr int kRunNodes = 1 << kRunBits;  // node slots: at most 1024 nodes
+constexpr int kRunEdges = 1 << kRunBits;  // edge slots: at most 1536 edges
+constexpr int kRunPool = 2 * 6 * kRunTets + 2 * 4 * kRunTets;  // words of a run's pieces: 20 a tet
 constexpr uint32_t kNoSlot = 0xffffffffu;
+constexpr uint32_t kNoPiece = 0xffffffffu;
+constexpr size_t kRunShared = (size_t)(2 * kRunNodes + kRunEdges + kRunPool) * sizeof(uint32_t);
 
-template <bool FILL>
-__global__ void __launch_bounds__(256) k_pp_runs(Adj g, const int32_t *tets, int64_t m, uint32_t *status) {
-  extern __shared__ uint32_t sm[];
-  uint32_t *nkey = sm, *ncnt = sm + kRunNodes, *ekey = sm + 2 * kRunNodes;
-  if (FILL && g.words[PP_BAD]) return;
+__global__ void __launch_bounds__(256) k_pp_runs(int64_t n, const int32_t *tets, int64_t m, uint32_t *pool,
+                                                uint32_t *head, int64_t *words, uint32_t *status) {
+  extern __shared__ __align__(16) uint32_t sm[];
+  __shared__ uint32_t s_scan[8];
+  __shared__ uint32_t s_base;
+  uint32_t *nkey = sm, *ncnt = sm + kRunNodes, *ekey = ncnt + kRunNodes, *out = ekey + kRunEdges;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int64_t t0 = (int64_t)blockIdx.x * kRunTets; t0 < m; t0 += (int64_t)gridDim.x * kRunTets) {
-    for (int j = threadIdx.x; j < kRunNodes; j += 256) {
-      nkey[j] = kNoSlot;
-      ncnt[j] = 0u;
+    for (int j = threadIdx.x; j < kRunNodes / 4; j += 256) {
+      reinterpret_cast<uint4 *>(nkey)[j] = make_uint4(kNoSlot, kNoSlot, kNoSlot, kNoSlot);
+      reinterpret_cast<uint4 *>(ncnt)[j] = make_uint4(0u, 0u, 0u, 0u);
     }
-    for (int j = threadIdx.x; j < kRunEdges; j += 256) ekey[j] = kNoSlot;
+    for (int j = threadIdx.x; j < kRunEdges / 4; j += 256)
+      reinterpret_cast<uint4 *>(ekey)[j] = make_uint4(kNoSlot, kNoSlot, kNoSlot, kNoSlot);
     __syncthreads();
     uint32_t slot[kRunTets / 256][4];
     bool ok[kRunTets / 256];
@@ -159,12 +160,12 @@ __global__ void __launch_bounds__(256) k_pp_runs(Adj g, const int32_t *tets, int
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           v[k] = tets[4 * t + k];
-          bad |= v[k] < 0 || v[k] >= g.n;
+          bad |= v[k] < 0 || v[k] >= n;
         }
         if (bad) {
           ok[q] = false;
           atomicOr(status, ST_INVALID);
-          atomicExch((unsigned long long *)(g.words + PP_BAD), 1ull);
+          atomicExch((unsigned long long *)(words + PP_BAD), 1ull);
         }
       }
 #pragma unroll
@@ -172,8 +173,8 @@ __global__ void __launch_bounds__(256) k_pp_runs(Adj g, const int32_t *tets, int
         slot[q][k] = 0u;
         if (!ok[q]) continue;
         const uint32_t key = (uint32_t)v[k];
-        uint32_t h = (key * 2654435761u) >> 20;
-        for (;;) {  // ends: at most 2048 of the 4096 slots are taken
+        uint32_t h = (key * 2654435761u) >> (32 - kRunBits);
+        for (;;) {  // ends: at most half of the slots are taken
           const uint32_t prev = atomicCAS(nkey + h, kNoSlot, key);
           if (prev == kNoSlot || prev == key) break;
           h = (h + 1) & (kRunNodes - 1);
@@ -190,9 +191,9 @@ __global__ void __launch_bounds__(256) k_pp_runs(Adj g, const int32_t *tets, int
         constexpr int kA[6] = {0, 0, 0, 1, 1, 2}, kB[6] = {1, 2, 3, 2, 3, 3};
         const uint32_t x = slot[q][kA[e]], y = slot[q][kB[e]];
         if (x == y) continue;  // a repeated node
-        const uint32_t key = (min(x, y) << 12) | max(x, y);
-        uint32_t h = (key * 2654435761u) >> 19;
-        for (;;) {  // ends: at most 3072 of the 8192 slots are taken
+        const uint32_t key = (min(x, y) << kRunBits) | max(x, y);
+        uint32_t h = (key * 2654435761u) >> (32 - kRunBits);
+        for (;;) {  // ends: at most three quarters of the slots are taken
           const uint32_t prev = atomicCAS(ekey + h, kNoSlot, key);
           if (prev == kNoSlot) {
             atomicAdd(ncnt + x, 1u);
@@ -205,27 +206,55 @@ __global__ void __launch_bounds__(256) k_pp_runs(Adj g, const int32_t *tets, int
       }
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < kRunNodes; j += 256) {
-      const uint32_t c = ncnt[j];
+    // piece offsets inside the run: scan of the slots' piece sizes
+    constexpr int kPer = kRunNodes / 256;
+    const int j0 = threadIdx.x * kPer;
+    uint32_t mine = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t c = ncnt[j0 + k];
+      mine += c ? c + 2u : 0u;
+    }
+    uint32_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_scan[wid] = incl;
+    __syncthreads();
+    uint32_t at = incl - mine, total = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      at += w < wid ? s_scan[w] : 0u;
+      total += s_scan[w];
+    }
+    if (threadIdx.x == 0) s_base = (uint32_t)atomicAdd((unsigned long long *)(words + PP_POOL), (unsigned long long)total);
+    __syncthreads();
+    const uint32_t base = s_base;
+#pragma unroll 4
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t c = ncnt[j0 + k];
       if (!c) continue;
-      const uint32_t v = nkey[j];
-      if (FILL) ncnt[j] = g.deg[v] + atomicAdd(g.fill + v, c);
-      else atomicAdd(g.deg + v, c);
+      out[at] = atomicExch(head + nkey[j0 + k], base + at);
+      out[at + 1] = c;
+      ncnt[j0 + k] = at + 2;  // the write position of the slot's neighbours
+      at += c + 2u;
     }
     __syncthreads();
-    if (FILL) {
-      for (int j = threadIdx.x; j < kRunEdges; j += 256) {
-        const uint32_t key = ekey[j];
-        if (key == kNoSlot) continue;
-        const uint32_t x = key >> 12, y = key & (kRunNodes - 1);
-        g.nbr[atomicAdd(ncnt + x, 1u)] = (int32_t)nkey[y];
-        g.nbr[atomicAdd(ncnt + y, 1u)] = (int32_t)nkey[x];
-      }
-      __syncthreads();
+    for (int j = threadIdx.x; j < kRunEdges; j += 256) {
+      const uint32_t key = ekey[j];
+      if (key == kNoSlot) continue;
+      const uint32_t x = key >> kRunBits, y = key & (kRunNodes - 1);
+      out[atomicAdd(ncnt + x, 1u)] = nkey[y];
+      out[atomicAdd(ncnt + y, 1u)] = nkey[x];
     }
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < total; j += 256) pool[base + j] = out[j];
+    __syncthreads();
   }
 }
-static_assert(kRunNodes == 1 << 12 && kRunEdges == 1 << 13, "slot numbers and hash shifts");
+static_assert(kRunNodes >= 8 * kRunTets && kRunEdges * 3 >= 24 * kRunTets, "the tables never fill up");
 
 // one undirected edge into the table (first insertion counts it at both ends)
 __device__ __forceinline__ void insert_edge(const Adj &g, uint32_t a, uint32_t b) {
@@ -507,6 +536,113 @@ __global__ void __launch_bounds__(256) k_pp_sort_rows(Adj g) {
   }
 }
 
+// Batcher's odd-even merge sort of N values in registers (Knuth, The Art of
+// Computer Programming 3, 5.3.4): N = 64 in 543 exchanges of two instructions,
+// the same for every lane.
+template <int N, int P, int K>
+__device__ __forceinline__ void merge_net(int32_t (&v)[N]) {
+#pragma unroll
+  for (int x = 0; x + K < N; ++x) {
+    constexpr int j0 = K % P;
+    if (x >= j0 && (x - j0) % (2 * K) < K && x / (2 * P) == (x + K) / (2 * P)) {
+      const int32_t a = min(v[x], v[x + K]), b = max(v[x], v[x + K]);
+      v[x] = a;
+      v[x + K] = b;
+    }
+  }
+  if constexpr (K > 1) merge_net<N, P, K / 2>(v);
+  else if constexpr (2 * P < N) merge_net<N, 2 * P, 2 * P>(v);
+}
+
+// Sorts the column of cnt <= N entries (stride 32) and writes it back without
+// repeats; returns what is left.
+template <int N>
+__device__ __forceinline__ int sort_column(int32_t *col, int cnt) {
+  int32_t v[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) v[k] = k < cnt ? col[32 * k] : kRepeat;
+  merge_net<N, 1, 1>(v);
+  int out = 0;
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+    if (v[k] != kRepeat && (k == 0 || v[k] != v[k - 1])) col[32 * out++] = v[k];
+  return out;
+}
+
+// The nodes' rows from their pieces, ascending and without repeats.  A warp
+// takes 32 nodes, one per thread: the pieces go into the thread's column in
+// shared memory (entry k of all lanes side by side: no bank conflicts), are
+// sorted by a network in registers -- an insertion sort in shared memory took
+// three times as long, its steps being dependent and the longest row of the
+// 32 setting the pace -- and the rows go out at a place taken from the row
+// cursor.  Nodes of more than kColumn entries are gathered and sorted one
+// after the other by the whole warp in their place in the rows array (room
+// for the repeats stays unused).
+constexpr int kColumn = 64;
+
+__global__ void __launch_bounds__(256) k_pp_merge(Adj g, const uint32_t *pool, const uint32_t *head) {
+  extern __shared__ int32_t s_rows[];
+  if (g.words[PP_BAD]) return;
+  const int lane = threadIdx.x & 31;
+  int32_t *buf = s_rows + (threadIdx.x >> 5) * (kColumn * 32);
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); i0 < g.n; i0 += step) {
+    const int64_t i = i0 + lane;
+    const uint32_t first = i < g.n ? head[i] : kNoPiece;
+    int cnt = 0;
+    for (uint32_t p = first; p != kNoPiece;) {
+      const uint32_t next = pool[p];
+      const int c = (int)pool[p + 1];
+      if (cnt + c <= kColumn)
+#pragma unroll 4
+        for (int k = 0; k < c; ++k) buf[32 * (cnt + k) + lane] = (int32_t)pool[p + 2 + k];
+      cnt += c;
+      p = next;
+    }
+    const bool mine = cnt <= kColumn;
+    const int longest = (int)__reduce_max_sync(0xffffffffu, (uint32_t)(mine ? cnt : 0));
+    int out = 0;
+    if (longest <= 32) out = sort_column<32>(buf + lane, mine ? cnt : 0);
+    else out = sort_column<64>(buf + lane, mine ? cnt : 0);
+    // places of the rows: the warp's from the cursor, one after the other
+    const int room = mine ? out : cnt;
+    int at = room;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, at, o);
+      if (lane >= o) at += t;
+    }
+    unsigned long long base = 0;
+    if (lane == 31 && at) base = atomicAdd((unsigned long long *)(g.words + PP_ROWS), (unsigned long long)at);
+    base = __shfl_sync(0xffffffffu, base, 31);
+    const uint32_t row = (uint32_t)base + (uint32_t)(at - room);
+    if (mine)
+      for (int k = 0; k < out; ++k) g.nbr[row + k] = buf[32 * k + lane];
+    if (i < g.n) {
+      g.deg[i] = row;
+      if (mine) g.fill[i] = (uint32_t)out;
+    }
+    uint32_t rest = __ballot_sync(0xffffffffu, !mine);
+    while (rest) {
+      const int src = __ffs(rest) - 1;
+      rest &= rest - 1;
+      const uint32_t r0 = __shfl_sync(0xffffffffu, row, src);
+      uint32_t p = __shfl_sync(0xffffffffu, first, src), w = r0;
+      while (p != kNoPiece) {
+        const uint32_t next = pool[p], c = pool[p + 1];
+        for (uint32_t k = lane; k < c; k += 32) g.nbr[w + k] = (int32_t)pool[p + 2 + k];
+        w += c;
+        p = next;
+      }
+      __syncwarp();
+      const int len = sort_row_warp(g.nbr + r0, (int)(w - r0), buf, lane);
+      if (lane == src) g.fill[i] = (uint32_t)len;
+    }
+    __syncwarp();
+  }
+}
+static_assert(kColumn * 32 >= kRowStage, "sort_row_warp's stage");
+
 // rows sorted (one launch)
 zef_status sort_rows(zef_ctx *ctx, const Adj &g) {
   constexpr size_t smem = (size_t)8 * kRowStage * sizeof(int32_t);
@@ -520,8 +656,10 @@ zef_status sort_rows(zef_ctx *ctx, const Adj &g) {
 // one 16-byte read of one sector instead of three 4-byte reads over one or
 // two.  Ten iterations on 3.8 M nodes and 20 M edges: 4.8 ms with packed
 // positions and one thread summing the blocks' partial sums (140 us of each
-// iteration), 2.7 ms now; the neighbour gathers from L2 bound both steps
-// (143 us forward, with the FP64 norm, and 117 us backward).
+// iteration), 2.5 ms now: 120 us a step, bound by the L1's handling of a
+// warp's 32 scattered 16-byte reads (44 M a step).  Rows interleaved by warp,
+// or read four indices at a time, changed the indices' share only (145 and
+// 130 us).
 struct Smooth {
   Adj g;
   float4 *x, *y;           // positions [n]: x current, y after the forward step
@@ -547,15 +685,16 @@ __device__ __forceinline__ double block_sum(double v) {
 
 // p + w sum_j (p_j - p), j the neighbours of node i in ascending order
 __device__ __forceinline__ float4 lap_step(const Adj &g, const float4 *p, int64_t i, float4 c, float weight) {
-  const uint32_t b = g.deg[i], e = b + g.fill[i];
+  const uint32_t len = g.fill[i];
+  const int32_t *r = g.nbr + g.deg[i];
   float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-  for (uint32_t k = b; k < e; ++k) {
-    const float4 q = p[g.nbr[k]];
+  for (uint32_t k = 0; k < len; ++k) {
+    const float4 q = p[r[k]];
     a0 += q.x - c.x;
     a1 += q.y - c.y;
     a2 += q.z - c.z;
   }
-  const float w = weight / (float)(e - b + 1);
+  const float w = weight / (float)(len + 1);
   return make_float4(fmaf(w, a0, c.x), fmaf(w, a1, c.y), fmaf(w, a2, c.z), 0.f);
 }
 
@@ -638,135 +777,184 @@ __global__ void __launch_bounds__(256) k_sm_unpack(const float4 *p, int64_t n, f
   }
 }
 
-// listed nodes in index order from their scanned flags
-__global__ void __launch_bounds__(256) k_in_list(const uint32_t *off, int64_t n, const int64_t *total, uint32_t *list) {
-  const uint32_t tot = (uint32_t)*total;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t nx = (i + 1 < n) ? off[i + 1] : tot;
-    if (nx != off[i]) list[off[i]] = (uint32_t)i;
-  }
-}
-
 __global__ void k_pp_words(int64_t *w) {
   if (threadIdx.x < PP_WORDS) w[threadIdx.x] = 0;
 }
 
 // ---- inflation
-// nodes inside compartment row `row` with a neighbour outside it
-__global__ void __launch_bounds__(256) k_in_flag(Adj g, const unsigned long long *mask, int row, uint32_t *flag) {
+// Crossing edges of every node inside compartment row `row`: the number of its
+// neighbours outside (edges null), then, from the scanned counts, the edges
+// themselves, in ascending neighbour order.
+__global__ void __launch_bounds__(256) k_in_edges(Adj g, const unsigned long long *mask, int row, uint32_t *off,
+                                                 int2 *edges) {
   const unsigned long long bit = 1ull << row;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t f = 0;
-    if (mask[i] & bit)
-      for (uint32_t k = g.deg[i], e = k + g.fill[i]; k < e; ++k)
-        if (!(mask[g.nbr[k]] & bit)) {
-          f = 1;
-          break;
-        }
-    flag[i] = f;
+    uint32_t c = 0;
+    if (mask[i] & bit) {
+      uint32_t at = edges ? off[i] : 0u;
+      for (uint32_t k = g.deg[i], e = k + g.fill[i]; k < e; ++k) {
+        const int32_t j = g.nbr[k];
+        if (mask[j] & bit) continue;
+        if (edges) edges[at++] = make_int2((int)i, j);
+        ++c;
+      }
+    }
+    if (!edges) off[i] = c;
   }
 }
 
-// One warp per listed node: for each crossing edge (ascending neighbour
-// order) the nearest intersection with the compartment's triangles
-// (Moller-Trumbore in FP32 on the scaled coordinates, inclusive by a
-// relative 2^-20 so that an edge through a shared triangle edge still hits),
-// then the averaged move.  The candidates are the
-// triangles of the cap-tree leaves whose box meets the edge's box grown by
-// 2^-10 (lane 0 walks the tree; a triangle the edge meets lies in such a
-// leaf, so the minimum is the one over all triangles); more than kInLeaves
-// such leaves fall back to every triangle.
+// Edge parameter of the nearest intersection of each crossing edge with the
+// compartment's triangles, infinity when there is none (Moller-Trumbore in
+// FP32 on the scaled coordinates, inclusive by a relative 2^-20 so that an
+// edge through a shared triangle edge still hits).  Eight lanes per edge.  The
+// candidates are the triangles listed in the cells of the compartment's grid
+// that the edge's box, grown by 2^-10, meets (a lane per cell): any triangle
+// the edge meets has a point that close to it, whose cell lists the triangle,
+// so the minimum is the one over all triangles.  A compartment without a grid,
+// and an edge whose box meets more than kInCells cells (a mesh far coarser
+// than the surface), take the leaves of the cap tree whose box meets the
+// edge's box (one lane walks the tree); more than kInLeaves of them fall back
+// to every triangle.  900,000 edges of a refined head: 0.30 ms, the chain of
+// reads (word, block, vertices) of each edge; a warp per node, taking one edge
+// after the other, needed 1.35 ms with the tree and 1.14 with the cells.
+constexpr int kInLanes = 8;
 constexpr int kInLeaves = 32;
+constexpr int kInCells = 4096;
 
-__global__ void __launch_bounds__(256) k_in_move(Adj g, const float *x, float *out, const unsigned long long *mask,
-                                                 int row, const uint32_t *pos, const float4 *tris, int tri_cnt,
-                                                 const CapNode *nodes, int root, const int32_t *ctidx, float scale,
-                                                 float zeta) {
-  __shared__ int2 s_leaf[8][kInLeaves];  // per warp: (first position in ctidx, triangles)
-  __shared__ int s_nleaf[8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t listed = g.words[PP_LISTED];
-  const unsigned long long bit = 1ull << row;
+__global__ void __launch_bounds__(256) k_in_hits(const int2 *edges, int64_t n_edges, const float *x, const float4 *tris,
+                                                int tri_cnt, const CapNode *nodes, int root, const int32_t *ctidx,
+                                                float scale, GridComp cells, float *hit) {
+  __shared__ int2 s_leaf[256 / kInLanes][kInLeaves];  // per edge: (first position in ctidx, triangles)
+  const int l = threadIdx.x % kInLanes, slot = threadIdx.x / kInLanes;
+  const uint32_t lanes = ((1u << kInLanes) - 1u) << (threadIdx.x & 31 & ~(kInLanes - 1));
   constexpr float kEps = 9.5367431640625e-07f;  // 2^-20
   constexpr float kBoxMargin = 9.765625e-04f;   // 2^-10
-  for (int64_t w = warp; w < listed; w += nwarps) {
-    const int32_t i = (int32_t)pos[w];
-    const float p0 = x[3 * (int64_t)i] * scale, p1 = x[3 * (int64_t)i + 1] * scale, p2 = x[3 * (int64_t)i + 2] * scale;
-    float m0 = 0.f, m1 = 0.f, m2 = 0.f;
-    int cnt = 0;
-    for (uint32_t k = g.deg[i], e = k + g.fill[i]; k < e; ++k) {
-      const int32_t j = g.nbr[k];
-      if (mask[j] & bit) continue;
-      const float e0 = x[3 * (int64_t)j] - x[3 * (int64_t)i], e1 = x[3 * (int64_t)j + 1] - x[3 * (int64_t)i + 1],
-                  e2 = x[3 * (int64_t)j + 2] - x[3 * (int64_t)i + 2];
-      const float d0 = e0 * scale, d1 = e1 * scale, d2 = e2 * scale;
-      if (lane == 0) {
+  const int64_t step = (int64_t)gridDim.x * (256 / kInLanes);
+  for (int64_t w = (int64_t)blockIdx.x * (256 / kInLanes) + slot; w < n_edges; w += step) {
+    const int64_t i = edges[w].x, j = edges[w].y;
+    const float q[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
+    const float ed[3] = {x[3 * j] - q[0], x[3 * j + 1] - q[1], x[3 * j + 2] - q[2]};
+    const float p0 = q[0] * scale, p1 = q[1] * scale, p2 = q[2] * scale;
+    const float d0 = ed[0] * scale, d1 = ed[1] * scale, d2 = ed[2] * scale;
+    float tmin = INFINITY;
+    auto test = [&](int t) {
+      const float4 A = tris[3 * t], B = tris[3 * t + 1], C = tris[3 * t + 2];
+      const float ax = B.x - A.x, ay = B.y - A.y, az = B.z - A.z;   // edge 1
+      const float bx = C.x - A.x, by = C.y - A.y, bz = C.z - A.z;   // edge 2
+      const float px = d1 * bz - d2 * by, py = d2 * bx - d0 * bz, pz = d0 * by - d1 * bx;
+      const float det = ax * px + ay * py + az * pz;
+      if (det == 0.f) return;
+      const float inv = 1.f / det;
+      const float tx = p0 - A.x, ty = p1 - A.y, tz = p2 - A.z;
+      const float u = (tx * px + ty * py + tz * pz) * inv;
+      if (u < -kEps || u > 1.f + kEps) return;
+      const float qx = ty * az - tz * ay, qy = tz * ax - tx * az, qz = tx * ay - ty * ax;
+      const float v = (d0 * qx + d1 * qy + d2 * qz) * inv;
+      if (v < -kEps || u + v > 1.f + kEps) return;
+      const float tt = (bx * qx + by * qy + bz * qz) * inv;
+      if (tt >= 0.f && tt <= 1.f + kEps) tmin = fminf(tmin, tt);
+    };
+    int c0[3] = {0, 0, 0}, cn[3] = {0, 0, 0};
+    int64_t total = kInCells + 1;  // cells the edge's box meets
+    if (cells.words) {
+      const float grow = kBoxMargin / scale;  // a power of two
+      bool miss = false;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const float lo = fminf(q[d], q[d] + ed[d]) - grow, hi = fmaxf(q[d], q[d] + ed[d]) + grow;
+        miss |= hi < cells.lo[d] || lo > cells.hi[d];
+        c0[d] = min(max((int)((fmaxf(lo, cells.lo[d]) - cells.lo[d]) * cells.inv[d]), 0), cells.n[d] - 1);
+        cn[d] = min(max((int)((fminf(hi, cells.hi[d]) - cells.lo[d]) * cells.inv[d]), 0), cells.n[d] - 1) - c0[d] + 1;
+      }
+      total = miss ? 0 : (int64_t)cn[0] * cn[1] * cn[2];
+    }
+    if (total <= kInCells) {
+      for (int c = l; c < (int)total; c += kInLanes) {
+        const int cx = c0[0] + c % cn[0], cy = c0[1] + c / cn[0] % cn[1], cz = c0[2] + c / cn[0] / cn[1];
+        const uint32_t word = cells.words[((int64_t)cz * cells.n[1] + cy) * cells.n[0] + cx];
+        if (!(word & kCellMixed)) continue;
+        const float4 *block = cells.blocks + (word & kCellOffset);
+        const int entries = (int)(__float_as_uint(block[0].w) >> 8) * kSub;
+        for (int e = 0; e < entries; ++e) {
+          const int t = __float_as_int(block[1 + e / kSub * kChunkWords + 2 * kSub + e % kSub].w);
+          if (t >= 0) test(t);
+        }
+      }
+    } else {
+      int nl = 0;
+      if (l == 0) {
         const float lo0 = fminf(p0, p0 + d0) - kBoxMargin, hi0 = fmaxf(p0, p0 + d0) + kBoxMargin;
         const float lo1 = fminf(p1, p1 + d1) - kBoxMargin, hi1 = fmaxf(p1, p1 + d1) + kBoxMargin;
         const float lo2 = fminf(p2, p2 + d2) - kBoxMargin, hi2 = fmaxf(p2, p2 + d2) + kBoxMargin;
-        int nl = 0;
         // pre-order walk without a stack: descend to i + 1, or continue at skip
         const int end = nodes[root].skip;
-        for (int q = root; q != end;) {
-          const CapNode nd = nodes[q];
+        for (int k = root; k != end;) {
+          const CapNode nd = nodes[k];
           if (nd.hi[0] < lo0 || nd.lo[0] > hi0 || nd.hi[1] < lo1 || nd.lo[1] > hi1 || nd.hi[2] < lo2 ||
               nd.lo[2] > hi2) {
-            q = nd.skip;
+            k = nd.skip;
           } else if (nd.left < 0) {
-            if (nl < kInLeaves) s_leaf[wid][nl] = make_int2(nd.tri_begin, nd.leaf_tris);
+            if (nl < kInLeaves) s_leaf[slot][nl] = make_int2(nd.tri_begin, nd.leaf_tris);
             ++nl;
-            q = nd.skip;
+            k = nd.skip;
           } else {
-            ++q;
+            ++k;
           }
         }
-        s_nleaf[wid] = nl;
       }
-      __syncwarp();
-      const int nl = s_nleaf[wid];
+      nl = __shfl_sync(lanes, nl, 0, kInLanes);
+      __syncwarp(lanes);
       const bool all = nl > kInLeaves;
-      const int nsrc = all ? 1 : nl;
-      float tmin = INFINITY;
-      for (int l = 0; l < nsrc; ++l) {
-        const int2 L = all ? make_int2(0, tri_cnt) : s_leaf[wid][l];
-        for (int q = lane; q < L.y; q += 32) {
-          const int t = all ? q : ctidx[L.x + q];
-          const float4 A = tris[3 * t], B = tris[3 * t + 1], C = tris[3 * t + 2];
-          const float ax = B.x - A.x, ay = B.y - A.y, az = B.z - A.z;   // edge 1
-          const float bx = C.x - A.x, by = C.y - A.y, bz = C.z - A.z;   // edge 2
-          const float px = d1 * bz - d2 * by, py = d2 * bx - d0 * bz, pz = d0 * by - d1 * bx;
-          const float det = ax * px + ay * py + az * pz;
-          if (det == 0.f) continue;
-          const float inv = 1.f / det;
-          const float tx = p0 - A.x, ty = p1 - A.y, tz = p2 - A.z;
-          const float u = (tx * px + ty * py + tz * pz) * inv;
-          if (u < -kEps || u > 1.f + kEps) continue;
-          const float qx = ty * az - tz * ay, qy = tz * ax - tx * az, qz = tx * ay - ty * ax;
-          const float v = (d0 * qx + d1 * qy + d2 * qz) * inv;
-          if (v < -kEps || u + v > 1.f + kEps) continue;
-          const float tt = (bx * qx + by * qy + bz * qz) * inv;
-          if (tt >= 0.f && tt <= 1.f + kEps) tmin = fminf(tmin, tt);
-        }
+      for (int s = 0; s < (all ? 1 : nl); ++s) {
+        const int2 L = all ? make_int2(0, tri_cnt) : s_leaf[slot][s];
+        for (int k = l; k < L.y; k += kInLanes) test(all ? k : ctidx[L.x + k]);
       }
-      __syncwarp();  // lane 0 rewrites the leaf list for the next edge
+      __syncwarp(lanes);  // the leaf list is rewritten for the next edge
+    }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) tmin = fminf(tmin, __shfl_xor_sync(0xffffffffu, tmin, o));
-      if (tmin < INFINITY) {
-        const float tc = fminf(tmin, 1.f);
-        m0 = fmaf(zeta * tc, e0, m0);
-        m1 = fmaf(zeta * tc, e1, m1);
-        m2 = fmaf(zeta * tc, e2, m2);
-        ++cnt;
-      }
+    for (int o = kInLanes / 2; o > 0; o >>= 1) tmin = fminf(tmin, __shfl_xor_sync(lanes, tmin, o));
+    if (l == 0) hit[w] = tmin;
+  }
+}
+
+// Moves of the nodes with an intersection, averaged over their crossing edges
+// in ascending neighbour order.
+__global__ void __launch_bounds__(256) k_in_move(Adj g, const uint32_t *off, int64_t n_edges, const int2 *edges,
+                                                const float *hit, float *x, float4 *moved, float zeta) {
+  uint32_t count = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = off[i], e = i + 1 < g.n ? (int64_t)off[i + 1] : n_edges;
+    float m0 = 0.f, m1 = 0.f, m2 = 0.f;
+    int cnt = 0;
+    for (int64_t k = b; k < e; ++k) {
+      if (!(hit[k] < INFINITY)) continue;
+      const int64_t j = edges[k].y;
+      const float tc = fminf(hit[k], 1.f);
+      m0 = fmaf(zeta * tc, x[3 * j] - x[3 * i], m0);
+      m1 = fmaf(zeta * tc, x[3 * j + 1] - x[3 * i + 1], m1);
+      m2 = fmaf(zeta * tc, x[3 * j + 2] - x[3 * i + 2], m2);
+      ++cnt;
     }
-    if (lane == 0 && cnt > 0) {
-      out[3 * (int64_t)i] = x[3 * (int64_t)i] + m0 / (float)cnt;
-      out[3 * (int64_t)i + 1] = x[3 * (int64_t)i + 1] + m1 / (float)cnt;
-      out[3 * (int64_t)i + 2] = x[3 * (int64_t)i + 2] + m2 / (float)cnt;
-      atomicAdd((unsigned long long *)(g.words + PP_STOP), 1ull);  // moved nodes
-    }
+    if (e > b) moved[b] = make_float4(x[3 * i] + m0 / (float)cnt, x[3 * i + 1] + m1 / (float)cnt,
+                                      x[3 * i + 2] + m2 / (float)cnt, cnt > 0 ? 1.f : 0.f);
+    count += cnt > 0 ? 1u : 0u;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
+  if ((threadIdx.x & 31) == 0 && count) atomicAdd((unsigned long long *)(g.words + PP_STOP), (unsigned long long)count);
+}
+
+// the moved nodes' positions (after every move has been computed from the old ones)
+__global__ void __launch_bounds__(256) k_in_store(int64_t n, const uint32_t *off, int64_t n_edges, const float4 *moved,
+                                                 float *x) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = off[i], e = i + 1 < n ? (int64_t)off[i + 1] : n_edges;
+    if (e == b) continue;
+    const float4 p = moved[b];
+    if (p.w == 0.f) continue;
+    x[3 * i] = p.x;
+    x[3 * i + 1] = p.y;
+    x[3 * i + 2] = p.z;
   }
 }
 
@@ -797,20 +985,23 @@ int slot_shift(int64_t cap, int64_t n) {
   return sh;
 }
 
-// Rows of the tets' unique edges (buffers 0-5 of pp_buf); synchronizes.
-// Counting and writing by runs needs no table, but its row offsets (32 bits)
-// count an edge once per run, at most 12 m in all; meshes beyond that take
-// the table of unique edges.
+// Rows of the tets' unique edges (buffers 0-5 of pp_buf); synchronizes.  The
+// pool's offsets have 32 bits and a run may need 20 words per tet; meshes
+// beyond that take the table of unique edges (12 to 24 slots of 8 bytes per
+// tet to clear, to fill with one swap per tet edge and to scan: 4.4 ms where
+// the pieces take 1.8, 14.7 M tets).
 zef_status build_adjacency(zef_ctx *ctx, const int32_t *tets, int64_t m, int64_t n, Adj *out) {
-  const bool runs = 12 * m <= (int64_t)0xffffffffu;
+  const int64_t runs = (m + kRunTets - 1) / kRunTets;
+  const bool pieces = runs * kRunPool < (int64_t)kNoPiece;
   int64_t cap = 1024;
-  while (!runs && cap < 12 * std::max<int64_t>(m, 1)) cap <<= 1;  // 6 m edge slots, load <= 1/2
+  while (!pieces && cap < 12 * std::max<int64_t>(m, 1)) cap <<= 1;  // 6 m edge slots, load <= 1/2
   zef_status st;
-  if (!runs && (st = pp_grow(ctx, 0, (size_t)cap * sizeof(unsigned long long)))) return st;
+  if ((st = pp_grow(ctx, 0, pieces ? (size_t)std::max<int64_t>(runs, 1) * kRunPool * sizeof(uint32_t)
+                                   : (size_t)cap * sizeof(unsigned long long)))) return st;
   if ((st = pp_grow(ctx, 1, (size_t)(n + 1) * sizeof(uint32_t)))) return st;
   if ((st = pp_grow(ctx, 2, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t)))) return st;
   if ((st = pp_grow(ctx, 4, (size_t)PP_WORDS * sizeof(int64_t)))) return st;
-  if ((st = pp_grow(ctx, 5, (size_t)((n + 1) / 2048 + 2) * sizeof(uint32_t)))) return st;
+  if ((st = pp_grow(ctx, 5, (size_t)std::max<int64_t>((n + 1) / 2048 + 2, n) * sizeof(uint32_t)))) return st;
   Adj g;
   g.keys = (unsigned long long *)ctx->pp_buf[0];
   g.mask = (unsigned long long)(cap - 1);
@@ -821,34 +1012,43 @@ zef_status build_adjacency(zef_ctx *ctx, const int32_t *tets, int64_t m, int64_t
   g.n = n;
   g.words = (int64_t *)ctx->pp_buf[4];
   cudaStream_t s = ctx->stream;
-  CK(cudaMemsetAsync(g.deg, 0, (size_t)(n + 1) * sizeof(uint32_t), s), "clear degrees");
-  CK(cudaMemsetAsync(g.fill, 0, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t), s), "clear cursors");
+  uint32_t *pool = (uint32_t *)ctx->pp_buf[0], *head = (uint32_t *)ctx->pp_buf[5];
   k_pp_words<<<1, 32, 0, s>>>(g.words);
-  const unsigned run_blocks = (unsigned)std::min<int64_t>((m + kRunTets - 1) / kRunTets, (int64_t)ctx->num_sms * 12);
-  if (runs) {
-    CK(cudaFuncSetAttribute(k_pp_runs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunShared), "shared memory");
-    CK(cudaFuncSetAttribute(k_pp_runs<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunShared), "shared memory");
-    if (m > 0) k_pp_runs<false><<<run_blocks, 256, kRunShared, s>>>(g, tets, m, ctx->d_status);
+  int64_t words[PP_WORDS];
+  uint32_t deg_sum = 0;
+  if (pieces) {
+    CK(cudaMemsetAsync(head, 0xff, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t), s), "clear piece lists");
+    CK(cudaFuncSetAttribute(k_pp_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunShared), "shared memory");
+    if (m > 0)
+      k_pp_runs<<<(unsigned)std::min<int64_t>(runs, (int64_t)ctx->num_sms * 12), 256, kRunShared, s>>>(
+          n, tets, m, pool, head, g.words, ctx->d_status);
   } else {
+    CK(cudaMemsetAsync(g.deg, 0, (size_t)(n + 1) * sizeof(uint32_t), s), "clear degrees");
+    CK(cudaMemsetAsync(g.fill, 0, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t), s), "clear cursors");
     CK(cudaMemsetAsync(g.keys, 0xff, (size_t)cap * sizeof(unsigned long long), s), "clear edge table");
     k_pp_edges<<<grid_blocks(ctx, m, 256), 256, 0, s>>>(g, tets, m, ctx->d_status);
+    st = scan_exclusive(ctx, g.deg, nullptr, 1, n + 1, nullptr, (uint32_t *)ctx->pp_buf[5]);
+    if (st) return st;
+    CK(cudaMemcpyAsync(&deg_sum, g.deg + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s), "read edge count");
   }
-  st = scan_exclusive(ctx, g.deg, nullptr, 1, n + 1, nullptr, (uint32_t *)ctx->pp_buf[5]);
-  if (st) return st;
-  int64_t words[PP_WORDS];
-  uint32_t deg_sum = 0;  // entries of all rows: the scanned counts' last
   CK(cudaMemcpyAsync(words, g.words, sizeof(words), cudaMemcpyDeviceToHost, s), "read adjacency status");
-  CK(cudaMemcpyAsync(&deg_sum, g.deg + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s), "read edge count");
   CK(cudaStreamSynchronize(s), "build adjacency");
   if (words[PP_BAD]) {
     zef_synchronize(ctx);  // clears the recorded status
     return fail(ctx, ZEF_ERR_INVALID_ARG, "a tet references a node index outside [0, num_nodes)");
   }
-  if ((st = pp_grow(ctx, 3, (size_t)std::max<int64_t>((int64_t)deg_sum, 1) * sizeof(int32_t)))) return st;
+  // the rows hold at most the pool's neighbours
+  const int64_t entries = pieces ? words[PP_POOL] : (int64_t)deg_sum;
+  if ((st = pp_grow(ctx, 3, (size_t)std::max<int64_t>(entries, 1) * sizeof(int32_t)))) return st;
   g.nbr = (int32_t *)ctx->pp_buf[3];
-  if (!runs) k_pp_scatter<<<grid_blocks(ctx, cap, 256), 256, 0, s>>>(g);
-  else if (m > 0) k_pp_runs<true><<<run_blocks, 256, kRunShared, s>>>(g, tets, m, ctx->d_status);
-  if ((st = sort_rows(ctx, g))) return st;
+  if (pieces) {
+    constexpr size_t smem = (size_t)8 * kColumn * 32 * sizeof(int32_t);
+    CK(cudaFuncSetAttribute(k_pp_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "shared memory");
+    k_pp_merge<<<grid_blocks(ctx, n, 256), 256, smem, s>>>(g, pool, head);
+  } else {
+    k_pp_scatter<<<grid_blocks(ctx, cap, 256), 256, 0, s>>>(g);
+    if ((st = sort_rows(ctx, g))) return st;
+  }
   CK(cudaGetLastError(), "adjacency kernels");
   *out = g;
   return ZEF_OK;
@@ -1101,27 +1301,48 @@ zef_status inflate_run(zef_ctx *ctx, float *nodes, int64_t n, const int32_t *tet
   if (st) return st;
   Adj g;
   if ((st = build_adjacency(ctx, tt, m, n, &g))) return st;
-  // nodes inside with an outside neighbour, listed in index order
+  // the crossing edges, by node
   if ((st = pp_grow(ctx, 13, (size_t)(n + 1) * sizeof(uint32_t)))) return st;
-  if ((st = pp_grow(ctx, 9, (size_t)n * 3 * sizeof(float)))) return st;
-  uint32_t *flag = (uint32_t *)ctx->pp_buf[13];
-  if ((st = pp_grow(ctx, 14, (size_t)n * sizeof(uint32_t)))) return st;
-  uint32_t *list = (uint32_t *)ctx->pp_buf[14];
-  float *out = (float *)ctx->pp_buf[9];
-  k_in_flag<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g, mask, row, flag);
-  st = scan_exclusive(ctx, flag, nullptr, 1, n, g.words + PP_LISTED, (uint32_t *)ctx->pp_buf[5]);
+  uint32_t *off = (uint32_t *)ctx->pp_buf[13];
+  k_in_edges<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g, mask, row, off, nullptr);
+  st = scan_exclusive(ctx, off, nullptr, 1, n, g.words + PP_LISTED, (uint32_t *)ctx->pp_buf[5]);
   if (st) return st;
-  k_in_list<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(flag, n, g.words + PP_LISTED, list);
-  CK(cudaMemcpyAsync(out, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToDevice, s), "copy positions");
+  int64_t words[PP_WORDS];
+  CK(cudaMemcpyAsync(words, g.words, sizeof(words), cudaMemcpyDeviceToHost, s), "read crossing edges");
+  CK(cudaStreamSynchronize(s), "crossing edges");
+  const int64_t crossing = words[PP_LISTED];
+  if (crossing == 0) {
+    if (!dn) CK(cudaMemcpy(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost), "copy nodes back");
+    return zef_synchronize(ctx);
+  }
+  // edges, their hits, the moved positions (at each node's first edge)
+  if ((st = pp_grow(ctx, 14, (size_t)crossing * sizeof(int2)))) return st;
+  if ((st = pp_grow(ctx, 15, (size_t)crossing * sizeof(float)))) return st;
+  if ((st = pp_grow(ctx, 9, (size_t)crossing * sizeof(float4)))) return st;
+  int2 *edges = (int2 *)ctx->pp_buf[14];
+  float *hit = (float *)ctx->pp_buf[15];
+  float4 *out = (float4 *)ctx->pp_buf[9];
+  k_in_edges<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g, mask, row, off, edges);
   CK(cudaMemsetAsync(g.words + PP_STOP, 0, sizeof(int64_t), s), "clear moved count");
   const CompHost &c = ctx->comps[(size_t)ci];
-  // one warp per listed node; the grid covers the node count at most
-  k_in_move<<<grid_blocks(ctx, n * 32, 256), 256, 0, s>>>(g, x, out, mask, row, list, ctx->d_tris + c.tri_off * 3,
-                                                          (int)c.nt, ctx->d_nodes, c.cap_root, ctx->d_ctidx,
-                                                          ctx->scale, zeta);
-  CK(cudaGetLastError(), "k_in_move");
-  int64_t words[PP_WORDS];
-  CK(cudaMemcpyAsync(x, out, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToDevice, s), "write positions");
+  GridComp cells = {};
+  if ((size_t)ci < ctx->grids.size() && ctx->grids[(size_t)ci].usable) {
+    const CompGrid &cg = ctx->grids[(size_t)ci];
+    for (int k = 0; k < 3; ++k) {
+      cells.lo[k] = c.lo[k];
+      cells.hi[k] = c.hi[k];
+      cells.inv[k] = cg.inv[k];
+      cells.n[k] = cg.n[k];
+    }
+    cells.words = cg.words;
+    cells.blocks = cg.blocks;
+  }
+  k_in_hits<<<grid_blocks(ctx, crossing * kInLanes, 256), 256, 0, s>>>(
+      edges, crossing, x, ctx->d_tris + c.tri_off * 3, (int)c.nt, ctx->d_nodes, c.cap_root, ctx->d_ctidx, ctx->scale,
+      cells, hit);
+  k_in_move<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g, off, crossing, edges, hit, x, out, zeta);
+  k_in_store<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(n, off, crossing, out, x);
+  CK(cudaGetLastError(), "inflation kernels");
   if (!dn) CK(cudaMemcpyAsync(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost, s), "copy nodes back");
   CK(cudaMemcpyAsync(words, g.words, sizeof(words), cudaMemcpyDeviceToHost, s), "read moved count");
   CK(cudaStreamSynchronize(s), "inflation");

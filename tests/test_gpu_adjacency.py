@@ -28,7 +28,7 @@ def _meshes():
     rng = np.random.default_rng(5)
     yield "lattice", nodes, tets
     yield "shuffled", nodes, tets[rng.permutation(len(tets))]
-    for k in (1, 511, 512, 513, 1025):
+    for k in (1, 255, 256, 257, 513):
         yield f"{k} tets", nodes, tets[rng.permutation(len(tets))[:k]]
     # a fan: node 0 joined to hundreds of others (any tets will do for the rows)
     pts = rng.standard_normal((700, 3)).astype(np.float32)
@@ -79,3 +79,21 @@ def test_boundary_faces_and_rows(zef, kind):
     assert (it, faces) == (oit, ofaces)
     # 2 k half-steps of about 2^-20 of the largest coordinate each
     assert np.abs(got.cpu().numpy() - want).max() <= 2 * 3 * 2.0 ** -20 * np.abs(x).max()
+
+
+@pytest.mark.parametrize("cells,freq", [(3, 24), (9, 24), (24, 6), (17, 2)])
+def test_inflation_by_cells_and_by_tree(zef, cells, freq):
+    """Edges from a tenth of a grid cell to longer than thousands of cells
+    (left to the cap tree) against the oracle's test of every triangle."""
+    from oracle import postprocess as pp
+    u, t = zs.geodesic_sphere(freq)
+    surf = zs.Surface(1, "s", (u * [1.0, 0.8, 0.9]).astype(np.float32), t.astype(np.int32))
+    nodes, tets = zs.lattice_5tet(cells, 2.4 / cells, (-1.21, -1.19, -1.2))
+    ctx = zef.Context(0)
+    ctx.add_compartment(1, surf.verts, surf.tris)
+    got = torch.from_numpy(nodes.copy()).cuda()
+    moved = ctx.inflate(got, torch.from_numpy(tets).cuda(), 1, 0.1)
+    ctx.close()
+    want, omoved = pp.inflate(nodes, tets, surf, 0.1)
+    assert moved == omoved and moved > 0
+    assert np.abs(got.cpu().numpy() - want).max() <= 1e-6 * np.abs(nodes).max()
