@@ -2,7 +2,7 @@
 // smoothing (Sec. 2.2.1) and inflation towards a compartment surface
 // (Sec. 2.2.2).
 //
-// Both work on the mesh's unique edges, gathered once per call into rows of
+// Smoothing works on the mesh's unique edges, gathered once per call into rows of
 // neighbours per node: blocks take runs of tets, find the unique edges of
 // their run in shared memory and leave each node's neighbours in the run as a
 // piece linked to the node; a node's row is its pieces merged, ascending and
@@ -24,8 +24,8 @@
 // iteration, so that only the boundary nodes move.
 //
 // Inflation: the nodes are labeled (inside bits of every compartment); the
-// edges from a node inside compartment c to a neighbour outside are listed,
-// eight lanes per edge find its intersection with c's triangles nearest to the
+// edges from a node inside compartment c to a node outside are gathered from
+// the tets through a table of that size and listed by node, eight lanes per edge find its intersection with c's triangles nearest to the
 // inside node, and the node moves by zeta t (x_j - x_i) averaged over its
 // crossing edges, t the edge parameter of that intersection.
 #include <cuda_runtime.h>
@@ -50,7 +50,7 @@ namespace {
 constexpr unsigned long long kNoKey = ~0ull;
 __constant__ int kEdgeLocal[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
 // words of the post-processing statistics (device)
-enum PpWord { PP_CAND = 0, PP_BAD, PP_ITER, PP_STOP, PP_LISTED, PP_FACES, PP_FULL, PP_POOL, PP_ROWS, PP_WORDS };
+enum PpWord { PP_CAND = 0, PP_BAD, PP_ITER, PP_STOP, PP_FACES, PP_FULL, PP_POOL, PP_ROWS, PP_WORDS };
 
 __device__ __forceinline__ unsigned long long pp_mix(unsigned long long x) {
   x ^= x >> 33;
@@ -782,24 +782,92 @@ __global__ void k_pp_words(int64_t *w) {
 }
 
 // ---- inflation
-// Crossing edges of every node inside compartment row `row`: the number of its
-// neighbours outside (edges null), then, from the scanned counts, the edges
-// themselves, in ascending neighbour order.
-__global__ void __launch_bounds__(256) k_in_edges(Adj g, const unsigned long long *mask, int row, uint32_t *off,
-                                                 int2 *edges) {
-  const unsigned long long bit = 1ull << row;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t c = 0;
-    if (mask[i] & bit) {
-      uint32_t at = edges ? off[i] : 0u;
-      for (uint32_t k = g.deg[i], e = k + g.fill[i]; k < e; ++k) {
-        const int32_t j = g.nbr[k];
-        if (mask[j] & bit) continue;
-        if (edges) edges[at++] = make_int2((int)i, j);
-        ++c;
-      }
+// ---- crossing edges: (inside node, outside node) pairs of the tets, each once
+__global__ void __launch_bounds__(256) k_in_bits(const unsigned long long *mask, int row, int64_t n, uint8_t *inside) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    inside[i] = (uint8_t)(mask[i] >> row & 1ull);
+}
+
+__device__ __forceinline__ uint32_t inside_bits(const uint8_t *inside, const int32_t (&v)[4]) {
+  uint32_t b = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) b |= inside[v[k]] ? 1u << k : 0u;
+  return b;
+}
+
+// their number with repeats, for the table's size
+__global__ void __launch_bounds__(256) k_in_count(const int32_t *tets, int64_t m, int64_t n, const uint8_t *inside,
+                                                 int64_t *words, uint32_t *status) {
+  uint32_t c = 0;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
+    int32_t v[4];
+    if (!load_tet(tets, t, n, v)) {
+      atomicOr(status, ST_INVALID);
+      atomicExch((unsigned long long *)(words + PP_BAD), 1ull);
+      continue;
     }
-    if (!edges) off[i] = c;
+    const uint32_t k = __popc(inside_bits(inside, v));
+    c += k * (4u - k);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long *)(words + PP_CAND), (unsigned long long)c);
+}
+
+// into the table (more slots than pairs); a pair's first insertion counts it
+// at the inside node
+__global__ void __launch_bounds__(256) k_in_insert(const int32_t *tets, int64_t m, int64_t n, const uint8_t *inside,
+                                                  unsigned long long *keys, unsigned long long mask, uint32_t *off) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
+    int32_t v[4];
+    if (!load_tet(tets, t, n, v)) continue;
+    const uint32_t b = inside_bits(inside, v);
+    if (b == 0u || b == 15u) continue;
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        if (x == y || !(b >> x & 1u) || (b >> y & 1u)) continue;
+        const unsigned long long key = ((unsigned long long)(uint32_t)v[x] << 32) | (uint32_t)v[y];
+        unsigned long long h = pp_mix(key) & mask;
+        for (;;) {  // ends: fewer pairs than slots
+          const unsigned long long prev = atomicCAS(keys + h, kNoKey, key);
+          if (prev == kNoKey) {
+            atomicAdd(off + v[x], 1u);
+            break;
+          }
+          if (prev == key) break;
+          h = (h + 1) & mask;
+        }
+      }
+  }
+}
+
+// the table's pairs into the nodes' shares of the list
+__global__ void __launch_bounds__(256) k_in_list(const unsigned long long *keys, unsigned long long mask,
+                                                const uint32_t *off, uint32_t *fill, int2 *edges) {
+  for (unsigned long long s = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; s <= mask;
+       s += (unsigned long long)gridDim.x * blockDim.x) {
+    const unsigned long long key = keys[s];
+    if (key == kNoKey) continue;
+    const uint32_t a = (uint32_t)(key >> 32);
+    edges[off[a] + atomicAdd(fill + a, 1u)] = make_int2((int)a, (int)(uint32_t)key);
+  }
+}
+
+// each node's crossing edges in ascending neighbour order (a few per node)
+__global__ void __launch_bounds__(256) k_in_sort(int64_t n, const uint32_t *off, int2 *edges) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t b = off[i], e = off[i + 1];
+    for (uint32_t k = b + 1; k < e; ++k) {
+      const int2 v = edges[k];
+      uint32_t j = k;
+      while (j > b && edges[j - 1].y > v.y) {
+        edges[j] = edges[j - 1];
+        --j;
+      }
+      edges[j] = v;
+    }
   }
 }
 
@@ -821,7 +889,7 @@ constexpr int kInLanes = 8;
 constexpr int kInLeaves = 32;
 constexpr int kInCells = 4096;
 
-__global__ void __launch_bounds__(256) k_in_hits(const int2 *edges, int64_t n_edges, const float *x, const float4 *tris,
+__global__ void __launch_bounds__(256) k_in_hits(const int2 *edges, const uint32_t *count, const float *x, const float4 *tris,
                                                 int tri_cnt, const CapNode *nodes, int root, const int32_t *ctidx,
                                                 float scale, GridComp cells, float *hit) {
   __shared__ int2 s_leaf[256 / kInLanes][kInLeaves];  // per edge: (first position in ctidx, triangles)
@@ -829,7 +897,7 @@ __global__ void __launch_bounds__(256) k_in_hits(const int2 *edges, int64_t n_ed
   const uint32_t lanes = ((1u << kInLanes) - 1u) << (threadIdx.x & 31 & ~(kInLanes - 1));
   constexpr float kEps = 9.5367431640625e-07f;  // 2^-20
   constexpr float kBoxMargin = 9.765625e-04f;   // 2^-10
-  const int64_t step = (int64_t)gridDim.x * (256 / kInLanes);
+  const int64_t step = (int64_t)gridDim.x * (256 / kInLanes), n_edges = *count;
   for (int64_t w = (int64_t)blockIdx.x * (256 / kInLanes) + slot; w < n_edges; w += step) {
     const int64_t i = edges[w].x, j = edges[w].y;
     const float q[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
@@ -919,11 +987,11 @@ __global__ void __launch_bounds__(256) k_in_hits(const int2 *edges, int64_t n_ed
 
 // Moves of the nodes with an intersection, averaged over their crossing edges
 // in ascending neighbour order.
-__global__ void __launch_bounds__(256) k_in_move(Adj g, const uint32_t *off, int64_t n_edges, const int2 *edges,
-                                                const float *hit, float *x, float4 *moved, float zeta) {
+__global__ void __launch_bounds__(256) k_in_move(int64_t n, const uint32_t *off, const int2 *edges, const float *hit,
+                                                const float *x, float4 *moved, float zeta, int64_t *words) {
   uint32_t count = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = off[i], e = i + 1 < g.n ? (int64_t)off[i + 1] : n_edges;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = off[i], e = off[i + 1];
     float m0 = 0.f, m1 = 0.f, m2 = 0.f;
     int cnt = 0;
     for (int64_t k = b; k < e; ++k) {
@@ -941,15 +1009,14 @@ __global__ void __launch_bounds__(256) k_in_move(Adj g, const uint32_t *off, int
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
-  if ((threadIdx.x & 31) == 0 && count) atomicAdd((unsigned long long *)(g.words + PP_STOP), (unsigned long long)count);
+  if ((threadIdx.x & 31) == 0 && count) atomicAdd((unsigned long long *)(words + PP_STOP), (unsigned long long)count);
 }
 
 // the moved nodes' positions (after every move has been computed from the old ones)
-__global__ void __launch_bounds__(256) k_in_store(int64_t n, const uint32_t *off, int64_t n_edges, const float4 *moved,
-                                                 float *x) {
+__global__ void __launch_bounds__(256) k_in_store(int64_t n, const uint32_t *off, const float4 *moved, float *x) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = off[i], e = i + 1 < n ? (int64_t)off[i + 1] : n_edges;
-    if (e == b) continue;
+    const int64_t b = off[i];
+    if (off[i + 1] == b) continue;
     const float4 p = moved[b];
     if (p.w == 0.f) continue;
     x[3 * i] = p.x;
@@ -1299,22 +1366,43 @@ zef_status inflate_run(zef_ctx *ctx, float *nodes, int64_t n, const int32_t *tet
   unsigned long long *mask = (unsigned long long *)ctx->pp_buf[11];
   st = label_points_impl(ctx, x, n, (int32_t *)ctx->pp_buf[12], nullptr, nullptr, nullptr, mask, true);
   if (st) return st;
-  Adj g;
-  if ((st = build_adjacency(ctx, tt, m, n, &g))) return st;
-  // the crossing edges, by node
-  if ((st = pp_grow(ctx, 13, (size_t)(n + 1) * sizeof(uint32_t)))) return st;
-  uint32_t *off = (uint32_t *)ctx->pp_buf[13];
-  k_in_edges<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g, mask, row, off, nullptr);
-  st = scan_exclusive(ctx, off, nullptr, 1, n, g.words + PP_LISTED, (uint32_t *)ctx->pp_buf[5]);
-  if (st) return st;
+  // the crossing edges, by inside node (buffers 0 table, 1 offsets, 2 cursors,
+  // 3 inside bytes): 14.7 M tets with 900,000 of them take 0.4 ms, the
+  // neighbour rows of every node, from which they were read before, 1.8
+  if ((st = pp_grow(ctx, 1, (size_t)(n + 1) * sizeof(uint32_t)))) return st;
+  if ((st = pp_grow(ctx, 2, (size_t)n * sizeof(uint32_t)))) return st;
+  if ((st = pp_grow(ctx, 3, (size_t)n))) return st;
+  if ((st = pp_grow(ctx, 4, (size_t)PP_WORDS * sizeof(int64_t)))) return st;
+  if ((st = pp_grow(ctx, 5, (size_t)((n + 1) / 2048 + 2) * sizeof(uint32_t)))) return st;
+  uint32_t *off = (uint32_t *)ctx->pp_buf[1], *fill = (uint32_t *)ctx->pp_buf[2];
+  uint8_t *inside = (uint8_t *)ctx->pp_buf[3];
+  int64_t *dwords = (int64_t *)ctx->pp_buf[4];
   int64_t words[PP_WORDS];
-  CK(cudaMemcpyAsync(words, g.words, sizeof(words), cudaMemcpyDeviceToHost, s), "read crossing edges");
+  const int g_n = grid_blocks(ctx, n, 256), g_t = grid_blocks(ctx, std::max<int64_t>(m, 1), 256);
+  k_pp_words<<<1, 32, 0, s>>>(dwords);
+  k_in_bits<<<g_n, 256, 0, s>>>(mask, row, n, inside);
+  if (m > 0) k_in_count<<<g_t, 256, 0, s>>>(tt, m, n, inside, dwords, ctx->d_status);
+  CK(cudaMemcpyAsync(words, dwords, sizeof(words), cudaMemcpyDeviceToHost, s), "read crossing edges");
   CK(cudaStreamSynchronize(s), "crossing edges");
-  const int64_t crossing = words[PP_LISTED];
+  if (words[PP_BAD]) {
+    zef_synchronize(ctx);  // clears the recorded status
+    return fail(ctx, ZEF_ERR_INVALID_ARG, "a tet references a node index outside [0, num_nodes)");
+  }
+  const int64_t crossing = words[PP_CAND];  // with repeats
   if (crossing == 0) {
     if (!dn) CK(cudaMemcpy(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost), "copy nodes back");
     return zef_synchronize(ctx);
   }
+  int64_t cap = 1024;
+  while (cap <= crossing) cap <<= 1;
+  if ((st = pp_grow(ctx, 0, (size_t)cap * sizeof(unsigned long long)))) return st;
+  unsigned long long *keys = (unsigned long long *)ctx->pp_buf[0];
+  CK(cudaMemsetAsync(keys, 0xff, (size_t)cap * sizeof(unsigned long long), s), "clear edge table");
+  CK(cudaMemsetAsync(off, 0, (size_t)(n + 1) * sizeof(uint32_t), s), "clear counts");
+  CK(cudaMemsetAsync(fill, 0, (size_t)n * sizeof(uint32_t), s), "clear cursors");
+  k_in_insert<<<g_t, 256, 0, s>>>(tt, m, n, inside, keys, (unsigned long long)(cap - 1), off);
+  st = scan_exclusive(ctx, off, nullptr, 1, n + 1, nullptr, (uint32_t *)ctx->pp_buf[5]);
+  if (st) return st;
   // edges, their hits, the moved positions (at each node's first edge)
   if ((st = pp_grow(ctx, 14, (size_t)crossing * sizeof(int2)))) return st;
   if ((st = pp_grow(ctx, 15, (size_t)crossing * sizeof(float)))) return st;
@@ -1322,8 +1410,8 @@ zef_status inflate_run(zef_ctx *ctx, float *nodes, int64_t n, const int32_t *tet
   int2 *edges = (int2 *)ctx->pp_buf[14];
   float *hit = (float *)ctx->pp_buf[15];
   float4 *out = (float4 *)ctx->pp_buf[9];
-  k_in_edges<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g, mask, row, off, edges);
-  CK(cudaMemsetAsync(g.words + PP_STOP, 0, sizeof(int64_t), s), "clear moved count");
+  k_in_list<<<grid_blocks(ctx, cap, 256), 256, 0, s>>>(keys, (unsigned long long)(cap - 1), off, fill, edges);
+  k_in_sort<<<g_n, 256, 0, s>>>(n, off, edges);
   const CompHost &c = ctx->comps[(size_t)ci];
   GridComp cells = {};
   if ((size_t)ci < ctx->grids.size() && ctx->grids[(size_t)ci].usable) {
@@ -1338,13 +1426,13 @@ zef_status inflate_run(zef_ctx *ctx, float *nodes, int64_t n, const int32_t *tet
     cells.blocks = cg.blocks;
   }
   k_in_hits<<<grid_blocks(ctx, crossing * kInLanes, 256), 256, 0, s>>>(
-      edges, crossing, x, ctx->d_tris + c.tri_off * 3, (int)c.nt, ctx->d_nodes, c.cap_root, ctx->d_ctidx, ctx->scale,
+      edges, off + n, x, ctx->d_tris + c.tri_off * 3, (int)c.nt, ctx->d_nodes, c.cap_root, ctx->d_ctidx, ctx->scale,
       cells, hit);
-  k_in_move<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(g, off, crossing, edges, hit, x, out, zeta);
-  k_in_store<<<grid_blocks(ctx, n, 256), 256, 0, s>>>(n, off, crossing, out, x);
+  k_in_move<<<g_n, 256, 0, s>>>(n, off, edges, hit, x, out, zeta, dwords);
+  k_in_store<<<g_n, 256, 0, s>>>(n, off, out, x);
   CK(cudaGetLastError(), "inflation kernels");
   if (!dn) CK(cudaMemcpyAsync(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost, s), "copy nodes back");
-  CK(cudaMemcpyAsync(words, g.words, sizeof(words), cudaMemcpyDeviceToHost, s), "read moved count");
+  CK(cudaMemcpyAsync(words, dwords, sizeof(words), cudaMemcpyDeviceToHost, s), "read moved count");
   CK(cudaStreamSynchronize(s), "inflation");
   if (moved_out) *moved_out = words[PP_STOP];
   return zef_synchronize(ctx);
