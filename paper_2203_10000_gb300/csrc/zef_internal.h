@@ -251,10 +251,12 @@ enum Counter {
   CNT_CL_ITER,        // closure passes of the level
   CNT_CL_GREEN,       // tets split along one to three edges
   CNT_CL_GEXTRA,      // children those splits add
+  CNT_RF_MASK,        // refinement: slots of the level's edge table - 1
+  CNT_RF_SHIFT,       // log2 of the slots per node of its placement, 0: hashed over the table
   CNT_LANE_TILES,     // cap trees: (tile, compartment) pairs evaluated by per-lane walks
   CNT_PEND,           // cell grid: points whose label the field leaves open
   CNT_UNC_LIST,       // uncertain pairs appended to the pair list (may exceed its capacity)
-  CNT_COUNT_ = 32
+  CNT_COUNT_ = 40
 };
 
 // zef_label_opts.kernel -> kernel template form: 0 (default) cap trees = 2,
@@ -350,8 +352,8 @@ struct zef_ctx {
   uint64_t rb_key = 0;
 
   // refinement scratch
-  void *rf_buf[10] = {};
-  size_t rf_cap[10] = {};
+  void *rf_buf[11] = {};
+  size_t rf_cap[11] = {};
   cudaGraphExec_t rf_exec = nullptr;
   uint64_t rf_key = 0;
 };

@@ -75,7 +75,8 @@ struct RF {
   unsigned long long *hkeys;
   uint32_t *hvals;
   int32_t *hids;
-  unsigned long long hmask;
+  uint32_t *slots;   // [6 fmax] table slot of every flagged tet's edge
+  unsigned long long hmask;  // slots held - 1; a level uses cnt[CNT_RF_MASK] + 1 of them
   int64_t node_cap, tet_cap, fmax;
   uint32_t *status;
   int64_t *lstats;
@@ -104,12 +105,39 @@ __device__ __forceinline__ bool is_flagged(const RF &r, int64_t t, int64_t M, ui
   return nx != s;
 }
 
+// Edge table of one level: cnt[CNT_RF_MASK] + 1 slots, sized on the device by
+// the level's flagged tets (conforming: all that are held, since the closure
+// flags tets while it fills the table).  Where a node has at least eight
+// slots an edge's first probe is in the run of its lower node, picked by a
+// hash of the other: the edges of neighbouring tets, whose nodes have nearby
+// numbers, then share lines; otherwise it is a hash of the edge.
+struct EdgeTable {
+  unsigned long long mask;
+  int shift;
+};
+__device__ __forceinline__ EdgeTable edge_table(const RF &r) {
+  EdgeTable t;
+  t.mask = (unsigned long long)r.cnt[CNT_RF_MASK];
+  t.shift = (int)r.cnt[CNT_RF_SHIFT];
+  return t;
+}
+__device__ __forceinline__ unsigned long long first_slot(const EdgeTable &t, unsigned long long key) {
+  if (!t.shift) return mix64(key) & t.mask;
+  return (((key >> 32) << t.shift) | (mix64(key & 0xffffffffull) & ((1ull << t.shift) - 1ull))) & t.mask;
+}
+__device__ __forceinline__ void set_table(const RF &r, unsigned long long mask) {
+  int shift = 0;
+  while (((unsigned long long)max(r.cnt[CNT_NODES], (int64_t)1) << (shift + 1)) <= mask + 1) ++shift;
+  r.cnt[CNT_RF_MASK] = (int64_t)mask;
+  r.cnt[CNT_RF_SHIFT] = shift >= 3 ? shift : 0;
+}
+
 // slot of a key known to be in the table (bounded probe)
-__device__ __forceinline__ unsigned long long find_slot(const RF &r, unsigned long long key) {
-  unsigned long long h = mix64(key) & r.hmask;
-  for (unsigned long long it = 0; it <= r.hmask; ++it) {
+__device__ __forceinline__ unsigned long long find_slot(const RF &r, const EdgeTable &tab, unsigned long long key) {
+  unsigned long long h = first_slot(tab, key);
+  for (unsigned long long it = 0; it <= tab.mask; ++it) {
     if (r.hkeys[h] == key) return h;
-    h = (h + 1) & r.hmask;
+    h = (h + 1) & tab.mask;
   }
   return 0;  // unreachable when the key was inserted
 }
@@ -126,27 +154,29 @@ __global__ void k_rf_init(int64_t *cnt, int64_t n, int64_t m) {
 
 // ---- conforming closure
 // true when the key is in the table (bounded probe)
-__device__ __forceinline__ bool edge_present(const RF &r, unsigned long long key) {
-  unsigned long long h = mix64(key) & r.hmask;
-  for (unsigned long long it = 0; it <= r.hmask; ++it) {
+__device__ __forceinline__ bool edge_present(const RF &r, const EdgeTable &tab, unsigned long long key) {
+  unsigned long long h = first_slot(tab, key);
+  for (unsigned long long it = 0; it <= tab.mask; ++it) {
     const unsigned long long k = r.hkeys[h];
     if (k == key) return true;
     if (k == kEmpty) return false;
-    h = (h + 1) & r.hmask;
+    h = (h + 1) & tab.mask;
   }
   return false;
 }
 
-__device__ __forceinline__ int split_mask(const RF &r, const int32_t *v) {
+__device__ __forceinline__ int split_mask(const RF &r, const EdgeTable &tab, const int32_t *v) {
   int m = 0;
 #pragma unroll
   for (int e = 0; e < 6; ++e)
-    if (edge_present(r, edge_key(v[c_edge[e][0]], v[c_edge[e][1]]))) m |= 1 << e;
+    if (edge_present(r, tab, edge_key(v[c_edge[e][0]], v[c_edge[e][1]]))) m |= 1 << e;
   return m;
 }
 
-__global__ void k_cl_reset(int64_t *cnt) {
+__global__ void k_cl_reset(RF r) {
+  int64_t *cnt = r.cnt;
   if (threadIdx.x == 0) {
+    set_table(r, r.hmask);
     cnt[CNT_LEVEL_SEED] = cnt[CNT_CL_CHANGED] = cnt[CNT_CL_ITER] = 0;
     cnt[CNT_CL_GREEN] = cnt[CNT_CL_GEXTRA] = 0;
   }
@@ -169,16 +199,17 @@ __global__ void __launch_bounds__(256) k_cl_seed(RF r) {
 __global__ void __launch_bounds__(256) k_cl_insert(RF r) {
   if (r.cnt[CNT_ABORT]) return;
   const int64_t M = r.cnt[CNT_TETS];
+  const EdgeTable tab = edge_table(r);
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < M; t += (int64_t)gridDim.x * blockDim.x) {
     if (r.state[t] != 2) continue;
     const int32_t *v = r.tets + 4 * t;
     for (int e = 0; e < 6; ++e) {
       const unsigned long long key = edge_key(v[c_edge[e][0]], v[c_edge[e][1]]);
-      unsigned long long h = mix64(key) & r.hmask;
-      for (unsigned long long it = 0; it <= r.hmask; ++it) {
+      unsigned long long h = first_slot(tab, key);
+      for (unsigned long long it = 0; it <= tab.mask; ++it) {
         const unsigned long long prev = atomicCAS(r.hkeys + h, kEmpty, key);
         if (prev == kEmpty || prev == key) break;
-        h = (h + 1) & r.hmask;
+        h = (h + 1) & tab.mask;
       }
     }
     r.state[t] = 1;
@@ -193,7 +224,7 @@ __global__ void __launch_bounds__(256) k_cl_check(RF r) {
     const int64_t t = t0 + threadIdx.x;
     bool promote = false;
     if (t < M && r.state[t] == 0) {
-      promote = c_gn[split_mask(r, r.tets + 4 * t)] < 0;
+      promote = c_gn[split_mask(r, edge_table(r), r.tets + 4 * t)] < 0;
       if (promote) r.state[t] = 2;
     }
     const unsigned b = __ballot_sync(0xffffffffu, promote);
@@ -230,7 +261,7 @@ __global__ void __launch_bounds__(256) k_cl_gcount(RF r) {
   for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x; t0 < M; t0 += (int64_t)gridDim.x * blockDim.x) {
     const int64_t t = t0 + threadIdx.x;
     int n = 0;
-    if (t < M && !ab && r.state[t] == 0) n = c_gn[split_mask(r, r.tets + 4 * t)];
+    if (t < M && !ab && r.state[t] == 0) n = c_gn[split_mask(r, edge_table(r), r.tets + 4 * t)];
     if (t < M) r.gx[t] = n > 1 ? (uint32_t)(n - 1) : 0u;
     const unsigned b = __ballot_sync(0xffffffffu, n > 1);
     if ((threadIdx.x & 31) == 0 && b)
@@ -275,44 +306,60 @@ __global__ void k_rf_check(RF r) {
     atomicOr(r.status, ST_CAPACITY);
   }
   r.cnt[CNT_OWN_LEN] = r.cnt[CNT_ABORT] ? 0 : 6 * F;
+  if (!r.state) {  // 6 F edges, load at most 1/2
+    unsigned long long size = 1024;
+    while (size < 12ull * (unsigned long long)(r.cnt[CNT_ABORT] ? 0 : F)) size <<= 1;
+    set_table(r, size - 1);
+  }
+}
+
+// the level's part of the table
+__global__ void __launch_bounds__(256) k_rf_clear(RF r) {
+  if (r.cnt[CNT_ABORT]) return;
+  const int64_t n = r.cnt[CNT_RF_MASK] + 1;  // a multiple of four
+  const ulonglong2 k = make_ulonglong2(kEmpty, kEmpty);
+  const uint4 v = make_uint4(~0u, ~0u, ~0u, ~0u);
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n / 4; j += (int64_t)gridDim.x * blockDim.x) {
+    reinterpret_cast<ulonglong2 *>(r.hkeys)[2 * j] = k;
+    reinterpret_cast<ulonglong2 *>(r.hkeys)[2 * j + 1] = k;
+    reinterpret_cast<uint4 *>(r.hvals)[j] = v;
+  }
 }
 
 __global__ void __launch_bounds__(256) k_rf_insert(RF r) {
   if (r.cnt[CNT_ABORT]) return;
   const int64_t M = r.cnt[CNT_TETS];
+  const EdgeTable tab = edge_table(r);
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < M; t += (int64_t)gridDim.x * blockDim.x) {
     uint32_t rank;
     if (!is_flagged(r, t, M, &rank)) continue;
-    const int32_t *v = r.tets + 4 * t;
+    const int4 q = reinterpret_cast<const int4 *>(r.tets)[t];
+    const int32_t v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
     for (int e = 0; e < 6; ++e) {
-      const unsigned long long key = edge_key(v[c_edge[e][0]], v[c_edge[e][1]]);
+      constexpr int kA[6] = {0, 0, 0, 1, 1, 2}, kB[6] = {1, 2, 3, 2, 3, 3};
+      const unsigned long long key = edge_key(v[kA[e]], v[kB[e]]);
       const uint32_t code = rank * 6u + (uint32_t)e;
-      unsigned long long h = mix64(key) & r.hmask;
-      for (unsigned long long it = 0; it <= r.hmask; ++it) {
+      unsigned long long h = first_slot(tab, key);
+      for (unsigned long long it = 0; it <= tab.mask; ++it) {
         const unsigned long long prev = atomicCAS(r.hkeys + h, kEmpty, key);
         if (prev == kEmpty || prev == key) {
           atomicMin(r.hvals + h, code);
           break;
         }
-        h = (h + 1) & r.hmask;
+        h = (h + 1) & tab.mask;
       }
+      r.slots[code] = (uint32_t)h;
     }
   }
 }
 
+// one thread per edge of a flagged tet: does its code own the edge
 __global__ void __launch_bounds__(256) k_rf_owner(RF r) {
   if (r.cnt[CNT_ABORT]) return;
-  const int64_t M = r.cnt[CNT_TETS];
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < M; t += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t rank;
-    if (!is_flagged(r, t, M, &rank)) continue;
-    const int32_t *v = r.tets + 4 * t;
-    for (int e = 0; e < 6; ++e) {
-      const unsigned long long key = edge_key(v[c_edge[e][0]], v[c_edge[e][1]]);
-      const uint32_t code = rank * 6u + (uint32_t)e;
-      r.owned[code] = (r.hvals[find_slot(r, key)] == code) ? 1u : 0u;
-    }
-  }
+  const int64_t len = r.cnt[CNT_OWN_LEN];
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < len; c += (int64_t)gridDim.x * blockDim.x)
+    r.owned[c] = r.hvals[r.slots[c]] == (uint32_t)c ? 1u : 0u;
 }
 
 // after the owner scan: node capacity, and the counts of the label pipeline
@@ -329,23 +376,19 @@ __global__ void k_rf_check2(RF r) {
 
 __global__ void __launch_bounds__(256) k_rf_nodes(RF r) {
   if (r.cnt[CNT_ABORT]) return;
-  const int64_t M = r.cnt[CNT_TETS], N = r.cnt[CNT_NODES];
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < M; t += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t rank;
-    if (!is_flagged(r, t, M, &rank)) continue;
-    const int32_t *v = r.tets + 4 * t;
-    for (int e = 0; e < 6; ++e) {
-      const int32_t a = v[c_edge[e][0]], b = v[c_edge[e][1]];
-      const unsigned long long key = edge_key(a, b);
-      const uint32_t code = rank * 6u + (uint32_t)e;
-      const unsigned long long slot = find_slot(r, key);
-      if (r.hvals[slot] != code) continue;
-      const int64_t id = N + r.owned[code];
-      r.hids[slot] = (int32_t)id;
-      const int32_t lo = min(a, b), hi = max(a, b);
-      for (int k = 0; k < 3; ++k)
-        r.nodes[3 * id + k] = __fmul_rn(__fadd_rn(r.nodes[3 * (int64_t)lo + k], r.nodes[3 * (int64_t)hi + k]), 0.5f);
-    }
+  // one thread per edge of a flagged tet; the scanned owner flags step at an
+  // owner, whose edge stands in the table under its slot
+  const int64_t N = r.cnt[CNT_NODES], len = r.cnt[CNT_OWN_LEN];
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < len; c += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t at = r.owned[c], next = c + 1 < len ? r.owned[c + 1] : (uint32_t)r.cnt[CNT_LEVEL_NEW];
+    if (at == next) continue;
+    const uint32_t slot = r.slots[c];
+    const unsigned long long key = r.hkeys[slot];
+    const int64_t id = N + at;
+    r.hids[slot] = (int32_t)id;
+    const int64_t lo = (int64_t)(key >> 32), hi = (int64_t)(key & 0xffffffffull);
+    for (int k = 0; k < 3; ++k)
+      r.nodes[3 * id + k] = __fmul_rn(__fadd_rn(r.nodes[3 * lo + k], r.nodes[3 * hi + k]), 0.5f);
   }
 }
 
@@ -361,9 +404,13 @@ __global__ void __launch_bounds__(256) k_rf_children(RF r) {
     uint32_t rank;
     if (!is_flagged(r, t, M, &rank)) continue;
     int32_t loc[10];
-    for (int k = 0; k < 4; ++k) loc[k] = r.tets[4 * t + k];
-    for (int e = 0; e < 6; ++e)
-      loc[4 + e] = r.hids[find_slot(r, edge_key(loc[c_edge[e][0]], loc[c_edge[e][1]]))];
+    const int4 q4 = reinterpret_cast<const int4 *>(r.tets)[t];
+    loc[0] = q4.x;
+    loc[1] = q4.y;
+    loc[2] = q4.z;
+    loc[3] = q4.w;
+#pragma unroll
+    for (int e = 0; e < 6; ++e) loc[4 + e] = r.hids[r.slots[(int64_t)rank * 6 + e]];
     float l[3];
     for (int d = 0; d < 3; ++d)
       l[d] = len2_rn(r.nodes + 3 * (int64_t)loc[c_diag[d][0]], r.nodes + 3 * (int64_t)loc[c_diag[d][1]]);
@@ -387,11 +434,12 @@ __global__ void __launch_bounds__(256) k_cl_children(RF r) {
     if (r.state[t] != 0) continue;
     int32_t loc[10];
     for (int k = 0; k < 4; ++k) loc[k] = r.tets[4 * t + k];
-    const int mask = split_mask(r, loc);
+    const EdgeTable tab = edge_table(r);
+    const int mask = split_mask(r, tab, loc);
     const int n = c_gn[mask];
     if (n <= 0) continue;
     for (int e = 0; e < 6; ++e)
-      loc[4 + e] = ((mask >> e) & 1) ? r.hids[find_slot(r, edge_key(loc[c_edge[e][0]], loc[c_edge[e][1]]))] : -1;
+      loc[4 + e] = ((mask >> e) & 1) ? r.hids[find_slot(r, tab, edge_key(loc[c_edge[e][0]], loc[c_edge[e][1]]))] : -1;
     int alt = 0;
     if (n == 3) {
       const float d0 = len2_rn(r.nodes + 3 * (int64_t)loc[c_gdg[mask][0][0]], r.nodes + 3 * (int64_t)loc[c_gdg[mask][0][1]]);
@@ -619,6 +667,7 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
   if ((st = grow(ctx, 1, (size_t)std::max<int64_t>(6 * fmax, 1) * sizeof(uint32_t)))) return st;  // owned
   if ((st = grow(ctx, 2, (size_t)hcap * (sizeof(unsigned long long) + 2 * sizeof(uint32_t))))) return st;
   if ((st = grow(ctx, 3, (size_t)bs_len * sizeof(uint32_t)))) return st;
+  if ((st = grow(ctx, 10, (size_t)std::max<int64_t>(6 * fmax, 1) * sizeof(uint32_t)))) return st;  // slots
   if ((st = grow(ctx, 4, (size_t)std::max(levels, 1) * kLevelStats * sizeof(int64_t)))) return st;
   if (conforming) {
     if ((st = grow(ctx, 8, (size_t)std::max<int64_t>(tcap, 1)))) return st;                     // state
@@ -674,6 +723,7 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
   r.hvals = (uint32_t *)(r.hkeys + hcap);
   r.hids = (int32_t *)(r.hvals + hcap);
   r.hmask = (unsigned long long)(hcap - 1);
+  r.slots = (uint32_t *)ctx->rf_buf[10];
   r.node_cap = ncap;
   r.tet_cap = tcap;
   r.fmax = fmax;
@@ -695,7 +745,7 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
                        (uint64_t)shape.ppt, (uint64_t)shape.variant, (uint64_t)opts.precision, fbits(opts.margin),
                        fbits(opts.winding_tol), (uint64_t)opts.flags, (uint64_t)grid, (uint64_t)(uintptr_t)b.pending,
                        (uint64_t)b.cap_pending, (uint64_t)(uintptr_t)ctx->d_entries, (uint64_t)conforming, ctx->gen,
-                       (uint64_t)(uintptr_t)r.state, (uint64_t)(uintptr_t)r.gx})
+                       (uint64_t)(uintptr_t)r.state, (uint64_t)(uintptr_t)r.gx, (uint64_t)(uintptr_t)r.slots})
       key = hash_mix(key, v);
     if (!ctx->rf_exec || ctx->rf_key != key) {
       if (ctx->rf_exec) {
@@ -713,14 +763,14 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
       cudaError_t ce = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
       st = ZEF_OK;
       if (ce == cudaSuccess) {
-        const int g_t = grid_blocks(ctx, tcap, 256);
+        const int g_t = grid_blocks(ctx, tcap, 256), g_e = grid_blocks(ctx, std::max<int64_t>(6 * fmax, 1), 256);
         for (int lv = 0; lv < levels && st == ZEF_OK; ++lv) {
           k_rf_flag<<<g_t, 256, 0, cap>>>(r);
           if (conforming) {
             // closure: the red set grows until every other tet has a green pattern
             cudaMemsetAsync(r.hkeys, 0xff, (size_t)hcap * sizeof(unsigned long long), cap);
             cudaMemsetAsync(r.hvals, 0xff, (size_t)hcap * sizeof(uint32_t), cap);
-            k_cl_reset<<<1, 32, 0, cap>>>(b.counters);
+            k_cl_reset<<<1, 32, 0, cap>>>(r);
             k_cl_seed<<<g_t, 256, 0, cap>>>(r);
             st = capture_while(ctx, cap, aux, [&](cudaStream_t s, cudaGraphConditionalHandle h) {
               k_cl_insert<<<g_t, 256, 0, s>>>(r);
@@ -733,12 +783,9 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
           st = scan_exclusive(ctx, r.flags, b.counters + CNT_TETS, 1, tcap, b.counters + CNT_LEVEL_FLAGGED, bsums);
           if (st) break;
           k_rf_check<<<1, 32, 0, cap>>>(r);
-          if (!conforming) {
-            cudaMemsetAsync(r.hkeys, 0xff, (size_t)hcap * sizeof(unsigned long long), cap);
-            cudaMemsetAsync(r.hvals, 0xff, (size_t)hcap * sizeof(uint32_t), cap);
-          }
+          if (!conforming) k_rf_clear<<<grid_blocks(ctx, hcap / 4, 256), 256, 0, cap>>>(r);
           k_rf_insert<<<g_t, 256, 0, cap>>>(r);
-          k_rf_owner<<<g_t, 256, 0, cap>>>(r);
+          k_rf_owner<<<g_e, 256, 0, cap>>>(r);
           st = scan_exclusive(ctx, r.owned, b.counters + CNT_OWN_LEN, 1, std::max<int64_t>(6 * fmax, 1),
                               b.counters + CNT_LEVEL_NEW, bsums);
           if (st) break;
@@ -749,7 +796,7 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
             if (st) break;
             k_cl_check3<<<1, 32, 0, cap>>>(r);
           }
-          k_rf_nodes<<<g_t, 256, 0, cap>>>(r);
+          k_rf_nodes<<<g_e, 256, 0, cap>>>(r);
           LabelPlan p;
           p.pts = nodes;
           p.labels = labels;
