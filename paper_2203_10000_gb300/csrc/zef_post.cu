@@ -814,32 +814,55 @@ __global__ void __launch_bounds__(256) k_in_count(const int32_t *tets, int64_t m
   if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long *)(words + PP_CAND), (unsigned long long)c);
 }
 
-// into the table (more slots than pairs); a pair's first insertion counts it
-// at the inside node
-__global__ void __launch_bounds__(256) k_in_insert(const int32_t *tets, int64_t m, int64_t n, const uint8_t *inside,
+// the pairs, with repeats, into a list (a place per warp from the cursor)
+__global__ void __launch_bounds__(256) k_in_pairs(const int32_t *tets, int64_t m, int64_t n, const uint8_t *inside,
+                                                 unsigned long long *pairs, int64_t *words) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); t0 < m; t0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = t0 + lane;
+    int32_t v[4] = {0, 0, 0, 0};
+    uint32_t b = 0;
+    if (t < m && load_tet(tets, t, n, v)) b = inside_bits(inside, v);
+    const int c = __popc(b) * (4 - __popc(b));
+    if (!__any_sync(0xffffffffu, c != 0)) continue;
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    unsigned long long at = 0;
+    if (lane == 31) at = atomicAdd((unsigned long long *)(words + PP_POOL), (unsigned long long)incl);
+    at = __shfl_sync(0xffffffffu, at, 31) + (unsigned long long)(incl - c);
+    if (c)
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          if (x != y && (b >> x & 1u) && !(b >> y & 1u))
+            pairs[at++] = ((unsigned long long)(uint32_t)v[x] << 32) | (uint32_t)v[y];
+  }
+}
+
+// the list into the table (more slots than pairs), one thread per pair; a
+// pair's first insertion counts it at the inside node.  (A thread per tet
+// waited for up to four swaps in turn, in warps of few crossing tets: 0.63 ms
+// for 14.7 M tets.)
+__global__ void __launch_bounds__(256) k_in_insert(const unsigned long long *pairs, const int64_t *count,
                                                   unsigned long long *keys, unsigned long long mask, uint32_t *off) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
-    int32_t v[4];
-    if (!load_tet(tets, t, n, v)) continue;
-    const uint32_t b = inside_bits(inside, v);
-    if (b == 0u || b == 15u) continue;
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        if (x == y || !(b >> x & 1u) || (b >> y & 1u)) continue;
-        const unsigned long long key = ((unsigned long long)(uint32_t)v[x] << 32) | (uint32_t)v[y];
-        unsigned long long h = pp_mix(key) & mask;
-        for (;;) {  // ends: fewer pairs than slots
-          const unsigned long long prev = atomicCAS(keys + h, kNoKey, key);
-          if (prev == kNoKey) {
-            atomicAdd(off + v[x], 1u);
-            break;
-          }
-          if (prev == key) break;
-          h = (h + 1) & mask;
-        }
+  const int64_t len = *count;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < len; k += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned long long key = pairs[k];
+    unsigned long long h = pp_mix(key) & mask;
+    for (;;) {  // ends: fewer pairs than slots
+      const unsigned long long prev = atomicCAS(keys + h, kNoKey, key);
+      if (prev == kNoKey) {
+        atomicAdd(off + (uint32_t)(key >> 32), 1u);
+        break;
       }
+      if (prev == key) break;
+      h = (h + 1) & mask;
+    }
   }
 }
 
@@ -1400,7 +1423,11 @@ zef_status inflate_run(zef_ctx *ctx, float *nodes, int64_t n, const int32_t *tet
   CK(cudaMemsetAsync(keys, 0xff, (size_t)cap * sizeof(unsigned long long), s), "clear edge table");
   CK(cudaMemsetAsync(off, 0, (size_t)(n + 1) * sizeof(uint32_t), s), "clear counts");
   CK(cudaMemsetAsync(fill, 0, (size_t)n * sizeof(uint32_t), s), "clear cursors");
-  k_in_insert<<<g_t, 256, 0, s>>>(tt, m, n, inside, keys, (unsigned long long)(cap - 1), off);
+  if ((st = pp_grow(ctx, 16, (size_t)crossing * sizeof(unsigned long long)))) return st;
+  unsigned long long *pairs = (unsigned long long *)ctx->pp_buf[16];
+  k_in_pairs<<<g_t, 256, 0, s>>>(tt, m, n, inside, pairs, dwords);
+  k_in_insert<<<grid_blocks(ctx, crossing, 256), 256, 0, s>>>(pairs, dwords + PP_POOL, keys, (unsigned long long)(cap - 1),
+                                                              off);
   st = scan_exclusive(ctx, off, nullptr, 1, n + 1, nullptr, (uint32_t *)ctx->pp_buf[5]);
   if (st) return st;
   // edges, their hits, the moved positions (at each node's first edge)
