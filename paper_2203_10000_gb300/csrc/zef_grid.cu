@@ -510,7 +510,8 @@ constexpr int kGlTile = 32 * kGlP;
 constexpr int kGlQueue = 32 + kGlTile;  // fewer than 32 left over, one tile's more
 constexpr int kGsP = 4;               // streaming kernel
 constexpr int kGsTile = 32 * kGsP;
-constexpr int kGsQueue = 64 + kGsTile;
+constexpr int kGsFlush = 256;         // listed together (each addition to the one cursor costs about a nanosecond)
+constexpr int kGsQueue = kGsFlush + kGsTile;
 constexpr int kGlMaxIters = 32;       // consecutive tiles of a warp
 constexpr int kLanes = 4;             // lanes per point of the crossing tests
 
@@ -792,7 +793,7 @@ __global__ void __launch_bounds__(kGlThreads, 4) k_grid_label(GridArgs a) {
 // Two launches (large calls).  Streaming: labels of the points that the field
 // decides (12 bytes in, 4 out per point, the field from L2; few registers, so
 // many loads in flight); the indices of the others are listed, a warp's
-// consecutive points in runs of at least 64.
+// consecutive points in runs of at least kGsFlush.
 template <bool WIDE>
 __global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
   using M = typename FieldCell<WIDE>::M;
@@ -841,7 +842,7 @@ __global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
       if (open) s_q[wid][queued + __popc(ob & ((1u << lane) - 1u))] = (int32_t)i;
       queued += __popc(ob);
     }
-    if (queued >= 64 || (base + kGsTile >= end && queued > 0)) {
+    if (queued >= kGsFlush || (base + kGsTile >= end && queued > 0)) {
       __syncwarp();
       unsigned long long at = 0;
       if (lane == 0) at = atomicAdd((unsigned long long *)(a.counters + CNT_PEND), (unsigned long long)queued);

@@ -274,6 +274,34 @@ __device__ __forceinline__ void insert_edge(const Adj &g, uint32_t a, uint32_t b
   atomicExch((unsigned long long *)(g.words + PP_FULL), 1ull);  // cannot happen at load <= 1/2
 }
 
+// First of cnt places from the cursor for every thread of a 256-thread block
+// (all threads call): one addition per block.  (One per warp costs 0.8 ns
+// each, all of them on one word: 0.37 ms for 0.46 M warps.)
+__device__ __forceinline__ unsigned long long block_places(uint32_t cnt, int64_t *cursor) {
+  __shared__ uint32_t s_warp[8];
+  __shared__ unsigned long long s_base;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t incl = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (lane == 31) s_warp[wid] = incl;
+  __syncthreads();
+  uint32_t before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    before += w < wid ? s_warp[w] : 0u;
+    total += s_warp[w];
+  }
+  if (threadIdx.x == 0 && total) s_base = atomicAdd((unsigned long long *)cursor, (unsigned long long)total);
+  __syncthreads();
+  const unsigned long long base = s_base;
+  __syncthreads();  // before the next call's writes
+  return base + before + (incl - cnt);
+}
+
 // ---- tissue-boundary faces
 struct FaceTab {
   unsigned long long *keys;  // [2 * (mask + 1)]: (a | b << 32, c) of the sorted triple, all ones when empty
@@ -370,61 +398,82 @@ __global__ void __launch_bounds__(256) k_sf_count(const int32_t *tets, int64_t m
   if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long *)(words + PP_CAND), (unsigned long long)c);
 }
 
-// the faces of mixed nodes into the table with their tets' element labels
-__global__ void __launch_bounds__(256) k_sf_faces(FaceTab f, const int32_t *tets, const int32_t *labels, int64_t m,
-                                                 int64_t n, const uint8_t *mixed, int64_t *words) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
-    int32_t v[4];
-    if (!load_tet(tets, t, n, v)) continue;
-    const uint32_t mb = mixed_bits(mixed, v);
-    if (__popc(mb) < 3) continue;
+// A face of three mixed nodes: sorted node triple and its tet's element label.
+struct __align__(16) FaceItem {
+  uint32_t a, b, c;
+  int32_t label;
+};
+
+// the faces of mixed nodes into a list
+__global__ void __launch_bounds__(256) k_sf_list(const int32_t *tets, const int32_t *labels, int64_t m, int64_t n,
+                                                const uint8_t *mixed, FaceItem *items, int64_t *words) {
+  for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x; t0 < m; t0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = t0 + threadIdx.x;
+    int32_t v[4] = {0, 0, 0, 0};
+    uint32_t mb = 0;
+    if (t < m && load_tet(tets, t, n, v)) mb = mixed_bits(mixed, v);
+    const uint32_t cnt = __popc(mb) == 4 ? 4u : __popc(mb) == 3 ? 1u : 0u;
+    unsigned long long at = block_places(cnt, words + PP_POOL);
+    if (!cnt) continue;
     const int32_t lab = labels[t];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       // face q leaves out vertex 3 - q
       if ((mb | 1u << (3 - q)) != 0xfu) continue;
-      uint32_t a = (uint32_t)v[q == 3 ? 1 : 0], b = (uint32_t)v[q >= 2 ? 2 : 1], c = (uint32_t)v[q >= 1 ? 3 : 2];
-      uint32_t lo = min(a, min(b, c)), hi = max(a, max(b, c));
-      const uint32_t mid = a ^ b ^ c ^ lo ^ hi;
-      a = lo;
-      b = mid;
-      c = hi;
-      const unsigned long long klo = (unsigned long long)a | ((unsigned long long)b << 32), khi = c;
-      unsigned long long h = pp_mix(klo ^ pp_mix(khi)) & f.mask;
-      bool placed = false;
-      for (unsigned long long it = 0; it <= f.mask; ++it) {
-        unsigned long long olo, ohi;
-        cas128(f.keys + 2 * h, kNoKey, kNoKey, klo, khi, olo, ohi);
-        if ((olo == kNoKey && ohi == kNoKey) || (olo == klo && ohi == khi)) {
-          atomicMin(f.lo + h, lab);
-          atomicMax(f.hi + h, lab);
-          placed = true;
-          break;
-        }
-        h = (h + 1) & f.mask;
-      }
-      if (!placed) atomicExch((unsigned long long *)(words + PP_FULL), 1ull);
+      const uint32_t a = (uint32_t)v[q == 3 ? 1 : 0], b = (uint32_t)v[q >= 2 ? 2 : 1], c = (uint32_t)v[q >= 1 ? 3 : 2];
+      FaceItem f;
+      f.a = min(a, min(b, c));
+      f.c = max(a, max(b, c));
+      f.b = a ^ b ^ c ^ f.a ^ f.c;
+      f.label = lab;
+      items[at++] = f;
     }
   }
 }
 
-// the boundary faces (two tets, different labels) and their edges
-__global__ void __launch_bounds__(256) k_sf_edges(FaceTab f, Adj g) {
-  uint32_t faces = 0;
-  for (unsigned long long s = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; s <= f.mask;
-       s += (unsigned long long)gridDim.x * blockDim.x) {
-    const unsigned long long klo = f.keys[2 * s];
-    if (klo == kNoKey || f.lo[s] == f.hi[s]) continue;
-    const uint32_t a = (uint32_t)(klo & 0xffffffffu), b = (uint32_t)(klo >> 32), c = (uint32_t)f.keys[2 * s + 1];
-    ++faces;
-    insert_edge(g, a, b);
-    insert_edge(g, a, c);
-    insert_edge(g, b, c);
+// the listed faces into the table, one thread each
+__global__ void __launch_bounds__(256) k_sf_faces(FaceTab f, const FaceItem *items, int64_t *words) {
+  const int64_t len = words[PP_POOL];
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < len; k += (int64_t)gridDim.x * blockDim.x) {
+    const FaceItem it = items[k];
+    const unsigned long long klo = (unsigned long long)it.a | ((unsigned long long)it.b << 32), khi = it.c;
+    unsigned long long h = pp_mix(klo ^ pp_mix(khi)) & f.mask;
+    bool placed = false;
+    for (unsigned long long p = 0; p <= f.mask; ++p) {
+      unsigned long long olo, ohi;
+      cas128(f.keys + 2 * h, kNoKey, kNoKey, klo, khi, olo, ohi);
+      if ((olo == kNoKey && ohi == kNoKey) || (olo == klo && ohi == khi)) {
+        atomicMin(f.lo + h, it.label);
+        atomicMax(f.hi + h, it.label);
+        placed = true;
+        break;
+      }
+      h = (h + 1) & f.mask;
+    }
+    if (!placed) atomicExch((unsigned long long *)(words + PP_FULL), 1ull);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) faces += __shfl_xor_sync(0xffffffffu, faces, o);
-  if ((threadIdx.x & 31) == 0 && faces)
-    atomicAdd((unsigned long long *)(g.words + PP_FACES), (unsigned long long)faces);
+}
+
+// the boundary faces (two tets, different labels) into a list
+__global__ void __launch_bounds__(256) k_sf_boundary(FaceTab f, uint4 *faces, int64_t *words) {
+  for (unsigned long long s0 = blockIdx.x * (unsigned long long)blockDim.x; s0 <= f.mask;
+       s0 += (unsigned long long)gridDim.x * blockDim.x) {  // the table's size is a multiple of 256
+    const unsigned long long s = s0 + threadIdx.x;
+    const ulonglong2 k = reinterpret_cast<const ulonglong2 *>(f.keys)[s];
+    const bool is = k.x != kNoKey && f.lo[s] != f.hi[s];
+    const unsigned long long at = block_places(is ? 1u : 0u, words + PP_FACES);
+    if (is) faces[at] = make_uint4((uint32_t)k.x, (uint32_t)(k.x >> 32), (uint32_t)k.y, 0u);
+  }
+}
+
+// their edges into the edge table, one thread per edge
+__global__ void __launch_bounds__(256) k_sf_edges(const uint4 *faces, Adj g) {
+  const int64_t len = 3 * g.words[PP_FACES];
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < len; k += (int64_t)gridDim.x * blockDim.x) {
+    const uint4 f = faces[k / 3];
+    const int e = (int)(k % 3);
+    insert_edge(g, e == 2 ? f.y : f.x, e == 0 ? f.y : f.z);
+  }
 }
 
 __global__ void __launch_bounds__(256) k_pp_scatter(Adj g) {
@@ -658,8 +707,8 @@ zef_status sort_rows(zef_ctx *ctx, const Adj &g) {
 // positions and one thread summing the blocks' partial sums (140 us of each
 // iteration), 2.5 ms now: 120 us a step, bound by the L1's handling of a
 // warp's 32 scattered 16-byte reads (44 M a step).  Rows interleaved by warp,
-// or read four indices at a time, changed the indices' share only (145 and
-// 130 us).
+// indices read four at a time, or staged in shared memory by the warp, took
+// 145, 130 and 140.
 struct Smooth {
   Adj g;
   float4 *x, *y;           // positions [n]: x current, y after the forward step
@@ -814,26 +863,16 @@ __global__ void __launch_bounds__(256) k_in_count(const int32_t *tets, int64_t m
   if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long *)(words + PP_CAND), (unsigned long long)c);
 }
 
-// the pairs, with repeats, into a list (a place per warp from the cursor)
+// the pairs, with repeats, into a list
 __global__ void __launch_bounds__(256) k_in_pairs(const int32_t *tets, int64_t m, int64_t n, const uint8_t *inside,
                                                  unsigned long long *pairs, int64_t *words) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); t0 < m; t0 += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t t = t0 + lane;
+  for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x; t0 < m; t0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = t0 + threadIdx.x;
     int32_t v[4] = {0, 0, 0, 0};
     uint32_t b = 0;
     if (t < m && load_tet(tets, t, n, v)) b = inside_bits(inside, v);
-    const int c = __popc(b) * (4 - __popc(b));
-    if (!__any_sync(0xffffffffu, c != 0)) continue;
-    int incl = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += u;
-    }
-    unsigned long long at = 0;
-    if (lane == 31) at = atomicAdd((unsigned long long *)(words + PP_POOL), (unsigned long long)incl);
-    at = __shfl_sync(0xffffffffu, at, 31) + (unsigned long long)(incl - c);
+    const uint32_t c = __popc(b) * (4 - __popc(b));
+    unsigned long long at = block_places(c, words + PP_POOL);
     if (c)
 #pragma unroll
       for (int x = 0; x < 4; ++x)
@@ -1202,12 +1241,13 @@ zef_status smooth_loop(zef_ctx *ctx, float *x, int64_t n, const Adj &g, const ui
   return ZEF_OK;
 }
 
-// Rows of the tissue-boundary faces' edges (buffers 0-5 as build_adjacency, 14
-// for the face table, 15 and 16 for the nodes' labels and marks);
-// synchronizes.  14.7 M tets of a refined head with 1.6 M boundary faces:
-// 0.6 + 6.1 ms clearing a table for, and inserting, all 59 M faces, and 4.0 ms
-// scanning it with one counter for all faces, before the faces were chosen by
-// their nodes.
+// Rows of the tissue-boundary faces' edges (buffers 0-5 as build_adjacency, 11
+// for the listed faces, 14 for the face table, 15 and 16 for the nodes' labels
+// and marks); synchronizes.  14.7 M tets of a refined head with 1.6 M boundary
+// faces: 0.6 + 6.1 ms clearing a table for, and inserting, all 59 M faces, and
+// 4.0 ms scanning it with one counter for all faces, before the faces were
+// chosen by their nodes; 0.50 and 0.41 ms for table and edges with a thread
+// per tet and per table slot, waiting for several swaps in turn.
 zef_status build_surface_adjacency(zef_ctx *ctx, const int32_t *tets, const int32_t *labels, int64_t m, int64_t n,
                                    Adj *out, int64_t *faces) {
   zef_status st;
@@ -1247,6 +1287,8 @@ zef_status build_surface_adjacency(zef_ctx *ctx, const int32_t *tets, const int3
   while (cap < 3 * cand) cap <<= 1;       // a boundary face was counted twice: at most 3/2 cand edges, load <= 1/2
   if ((st = pp_grow(ctx, 14, (size_t)fcap * (2 * sizeof(unsigned long long) + 2 * sizeof(int32_t))))) return st;
   if ((st = pp_grow(ctx, 0, (size_t)cap * sizeof(unsigned long long)))) return st;
+  if ((st = pp_grow(ctx, 11, (size_t)cand * sizeof(FaceItem)))) return st;
+  FaceItem *items = (FaceItem *)ctx->pp_buf[11];
   FaceTab f;
   f.keys = (unsigned long long *)ctx->pp_buf[14];
   f.lo = (int32_t *)(f.keys + 2 * fcap);
@@ -1265,8 +1307,11 @@ zef_status build_surface_adjacency(zef_ctx *ctx, const int32_t *tets, const int3
   CK(cudaMemsetAsync(g.keys, 0xff, (size_t)cap * sizeof(unsigned long long), s), "clear edge table");
   CK(cudaMemsetAsync(g.deg, 0, (size_t)(n + 1) * sizeof(uint32_t), s), "clear degrees");
   CK(cudaMemsetAsync(g.fill, 0, (size_t)std::max<int64_t>(n, 1) * sizeof(uint32_t), s), "clear cursors");
-  k_sf_faces<<<grid_blocks(ctx, m, 256), 256, 0, s>>>(f, tets, labels, m, n, mixed, dwords);
-  k_sf_edges<<<grid_blocks(ctx, fcap, 256), 256, 0, s>>>(f, g);
+  k_sf_list<<<grid_blocks(ctx, m, 256), 256, 0, s>>>(tets, labels, m, n, mixed, items, dwords);
+  k_sf_faces<<<grid_blocks(ctx, cand, 256), 256, 0, s>>>(f, items, dwords);
+  // the list of candidates is free again: at most half as many boundary faces
+  k_sf_boundary<<<grid_blocks(ctx, fcap, 256), 256, 0, s>>>(f, (uint4 *)items, dwords);
+  k_sf_edges<<<grid_blocks(ctx, 3 * cand / 2, 256), 256, 0, s>>>((const uint4 *)items, g);
   st = scan_exclusive(ctx, g.deg, nullptr, 1, n + 1, nullptr, (uint32_t *)ctx->pp_buf[5]);
   if (st) return st;
   uint32_t deg_sum = 0;
