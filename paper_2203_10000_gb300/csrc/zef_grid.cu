@@ -25,7 +25,7 @@
 // at registration and stored rounded to FP32 with a bound E on the error of
 // the FP32 dot products, so a test is nine multiply-adds and a few compares.
 // A decision is taken only from quantities beyond their bounds.  Anything
-// else -- a point within about 1e-6 cell widths of a triangle's plane inside
+// else -- a point within about 1e-5 cell widths of a triangle's plane inside
 // the triangle, a segment that close to an edge -- is re-evaluated in FP64
 // from the vertices (again with a bound), and what FP64 cannot decide either
 // (a point on the surface) by the FP64 solid angle over the cap tree, as the
@@ -72,6 +72,10 @@ constexpr uint32_t kMixed = kCellMixed;
 constexpr uint32_t kUnknown = 0x40000000u;
 constexpr int kChunkShift = kCellChunkShift;
 constexpr uint32_t kOffsetMask = kCellOffset;
+// W = v_ab + v_bc + v_ca - V, the point's side of the plane, is off by at most
+// 8 E; four times that is left to FP64, so that it decides wherever the point is
+// within about 1e-5 cell widths of a triangle.
+constexpr float kPlane = 32.f;
 constexpr int kNoK = -128;  // block header: the anchor's winding number is unknown
 // A block: a header (anchor x, y, z; k in the low 8 bits of w and the number
 // of chunks above), then chunks of kSub entries: kSub first words (a x b, V),
@@ -238,7 +242,7 @@ __global__ void __launch_bounds__(256) k_gr_finish(const float4 *tris, float to_
     }
     for (uint32_t j = b + lane; j < b + chunks * kSub; j += 32) {
       float4 *o = block + 1 + (j - b) / kSub * kChunkWords + (j - b) % kSub;
-      if (j >= e) {  // V > E > 0 and W = -V < -8 E: the segment ends before the plane
+      if (j >= e) {  // V > E > 0 and W = -V < -kPlane E: the segment ends before the plane
         o[0] = make_float4(0.f, 0.f, 0.f, 1.f);
         o[kSub] = make_float4(0.f, 0.f, 0.f, 0.01f);
         o[2 * kSub] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
@@ -600,7 +604,7 @@ __device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, c
             const float v0 = fmaf(n0.x, dx, fmaf(n0.y, dy, n0.z * dz));
             const float v1 = fmaf(n1.x, dx, fmaf(n1.y, dy, n1.z * dz));
             const float v2 = fmaf(n2.x, dx, fmaf(n2.y, dy, n2.z * dz));
-            const float V = n0.w, E = n1.w, EW = 8.f * n1.w, W = (v0 + v1 + v2) - V;
+            const float V = n0.w, E = n1.w, EW = kPlane * n1.w, W = (v0 + v1 + v2) - V;
             const float mn = fminf(v0, fminf(v1, v2)), mx = fmaxf(v0, fmaxf(v1, v2));
             const bool vp = V > E, vn = V < -E, wp = W > EW, wn = W < -EW;
             const bool cross_out = vp && wp && mn > E, cross_in = vn && wn && mx < -E;
@@ -660,9 +664,10 @@ __device__ __forceinline__ typename FieldCell<WIDE>::T field_cell(const GridArgs
   c.y = 0;
   *in_box = x >= a.ub.lo[0] && x <= a.ub.hi[0] && y >= a.ub.lo[1] && y <= a.ub.hi[1] && z >= a.ub.lo[2] && z <= a.ub.hi[2];
   if (*in_box) {
-    const int cx = axis_cell(x, a.field.lo[0], a.field.inv[0], a.field.n[0]),
-              cy = axis_cell(y, a.field.lo[1], a.field.inv[1], a.field.n[1]),
-              cz = axis_cell(z, a.field.lo[2], a.field.inv[2], a.field.n[2]);
+    // x >= lo: no cell below the first
+    const int cx = min((int)((x - a.field.lo[0]) * a.field.inv[0]), a.field.n[0] - 1),
+              cy = min((int)((y - a.field.lo[1]) * a.field.inv[1]), a.field.n[1] - 1),
+              cz = min((int)((z - a.field.lo[2]) * a.field.inv[2]), a.field.n[2] - 1);
     c = __ldg(reinterpret_cast<const typename FieldCell<WIDE>::T *>(a.field.cells) +
               ((cz * a.field.n[1] + cy) * a.field.n[0] + cx));
   }
@@ -793,56 +798,81 @@ __global__ void __launch_bounds__(kGlThreads, 4) k_grid_label(GridArgs a) {
 // Two launches (large calls).  Streaming: labels of the points that the field
 // decides (12 bytes in, 4 out per point, the field from L2; few registers, so
 // many loads in flight); the indices of the others are listed, a warp's
-// consecutive points in runs of at least kGsFlush.
-template <bool WIDE>
+// consecutive points in runs of at least kGsFlush.  PLAIN: labels alone, no
+// solid angles, inside bits or statistics -- the issue slots bound the
+// streaming (four of five busy at 116 instructions per 32 points), so that
+// form leaves everything else out.
+template <bool WIDE, bool PLAIN>
 __global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
   using M = typename FieldCell<WIDE>::M;
-  __shared__ int32_t s_id[ZEF_MAX_COMPARTMENTS];
+  __shared__ int32_t s_id[ZEF_MAX_COMPARTMENTS + 1];  // label by the number of the first row + 1, 0: none
   __shared__ int32_t s_q[kGlWarps][kGsQueue];
   __shared__ unsigned long long s_stat[kGlWarps][GS_COUNT];
-  for (int j = threadIdx.x; j < a.ncomp; j += kGlThreads) s_id[j] = a.row_ids[j];
+  for (int j = threadIdx.x; j <= a.ncomp; j += kGlThreads) s_id[j] = j ? a.row_ids[j - 1] : 0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   __syncthreads();
   const int64_t n = a.n_host >= 0 ? a.n_host : a.counters[CNT_N];
   const int64_t off = a.n_host >= 0 ? 0 : a.counters[CNT_OFF];
-  const float *pts = a.pts + 3 * off;
   int queued = 0;
   LaneStats st;
   const int64_t first = ((int64_t)blockIdx.x * kGlWarps + wid) * a.iters * kGsTile;
-  const int64_t end = min(n, first + (int64_t)a.iters * kGsTile);
-  for (int64_t base = first; base < end; base += kGsTile) {
+  const int count = (int)(min(n, first + (int64_t)a.iters * kGsTile) - first);  // this warp's points, if positive
+  const float *p = a.pts + 3 * (off + first + lane);
+  int32_t *lab = a.labels + off + first + lane;
+  for (int base = 0; base < count; base += kGsTile, p += 3 * kGsTile, lab += kGsTile) {
     float x[kGsP], y[kGsP], z[kGsP];
     bool in_box[kGsP];
     typename FieldCell<WIDE>::T c[kGsP];
+    if (base + kGsTile <= count) {
 #pragma unroll
-    for (int u = 0; u < kGsP; ++u) {
-      const int64_t i = base + 32 * u + lane;
-      x[u] = y[u] = z[u] = __int_as_float(0x7fc00000);
-      if (i < end) {
-        x[u] = __ldcs(pts + 3 * i);
-        y[u] = __ldcs(pts + 3 * i + 1);
-        z[u] = __ldcs(pts + 3 * i + 2);
+      for (int u = 0; u < kGsP; ++u) {
+        x[u] = __ldcs(p + 96 * u);
+        y[u] = __ldcs(p + 96 * u + 1);
+        z[u] = __ldcs(p + 96 * u + 2);
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < kGsP; ++u) {
+        x[u] = y[u] = z[u] = __int_as_float(0x7fc00000);
+        if (base + 32 * u + lane < count) {
+          x[u] = p[96 * u];
+          y[u] = p[96 * u + 1];
+          z[u] = p[96 * u + 2];
+        }
       }
     }
 #pragma unroll
     for (int u = 0; u < kGsP; ++u) c[u] = field_cell<WIDE>(a, x[u], y[u], z[u], &in_box[u]);
 #pragma unroll
     for (int u = 0; u < kGsP; ++u) {
-      const int64_t i = base + 32 * u + lane;
       const M ins = c[u].x, mix = c[u].y;
-      const bool fin = isfinite(x[u]) && isfinite(y[u]) && isfinite(z[u]);
-      const bool open = open_rows<M>(ins, mix, a.early) != 0;
-      if (a.stats) {
-        st.coh += sizeof(M) == 8 ? __popcll(ins) : __popc((uint32_t)ins);
-        st.nin += in_box[u] ? 1 : 0;
-        st.nonfin += i < end && !fin ? 1 : 0;
+      const int row1 = sizeof(M) == 8 ? __ffsll((long long)ins) : __ffs((int)ins);
+      if (PLAIN) {
+        // a point with a non-finite coordinate is in no box
+        const bool open = open_rows<M>(ins, mix, 1) != 0;
+        int32_t l = s_id[row1];
+        if (!in_box[u] && !(isfinite(x[u]) && isfinite(y[u]) && isfinite(z[u]))) l = -1;
+        if (!open && base + 32 * u + lane < count) lab[32 * u] = l;
+        const uint32_t ob = __ballot_sync(0xffffffffu, open);
+        if (open) s_q[wid][queued + __popc(ob & ((1u << lane) - 1u))] = (int32_t)(first + base + 32 * u + lane);
+        queued += __popc(ob);
+      } else {
+        const int64_t i = first + base + 32 * u + lane;
+        const bool valid = base + 32 * u + lane < count;
+        const bool fin = isfinite(x[u]) && isfinite(y[u]) && isfinite(z[u]);
+        const bool open = open_rows<M>(ins, mix, a.early) != 0;
+        if (a.stats) {
+          st.coh += sizeof(M) == 8 ? __popcll(ins) : __popc((uint32_t)ins);
+          st.nin += in_box[u] ? 1 : 0;
+          st.nonfin += valid && !fin ? 1 : 0;
+        }
+        if (valid) field_store<WIDE>(a, s_id + 1, off, i, ins, mix, fin, open);
+        const uint32_t ob = __ballot_sync(0xffffffffu, open);
+        if (open) s_q[wid][queued + __popc(ob & ((1u << lane) - 1u))] = (int32_t)i;
+        queued += __popc(ob);
       }
-      if (i < end) field_store<WIDE>(a, s_id, off, i, ins, mix, fin, open);
-      const uint32_t ob = __ballot_sync(0xffffffffu, open);
-      if (open) s_q[wid][queued + __popc(ob & ((1u << lane) - 1u))] = (int32_t)i;
-      queued += __popc(ob);
     }
-    if (queued >= kGsFlush || (base + kGsTile >= end && queued > 0)) {
+    if (queued >= kGsFlush || (base + kGsTile >= count && queued > 0)) {
       __syncwarp();
       unsigned long long at = 0;
       if (lane == 0) at = atomicAdd((unsigned long long *)(a.counters + CNT_PEND), (unsigned long long)queued);
@@ -852,7 +882,7 @@ __global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
       __syncwarp();
     }
   }
-  if (a.stats) flush_stats(a, st, s_stat, wid, lane);
+  if (!PLAIN && a.stats) flush_stats(a, st, s_stat, wid, lane);
 }
 
 // The listed points, 32 at a time.
@@ -973,13 +1003,12 @@ zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
     a.iters = (int)std::min<int64_t>(kGlMaxIters, std::max<int64_t>(1, tiles / ((int64_t)ctx->num_sms * 16 * kGlWarps)));
     const unsigned blocks = (unsigned)((tiles + (int64_t)a.iters * kGlWarps - 1) / ((int64_t)a.iters * kGlWarps));
     const unsigned pblocks = (unsigned)std::min<int64_t>((plan.n_cap + kGlThreads - 1) / kGlThreads, (int64_t)ctx->num_sms * 16);
-    if (wide) {
-      k_grid_stream<true><<<blocks, kGlThreads, 0, s>>>(a);
-      k_grid_pending<true><<<pblocks, kGlThreads, 0, s>>>(a);
-    } else {
-      k_grid_stream<false><<<blocks, kGlThreads, 0, s>>>(a);
-      k_grid_pending<false><<<pblocks, kGlThreads, 0, s>>>(a);
-    }
+    const bool plain = !a.omega && !a.masks && !a.stats && a.early;
+    auto stream = wide ? (plain ? k_grid_stream<true, true> : k_grid_stream<true, false>)
+                       : (plain ? k_grid_stream<false, true> : k_grid_stream<false, false>);
+    stream<<<blocks, kGlThreads, 0, s>>>(a);
+    if (wide) k_grid_pending<true><<<pblocks, kGlThreads, 0, s>>>(a);
+    else k_grid_pending<false><<<pblocks, kGlThreads, 0, s>>>(a);
     ctx->launches += 2;
   } else {
     a.iters = 1;
