@@ -193,8 +193,9 @@ zef_status zef_create(zef_ctx **out, int device, void *cuda_stream) {
     if (e != cudaSuccess) { st = cuda_fail(ctx, e, "cudaMalloc(status)"); break; }
     e = cudaMemset(ctx->d_status, 0, 4 * sizeof(uint32_t));
     if (e != cudaSuccess) { st = cuda_fail(ctx, e, "cudaMemset(status)"); break; }
-    e = cudaMallocHost(&ctx->h_counters, CNT_COUNT_ * sizeof(int64_t));
+    e = cudaMallocHost(&ctx->h_counters, CNT_COUNT_ * sizeof(int64_t) + 16);
     if (e != cudaSuccess) { st = cuda_fail(ctx, e, "cudaMallocHost"); break; }
+    ctx->h_status = reinterpret_cast<uint32_t *>(ctx->h_counters + CNT_COUNT_);
     if ((st = upload_dop_directions(ctx)) != ZEF_OK) break;
     for (auto &ev : ctx->ev) {
       e = cudaEventCreate(&ev);
@@ -252,6 +253,7 @@ void zef_destroy(zef_ctx *ctx) {
   if (ctx->rb_exec) cudaGraphExecDestroy(ctx->rb_exec);
   if (ctx->rf_exec) cudaGraphExecDestroy(ctx->rf_exec);
   if (ctx->h_counters) cudaFreeHost(ctx->h_counters);
+  if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
   for (auto &ev : ctx->ev)
     if (ev) cudaEventDestroy(ev);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
@@ -527,13 +529,16 @@ zef_status zef_synchronize(zef_ctx *ctx) {
   if (!ctx) return ZEF_ERR_INVALID_ARG;
   if (ctx->device == ZEF_HOST_ONLY) return ZEF_OK;
   DeviceGuard g(ctx->device);
+  // the status words come over behind the work: one wait instead of two (every
+  // kernel runs on the context's stream)
+  CK(cudaMemcpyAsync(ctx->h_status, ctx->d_status, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream),
+     "read status");
   CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
   if (ctx->s_in) {
     CK(cudaStreamSynchronize(ctx->s_in), "cudaStreamSynchronize(copy-in)");
     CK(cudaStreamSynchronize(ctx->s_out), "cudaStreamSynchronize(copy-out)");
   }
-  uint32_t st[2] = {0, 0};
-  CK(cudaMemcpy(st, ctx->d_status, sizeof(st), cudaMemcpyDeviceToHost), "read status");
+  const uint32_t st[2] = {ctx->h_status[0], ctx->h_status[1]};
   if (st[0]) {
     CK(cudaMemset(ctx->d_status, 0, 2 * sizeof(uint32_t)), "clear status");
     if (st[0] & ST_TIMEOUT)
@@ -761,6 +766,10 @@ zef_status label_points_async_impl(zef_ctx *ctx, const float *pts, int64_t n, in
   return ZEF_OK;
 }
 
+constexpr int64_t kPinnedPoints = 1 << 16;
+static zef_status read_stats(zef_ctx *ctx, int64_t n, const zef_label_opts &o, const LaunchShape &shape,
+                             int64_t launches, zef_label_stats *stats);
+
 zef_status label_points_impl(zef_ctx *ctx, const float *pts, int64_t n, int32_t *labels, float *omega,
                              const zef_label_opts *opts, zef_label_stats *stats, unsigned long long *d_masks,
                              bool full_masks) {
@@ -776,8 +785,27 @@ zef_status label_points_impl(zef_ctx *ctx, const float *pts, int64_t n, int32_t 
   const int C = (int)ctx->comps.size();
   bool dpts = is_device_ptr(pts, ctx->device);
   bool dlab = is_device_ptr(labels, ctx->device);
-  st = reserve_call(ctx, n, o, !dpts || !dlab);
+  // Small host calls: the kernel reads the points from, and writes the labels
+  // to, pinned host memory, so the call is two host copies, one launch and one
+  // wait.
+  const bool small = !dpts && !dlab && !omega && n <= kPinnedPoints && grid_serves(ctx, o);
+  st = reserve_call(ctx, n, o, (!dpts || !dlab) && !small);
   if (st) return st;
+  if (small) {
+    if (!ctx->h_stage)
+      CK(cudaMallocHost(&ctx->h_stage, (size_t)kPinnedPoints * (3 * sizeof(float) + sizeof(int32_t))),
+         "cudaMallocHost(staging)");
+    float *hp = reinterpret_cast<float *>(ctx->h_stage);
+    int32_t *hl = reinterpret_cast<int32_t *>(hp + 3 * kPinnedPoints);
+    std::memcpy(hp, pts, (size_t)n * 3 * sizeof(float));
+    LaunchShape shape;
+    int64_t launches = 0;
+    st = enqueue_labeling(ctx, hp, n, hl, nullptr, o, d_masks, full_masks, stats != nullptr, &shape, &launches);
+    if (!st) st = zef_synchronize(ctx);
+    if (st) return st;
+    std::memcpy(labels, hl, (size_t)n * sizeof(int32_t));
+    return stats ? read_stats(ctx, n, o, shape, launches, stats) : ZEF_OK;
+  }
   bool dom = omega ? is_device_ptr(omega, ctx->device) : true;
   LabelBuffers &b = ctx->lb;
   const float *d_pts = pts;
@@ -812,36 +840,40 @@ zef_status label_points_impl(zef_ctx *ctx, const float *pts, int64_t n, int32_t 
     st = zef_synchronize(ctx);
     if (st) return st;
   }
-  if (stats) {
-    CK(cudaMemcpy(ctx->h_counters, b.counters, CNT_COUNT_ * sizeof(int64_t), cudaMemcpyDeviceToHost),
-       "read counters");
-    const int64_t *h = ctx->h_counters;
-    stats->points = n;
-    stats->nonfinite_points = h[CNT_NONFINITE];
-    int64_t tt = 0;
-    for (auto &c : ctx->comps) tt += c.nt;
-    stats->pairs_nominal = n * tt;
-    stats->pairs_rescued = h[CNT_PAIRS_RESCUE];
-    stats->pairs_evaluated = h[CNT_PAIRS_EVAL] + h[CNT_PAIRS_RESCUE];
-    stats->uncertain_pairs = h[CNT_UNC];
-    stats->work_items = h[CNT_ITEMS];
-    // the cell grid's tiles: 64 consecutive points each, as many as the
-    // points inside the union box would fill
-    stats->tiles = grid_serves(ctx, o) ? (h[CNT_NIN] + 63) / 64 : h[CNT_TILES];
-    stats->coherent_pairs = h[CNT_COHERENT];
-    stats->representative_pairs = h[CNT_REP_PAIRS];
-    stats->lane_walk_items = h[CNT_LANE_TILES];
-    stats->kernel_launches = launches;
-    stats->block_threads = shape.threads;
-    stats->points_per_thread = shape.ppt;
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[5]);
-    stats->ms_total = ms;
-    cudaEventElapsedTime(&ms, ctx->ev[1], ctx->ev[2]);
-    stats->ms_label = ms;
-    cudaEventElapsedTime(&ms, ctx->ev[3], ctx->ev[4]);
-    stats->ms_rescue = ms;
-  }
+  return stats ? read_stats(ctx, n, o, shape, launches, stats) : ZEF_OK;
+}
+
+// the statistics of a synchronized call
+static zef_status read_stats(zef_ctx *ctx, int64_t n, const zef_label_opts &o, const LaunchShape &shape,
+                             int64_t launches, zef_label_stats *stats) {
+  CK(cudaMemcpy(ctx->h_counters, ctx->lb.counters, CNT_COUNT_ * sizeof(int64_t), cudaMemcpyDeviceToHost),
+     "read counters");
+  const int64_t *h = ctx->h_counters;
+  stats->points = n;
+  stats->nonfinite_points = h[CNT_NONFINITE];
+  int64_t tt = 0;
+  for (auto &c : ctx->comps) tt += c.nt;
+  stats->pairs_nominal = n * tt;
+  stats->pairs_rescued = h[CNT_PAIRS_RESCUE];
+  stats->pairs_evaluated = h[CNT_PAIRS_EVAL] + h[CNT_PAIRS_RESCUE];
+  stats->uncertain_pairs = h[CNT_UNC];
+  stats->work_items = h[CNT_ITEMS];
+  // the cell grid's tiles: 64 consecutive points each, as many as the
+  // points inside the union box would fill
+  stats->tiles = grid_serves(ctx, o) ? (h[CNT_NIN] + 63) / 64 : h[CNT_TILES];
+  stats->coherent_pairs = h[CNT_COHERENT];
+  stats->representative_pairs = h[CNT_REP_PAIRS];
+  stats->lane_walk_items = h[CNT_LANE_TILES];
+  stats->kernel_launches = launches;
+  stats->block_threads = shape.threads;
+  stats->points_per_thread = shape.ppt;
+  float ms = 0.f;
+  cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[5]);
+  stats->ms_total = ms;
+  cudaEventElapsedTime(&ms, ctx->ev[1], ctx->ev[2]);
+  stats->ms_label = ms;
+  cudaEventElapsedTime(&ms, ctx->ev[3], ctx->ev[4]);
+  stats->ms_rescue = ms;
   return ZEF_OK;
 }
 

@@ -308,6 +308,8 @@ struct zef_ctx {
   uint32_t *d_status = nullptr;       // [2]
   zef::LabelBuffers lb;
   int64_t *h_counters = nullptr;      // pinned mirror of the counters
+  uint32_t *h_status = nullptr;       // pinned mirror of the status words
+  unsigned char *h_stage = nullptr;   // pinned points and labels of small host calls
 
   cudaEvent_t ev[6] = {};
   std::vector<zef::CompGrid> grids;   // cell grids, by compartment
