@@ -104,8 +104,22 @@ struct Geom {
 
 __device__ __forceinline__ float4 raw_vertex(float4 v, float s) { return make_float4(v.x * s, v.y * s, v.z * s, 0.f); }
 
+// True when the projections of the triangle (vertices v relative to the cell's
+// centre) and of the cell (half extents r) on axis edge x e_d separate them.
+// FP32: its error, a few 2^-24 of the triangle's size (at most kMaxAxis cells),
+// is far below the growth in r.
+__device__ __forceinline__ bool axis_separates(const float (&v)[3][3], const float (&edge)[3], int d, const float (&r)[3]) {
+  const int d1 = (d + 1) % 3, d2 = (d + 2) % 3;  // e_d x edge = (0, -edge_d2, edge_d1) on (d, d1, d2)
+  const float a1 = -edge[d2], a2 = edge[d1];
+  const float p0 = a1 * v[0][d1] + a2 * v[0][d2], p1 = a1 * v[1][d1] + a2 * v[1][d2], p2 = a1 * v[2][d1] + a2 * v[2][d2];
+  const float reach = fabsf(a1) * r[d1] + fabsf(a2) * r[d2];
+  return fminf(p0, fminf(p1, p2)) > reach || fmaxf(p0, fmaxf(p1, p2)) < -reach;
+}
+
 // Triangles of every cell: one warp per triangle, the lanes over the cells of
-// its box; a cell counts when the triangle's plane meets the grown cell.  The
+// its box; a cell counts unless one of the separating axes of a triangle and a
+// box (the box's own by the choice of the cells, the triangle's normal, the
+// products of their edges) separates the triangle from the grown cell.  The
 // first pass counts (list null), the second, from the scanned counts, fills:
 // one kernel, so that both take the same cells.
 __global__ void __launch_bounds__(256) k_gr_refs(const float4 *tris, float to_raw, int nt, Geom g, uint32_t *cnt,
@@ -142,6 +156,24 @@ __global__ void __launch_bounds__(256) k_gr_refs(const float4 *tris, float to_ra
       const double dist = nrm[0] * (g.lo[0] + (x + 0.5) * g.h[0] - A[0]) + nrm[1] * (g.lo[1] + (y + 0.5) * g.h[1] - A[1]) +
                           nrm[2] * (g.lo[2] + (z + 0.5) * g.h[2] - A[2]);
       if (fabs(dist) > reach) continue;
+      const double ctr[3] = {g.lo[0] + (x + 0.5) * g.h[0], g.lo[1] + (y + 0.5) * g.h[1], g.lo[2] + (z + 0.5) * g.h[2]};
+      float rel[3][3], half[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        rel[k][0] = (float)(v[k].x - ctr[0]);
+        rel[k][1] = (float)(v[k].y - ctr[1]);
+        rel[k][2] = (float)(v[k].z - ctr[2]);
+        half[k] = (float)(g.h[k] * (0.5 + kGrow));
+      }
+      bool apart = false;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const float edge[3] = {rel[(k + 1) % 3][0] - rel[k][0], rel[(k + 1) % 3][1] - rel[k][1],
+                               rel[(k + 1) % 3][2] - rel[k][2]};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) apart |= axis_separates(rel, edge, d, half);
+      }
+      if (apart) continue;
       const int64_t c = ((int64_t)z * g.n[1] + y) * g.n[0] + x;
       const uint32_t pos = atomicAdd(cnt + c, 1u);
       if (list) list[pos] = (int32_t)t;
@@ -1033,9 +1065,13 @@ void grid_free(zef_ctx *ctx) {
     if (g.blob) cudaFree(g.blob);
   ctx->grids.clear();
   if (ctx->d_grid) cudaFree(ctx->d_grid);
-  if (ctx->field.cells) cudaFree(ctx->field.cells);
+  if (ctx->field_mem) cudaFree(ctx->field_mem);
+  for (void *&p : ctx->gr_buf) {
+    if (p) cudaFree(p);
+    p = nullptr;
+  }
   ctx->d_grid = nullptr;
-  ctx->field.cells = nullptr;
+  ctx->field.cells = ctx->field_mem = nullptr;
 }
 
 // Cell grid of compartment c (uploaded, with its cap tree).  Cells are one
@@ -1087,14 +1123,22 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   const int64_t bs = cells / 2048 + 2;
   const size_t o_flag = (size_t)cells * 4, o_sum = o_flag + (size_t)cells * 4, o_tot = (o_sum + (size_t)bs * 4 + 15) & ~(size_t)15,
                o_anch = o_tot + 32, o_om = o_anch + (size_t)cells * 12, bytes = o_om + (size_t)cells * 4;
-  unsigned char *tmp = nullptr;
   auto no_memory = [&](cudaError_t e) {
     cudaGetLastError();
-    if (tmp) cudaFree(tmp);
     return e == cudaErrorMemoryAllocation ? ZEF_OK : cuda_fail(ctx, e, "cell grid");
   };
-  cudaError_t e = cudaMalloc(&tmp, bytes);
+  auto scratch = [](void **p, size_t *cap, size_t need) {
+    if (*cap >= need) return cudaSuccess;
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+    *cap = 0;
+    const cudaError_t e = cudaMalloc(p, need);
+    if (e == cudaSuccess) *cap = need;
+    return e;
+  };
+  cudaError_t e = scratch(&ctx->gr_buf[0], &ctx->gr_cap[0], bytes);
   if (e != cudaSuccess) return no_memory(e);
+  unsigned char *tmp = (unsigned char *)ctx->gr_buf[0];
   uint32_t *cnt = (uint32_t *)tmp, *flag = (uint32_t *)(tmp + o_flag), *bsum = (uint32_t *)(tmp + o_sum);
   int64_t *tot = (int64_t *)(tmp + o_tot);
   float *anchor = (float *)(tmp + o_anch), *omega = (float *)(tmp + o_om);
@@ -1112,25 +1156,17 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) zs = cuda_fail(ctx, e, "cell grid");
   }
-  if (zs) {
-    cudaFree(tmp);
-    return zs;
-  }
+  if (zs) return zs;
   const int64_t refs = totals[0], words16 = totals[1];
-  if (totals[2] > kMaxList || refs > 64 * (int64_t)nt + 65536 || words16 > (int64_t)kOffsetMask) {
-    cudaFree(tmp);
+  if (totals[2] > kMaxList || refs > 64 * (int64_t)nt + 65536 || words16 > (int64_t)kOffsetMask)
     return ZEF_OK;
-  }
   // blocks and words; the triangle lists are scratch
   const size_t p_word = (size_t)words16 * 16, p_end = p_word + (size_t)cells * 4;
   unsigned char *blob = nullptr;
-  int32_t *list = nullptr;
-  e = cudaMalloc(&list, std::max<size_t>((size_t)refs * 4, 16));
+  e = scratch(&ctx->gr_buf[1], &ctx->gr_cap[1], std::max<size_t>((size_t)refs * 4, 16));
   if (e == cudaSuccess) e = cudaMalloc(&blob, p_end);
-  if (e != cudaSuccess) {
-    if (list) cudaFree(list);
-    return no_memory(e);
-  }
+  if (e != cudaSuccess) return no_memory(e);
+  int32_t *list = (int32_t *)ctx->gr_buf[1];
   k_gr_refs<<<g_t, 256, 0, st>>>(tris, to_raw, nt, g, cnt, list);  // cnt: list starts -> ends
   k_gr_anchor<<<g_w, 256, 0, st>>>(tris, to_raw, g, cells, cnt, list, anchor);
   // the anchors' solid angles of this compartment alone
@@ -1160,8 +1196,6 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   if (zs) {
     cudaStreamSynchronize(st);
     cudaFree(blob);
-    cudaFree(list);
-    cudaFree(tmp);
     if (zs != ZEF_ERR_OOM) return zs;
     cudaGetLastError();
     return ZEF_OK;
@@ -1170,8 +1204,6 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
                                    (float4 *)blob);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(tmp);
-  cudaFree(list);
   if (e != cudaSuccess) {
     cudaFree(blob);
     return cuda_fail(ctx, e, "cell grid");
@@ -1222,7 +1254,6 @@ zef_status grid_update(zef_ctx *ctx) {
 
   // the label field: cells as wide as the finest compartment grid's, at most
   // kMaxField of them (one or two 64-bit words each: it stays in L2)
-  if (ctx->field.cells) cudaFree(ctx->field.cells);
   ctx->field.cells = nullptr;
   LabelField f = {};
   float ext[3], longest = 0.f;
@@ -1251,12 +1282,20 @@ zef_status grid_update(zef_ctx *ctx) {
     f.inv[k] = ext[k] > 0.f ? (float)(f.n[k] / (double)ext[k]) : 0.f;
   }
   const bool wide = C > 32;
-  cudaError_t e = cudaMalloc(&f.cells, (size_t)cells * (wide ? sizeof(ulonglong2) : sizeof(uint2)));
-  if (e == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    return ZEF_OK;  // no field: the general kernels
+  const size_t need = (size_t)cells * (wide ? sizeof(ulonglong2) : sizeof(uint2));
+  if (ctx->field_cap < need) {
+    if (ctx->field_mem) cudaFree(ctx->field_mem);
+    ctx->field_mem = nullptr;
+    ctx->field_cap = 0;
+    cudaError_t e = cudaMalloc(&ctx->field_mem, need);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      return ZEF_OK;  // no field: the general kernels
+    }
+    CK(e, "cudaMalloc(label field)");
+    ctx->field_cap = need;
   }
-  CK(e, "cudaMalloc(label field)");
+  f.cells = ctx->field_mem;
   ctx->field = f;
   const int g_f = grid_blocks(ctx, cells, 256);
   if (wide) k_gr_field<true><<<g_f, 256, 0, ctx->stream>>>(f, ctx->d_grid, (int)C);

@@ -315,6 +315,10 @@ struct zef_ctx {
   std::vector<zef::CompGrid> grids;   // cell grids, by compartment
   zef::GridComp *d_grid = nullptr;    // by priority row
   zef::LabelField field = {};
+  void *field_mem = nullptr;          // its cells (grow-only)
+  size_t field_cap = 0;
+  void *gr_buf[2] = {};               // scratch of the grids' construction (grow-only)
+  size_t gr_cap[2] = {};
   zef::UnionBox ubox = {};            // union box of the surfaces (unscaled), set at upload
   int64_t launches = 0;               // kernels launched by the labeling pipeline (running count)
 
