@@ -760,7 +760,7 @@ __global__ void __launch_bounds__(256) k_sm_forward(Smooth s) {
     float4 o = c;
     if (!(s.fixed && s.fixed[i])) o = lap_step(s.g, s.x, i, c, s.lambda);
     s.y[i] = o;
-    if (NORM) {
+    if (NORM && s.g.fill[i]) {  // a node without neighbours does not move
       const double d0 = (double)o.x - c.x, d1 = (double)o.y - c.y, d2 = (double)o.z - c.z;
       acc += d0 * d0 + d1 * d1 + d2 * d2;
     } else {

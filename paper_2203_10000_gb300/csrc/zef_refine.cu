@@ -76,6 +76,7 @@ struct RF {
   uint32_t *hvals;
   int32_t *hids;
   uint32_t *slots;   // [6 fmax] table slot of every flagged tet's edge
+  int32_t *list;     // [fmax] the flagged tets by rank
   unsigned long long hmask;  // slots held - 1; a level uses cnt[CNT_RF_MASK] + 1 of them
   int64_t node_cap, tet_cap, fmax;
   uint32_t *status;
@@ -326,31 +327,38 @@ __global__ void __launch_bounds__(256) k_rf_clear(RF r) {
   }
 }
 
-__global__ void __launch_bounds__(256) k_rf_insert(RF r) {
+// the flagged tets by rank
+__global__ void __launch_bounds__(256) k_rf_list(RF r) {
   if (r.cnt[CNT_ABORT]) return;
   const int64_t M = r.cnt[CNT_TETS];
-  const EdgeTable tab = edge_table(r);
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < M; t += (int64_t)gridDim.x * blockDim.x) {
     uint32_t rank;
-    if (!is_flagged(r, t, M, &rank)) continue;
-    const int4 q = reinterpret_cast<const int4 *>(r.tets)[t];
-    const int32_t v[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int e = 0; e < 6; ++e) {
-      constexpr int kA[6] = {0, 0, 0, 1, 1, 2}, kB[6] = {1, 2, 3, 2, 3, 3};
-      const unsigned long long key = edge_key(v[kA[e]], v[kB[e]]);
-      const uint32_t code = rank * 6u + (uint32_t)e;
-      unsigned long long h = first_slot(tab, key);
-      for (unsigned long long it = 0; it <= tab.mask; ++it) {
-        const unsigned long long prev = atomicCAS(r.hkeys + h, kEmpty, key);
-        if (prev == kEmpty || prev == key) {
-          atomicMin(r.hvals + h, code);
-          break;
-        }
-        h = (h + 1) & tab.mask;
+    if (is_flagged(r, t, M, &rank)) r.list[rank] = (int32_t)t;
+  }
+}
+
+// one thread per edge of a flagged tet (a thread per tet waited for six swaps
+// in turn, in warps of which half the tets are not flagged: 0.36 ms for the
+// 9.8 M edges of a third level, 0.16 now)
+__global__ void __launch_bounds__(256) k_rf_insert(RF r) {
+  if (r.cnt[CNT_ABORT]) return;
+  const int64_t len = r.cnt[CNT_OWN_LEN];
+  const EdgeTable tab = edge_table(r);
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < len; c += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t rank = c / 6;
+    const int e = (int)(c - 6 * rank);
+    const int32_t *v = r.tets + 4 * (int64_t)r.list[rank];
+    const unsigned long long key = edge_key(v[e < 3 ? 0 : e < 5 ? 1 : 2], v[e < 3 ? e + 1 : e < 5 ? e - 1 : 3]);
+    unsigned long long h = first_slot(tab, key);
+    for (unsigned long long it = 0; it <= tab.mask; ++it) {
+      const unsigned long long prev = atomicCAS(r.hkeys + h, kEmpty, key);
+      if (prev == kEmpty || prev == key) {
+        atomicMin(r.hvals + h, (uint32_t)c);
+        break;
       }
-      r.slots[code] = (uint32_t)h;
+      h = (h + 1) & tab.mask;
     }
+    r.slots[c] = (uint32_t)h;
   }
 }
 
@@ -399,10 +407,9 @@ __device__ __forceinline__ float len2_rn(const float *p, const float *q) {
 
 __global__ void __launch_bounds__(256) k_rf_children(RF r) {
   if (r.cnt[CNT_ABORT]) return;
-  const int64_t M = r.cnt[CNT_TETS];
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < M; t += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t rank;
-    if (!is_flagged(r, t, M, &rank)) continue;
+  const int64_t M = r.cnt[CNT_TETS], F = r.cnt[CNT_LEVEL_FLAGGED];
+  for (int64_t rank = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; rank < F; rank += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = r.list[rank];
     int32_t loc[10];
     const int4 q4 = reinterpret_cast<const int4 *>(r.tets)[t];
     loc[0] = q4.x;
@@ -410,7 +417,7 @@ __global__ void __launch_bounds__(256) k_rf_children(RF r) {
     loc[2] = q4.z;
     loc[3] = q4.w;
 #pragma unroll
-    for (int e = 0; e < 6; ++e) loc[4 + e] = r.hids[r.slots[(int64_t)rank * 6 + e]];
+    for (int e = 0; e < 6; ++e) loc[4 + e] = r.hids[r.slots[rank * 6 + e]];
     float l[3];
     for (int d = 0; d < 3; ++d)
       l[d] = len2_rn(r.nodes + 3 * (int64_t)loc[c_diag[d][0]], r.nodes + 3 * (int64_t)loc[c_diag[d][1]]);
@@ -418,7 +425,7 @@ __global__ void __launch_bounds__(256) k_rf_children(RF r) {
     if (l[1] < l[diag]) diag = 1;
     if (l[2] < l[diag]) diag = 2;
     for (int c = 0; c < 8; ++c) {
-      const int64_t dst = c == 0 ? t : M + 7 * (int64_t)rank + (c - 1);
+      const int64_t dst = c == 0 ? t : M + 7 * rank + (c - 1);
       const int4 q = make_int4(loc[c_child[diag][c][0]], loc[c_child[diag][c][1]], loc[c_child[diag][c][2]],
                                loc[c_child[diag][c][3]]);
       reinterpret_cast<int4 *>(r.tets)[dst] = q;
@@ -667,7 +674,7 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
   if ((st = grow(ctx, 1, (size_t)std::max<int64_t>(6 * fmax, 1) * sizeof(uint32_t)))) return st;  // owned
   if ((st = grow(ctx, 2, (size_t)hcap * (sizeof(unsigned long long) + 2 * sizeof(uint32_t))))) return st;
   if ((st = grow(ctx, 3, (size_t)bs_len * sizeof(uint32_t)))) return st;
-  if ((st = grow(ctx, 10, (size_t)std::max<int64_t>(6 * fmax, 1) * sizeof(uint32_t)))) return st;  // slots
+  if ((st = grow(ctx, 10, (size_t)std::max<int64_t>(7 * fmax, 1) * sizeof(uint32_t)))) return st;  // slots, list
   if ((st = grow(ctx, 4, (size_t)std::max(levels, 1) * kLevelStats * sizeof(int64_t)))) return st;
   if (conforming) {
     if ((st = grow(ctx, 8, (size_t)std::max<int64_t>(tcap, 1)))) return st;                     // state
@@ -724,6 +731,7 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
   r.hids = (int32_t *)(r.hvals + hcap);
   r.hmask = (unsigned long long)(hcap - 1);
   r.slots = (uint32_t *)ctx->rf_buf[10];
+  r.list = (int32_t *)(r.slots + 6 * fmax);
   r.node_cap = ncap;
   r.tet_cap = tcap;
   r.fmax = fmax;
@@ -784,7 +792,8 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
           if (st) break;
           k_rf_check<<<1, 32, 0, cap>>>(r);
           if (!conforming) k_rf_clear<<<grid_blocks(ctx, hcap / 4, 256), 256, 0, cap>>>(r);
-          k_rf_insert<<<g_t, 256, 0, cap>>>(r);
+          k_rf_list<<<g_t, 256, 0, cap>>>(r);
+          k_rf_insert<<<g_e, 256, 0, cap>>>(r);
           k_rf_owner<<<g_e, 256, 0, cap>>>(r);
           st = scan_exclusive(ctx, r.owned, b.counters + CNT_OWN_LEN, 1, std::max<int64_t>(6 * fmax, 1),
                               b.counters + CNT_LEVEL_NEW, bsums);
@@ -810,7 +819,7 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
           p.timed = false;
           st = label_enqueue(ctx, p);
           if (st) break;
-          k_rf_children<<<g_t, 256, 0, cap>>>(r);
+          k_rf_children<<<grid_blocks(ctx, std::max<int64_t>(fmax, 1), 256), 256, 0, cap>>>(r);
           if (conforming) k_cl_children<<<g_t, 256, 0, cap>>>(r);
           k_rf_advance<<<1, 32, 0, cap>>>(r, lv);
         }
