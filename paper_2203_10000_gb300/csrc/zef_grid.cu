@@ -418,14 +418,50 @@ __device__ __noinline__ bool resolve64(const GridArgs &a, const GridComp &g, uin
   // leaves whose box holds it
   const DevComp *cp = a.comps + g.comp;
   const float px = x * a.scale, py = y * a.scale, pz = z * a.scale;
-  // the groups of four entries in the order of the list kernel's block of 256
+  // The groups of four entries in the order of the list kernel's block of 256
   // threads (thread g mod 256 takes group g; the sums of each 32 threads, then
   // of the eight in turn), so that a point on the surface, whose Omega is 2 pi
-  // up to rounding, gets that kernel's rounding
+  // up to rounding, gets that kernel's rounding.  The walk's segments are a
+  // few groups each: every lane holds one, and each time they hold 32 groups
+  // together the lanes take one each (segment by segment a pair took 0.4 ms).
   double part[8];
 #pragma unroll
   for (int w = 0; w < 8; ++w) part[w] = 0.0;
-  int K = 0, tris = 0, g0 = 0;
+  int K = 0, tris = 0;
+  int seg_b = 0, seg_n = 0;           // this lane's segment: first entry, groups left
+  int segs = 0, held = 0, round = 0;  // segments and groups held, batches taken
+  auto take = [&]() {                 // the first 32 groups held (fewer at the end)
+    int end = seg_n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += t;
+    }
+    const int first = end - seg_n;
+    int pos = -1;
+    for (int q = 0; q < segs; ++q) {
+      const int f = __shfl_sync(0xffffffffu, first, q), e = __shfl_sync(0xffffffffu, end, q),
+                b = __shfl_sync(0xffffffffu, seg_b, q);
+      if (lane >= f && lane < e) pos = b + 4 * (lane - f);
+    }
+    if (pos >= 0) {
+      const double h = group64(a.cseg, pos, px, py, pz, &K);
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (q == (round & 7)) part[q] += h;
+    }
+    ++round;
+    const int used = min(max(32 - first, 0), seg_n);
+    seg_b += 4 * used;
+    seg_n -= used;
+    held = max(held - 32, 0);
+    // the empty segments are the first ones
+    const int gone = __popc(__ballot_sync(0xffffffffu, lane < segs && seg_n == 0));
+    const int nb = __shfl_sync(0xffffffffu, seg_b, (lane + gone) & 31), nn = __shfl_sync(0xffffffffu, seg_n, (lane + gone) & 31);
+    segs -= gone;
+    seg_b = nb;
+    seg_n = lane < segs ? nn : 0;
+  };
   const int root = cp->cap_root, end = a.nodes[root].skip;
   for (int i = root; i != end;) {
     const CapNode nd = a.nodes[i];
@@ -441,15 +477,16 @@ __device__ __noinline__ bool resolve64(const GridArgs &a, const GridComp &g, uin
     }
     tris += far ? nd.cap_tris : nd.leaf_tris;
     i = nd.skip;
-    for (int j = (lane - g0) & 31; j < c / 4; j += 32) {
-      const double h = group64(a.cseg, b + 4 * j, px, py, pz, &K);
-      const int w = ((g0 + j) >> 5) & 7;
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (q == w) part[q] += h;
+    if (c < 4) continue;
+    if (lane == segs) {  // at most 31 are held here: a segment has at least one group
+      seg_b = b;
+      seg_n = c / 4;
     }
-    g0 += c / 4;
+    ++segs;
+    held += c / 4;
+    while (held >= 32) take();
   }
+  if (held > 0) take();
   double sum = 0.0;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
@@ -1096,12 +1133,17 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   double w = 1.0 * std::sqrt(h.area / (0.43 * (double)h.nt));
   w = std::min(w, (double)longest / 8.0);
   w = std::max(w, (double)longest / kMaxAxis);
+  // a cell is many float32 steps wide on every axis it divides, so that its
+  // anchor, rounded to float32, stays inside
+  double finest[3];
+  for (int k = 0; k < 3; ++k)
+    finest[k] = std::max(1.0, std::floor((double)ext[k] * 65536.0 / std::max(std::fabs(h.lo[k]), std::fabs(h.hi[k]))));
   Geom g;
   int64_t cells = 0;
   for (;; w *= 1.1) {
     cells = 1;
     for (int k = 0; k < 3; ++k) {
-      g.n[k] = (int)std::min<double>(kMaxAxis, std::max(1.0, std::ceil(ext[k] / w)));
+      g.n[k] = (int)std::min<double>(std::min<double>(kMaxAxis, finest[k]), std::max(1.0, std::ceil(ext[k] / w)));
       cells *= g.n[k];
     }
     if (cells <= kMaxCells) break;
@@ -1224,12 +1266,16 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
 // priority order (the surfaces are uploaded).
 zef_status grid_update(zef_ctx *ctx) {
   const size_t C = ctx->comps.size();
+  const int64_t held = ctx->lb.cap_points;
   while (ctx->grids.size() < C) {
     CompGrid g;
     zef_status st = grid_build(ctx, ctx->grids.size(), &g);
     if (st) return st;
     ctx->grids.push_back(g);
   }
+  // the anchors' work buffers, where they are large: calls that the grids
+  // serve need none
+  if (ctx->lb.cap_points > held && ctx->lb.cap_points > (int64_t)1 << 20) label_release(ctx);
   if (!ctx->d_grid) CK(cudaMalloc(&ctx->d_grid, ZEF_MAX_COMPARTMENTS * sizeof(GridComp)), "cudaMalloc(cell grids)");
   std::vector<GridComp> d(C);
   for (size_t c = 0; c < C; ++c) {

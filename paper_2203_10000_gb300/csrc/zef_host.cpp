@@ -1043,6 +1043,8 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
   if (!ctx->dirty) return ZEF_OK;
   const int C = (int)ctx->comps.size();
   if (C == 0) return ZEF_OK;
+  // labelings still running read what is overwritten here
+  CK(cudaStreamSynchronize(ctx->stream), "wait before the upload");
   int64_t ne = (int64_t)ctx->h_entries.size();
   int64_t ntv = (int64_t)ctx->h_tris.size();
   if (ctx->d_entries_cap < ne) {

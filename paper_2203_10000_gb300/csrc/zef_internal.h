@@ -401,6 +401,7 @@ struct LabelPlan {
 zef_status label_reserve_counters(zef_ctx *ctx);
 zef_status label_reserve_stage(zef_ctx *ctx, int64_t n);
 zef_status label_reserve(zef_ctx *ctx, int64_t n_cap);
+void label_release(zef_ctx *ctx);  // the general kernels' work buffers
 zef_status label_enqueue(zef_ctx *ctx, const LabelPlan &plan);
 zef_status label_set_count(zef_ctx *ctx, int64_t n, int64_t off);
 zef_status launch_wait_probe(zef_ctx *ctx, int64_t limit_ns);

@@ -2892,6 +2892,25 @@ zef_status label_reserve_stage(zef_ctx *ctx, int64_t n) {
   return ZEF_OK;
 }
 
+void label_release(zef_ctx *ctx) {
+  LabelBuffers &b = ctx->lb;
+  cudaStreamSynchronize(ctx->stream);
+  auto fr = [](auto *&p) {
+    if (p) cudaFree(p);
+    p = nullptr;
+  };
+  fr(b.spts);
+  fr(b.perm);
+  fr(b.keys);
+  fr(b.in_mask);
+  fr(b.unc_mask);
+  fr(b.tile_box);
+  fr(b.flags);
+  fr(b.items);
+  fr(b.block_sums);
+  b.cap_points = b.cap_tiles = b.cap_items = 0;
+}
+
 // work buffers of the general kernels
 zef_status label_reserve(zef_ctx *ctx, int64_t n_cap) {
   LabelBuffers &b = ctx->lb;

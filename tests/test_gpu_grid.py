@@ -48,6 +48,8 @@ def _surfaces(name):
         return [_surf(*_join(_sphere(1.0, 6), _sphere(1.0, 6, c=(0.7, 0.1, 0.0))))]
     if name == "far_small":      # a small surface far from the origin
         return [_surf(*_sphere(0.5, 7, c=(300.0, -200.0, 100.0)))]
+    if name == "far_fine":       # cells of a few float32 steps
+        return [_surf(*_sphere(0.5, 12, c=(30000.0, -20000.0, 100.0)))]
     if name == "tiny":
         return [_surf(*_sphere(3e-5, 7, c=(1e-4, 0, 0)))]
     if name == "flat":           # one cell thick
@@ -60,7 +62,7 @@ def _surfaces(name):
     raise KeyError(name)
 
 
-NAMES = ["box", "box_grid", "tetra", "torus", "shell", "double", "far_small", "tiny", "flat", "mixed_sizes"]
+NAMES = ["box", "box_grid", "tetra", "torus", "shell", "double", "far_small", "far_fine", "tiny", "flat", "mixed_sizes"]
 
 
 def _points(surfs, n, seed):
@@ -128,7 +130,7 @@ def test_grid_labels_equal_general_kernels_and_oracle(zef, name):
     assert st["kernel_launches"] <= 2 < gst["kernel_launches"]      # the grid path, the tile kernels
     olab, oom = oracle.label_points(pts, surfs, prio)
     off = _off_surface(oracle, pts, surfs, prio, oom)
-    assert off.sum() > 0.6 * len(pts)
+    assert off.sum() > (0.1 if name == "far_fine" else 0.6) * len(pts)
     for kind, got in (("grid", lab), ("grid, early exit", early), ("general", glab), ("general, early exit", gearly)):
         bad = off & (got != olab)
         assert not bad.any(), (kind, int(bad.sum()), pts[bad][:3], got[bad][:3], olab[bad][:3])
