@@ -1275,7 +1275,7 @@ zef_status grid_update(zef_ctx *ctx) {
   }
   // the anchors' work buffers, where they are large: calls that the grids
   // serve need none
-  if (ctx->lb.cap_points > held && ctx->lb.cap_points > (int64_t)1 << 20) label_release(ctx);
+  if (ctx->lb.cap_points > held && ctx->lb.cap_points > (int64_t)1 << 22) label_release(ctx);
   if (!ctx->d_grid) CK(cudaMalloc(&ctx->d_grid, ZEF_MAX_COMPARTMENTS * sizeof(GridComp)), "cudaMalloc(cell grids)");
   std::vector<GridComp> d(C);
   for (size_t c = 0; c < C; ++c) {

@@ -5,7 +5,9 @@
 // Omega_t = 2 atan2(N, D); p is inside when Omega > 2 pi; the first
 // compartment of the priority list that encloses p labels it.
 //
-// Pipeline of one call (all on the context stream, no host round trip):
+// The general kernels: they sum the anchors of the cell grids at registration
+// and serve the calls that the grids (zef_grid.cu, the default path) do not.
+// Pipeline of one such call (all on the context stream, no host round trip):
 //   k_prepare      point count and offset of this call
 //   k_reset        counters, work histogram, split-pair completion counts
 //   k_keys         binning key of every point: its 21-bit Morton cell in the
