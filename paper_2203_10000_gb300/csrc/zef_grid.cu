@@ -36,10 +36,10 @@
 // 24 compartments); here such a point costs about a dozen crossing tests held
 // by the lanes of one warp, and every other point one word per compartment.
 // No sort of the points and no work list: one launch, two for large calls.
-// 56.2 M points in 24 compartments take 0.63 ms (58 ms with the tile kernels,
+// 56.2 M points in 24 compartments take 0.57 ms (58 ms with the tile kernels,
 // 2.4 ms when every compartment met by a warp was looked up and its cells
 // taken one after the other), 20.5 M in 20 small structures 0.10 ms (2.8),
-// 36,864 with solid angles 9.5 us (259).  What bounds them now: the streaming
+// 36,864 with solid angles 8.3 us (258).  What bounds them now: the streaming
 // kernel is near half the copy bandwidth (12 + 4 bytes a point), the open
 // points' kernel waits on its two dependent L2 reads per point.
 #include <cuda_runtime.h>
