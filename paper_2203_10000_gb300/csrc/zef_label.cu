@@ -2922,6 +2922,7 @@ zef_status label_reserve(zef_ctx *ctx, int64_t n_cap) {
   zef_status st;
   if (b.cap_points < n_cap) {
     int64_t cap = std::max<int64_t>(n_cap, 1024);
+    b.cap_points = 0;  // until all of them are there: an allocation may fail half-way
     auto realloc = [&](void **p, size_t bytes) -> zef_status {
       if (*p) cudaFree(*p);
       *p = nullptr;

@@ -1,0 +1,119 @@
+// Host code of the library on the runtime of fake_cudart.cpp: one scenario
+// per name; prints what is wrong and exits 1, or exits 0.
+#include <cstdio>
+#include <cstring>
+#include <string>
+#include <vector>
+
+#include "fake_cudart.h"
+#include "zef_internal.h"
+
+using namespace zef;
+
+namespace {
+
+int g_bad = 0;
+#define CHECK(cond, ...)          \
+  do {                            \
+    if (!(cond)) {                \
+      ++g_bad;                    \
+      std::printf(__VA_ARGS__);   \
+      std::printf("\n");          \
+    }                             \
+  } while (0)
+
+// an octahedron of radius r, every face cut into m^2 triangles by its planes
+struct Surface {
+  std::vector<float> v;
+  std::vector<int32_t> t;
+};
+Surface octahedron(float r, int m) {
+  Surface s;
+  std::vector<std::vector<int>> keys;
+  auto vertex = [&](int x, int y, int z) {
+    const std::vector<int> k = {x, y, z};
+    for (size_t i = 0; i < keys.size(); ++i)
+      if (keys[i] == k) return (int32_t)i;
+    keys.push_back(k);
+    for (int c : k) s.v.push_back(r * (float)c / (float)m);
+    return (int32_t)(keys.size() - 1);
+  };
+  for (int o = 0; o < 8; ++o) {
+    const int sx = o & 1 ? -1 : 1, sy = o & 2 ? -1 : 1, sz = o & 4 ? -1 : 1;
+    const bool flip = sx * sy * sz < 0;
+    auto at = [&](int i, int j) { return vertex(sx * i, sy * j, sz * (m - i - j)); };
+    auto add = [&](int32_t a, int32_t b, int32_t c) {
+      s.t.insert(s.t.end(), {a, flip ? c : b, flip ? b : c});
+    };
+    for (int i = 0; i < m; ++i)
+      for (int j = 0; i + j < m; ++j) {
+        add(at(i + 1, j), at(i, j + 1), at(i, j));
+        if (i + j + 1 < m) add(at(i + 1, j), at(i + 1, j + 1), at(i, j + 1));
+      }
+  }
+  return s;
+}
+
+zef_status add(zef_ctx *ctx, int id, const Surface &s) {
+  return zef_add_compartment(ctx, id, s.v.data(), (int64_t)s.v.size() / 3, s.t.data(), (int64_t)s.t.size() / 3, 0);
+}
+
+// no capacity is claimed for a buffer that is not there
+void check_buffers(const LabelBuffers &b, long k, const char *when) {
+  CHECK(!b.cap_points || (b.spts && b.perm && b.keys && b.in_mask && b.unc_mask),
+        "allocation %ld failed, %s: %lld points without their buffers", k, when, (long long)b.cap_points);
+  CHECK(!b.cap_items || (b.tile_box && b.flags && b.items && b.block_sums),
+        "allocation %ld failed, %s: %lld items without their buffers", k, when, (long long)b.cap_items);
+  CHECK(!b.cap_stage || (b.labels_tmp && b.pts_tmp), "allocation %ld failed, %s: no staging", k, when);
+  CHECK(!b.cap_pending || b.pending, "allocation %ld failed, %s: no list", k, when);
+}
+
+// Every device allocation of a registration, and of a call behind it, fails
+// once in turn: whatever the call returns, the context stays usable.
+int out_of_memory() {
+  const Surface small = octahedron(1.f, 2), large = octahedron(2.f, 24);
+  const std::vector<float> pts(3 * 5000, 0.25f);
+  std::vector<int32_t> lab(5000);
+  zef_label_opts general;
+  std::memset(&general, 0, sizeof(general));
+  general.block_threads = 256;
+  general.points_per_thread = 2;
+  long last = 1;
+  for (long k = 0; k < last; ++k) {
+    zef_ctx *ctx = nullptr;
+    CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+    CHECK(add(ctx, 1, small) == ZEF_OK, "first surface: %s", zef_last_error(ctx));
+    fake_fail_alloc(k);
+    const zef_status reg = add(ctx, 2, large);
+    check_buffers(ctx->lb, k, "after the registration");
+    zef_status call = ZEF_OK;
+    for (int n : {100, 5000})
+      if (!call) call = zef_label_points(ctx, pts.data(), n, lab.data(), nullptr, &general, nullptr);
+    if (fake_allocs() > last) last = fake_allocs();
+    fake_fail_alloc(-1);
+    CHECK(reg == ZEF_OK || reg == ZEF_ERR_OOM, "allocation %ld: registration returned %d", k, reg);
+    CHECK(call == ZEF_OK || call == ZEF_ERR_OOM, "allocation %ld: the call returned %d", k, call);
+    check_buffers(ctx->lb, k, "after the failure");
+    for (int n : {100, 5000}) {
+      const zef_status st = zef_label_points(ctx, pts.data(), n, lab.data(), nullptr, &general, nullptr);
+      CHECK(st == ZEF_OK, "allocation %ld failed: the next call of %d points returned %d: %s", k, n, st,
+            zef_last_error(ctx));
+      check_buffers(ctx->lb, k, "after the next call");
+      CHECK(ctx->lb.cap_points >= n, "allocation %ld failed: buffers of %lld points for %d", k,
+            (long long)ctx->lb.cap_points, n);
+    }
+    CHECK(add(ctx, 3, small) == ZEF_OK, "allocation %ld failed: the next surface: %s", k, zef_last_error(ctx));
+    check_buffers(ctx->lb, k, "after the next surface");
+    zef_destroy(ctx);
+  }
+  return 0;
+}
+
+}  // namespace
+
+int main(int argc, char **argv) {
+  const std::string name = argc > 1 ? argv[1] : "";
+  if (name == "out_of_memory") out_of_memory();
+  else return 2;
+  return g_bad ? 1 : 0;
+}
