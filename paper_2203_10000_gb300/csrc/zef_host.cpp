@@ -41,6 +41,7 @@ void dop_directions(float (*dirs)[3]) {
 zef_status cuda_fail(zef_ctx *ctx, cudaError_t e, const char *what) {
   std::string m = std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
   zef_status st = (e == cudaErrorMemoryAllocation) ? ZEF_ERR_OOM : ZEF_ERR_CUDA;
+  cudaGetLastError();  // reported here: the next call's launch check must not find it again
   return fail(ctx, st, m);
 }
 

@@ -93,6 +93,7 @@ int out_of_memory() {
     fake_fail_alloc(-1);
     CHECK(reg == ZEF_OK || reg == ZEF_ERR_OOM, "allocation %ld: registration returned %d", k, reg);
     CHECK(call == ZEF_OK || call == ZEF_ERR_OOM, "allocation %ld: the call returned %d", k, call);
+    CHECK(!reg || !call, "allocation %ld: one failure, reported by the registration and by the call", k);
     check_buffers(ctx->lb, k, "after the failure");
     for (int n : {100, 5000}) {
       const zef_status st = zef_label_points(ctx, pts.data(), n, lab.data(), nullptr, &general, nullptr);
