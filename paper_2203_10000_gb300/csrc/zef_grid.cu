@@ -1277,7 +1277,8 @@ zef_status grid_update(zef_ctx *ctx) {
   // serve need none
   if (ctx->lb.cap_points > held && ctx->lb.cap_points > (int64_t)1 << 22) label_release(ctx);
   if (!ctx->d_grid) CK(cudaMalloc(&ctx->d_grid, ZEF_MAX_COMPARTMENTS * sizeof(GridComp)), "cudaMalloc(cell grids)");
-  std::vector<GridComp> d(C);
+  std::vector<GridComp> &d = ctx->h_grid;  // outlives the copy
+  d.assign(C, GridComp{});
   for (size_t c = 0; c < C; ++c) {
     const CompHost &h = ctx->comps[c];
     const CompGrid &g = ctx->grids[c];
@@ -1296,7 +1297,8 @@ zef_status grid_update(zef_ctx *ctx) {
     r.blocks = g.blocks;
     r.tris = ctx->d_tris + h.tri_off * 3;
   }
-  CK(cudaMemcpy(ctx->d_grid, d.data(), C * sizeof(GridComp), cudaMemcpyHostToDevice), "upload cell grids");
+  CK(cudaMemcpyAsync(ctx->d_grid, d.data(), C * sizeof(GridComp), cudaMemcpyHostToDevice, ctx->stream),
+     "upload cell grids");
 
   // the label field: cells as wide as the finest compartment grid's, at most
   // kMaxField of them (one or two 64-bit words each: it stays in L2)

@@ -192,7 +192,7 @@ zef_status zef_create(zef_ctx **out, int device, void *cuda_stream) {
     }
     e = cudaMalloc(&ctx->d_status, 4 * sizeof(uint32_t));
     if (e != cudaSuccess) { st = cuda_fail(ctx, e, "cudaMalloc(status)"); break; }
-    e = cudaMemset(ctx->d_status, 0, 4 * sizeof(uint32_t));
+    e = cudaMemsetAsync(ctx->d_status, 0, 4 * sizeof(uint32_t), ctx->stream);
     if (e != cudaSuccess) { st = cuda_fail(ctx, e, "cudaMemset(status)"); break; }
     e = cudaMallocHost(&ctx->h_counters, CNT_COUNT_ * sizeof(int64_t) + 16);
     if (e != cudaSuccess) { st = cuda_fail(ctx, e, "cudaMallocHost"); break; }
@@ -1044,7 +1044,9 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
   if (!ctx->dirty) return ZEF_OK;
   const int C = (int)ctx->comps.size();
   if (C == 0) return ZEF_OK;
-  // labelings still running read what is overwritten here
+  // Labelings still running read what is overwritten here, and the copies below
+  // go to the context's stream: one on the legacy stream may still be on its
+  // way when it returns, and a non-blocking stream's kernels do not wait for it.
   CK(cudaStreamSynchronize(ctx->stream), "wait before the upload");
   int64_t ne = (int64_t)ctx->h_entries.size();
   int64_t ntv = (int64_t)ctx->h_tris.size();
@@ -1097,7 +1099,7 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
     CK(cudaMalloc(&ctx->d_nodes, std::max<size_t>(ns.size(), 1) * sizeof(CapNode)), "cudaMalloc(cap nodes)");
     ctx->d_nodes_cap = (int64_t)ns.size();
   }
-  if (!ns.empty()) CK(cudaMemcpy(ctx->d_nodes, ns.data(), ns.size() * sizeof(CapNode), cudaMemcpyHostToDevice), "upload cap nodes");
+  if (!ns.empty()) CK(cudaMemcpyAsync(ctx->d_nodes, ns.data(), ns.size() * sizeof(CapNode), cudaMemcpyHostToDevice, ctx->stream), "upload cap nodes");
   std::vector<Entry> gs(ctx->h_cseg);
   for (Entry &e : gs) {
     e.v.x *= s; e.v.y *= s; e.v.z *= s;
@@ -1109,7 +1111,7 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
     CK(cudaMalloc(&ctx->d_cseg, std::max<size_t>(gs.size(), 1) * sizeof(Entry)), "cudaMalloc(cap segments)");
     ctx->d_cseg_cap = (int64_t)gs.size();
   }
-  if (!gs.empty()) CK(cudaMemcpy(ctx->d_cseg, gs.data(), gs.size() * sizeof(Entry), cudaMemcpyHostToDevice), "upload cap segments");
+  if (!gs.empty()) CK(cudaMemcpyAsync(ctx->d_cseg, gs.data(), gs.size() * sizeof(Entry), cudaMemcpyHostToDevice, ctx->stream), "upload cap segments");
   if (ctx->d_ctidx_cap < (int64_t)ctx->h_ctidx.size()) {
     if (ctx->d_ctidx) cudaFree(ctx->d_ctidx);
     ctx->d_ctidx = nullptr;
@@ -1118,7 +1120,7 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
     ctx->d_ctidx_cap = (int64_t)ctx->h_ctidx.size();
   }
   if (!ctx->h_ctidx.empty())
-    CK(cudaMemcpy(ctx->d_ctidx, ctx->h_ctidx.data(), ctx->h_ctidx.size() * sizeof(int32_t), cudaMemcpyHostToDevice),
+    CK(cudaMemcpyAsync(ctx->d_ctidx, ctx->h_ctidx.data(), ctx->h_ctidx.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream),
        "upload cap-tree triangle order");
   // union box of the surfaces in the caller's coordinates: the binning keys'
   // range (a point outside it is outside every compartment's box)
@@ -1161,12 +1163,13 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
   std::iota(lpt.begin(), lpt.end(), 0);
   std::stable_sort(lpt.begin(), lpt.end(),
                    [&](int a, int b) { return ctx->comps[a].nt > ctx->comps[b].nt; });
-  CK(cudaMemcpy(ctx->d_dop, dop.data(), dop.size() * sizeof(float), cudaMemcpyHostToDevice), "upload dop");
-  CK(cudaMemcpy(ctx->d_entries, es.data(), ne * sizeof(Entry), cudaMemcpyHostToDevice), "upload entries");
-  CK(cudaMemcpy(ctx->d_tris, ts.data(), ntv * sizeof(float4), cudaMemcpyHostToDevice), "upload tris");
-  CK(cudaMemcpy(ctx->d_comps, dc.data(), C * sizeof(DevComp), cudaMemcpyHostToDevice), "upload comps");
-  CK(cudaMemcpy(ctx->d_row_ids, rows.data(), C * sizeof(int32_t), cudaMemcpyHostToDevice), "upload rows");
-  CK(cudaMemcpy(ctx->d_lpt, lpt.data(), C * sizeof(int32_t), cudaMemcpyHostToDevice), "upload lpt");
+  CK(cudaMemcpyAsync(ctx->d_dop, dop.data(), dop.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream), "upload dop");
+  CK(cudaMemcpyAsync(ctx->d_entries, es.data(), ne * sizeof(Entry), cudaMemcpyHostToDevice, ctx->stream), "upload entries");
+  CK(cudaMemcpyAsync(ctx->d_tris, ts.data(), ntv * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream), "upload tris");
+  CK(cudaMemcpyAsync(ctx->d_comps, dc.data(), C * sizeof(DevComp), cudaMemcpyHostToDevice, ctx->stream), "upload comps");
+  CK(cudaMemcpyAsync(ctx->d_row_ids, rows.data(), C * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream), "upload rows");
+  CK(cudaMemcpyAsync(ctx->d_lpt, lpt.data(), C * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream), "upload lpt");
+  CK(cudaStreamSynchronize(ctx->stream), "upload");  // the copies' host arrays end with this call
   ctx->dirty = false;
   ++ctx->gen;
   const zef_status st = grid_update(ctx);

@@ -314,6 +314,7 @@ struct zef_ctx {
   cudaEvent_t ev[6] = {};
   std::vector<zef::CompGrid> grids;   // cell grids, by compartment
   zef::GridComp *d_grid = nullptr;    // by priority row
+  std::vector<zef::GridComp> h_grid;  // its copy on the host
   zef::LabelField field = {};
   void *field_mem = nullptr;          // its cells (grow-only)
   size_t field_cap = 0;

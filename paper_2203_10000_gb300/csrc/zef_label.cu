@@ -2873,7 +2873,8 @@ zef_status label_reserve_counters(zef_ctx *ctx) {
   if (b.counters) return ZEF_OK;
   cudaError_t e = cudaMalloc(&b.counters, CNT_COUNT_ * sizeof(int64_t));
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(counters)");
-  cudaMemset(b.counters, 0, CNT_COUNT_ * sizeof(int64_t));
+  e = cudaMemsetAsync(b.counters, 0, CNT_COUNT_ * sizeof(int64_t), ctx->stream);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "clear counters");
   return ZEF_OK;
 }
 
@@ -3179,6 +3180,7 @@ zef_status upload_dop_directions(zef_ctx *ctx) {
   dop_directions(dirs);
   cudaError_t e = cudaMemcpyToSymbol(c_dop, dirs, sizeof(dirs));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_dop, dirs, sizeof(dirs));
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // before any kernel of a non-blocking stream
   if (e != cudaSuccess) return cuda_fail(ctx, e, "upload hull directions");
   return ZEF_OK;
 }

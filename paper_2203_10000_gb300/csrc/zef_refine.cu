@@ -685,9 +685,9 @@ zef_status refine_run(zef_ctx *ctx, zef_mesh *mesh, int32_t levels, const zef_la
       green_tables(gt);
       gt_ready = true;
     }
-    CK(cudaMemcpyToSymbol(c_gn, gt.n, sizeof(gt.n)), "upload closure table");
-    CK(cudaMemcpyToSymbol(c_gch, gt.ch, sizeof(gt.ch)), "upload closure table");
-    CK(cudaMemcpyToSymbol(c_gdg, gt.dg, sizeof(gt.dg)), "upload closure table");
+    CK(cudaMemcpyToSymbolAsync(c_gn, gt.n, sizeof(gt.n), 0, cudaMemcpyHostToDevice, ctx->stream), "upload closure table");
+    CK(cudaMemcpyToSymbolAsync(c_gch, gt.ch, sizeof(gt.ch), 0, cudaMemcpyHostToDevice, ctx->stream), "upload closure table");
+    CK(cudaMemcpyToSymbolAsync(c_gdg, gt.dg, sizeof(gt.dg), 0, cudaMemcpyHostToDevice, ctx->stream), "upload closure table");
   }
   const int64_t new_cap = std::max<int64_t>(1, std::min<int64_t>(6 * fmax, ncap - N0));
   if ((st = label_reserve_counters(ctx))) return st;

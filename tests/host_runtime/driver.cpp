@@ -110,11 +110,32 @@ int out_of_memory() {
   return 0;
 }
 
+// Copies and sets that the library's kernels read or overwrite are in order
+// with them, also on a non-blocking stream.
+int uploads() {
+  const Surface a = octahedron(1.f, 3), b = octahedron(2.f, 5);
+  const std::vector<float> pts(300, 0.25f);
+  std::vector<int32_t> lab(100);
+  const int32_t order[2] = {2, 1};
+  zef_ctx *ctx = nullptr;
+  std::string first;
+  CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+  CHECK(add(ctx, 1, a) == ZEF_OK && add(ctx, 2, b) == ZEF_OK, "surfaces: %s", zef_last_error(ctx));
+  CHECK(zef_compartment_priority(ctx, order, 2) == ZEF_OK, "priority: %s", zef_last_error(ctx));
+  CHECK(zef_label_points(ctx, pts.data(), 100, lab.data(), nullptr, nullptr, nullptr) == ZEF_OK, "labels: %s",
+        zef_last_error(ctx));
+  CHECK(fake_unordered(&first) == 0, "%ld launches beside a copy on the legacy stream, the first %s",
+        fake_unordered(nullptr), first.c_str());
+  zef_destroy(ctx);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
   const std::string name = argc > 1 ? argv[1] : "";
   if (name == "out_of_memory") out_of_memory();
+  else if (name == "uploads") uploads();
   else return 2;
   return g_bad ? 1 : 0;
 }

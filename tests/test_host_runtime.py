@@ -32,3 +32,7 @@ def _run(driver, scenario):
 
 def test_failed_allocations_leave_the_context_usable(driver):
     _run(driver, "out_of_memory")
+
+
+def test_uploads_are_ordered_with_the_kernels_that_read_them(driver):
+    _run(driver, "uploads")
