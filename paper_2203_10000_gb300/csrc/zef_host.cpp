@@ -541,7 +541,8 @@ zef_status zef_synchronize(zef_ctx *ctx) {
   }
   const uint32_t st[2] = {ctx->h_status[0], ctx->h_status[1]};
   if (st[0]) {
-    CK(cudaMemset(ctx->d_status, 0, 2 * sizeof(uint32_t)), "clear status");
+    // on the stream that reads them next: a clear on the legacy stream may come after that
+    CK(cudaMemsetAsync(ctx->d_status, 0, 2 * sizeof(uint32_t), ctx->stream), "clear status");
     if (st[0] & ST_TIMEOUT)
       return fail(ctx, ZEF_ERR_TIMEOUT, "a bounded device wait expired (site " + std::to_string(st[1]) + ")");
     if (st[0] & ST_INVALID)

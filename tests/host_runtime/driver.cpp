@@ -130,12 +130,33 @@ int uploads() {
   return 0;
 }
 
+// An error that a kernel recorded is reported once.
+int status_once() {
+  const std::vector<float> pts(300, 0.25f);
+  std::vector<int32_t> lab(100);
+  zef_ctx *ctx = nullptr;
+  CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+  CHECK(add(ctx, 1, octahedron(1.f, 3)) == ZEF_OK, "surface: %s", zef_last_error(ctx));
+  for (const uint32_t bit : {ST_TIMEOUT, ST_INVALID}) {
+    fake_on_launch("k_grid_label", [ctx, bit] { ctx->d_status[0] |= bit; });
+    CHECK(zef_label_points(ctx, pts.data(), 100, lab.data(), nullptr, nullptr, nullptr) ==
+              (bit == ST_TIMEOUT ? ZEF_ERR_TIMEOUT : ZEF_ERR_INVALID_ARG), "bit %u: not reported", bit);
+    fake_on_launch("", [] {});
+    CHECK(zef_synchronize(ctx) == ZEF_OK, "bit %u: reported twice: %s", bit, zef_last_error(ctx));
+    CHECK(zef_label_points(ctx, pts.data(), 100, lab.data(), nullptr, nullptr, nullptr) == ZEF_OK,
+          "bit %u: reported by the next call: %s", bit, zef_last_error(ctx));
+  }
+  zef_destroy(ctx);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
   const std::string name = argc > 1 ? argv[1] : "";
   if (name == "out_of_memory") out_of_memory();
   else if (name == "uploads") uploads();
+  else if (name == "status_once") status_once();
   else return 2;
   return g_bad ? 1 : 0;
 }

@@ -36,3 +36,7 @@ def test_failed_allocations_leave_the_context_usable(driver):
 
 def test_uploads_are_ordered_with_the_kernels_that_read_them(driver):
     _run(driver, "uploads")
+
+
+def test_a_recorded_error_is_reported_once(driver):
+    _run(driver, "status_once")
