@@ -1358,7 +1358,7 @@ zef_status taubin_run(zef_ctx *ctx, float *nodes, int64_t n, const int32_t *tets
   if ((st = build_adjacency(ctx, tt, m, n, &g))) return st;  // synchronizes
   int64_t words[PP_WORDS] = {0};
   if ((st = smooth_loop(ctx, x, n, g, fx, o, false, words))) return st;
-  if (!dn) CK(cudaMemcpy(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost), "copy nodes back");
+  if (!dn) CK(cudaMemcpyAsync(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost, s), "copy nodes back");
   if (iters_out) *iters_out = (int32_t)words[PP_ITER];
   return zef_synchronize(ctx);
 }
@@ -1396,7 +1396,7 @@ zef_status taubin_surface_run(zef_ctx *ctx, float *nodes, int64_t n, const int32
   if ((st = build_surface_adjacency(ctx, tt, lab, m, n, &g, &faces))) return st;  // synchronizes
   int64_t words[PP_WORDS] = {0};
   if (faces > 0 && (st = smooth_loop(ctx, x, n, g, nullptr, o, true, words))) return st;
-  if (!dn) CK(cudaMemcpy(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost), "copy nodes back");
+  if (!dn) CK(cudaMemcpyAsync(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost, s), "copy nodes back");
   if (iters_out) *iters_out = (int32_t)words[PP_ITER];
   if (faces_out) *faces_out = faces;
   return zef_synchronize(ctx);
@@ -1456,7 +1456,7 @@ zef_status inflate_run(zef_ctx *ctx, float *nodes, int64_t n, const int32_t *tet
   }
   const int64_t crossing = words[PP_CAND];  // with repeats
   if (crossing == 0) {
-    if (!dn) CK(cudaMemcpy(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost), "copy nodes back");
+    if (!dn) CK(cudaMemcpyAsync(nodes, x, (size_t)n * 3 * sizeof(float), cudaMemcpyDeviceToHost, s), "copy nodes back");
     return zef_synchronize(ctx);
   }
   int64_t cap = 1024;

@@ -150,6 +150,27 @@ int status_once() {
   return 0;
 }
 
+// Host meshes without tets: every entry point that works in place leaves the
+// nodes as they are.
+int no_tets() {
+  const std::vector<float> x = {0.1f, 0.2f, 0.3f, 1.f, 2.f, 3.f};
+  zef_smooth_opts o = {0.4f, 0.4f, 0.f, 3};
+  zef_ctx *ctx = nullptr;
+  CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+  CHECK(add(ctx, 1, octahedron(1.f, 3)) == ZEF_OK, "surface: %s", zef_last_error(ctx));
+  int32_t it = 0;
+  int64_t count = 0;
+  std::vector<float> y = x;
+  CHECK(zef_taubin_smooth_surface(ctx, y.data(), 2, nullptr, 0, nullptr, &o, &it, &count) == ZEF_OK, "boundaries: %s",
+        zef_last_error(ctx));
+  CHECK(y == x, "boundary smoothing without tets changed the nodes: %g %g %g", y[0], y[1], y[2]);
+  y = x;
+  CHECK(zef_inflate(ctx, y.data(), 2, nullptr, 0, 1, 0.05f, &count) == ZEF_OK, "inflation: %s", zef_last_error(ctx));
+  CHECK(y == x, "inflation without tets changed the nodes: %g %g %g", y[0], y[1], y[2]);
+  zef_destroy(ctx);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -157,6 +178,7 @@ int main(int argc, char **argv) {
   if (name == "out_of_memory") out_of_memory();
   else if (name == "uploads") uploads();
   else if (name == "status_once") status_once();
+  else if (name == "no_tets") no_tets();
   else return 2;
   return g_bad ? 1 : 0;
 }

@@ -40,3 +40,7 @@ def test_uploads_are_ordered_with_the_kernels_that_read_them(driver):
 
 def test_a_recorded_error_is_reported_once(driver):
     _run(driver, "status_once")
+
+
+def test_host_meshes_without_tets_keep_their_nodes(driver):
+    _run(driver, "no_tets")
