@@ -48,6 +48,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <string>
 #include <vector>
 
 #include "zef_fp64.cuh"
@@ -1245,7 +1246,23 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   k_gr_finish<<<g_w, 256, 0, st>>>(tris, to_raw, s, g, cells, cnt, flag, list, anchor, omega, (uint32_t *)(blob + p_word),
                                    (float4 *)blob);
   e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(ctx->h_status, ctx->d_status, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  // anchors whose sums were cut short: no grid from them.  The error is this
+  // call's; what an earlier call recorded beside it stays to be reported.
+  constexpr uint32_t cut = ST_TIMEOUT | ST_BOUNDS;
+  const uint32_t status = ctx->h_status[0];
+  if (e == cudaSuccess && (status & cut)) {
+    ctx->h_status[0] = status & ~cut;
+    e = cudaMemcpyAsync(ctx->d_status, ctx->h_status, sizeof(uint32_t), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) {
+      cudaFree(blob);
+      return fail(ctx, status & ST_TIMEOUT ? ZEF_ERR_TIMEOUT : ZEF_ERR_BOUNDS,
+                  "the solid angles of a cell grid's anchors were cut short (site " + std::to_string(ctx->h_status[1]) + ")");
+    }
+  }
   if (e != cudaSuccess) {
     cudaFree(blob);
     return cuda_fail(ctx, e, "cell grid");

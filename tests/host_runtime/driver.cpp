@@ -171,6 +171,28 @@ int no_tets() {
   return 0;
 }
 
+// Anchors whose solid angles were cut short by an expired wait make no grid:
+// the registration reports it, the next call builds the grid anew, and an
+// error of an earlier call stays to be reported.
+int anchors_cut_short() {
+  const std::vector<float> pts(300, 0.25f);
+  std::vector<int32_t> lab(100);
+  zef_ctx *ctx = nullptr;
+  CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+  fake_settle();
+  ctx->d_status[0] = ST_INVALID;
+  fake_on_launch("k_label32", [ctx] { ctx->d_status[0] |= ST_TIMEOUT; });
+  CHECK(add(ctx, 1, octahedron(1.f, 3)) == ZEF_ERR_TIMEOUT, "registration did not report the expired wait");
+  CHECK(ctx->grids.empty(), "a grid from anchors that were cut short");
+  fake_on_launch("", [] {});
+  CHECK(zef_synchronize(ctx) == ZEF_ERR_INVALID_ARG, "the earlier call's error is lost");
+  CHECK(zef_label_points(ctx, pts.data(), 100, lab.data(), nullptr, nullptr, nullptr) == ZEF_OK, "next call: %s",
+        zef_last_error(ctx));
+  CHECK(ctx->grids.size() == 1 && ctx->grids[0].usable, "the next call did not build the grid");
+  zef_destroy(ctx);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -179,6 +201,7 @@ int main(int argc, char **argv) {
   else if (name == "uploads") uploads();
   else if (name == "status_once") status_once();
   else if (name == "no_tets") no_tets();
+  else if (name == "anchors_cut_short") anchors_cut_short();
   else return 2;
   return g_bad ? 1 : 0;
 }

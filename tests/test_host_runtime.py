@@ -44,3 +44,7 @@ def test_a_recorded_error_is_reported_once(driver):
 
 def test_host_meshes_without_tets_keep_their_nodes(driver):
     _run(driver, "no_tets")
+
+
+def test_anchors_cut_short_make_no_grid(driver):
+    _run(driver, "anchors_cut_short")
