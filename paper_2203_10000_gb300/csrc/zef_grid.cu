@@ -65,6 +65,7 @@ namespace zef {
 namespace {
 
 constexpr float kFourPi = 12.5663706143591729539f;
+constexpr double kTwoPi64 = 6.283185307179586476925;
 // Cell word of a cell that triangles meet: the top bit, the chunks of its
 // block in two bits (0: more than three, see the block's header), and the
 // block's offset in 16-byte words.  Otherwise the winding number (8 bits), or
@@ -333,7 +334,9 @@ struct GridArgs {
   int early;                  // a point certainly inside needs no later compartment
   int stats;
   int iters;                  // streaming kernel: consecutive tiles of a warp
+  int tile;                   // fused kernel: points of a warp's step
   int32_t *pending;           // streaming kernel: indices of the points the field leaves open
+  OpenPoint *open;            // points for the FP64 solid angles
   UnionBox ub;
   LabelField field;
   uint32_t *status;
@@ -353,10 +356,10 @@ enum GridStat { GS_EVAL = 0, GS_COHERENT, GS_OWN, GS_ITEMS, GS_NONFINITE, GS_NIN
 
 // FP64 re-evaluation of one (point, compartment) pair by the whole warp: the
 // crossings from the vertices in FP64, each sign taken only beyond its
-// rounding bound; where that leaves one open, the FP64 solid angle over the
-// cap tree.  Returns whether the point is inside; *omega = Omega.
-__device__ __noinline__ bool resolve64(const GridArgs &a, const GridComp &g, uint32_t word, float x, float y, float z,
-                                       int lane, float *omega) {
+// rounding bound.  Returns whether that decides the pair; *k = the point's
+// winding number.
+__device__ __noinline__ bool crossings64(const GridArgs &a, const GridComp &g, uint32_t word, float x, float y, float z,
+                                         int lane, int *k) {
   if (word & kMixed) {
     const float4 *block = g.blocks + (word & kOffsetMask);
     const float4 r = block[0];
@@ -411,15 +414,21 @@ __device__ __noinline__ bool resolve64(const GridArgs &a, const GridComp &g, uin
         count_add(a, CNT_UNC, 1);
         count_add(a, CNT_PAIRS_RESCUE, (unsigned long long)tested);
       }
-      *omega = kFourPi * (float)(k0 + net);
-      return k0 + net >= 1;
+      *k = k0 + net;
+      return true;
     }
   }
+  return false;
+}
+
+// FP64 solid angle of one pair by the whole warp, over the cap tree: what the
+// crossings leave open (a point on the surface).
+__device__ __noinline__ double solid64(const GridArgs &a, const GridComp &g, float x, float y, float z, int lane) {
   // FP64 solid angle: the caps of the nodes whose box misses the point, the
   // leaves whose box holds it
   const DevComp *cp = a.comps + g.comp;
   const float px = x * a.scale, py = y * a.scale, pz = z * a.scale;
-  // The groups of four entries in the order of the list kernel's block of 256
+  // The groups of four entries in the order of k_grid_open's block of 256
   // threads (thread g mod 256 takes group g; the sums of each 32 threads, then
   // of the eight in turn), so that a point on the surface, whose Omega is 2 pi
   // up to rounding, gets that kernel's rounding.  The walk's segments are a
@@ -496,13 +505,176 @@ __device__ __noinline__ bool resolve64(const GridArgs &a, const GridComp &g, uin
     sum += part[q];
   }
   K = __reduce_add_sync(0xffffffffu, K);
-  const double om = 2.0 * (sum + 6.283185307179586476925 * (double)K);
+  const double om = 2.0 * (sum + kTwoPi64 * (double)K);
   if (lane == 0 && a.stats) {
     count_add(a, CNT_UNC, 1);
     count_add(a, CNT_PAIRS_RESCUE, (unsigned long long)tris);
   }
+  return om;
+}
+
+// Index of x on an axis of n cells; monotone in x, so the indices of a box's
+// ends bound those of its points.
+__device__ __forceinline__ int axis_cell(float x, float lo, float inv, int n) {
+  return min(max((int)((x - lo) * inv), 0), n - 1);
+}
+
+// Word of the cell that holds a point of the surface's box.
+__device__ __forceinline__ uint32_t cell_word(const GridArgs &a, const GridComp &g, float x, float y, float z) {
+  const int cx = axis_cell(x, g.lo[0], g.inv[0], g.n[0]), cy = axis_cell(y, g.lo[1], g.inv[1], g.n[1]),
+            cz = axis_cell(z, g.lo[2], g.inv[2], g.n[2]);
+  const int c = (cz * g.n[1] + cy) * g.n[0] + cx;  // at most kMaxCells
+  return ZEF_BOUNDS_OK(c >= 0 && c < g.n[0] * g.n[1] * g.n[2], a.status, 30) ? __ldg(g.words + c) : 0u;
+}
+
+// Both by the whole warp: whether the point is inside; *omega = Omega.
+__device__ __noinline__ bool resolve64(const GridArgs &a, const GridComp &g, uint32_t word, float x, float y, float z,
+                                       int lane, float *omega) {
+  int k = 0;
+  if (crossings64(a, g, word, x, y, z, lane, &k)) {
+    *omega = kFourPi * (float)k;
+    return k >= 1;
+  }
+  const double om = solid64(a, g, x, y, z, lane);
   *omega = (float)om;
-  return om > 6.283185307179586476925;
+  return om > kTwoPi64;
+}
+
+// The FP64 solid angle of one pair by a block of 256 threads.  The walk of the
+// cap tree goes down one level at a time: the list holds, in the tree's order,
+// the segments found so far and the nodes still to be opened, and each node is
+// replaced by its segment or its two children: a level is one read of every
+// thread's node and a scan, and eight warps share the FP64 pipe that bounds the
+// sum.  A vertex of a 20,000-triangle surface: 50 us, 115 by one warp.  Every
+// thread returns the same Omega; `lane` and `wid` are the thread's.
+constexpr int kOpenThreads = 256;
+constexpr int kOpenList = 1024;  // entries of a level; beyond that one warp walks as solid64 does
+
+struct OpenShared {
+  int2 seg[2][kOpenList];  // x: first entry, y: its groups of four, or x: node, y: 0
+  int first[kOpenList];    // groups before the segment
+  int scan[2][kOpenThreads / 32];
+  double part[kOpenThreads / 32];
+  int wraps[kOpenThreads / 32];
+  int decided, k;
+  double om;
+};
+
+// exclusive sum of v over the block in thread order; *total its sum
+__device__ __forceinline__ int block_exclusive(int v, int (&s_scan)[kOpenThreads / 32], int lane, int wid, int *total) {
+  int incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  __syncthreads();  // the last sum's readers are done
+  if (lane == 31) s_scan[wid] = incl;
+  __syncthreads();
+  int before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < kOpenThreads / 32; ++w) {
+    before += w < wid ? s_scan[w] : 0;
+    all += s_scan[w];
+  }
+  *total = all;
+  return before + incl - v;
+}
+
+__device__ double solid64_block(const GridArgs &a, const GridComp &g, float x, float y, float z, OpenShared &sh, int lane,
+                                int wid) {
+  const DevComp *cp = a.comps + g.comp;
+  const float px = x * a.scale, py = y * a.scale, pz = z * a.scale;
+  int cur = 0, len = 1, tris = 0;
+  if (threadIdx.x == 0) sh.seg[0][0] = make_int2(cp->cap_root, 0);
+  __syncthreads();
+  for (;;) {
+    int out = 0;
+    bool nodes = false;
+    for (int e0 = 0; e0 < len; e0 += kOpenThreads) {
+      const int e = e0 + (int)threadIdx.x;
+      int n = 0;
+      int2 o0 = make_int2(0, 0), o1 = make_int2(0, 0);
+      if (e < len) {
+        o0 = sh.seg[cur][e];
+        n = 1;
+        if (o0.y == 0) {
+          const CapNode nd = a.nodes[o0.x];
+          const bool far = nd.hi[0] < px || nd.lo[0] > px || nd.hi[1] < py || nd.lo[1] > py || nd.hi[2] < pz || nd.lo[2] > pz;
+          if (!far && nd.left >= 0) {
+            o1 = make_int2(nd.right, 0);
+            o0 = make_int2(o0.x + 1, 0);
+            n = 2;
+            nodes = true;
+          } else {
+            const int c = far ? nd.cap_cnt : nd.leaf_cnt;
+            tris += far ? nd.cap_tris : nd.leaf_tris;
+            o0 = make_int2(far ? nd.cap_begin : nd.leaf_begin, c / 4);
+            n = c >= 4 ? 1 : 0;
+          }
+        }
+      }
+      int total;
+      const int at = out + block_exclusive(n, sh.scan[0], lane, wid, &total);
+      if (n > 0 && at < kOpenList) sh.seg[cur ^ 1][at] = o0;
+      if (n > 1 && at + 1 < kOpenList) sh.seg[cur ^ 1][at + 1] = o1;
+      out += total;
+    }
+    len = out;
+    cur ^= 1;
+    const bool more = __syncthreads_or(nodes);
+    if (len > kOpenList || !more) break;
+  }
+  if (len > kOpenList) {
+    if (wid == 0) {
+      const double om = solid64(a, g, x, y, z, lane);
+      if (lane == 0) sh.om = om;
+    }
+    __syncthreads();
+    const double om = sh.om;
+    __syncthreads();
+    return om;
+  }
+  int groups = 0;
+  for (int e0 = 0; e0 < len; e0 += kOpenThreads) {
+    const int e = e0 + (int)threadIdx.x;
+    int total;
+    const int at = groups + block_exclusive(e < len ? sh.seg[cur][e].y : 0, sh.scan[1], lane, wid, &total);
+    if (e < len) sh.first[e] = at;
+    groups += total;
+  }
+  __syncthreads();
+  double part = 0.0;
+  int K = 0;
+  for (int j = (int)threadIdx.x; j < groups; j += kOpenThreads) {
+    int lo = 0, hi = len - 1;  // the last segment that starts at or before group j
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (sh.first[mid] <= j) lo = mid;
+      else hi = mid - 1;
+    }
+    part += group64(a.cseg, sh.seg[cur][lo].x + 4 * (j - sh.first[lo]), px, py, pz, &K);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  K = __reduce_add_sync(0xffffffffu, K);
+  tris = __reduce_add_sync(0xffffffffu, tris);
+  if (lane == 0) {
+    sh.part[wid] = part;
+    sh.wraps[wid] = K;
+    if (a.stats && tris) count_add(a, CNT_PAIRS_RESCUE, (unsigned long long)tris);
+  }
+  if (threadIdx.x == 0 && a.stats) count_add(a, CNT_UNC, 1);
+  __syncthreads();
+  double sum = 0.0;
+  K = 0;
+#pragma unroll
+  for (int w = 0; w < kOpenThreads / 32; ++w) {
+    sum += sh.part[w];
+    K += sh.wraps[w];
+  }
+  __syncthreads();
+  return 2.0 * (sum + kTwoPi64 * (double)K);
 }
 
 // ---- the label field: one cell grid over the union box of all surfaces.  A
@@ -521,12 +693,6 @@ struct FieldCell<true> {
   using T = ulonglong2;
   using M = unsigned long long;
 };
-
-// Index of x on an axis of n cells; monotone in x, so the indices of a box's
-// ends bound those of its points.
-__device__ __forceinline__ int axis_cell(float x, float lo, float inv, int n) {
-  return min(max((int)((x - lo) * inv), 0), n - 1);
-}
 
 template <bool WIDE>
 __global__ void __launch_bounds__(256) k_gr_field(LabelField f, const GridComp *grid, int ncomp) {
@@ -582,6 +748,7 @@ constexpr int kGlWarps = kGlThreads / 32;
 constexpr int kGlP = 2;               // fused kernel: points per lane and step
 constexpr int kGlTile = 32 * kGlP;
 constexpr int kGlQueue = 32 + kGlTile;  // fewer than 32 left over, one tile's more
+constexpr int kRun = 8;               // consecutive points of a warp (see run_point)
 constexpr int kGsP = 4;               // streaming kernel
 constexpr int kGsTile = 32 * kGsP;
 constexpr int kGsFlush = 256;         // listed together (each addition to the one cursor costs about a nanosecond)
@@ -617,7 +784,10 @@ struct Batch {
 // points in cells with triangles are then taken eight at a time, four lanes
 // each over the entries of the point's own cell (two dependent reads per
 // point -- word, block -- whatever cells and compartments the batch lies in).
-template <bool WIDE>
+// Pairs that the crossings leave open are taken to FP64 by the warp, one after
+// the other; with LIST, a point whose label needs one is listed for k_grid_open
+// instead, and one that the list does not hold is left to its second part.
+template <bool WIDE, bool LIST>
 __device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, const int32_t *s_id, Batch &sb, int wid,
                                        int lane, int64_t off, float x, float y, float z, int32_t i, bool have,
                                        typename FieldCell<WIDE>::M mask, typename FieldCell<WIDE>::M mix,
@@ -625,19 +795,14 @@ __device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, c
   using M = typename FieldCell<WIDE>::M;
   const int sub = lane / kLanes, ti = lane % kLanes;
   M pend = have ? open_rows<M>(mask, mix, a.early) : 0;
+  M left = 0;  // LIST: rows left open
   while (__any_sync(0xffffffffu, pend != 0)) {
     const bool mine = pend != 0;
     const int r = mine ? first_row(pend) : 0;
     pend &= pend - 1;
     const GridComp &g = s_g[r];
     const bool in = mine && x >= g.lo[0] && x <= g.hi[0] && y >= g.lo[1] && y <= g.hi[1] && z >= g.lo[2] && z <= g.hi[2];
-    uint32_t word = 0u;
-    if (in) {
-      const int cx = axis_cell(x, g.lo[0], g.inv[0], g.n[0]), cy = axis_cell(y, g.lo[1], g.inv[1], g.n[1]),
-                cz = axis_cell(z, g.lo[2], g.inv[2], g.n[2]);
-      const int c = (cz * g.n[1] + cy) * g.n[0] + cx;  // at most kMaxCells
-      if (ZEF_BOUNDS_OK(c >= 0 && c < g.n[0] * g.n[1] * g.n[2], a.status, 30)) word = __ldg(g.words + c);
-    }
+    const uint32_t word = in ? cell_word(a, g, x, y, z) : 0u;
     const bool mixed = (word & kMixed) != 0u;
     bool unc = (word & (kMixed | kUnknown)) == kUnknown;
     int k = (int)(signed char)(word & 0xffu);
@@ -699,17 +864,21 @@ __device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, c
     }
     float om = kFourPi * (float)k;
     bool inside = in && !unc && k >= 1;
-    uint32_t um = __ballot_sync(0xffffffffu, unc);
-    while (um) {
-      const int src = __ffs(um) - 1;
-      um &= um - 1;
-      float o64;
-      const bool i64 = resolve64(a, s_g[__shfl_sync(0xffffffffu, r, src)], __shfl_sync(0xffffffffu, word, src),
-                                 __shfl_sync(0xffffffffu, x, src), __shfl_sync(0xffffffffu, y, src),
-                                 __shfl_sync(0xffffffffu, z, src), lane, &o64);
-      if (lane == src) {
-        inside = i64;
-        om = o64;
+    if (LIST) {
+      if (unc) left |= (M)1 << r;
+    } else {
+      uint32_t um = __ballot_sync(0xffffffffu, unc);
+      while (um) {
+        const int src = __ffs(um) - 1;
+        um &= um - 1;
+        float o64;
+        const bool i64 = resolve64(a, s_g[__shfl_sync(0xffffffffu, r, src)], __shfl_sync(0xffffffffu, word, src),
+                                   __shfl_sync(0xffffffffu, x, src), __shfl_sync(0xffffffffu, y, src),
+                                   __shfl_sync(0xffffffffu, z, src), lane, &o64);
+        if (lane == src) {
+          inside = i64;
+          om = o64;
+        }
       }
     }
     if (inside) {
@@ -718,10 +887,44 @@ __device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, c
     }
     if (a.omega && mine) a.omega[(int64_t)r * a.omega_ld + i] = in ? om : 0.f;
   }
+  if (LIST) {
+    left = open_rows<M>(mask, left, a.early);
+    const uint32_t lm = __ballot_sync(0xffffffffu, left != 0);
+    if (lm) {
+      const int first = __ffs(lm) - 1;
+      unsigned long long at = 0;
+      if (lane == first) at = atomicAdd((unsigned long long *)(a.counters + CNT_OPEN), (unsigned long long)__popc(lm));
+      at = __shfl_sync(0xffffffffu, at, first) + __popc(lm & ((1u << lane) - 1u));
+      if (left && at < (unsigned long long)kOpenCap) {
+        OpenPoint p;
+        p.ins = mask;
+        p.open = left;
+        p.i = i;
+        a.open[at] = p;
+      }
+      if (left) have = false;
+    }
+  }
   if (have) {
     a.labels[off + i] = mask ? s_id[first_row(mask)] : 0;
     if (a.masks) a.masks[off + i] = mask;
   }
+}
+
+// Index of a warp's k-th point of tile t of `tiles`: runs of kRun consecutive
+// points, the runs of a tile `tiles` runs apart.  Points that the crossings
+// leave open -- points on a surface: electrodes are vertices of the scalp mesh,
+// mesh nodes may lie in a face -- cost an FP64 solid angle each, one after the
+// other in a warp, and come one behind the other: 64 vertices in 64 consecutive
+// points took 6.9 ms in one warp, 0.9 ms in eight (the general kernels: 4.1).
+// A run is three whole sectors of coordinates and one of labels.  (The pending
+// kernel keeps 32 neighbours together, whose cells share L1 lines -- 5.2 M
+// points 92 us in runs, 85 so -- and lists what stays open.)
+__device__ __forceinline__ int64_t run_point(int64_t t, int64_t tiles, int k) {
+  return kRun * ((k / kRun) * tiles + t) + k % kRun;
+}
+__device__ __forceinline__ int64_t run_tiles(int64_t n, int tile) {
+  return ((n + kRun - 1) / kRun + tile / kRun - 1) / (tile / kRun);
 }
 
 // Field cell of a point: zero outside the union box and for a non-finite
@@ -793,7 +996,7 @@ __device__ __forceinline__ void field_store(const GridArgs &a, const int32_t *s_
         a.omega[(int64_t)r * a.omega_ld + i] = !fin ? __int_as_float(0x7fc00000) : (ins >> r) & 1 ? kFourPi : 0.f;
 }
 
-// One launch (small calls): a warp reads 64 consecutive points, looks their
+// One launch (small calls): a warp reads the points of a tile, looks their
 // field cells up and writes the labels of the points that the field decides;
 // the others go to the warp's queue in shared memory, and whenever it holds
 // 32 they are decided together.
@@ -813,14 +1016,16 @@ __global__ void __launch_bounds__(kGlThreads, 4) k_grid_label(GridArgs a) {
   const float *pts = a.pts + 3 * off;
   int queued = 0;
   LaneStats st;
-  const int64_t step = (int64_t)gridDim.x * kGlWarps * kGlTile;
-  for (int64_t base = ((int64_t)blockIdx.x * kGlWarps + wid) * kGlTile;; base += step) {
-    const bool last = base >= n;  // warp-uniform: no points left, only the queue
+  const int64_t tiles = run_tiles(n, a.tile);
+  for (int64_t t = (int64_t)wid * gridDim.x + blockIdx.x;; t += (int64_t)gridDim.x * kGlWarps) {
+    const bool last = t >= tiles;  // warp-uniform: no points left, only the queue
 #pragma unroll
     for (int u = 0; u < kGlP; ++u) {
-      const int64_t i = base + 32 * u + lane;
+      if (32 * u >= a.tile) break;
+      const int64_t i = run_point(t, tiles, 32 * u + lane);
+      const bool valid = !last && i < n && 32 * u + lane < a.tile;
       float x = __int_as_float(0x7fc00000), y = x, z = x;
-      if (i < n) {
+      if (valid) {
         x = pts[3 * i];
         y = pts[3 * i + 1];
         z = pts[3 * i + 2];
@@ -832,9 +1037,9 @@ __global__ void __launch_bounds__(kGlThreads, 4) k_grid_label(GridArgs a) {
       if (a.stats) {
         st.coh += sizeof(M) == 8 ? __popcll(ins) : __popc((uint32_t)ins);
         st.nin += in_box ? 1 : 0;
-        st.nonfin += i < n && !fin ? 1 : 0;
+        st.nonfin += valid && !fin ? 1 : 0;
       }
-      if (i < n) field_store<WIDE>(a, s_id, off, i, ins, mix, fin, open);
+      if (valid) field_store<WIDE>(a, s_id, off, i, ins, mix, fin, open);
       const uint32_t ob = __ballot_sync(0xffffffffu, open);
       if (open) {
         Pending<WIDE> p;
@@ -852,7 +1057,7 @@ __global__ void __launch_bounds__(kGlThreads, 4) k_grid_label(GridArgs a) {
     while (queued >= 32 || (last && queued > 0)) {
       const Pending<WIDE> p = s_q[wid][lane];
       const int cnt = min(queued, 32);
-      decide<WIDE>(a, s_g, s_id, sb, wid, lane, off, p.x, p.y, p.z, p.i, lane < cnt, p.ins, p.mix, st.eval, st.own);
+      decide<WIDE, false>(a, s_g, s_id, sb, wid, lane, off, p.x, p.y, p.z, p.i, lane < cnt, p.ins, p.mix, st.eval, st.own);
       for (int j = lane; j + 32 < queued; j += 32) {
         const Pending<WIDE> t = s_q[wid][j + 32];
         s_q[wid][j] = t;
@@ -955,6 +1160,24 @@ __global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
   if (!PLAIN && a.stats) flush_stats(a, st, s_stat, wid, lane);
 }
 
+// 32 of the points that the streaming kernel listed, one per lane (entry j).
+template <bool WIDE, bool LIST>
+__device__ __forceinline__ void pending_batch(const GridArgs &a, const GridComp *s_g, const int32_t *s_id, Batch &sb, int wid,
+                                              int lane, int64_t off, int64_t j, int64_t m, LaneStats &st) {
+  const bool have = j < m;
+  const int32_t i = have ? a.pending[j] : 0;
+  float x = __int_as_float(0x7fc00000), y = x, z = x;
+  if (have) {
+    const float *p = a.pts + 3 * (off + i);
+    x = p[0];
+    y = p[1];
+    z = p[2];
+  }
+  bool in_box;
+  const auto c = field_cell<WIDE>(a, x, y, z, &in_box);
+  decide<WIDE, LIST>(a, s_g, s_id, sb, wid, lane, off, x, y, z, i, have, c.x, c.y, st.eval, st.own);
+}
+
 // The listed points, 32 at a time.
 template <bool WIDE>
 __global__ void __launch_bounds__(kGlThreads, 4) k_grid_pending(GridArgs a) {
@@ -962,33 +1185,103 @@ __global__ void __launch_bounds__(kGlThreads, 4) k_grid_pending(GridArgs a) {
   __shared__ int32_t s_id[ZEF_MAX_COMPARTMENTS];
   __shared__ Batch sb;
   __shared__ unsigned long long s_stat[kGlWarps][GS_COUNT];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // k_grid_open may be launched (it waits)
   const int64_t m = a.counters[CNT_PEND];
   if ((int64_t)blockIdx.x * kGlThreads >= m) return;
   load_grids(a, s_g, s_id);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   __syncthreads();
   const int64_t off = a.n_host >= 0 ? 0 : a.counters[CNT_OFF];
-  const float *pts = a.pts + 3 * off;
   LaneStats st;
-  for (int64_t j0 = (int64_t)blockIdx.x * kGlThreads + 32 * wid; j0 < m; j0 += (int64_t)gridDim.x * kGlThreads) {
-    const bool have = j0 + lane < m;
-    const int32_t i = have ? a.pending[j0 + lane] : 0;
-    float x = __int_as_float(0x7fc00000), y = x, z = x;
-    if (have) {
-      x = pts[3 * (int64_t)i];
-      y = pts[3 * (int64_t)i + 1];
-      z = pts[3 * (int64_t)i + 2];
-    }
-    bool in_box;
-    const auto c = field_cell<WIDE>(a, x, y, z, &in_box);
-    decide<WIDE>(a, s_g, s_id, sb, wid, lane, off, x, y, z, i, have, c.x, c.y, st.eval, st.own);
-  }
+  for (int64_t j0 = (int64_t)blockIdx.x * kGlThreads + 32 * wid; j0 < m; j0 += (int64_t)gridDim.x * kGlThreads)
+    pending_batch<WIDE, true>(a, s_g, s_id, sb, wid, lane, off, j0 + lane, m, st);
   if (a.stats) flush_stats(a, st, s_stat, wid, lane);
+}
+
+// The points that the crossings left open, one block each: the rows left open
+// in turn, the crossings in FP64 by one warp, then the solid angle by the
+// block.  (By the warp that met them, one pair after the other, 4,096
+// consecutive vertices took 11.7 ms.)  Where the list did not hold them all,
+// the pending points are taken once more, their open pairs by the warps.  The
+// last block leaves the lists empty, so that a call need not clear them first.
+template <bool WIDE>
+__global__ void __launch_bounds__(kOpenThreads) k_grid_open(GridArgs a) {
+  using M = typename FieldCell<WIDE>::M;
+  __shared__ union {
+    OpenShared open;
+    struct {
+      GridComp g[ZEF_MAX_COMPARTMENTS];
+      int32_t id[ZEF_MAX_COMPARTMENTS];
+      Batch batch;
+    } again;
+  } sh;
+  static_assert(kOpenThreads == kGlThreads, "the second part's batches");
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // for k_grid_pending, where launched beside it
+  const int64_t listed = a.counters[CNT_OPEN];
+  if (listed == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.counters[CNT_PEND] = 0;
+    return;
+  }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t off = a.n_host >= 0 ? 0 : a.counters[CNT_OFF];
+  const int64_t n = a.n_host >= 0 ? a.n_host : a.counters[CNT_N], m = a.counters[CNT_PEND];
+  if (listed > kOpenCap) {
+    load_grids(a, sh.again.g, sh.again.id);
+    __syncthreads();
+    LaneStats st;  // counted before
+    const int64_t tiles = run_tiles(m, 32);
+    for (int64_t t = (int64_t)wid * gridDim.x + blockIdx.x; t < tiles; t += (int64_t)gridDim.x * kGlWarps)
+      pending_batch<WIDE, false>(a, sh.again.g, sh.again.id, sh.again.batch, wid, lane, off, run_point(t, tiles, lane), m, st);
+  } else {
+    for (int64_t e = blockIdx.x; e < listed; e += gridDim.x) {
+      const OpenPoint p = a.open[e];
+      if (!ZEF_BOUNDS_OK(p.i >= 0 && p.i < n, a.status, 31)) continue;
+      const float *q = a.pts + 3 * (off + p.i);
+      const float x = q[0], y = q[1], z = q[2];
+      M mask = (M)p.ins, left = (M)p.open;
+      while (left) {
+        const int r = first_row(left);
+        left &= left - 1;
+        const GridComp &g = a.grid[r];
+        if (wid == 0) {
+          int k = 0;
+          const bool decided = crossings64(a, g, cell_word(a, g, x, y, z), x, y, z, lane, &k);
+          if (lane == 0) {
+            sh.open.decided = decided;
+            sh.open.k = k;
+          }
+        }
+        __syncthreads();
+        const bool decided = sh.open.decided;
+        const int k = sh.open.k;
+        __syncthreads();
+        const double om = decided ? 0.0 : solid64_block(a, g, x, y, z, sh.open, lane, wid);
+        const bool inside = decided ? k >= 1 : om > kTwoPi64;
+        if (threadIdx.x == 0 && a.omega) a.omega[(int64_t)r * a.omega_ld + p.i] = decided ? kFourPi * (float)k : (float)om;
+        if (inside) {
+          mask |= (M)1 << r;
+          if (a.early) left = 0;
+        }
+      }
+      if (threadIdx.x == 0) {
+        a.labels[off + p.i] = mask ? a.row_ids[first_row(mask)] : 0;
+        if (a.masks) a.masks[off + p.i] = mask;
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 &&
+      atomicAdd((unsigned long long *)(a.counters + CNT_OPEN_DONE), 1ull) == (unsigned long long)gridDim.x - 1ull) {
+    a.counters[CNT_PEND] = 0;
+    a.counters[CNT_OPEN] = 0;
+    a.counters[CNT_OPEN_DONE] = 0;
+  }
 }
 
 __global__ void k_grid_reset(int64_t *cnt) {
   constexpr int c[] = {CNT_ITEMS, CNT_UNC,      CNT_NONFINITE, CNT_PAIRS_EVAL, CNT_PAIRS_RESCUE,
-                       CNT_COHERENT, CNT_REP_PAIRS, CNT_LANE_TILES, CNT_NIN,     CNT_TILES, CNT_PEND};
+                       CNT_COHERENT, CNT_REP_PAIRS, CNT_LANE_TILES, CNT_NIN,     CNT_TILES,      CNT_PEND,
+                       CNT_OPEN,     CNT_OPEN_DONE};
   if (threadIdx.x < sizeof(c) / sizeof(c[0])) cnt[c[threadIdx.x]] = 0;
 }
 
@@ -1020,11 +1313,18 @@ bool grid_serves(const zef_ctx *ctx, const zef_label_opts &o) {
 // at most 65,536 points, never needs).
 constexpr int64_t kListedMin = 1 << 18;
 static_assert(kListedMin > ZEF_NOALLOC_MAX_POINTS, "the allocation-free entry point has no list");
-static bool grid_listed(const zef_ctx *ctx, int64_t n_cap) { return n_cap >= kListedMin && ctx->lb.cap_pending >= n_cap; }
+static bool grid_listed(const zef_ctx *ctx, int64_t n_cap) {
+  return n_cap >= kListedMin && ctx->lb.cap_pending >= n_cap && ctx->lb.open;
+}
 
 zef_status grid_reserve(zef_ctx *ctx, int64_t n_cap) {
   LabelBuffers &b = ctx->lb;
-  if (n_cap < kListedMin || b.cap_pending >= n_cap) return ZEF_OK;
+  if (n_cap < kListedMin) return ZEF_OK;
+  if (!b.open) {
+    const cudaError_t e = cudaMalloc(&b.open, kOpenCap * sizeof(OpenPoint));
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(points on a surface)");
+  }
+  if (b.cap_pending >= n_cap) return ZEF_OK;
   if (b.pending) cudaFree(b.pending);
   b.pending = nullptr;
   b.cap_pending = 0;
@@ -1059,14 +1359,17 @@ zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
   // The list serves calls that fill the GPU; below that one launch is shorter.
   const bool listed = grid_listed(ctx, plan.n_cap);
   a.pending = ctx->lb.pending;
+  a.open = ctx->lb.open;
   if (plan.timed) cudaEventRecord(ctx->ev[0], s);
-  if (a.stats || listed) {
+  if (a.stats || (listed && ctx->lb.lists_dirty)) {
     k_grid_reset<<<1, 32, 0, s>>>(ctx->lb.counters);
     ++ctx->launches;
   }
+  if (listed) ctx->lb.lists_dirty = true;  // until every kernel of this call is launched
   NvtxRange nvtx_stage("zef.label_kernel");
   if (plan.timed) cudaEventRecord(ctx->ev[1], s);
   const bool wide = a.ncomp > 32;
+  a.tile = kGlTile;
   if (listed) {
     const int64_t tiles = (plan.n_cap + kGsTile - 1) / kGsTile;
     // a warp's consecutive tiles list neighbouring points together
@@ -1081,20 +1384,47 @@ zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
     else k_grid_pending<false><<<pblocks, kGlThreads, 0, s>>>(a);
     ctx->launches += 2;
   } else {
+    // as few points per warp as 16 warps an SM allow, kRun to kGlTile (calls
+    // one behind the other, the three-layer head; with 8, 16, 32, 64: 5,000 points 8.2,
+    // 8.3, 8.3, 10.3 us; 36,864 10.3, 10.3, 8.3, 10.3; 65,536 with solid
+    // angles 16.5, 12.3, 10.3, 11.8; 200,000 with them 36, 25, 19, 14.5);
+    // neighbouring tiles go to different blocks
     a.iters = 1;
-    const unsigned blocks = (unsigned)std::max<int64_t>(1, (plan.n_cap + kGlWarps * kGlTile - 1) / (kGlWarps * kGlTile));
+    while (a.tile > kRun && plan.n_cap <= (int64_t)ctx->num_sms * 16 * (a.tile / 2)) a.tile /= 2;
+    const int64_t tiles = std::max<int64_t>(1, (plan.n_cap + a.tile - 1) / a.tile);
+    const unsigned blocks = (unsigned)std::min(tiles, std::max((int64_t)ctx->num_sms, (tiles + kGlWarps - 1) / kGlWarps));
     if (wide) k_grid_label<true><<<blocks, kGlThreads, 0, s>>>(a);
     else k_grid_label<false><<<blocks, kGlThreads, 0, s>>>(a);
     ++ctx->launches;
   }
+  if (plan.timed) cudaEventRecord(ctx->ev[2], s);
+  nvtx_stage.next("zef.rescue64");
+  if (plan.timed) cudaEventRecord(ctx->ev[3], s);
+  if (listed) {
+    // most calls have few such points or none: the launch overlaps the kernel
+    // before it (the library's own graphs, some with conditional nodes, and
+    // timed calls, with events in between, launch it the plain way).  5.2 M
+    // points: 84.8 us, 83.9 with the overlap; a million nodes with every row
+    // decided: 75.6 and 73.8
+    cudaLaunchAttribute overlap;
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctx->num_sms * 2);
+    cfg.blockDim = dim3(kOpenThreads);
+    cfg.stream = s;
+    cfg.attrs = &overlap;
+    cfg.numAttrs = plan.n_host >= 0 && !plan.timed ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, wide ? k_grid_open<true> : k_grid_open<false>, a);
+    ++ctx->launches;
+  }
   if (plan.timed) {
-    cudaEventRecord(ctx->ev[2], s);
-    cudaEventRecord(ctx->ev[3], s);
     cudaEventRecord(ctx->ev[4], s);
     cudaEventRecord(ctx->ev[5], s);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "k_grid_label launch");
+  ctx->lb.lists_dirty = false;
   return ZEF_OK;
 }
 

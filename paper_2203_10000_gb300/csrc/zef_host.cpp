@@ -246,7 +246,7 @@ void zef_destroy(zef_ctx *ctx) {
   LabelBuffers &b = ctx->lb;
   fr(b.spts); fr(b.perm); fr(b.keys); fr(b.in_mask); fr(b.unc_mask); fr(b.tile_box);
   fr(b.hist); fr(b.flags); fr(b.block_sums); fr(b.items); fr(b.unc_list); fr(b.counters);
-  fr(b.pending); fr(b.labels_tmp); fr(b.pts_tmp); fr(b.omega_tmp); fr(b.tune_pts);
+  fr(b.pending); fr(b.open); fr(b.labels_tmp); fr(b.pts_tmp); fr(b.omega_tmp); fr(b.tune_pts);
   fr(ctx->el_node_labels); fr(ctx->el_masks); fr(ctx->el_tets); fr(ctx->el_labels);
   for (auto &p : ctx->rf_buf) fr(p);
   for (auto &p : ctx->rb_buf) fr(p);

@@ -190,6 +190,13 @@ struct CompHost {
   double dop[kDop];  // max over the vertices of d_k . v (unscaled coordinates)
 };
 
+// A point that the cell grid leaves to the FP64 solid angles (zef_grid.cu).
+struct OpenPoint {
+  unsigned long long ins, open;  // rows it is inside of, rows to be decided
+  int32_t i;
+};
+constexpr int kOpenCap = 1 << 15;
+
 // Grow-only device buffers of the labeling pipeline.
 struct LabelBuffers {
   int64_t cap_points = 0;   // points the buffers hold
@@ -210,6 +217,8 @@ struct LabelBuffers {
   int64_t *counters = nullptr;  // device counters, see Counter enum
   int32_t *pending = nullptr;   // cell grid: points whose label the field leaves open
   int64_t cap_pending = 0;
+  OpenPoint *open = nullptr;    // cell grid: kOpenCap points for the FP64 solid angles
+  bool lists_dirty = false;     // the lists' counters may not be zero (a call failed half-way)
   int64_t cap_stage = 0;
   int32_t *labels_tmp = nullptr;
   float *pts_tmp = nullptr;     // staging for host inputs
@@ -254,7 +263,12 @@ enum Counter {
   CNT_RF_MASK,        // refinement: slots of the level's edge table - 1
   CNT_RF_SHIFT,       // log2 of the slots per node of its placement, 0: hashed over the table
   CNT_LANE_TILES,     // cap trees: (tile, compartment) pairs evaluated by per-lane walks
-  CNT_PEND,           // cell grid: points whose label the field leaves open
+  // cell grid (zero again when a call is over): points whose label the field
+  // leaves open, points listed for the FP64 solid angles (may exceed
+  // kOpenCap), blocks done with those
+  CNT_PEND,
+  CNT_OPEN,
+  CNT_OPEN_DONE,
   CNT_UNC_LIST,       // uncertain pairs appended to the pair list (may exceed its capacity)
   CNT_COUNT_ = 40
 };
