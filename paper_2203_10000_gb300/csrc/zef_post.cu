@@ -796,7 +796,8 @@ __device__ __forceinline__ float4 lap_step(const Adj &g, const float4 *p, int64_
 // y = x + lambda L(x) (fixed nodes keep x); block sums of |y - x|^2 in a fixed
 // order.  With xi = 0 only a sum of zero stops the loop, so NORM = false leaves
 // 1 when some node of the block moved, else 0, and does no FP64 work.
-template <bool NORM>
+// With BOUNDARY the norms run over the nodes that have a neighbour.
+template <bool NORM, bool BOUNDARY>
 __global__ void __launch_bounds__(256) k_sm_forward(Smooth s) {
   if (s.g.words[PP_STOP]) return;
   double acc = 0.0;
@@ -806,7 +807,8 @@ __global__ void __launch_bounds__(256) k_sm_forward(Smooth s) {
     float4 o = c;
     if (!(s.fixed && s.fixed[i])) o = lap_step(s.g, s.x, i, c, s.lambda);
     s.y[i] = o;
-    if (NORM && s.g.fill[i]) {  // a node without neighbours does not move
+    if (BOUNDARY && !s.g.fill[i]) continue;
+    if (NORM) {
       const double d0 = (double)o.x - c.x, d1 = (double)o.y - c.y, d2 = (double)o.z - c.z;
       acc += d0 * d0 + d1 * d1 + d2 * d2;
     } else {
@@ -837,7 +839,9 @@ __global__ void __launch_bounds__(256) k_sm_next(Smooth s) {
   if (threadIdx.x != 0) return;
   const int64_t it = ++s.g.words[PP_ITER];
   const double x0 = *s.x0;
-  const bool small = x0 > 0.0 ? sqrt(ss) / x0 <= (double)s.xi : true;
+  // an infinite coordinate: its difference, and so the ratio, is not a number,
+  // which is not small (and which the NORM = false form does not see)
+  const bool small = x0 > 0.0 ? !isinf(x0) && sqrt(ss) / x0 <= (double)s.xi : true;
   if (small || it >= s.max_iters || s.g.words[PP_BAD]) s.g.words[PP_STOP] = 1;
 }
 
@@ -1264,12 +1268,13 @@ zef_status smooth_loop(zef_ctx *ctx, float *x, int64_t n, const Adj &g, const ui
   sm.nblocks = nblocks;
   k_sm_pack<<<nblocks, threads, 0, s>>>(x, n, boundary_norm ? g.fill : nullptr, sm.x, partial);
   k_sm_norm<<<1, threads, 0, s>>>(partial, nblocks, partial + nblocks);
+  auto forward = o.xi > 0.f ? (boundary_norm ? k_sm_forward<true, true> : k_sm_forward<true, false>)
+                            : (boundary_norm ? k_sm_forward<false, true> : k_sm_forward<false, false>);
   int batch = o.xi > 0.f ? 1 : 32;
   for (int left = o.max_iters; left > 0;) {
     const int k = std::min(batch, left);
     for (int q = 0; q < k; ++q) {
-      if (o.xi > 0.f) k_sm_forward<true><<<nblocks, threads, 0, s>>>(sm);
-      else k_sm_forward<false><<<nblocks, threads, 0, s>>>(sm);
+      forward<<<nblocks, threads, 0, s>>>(sm);
       k_sm_backward<<<nblocks, threads, 0, s>>>(sm);
       k_sm_next<<<1, threads, 0, s>>>(sm);
     }
