@@ -80,7 +80,7 @@ constexpr uint32_t kOffsetMask = kCellOffset;
 constexpr float kPlane = 32.f;
 constexpr int kNoK = -128;  // block header: the anchor's winding number is unknown
 // A block: a header (anchor x, y, z; k in the low 8 bits of w and the number
-// of chunks above), then chunks of kSub entries: kSub first words (a x b, V),
+// of triangles above), then chunks of kSub entries: kSub first words (a x b, V),
 // kSub second (b x c, error bound), kSub third (c x a, triangle index), so
 // that kSub lanes read 128 bytes at a time.  The last chunk is filled up with
 // entries that the test calls a miss.
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(256) k_gr_finish(const float4 *tris, float to_
     float4 *block = blocks + off[c];
     if (lane == 0) {
       words[c] = kMixed | (chunks <= 3 ? chunks << kChunkShift : 0u) | off[c];
-      block[0] = make_float4(qx, qy, qz, __uint_as_float((chunks << 8) | ((uint32_t)(known ? (int)kf : kNoK) & 0xffu)));
+      block[0] = make_float4(qx, qy, qz, __uint_as_float(((e - b) << 8) | ((uint32_t)(known ? (int)kf : kNoK) & 0xffu)));
     }
     for (uint32_t j = b + lane; j < b + chunks * kSub; j += 32) {
       float4 *o = block + 1 + (j - b) / kSub * kChunkWords + (j - b) % kSub;
@@ -363,14 +363,13 @@ __device__ __noinline__ bool crossings64(const GridArgs &a, const GridComp &g, u
   if (word & kMixed) {
     const float4 *block = g.blocks + (word & kOffsetMask);
     const float4 r = block[0];
-    const int k0 = (int)(signed char)(__float_as_uint(r.w) & 0xffu), count = (int)(__float_as_uint(r.w) >> 8) * kSub;
+    const int k0 = (int)(signed char)(__float_as_uint(r.w) & 0xffu), count = (int)(__float_as_uint(r.w) >> 8);
     int net = 0, tested = 0;
     bool open = k0 == kNoK;
     if (!open) {
       const double dx = (double)x - r.x, dy = (double)y - r.y, dz = (double)z - r.z;
       for (int j = lane; j < count; j += 32) {
         const int64_t t = __float_as_int(block[1 + j / kSub * kChunkWords + 2 * kSub + j % kSub].w);
-        if (t < 0) continue;
         ++tested;
         double v[3][3];
 #pragma unroll
@@ -822,7 +821,7 @@ __device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, c
         const float4 h = __ldg(block);
         const float4 *t = block + 1 + ti;
         int chunks = (int)((w & ~kMixed) >> kChunkShift);
-        if (!chunks) chunks = (int)(__float_as_uint(h.w) >> 8);
+        if (!chunks) chunks = (int)(((__float_as_uint(h.w) >> 8) + kSub - 1) / kSub);
         const int k0 = (int)(signed char)(__float_as_uint(h.w) & 0xffu);
         const float dx = q.x - h.x, dy = q.y - h.y, dz = q.z - h.z;
         bool open = k0 == kNoK;
@@ -857,7 +856,7 @@ __device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, c
           k = kn;
           unc = ((bu >> ((rank - j0) * kLanes)) & ((1u << kLanes) - 1u)) != 0u;
         }
-        if (a.stats && j0 + sub < np && ti == 0) st_eval += (uint32_t)chunks * kSub;
+        if (a.stats && j0 + sub < np && ti == 0) st_eval += __float_as_uint(h.w) >> 8;
       }
       __syncwarp();
       ++st_own;

@@ -1054,11 +1054,8 @@ __global__ void __launch_bounds__(256) k_in_hits(const int2 *edges, const uint32
         const uint32_t word = cells.words[((int64_t)cz * cells.n[1] + cy) * cells.n[0] + cx];
         if (!(word & kCellMixed)) continue;
         const float4 *block = cells.blocks + (word & kCellOffset);
-        const int entries = (int)(__float_as_uint(block[0].w) >> 8) * kSub;
-        for (int e = 0; e < entries; ++e) {
-          const int t = __float_as_int(block[1 + e / kSub * kChunkWords + 2 * kSub + e % kSub].w);
-          if (t >= 0) test(t);
-        }
+        const int entries = (int)(__float_as_uint(block[0].w) >> 8);
+        for (int e = 0; e < entries; ++e) test(__float_as_int(block[1 + e / kSub * kChunkWords + 2 * kSub + e % kSub].w));
       }
     } else {
       int nl = 0;
