@@ -329,6 +329,10 @@ struct GridArgs {
   const GridComp *grid;       // by priority row
   const int32_t *row_ids;
   int64_t *counters;
+#ifdef ZEF_DEBUG_BOUNDS
+  int64_t n_nodes, n_cseg;    // cap-tree nodes and segment entries
+  int64_t pend_cap;           // entries of `pending`
+#endif
   int64_t n_host;             // points, or -1: counters[CNT_N] from counters[CNT_OFF] on
   int ncomp;
   int early;                  // a point certainly inside needs no later compartment
@@ -370,6 +374,7 @@ __device__ __noinline__ bool crossings64(const GridArgs &a, const GridComp &g, u
       const double dx = (double)x - r.x, dy = (double)y - r.y, dz = (double)z - r.z;
       for (int j = lane; j < count; j += 32) {
         const int64_t t = __float_as_int(block[1 + j / kSub * kChunkWords + 2 * kSub + j % kSub].w);
+        if (!ZEF_BOUNDS_OK(t >= 0 && t < a.comps[g.comp].tri_cnt, a.status, 34)) continue;
         ++tested;
         double v[3][3];
 #pragma unroll
@@ -453,7 +458,7 @@ __device__ __noinline__ double solid64(const GridArgs &a, const GridComp &g, flo
                 b = __shfl_sync(0xffffffffu, seg_b, q);
       if (lane >= f && lane < e) pos = b + 4 * (lane - f);
     }
-    if (pos >= 0) {
+    if (pos >= 0 && ZEF_BOUNDS_OK((int64_t)pos + 4 <= a.n_cseg, a.status, 36)) {
       const double h = group64(a.cseg, pos, px, py, pz, &K);
 #pragma unroll
       for (int q = 0; q < 8; ++q)
@@ -473,6 +478,7 @@ __device__ __noinline__ double solid64(const GridArgs &a, const GridComp &g, flo
   };
   const int root = cp->cap_root, end = a.nodes[root].skip;
   for (int i = root; i != end;) {
+    if (!ZEF_BOUNDS_OK(i >= 0 && i < a.n_nodes, a.status, 35)) break;
     const CapNode nd = a.nodes[i];
     const bool far = nd.hi[0] < px || nd.lo[0] > px || nd.hi[1] < py || nd.lo[1] > py || nd.hi[2] < pz || nd.lo[2] > pz;
     int b = nd.cap_begin, c = nd.cap_cnt;
@@ -523,7 +529,13 @@ __device__ __forceinline__ uint32_t cell_word(const GridArgs &a, const GridComp 
   const int cx = axis_cell(x, g.lo[0], g.inv[0], g.n[0]), cy = axis_cell(y, g.lo[1], g.inv[1], g.n[1]),
             cz = axis_cell(z, g.lo[2], g.inv[2], g.n[2]);
   const int c = (cz * g.n[1] + cy) * g.n[0] + cx;  // at most kMaxCells
-  return ZEF_BOUNDS_OK(c >= 0 && c < g.n[0] * g.n[1] * g.n[2], a.status, 30) ? __ldg(g.words + c) : 0u;
+  if (!ZEF_BOUNDS_OK(c >= 0 && c < g.n[0] * g.n[1] * g.n[2], a.status, 30)) return 0u;
+  const uint32_t w = __ldg(g.words + c);
+  // the words lie behind the blocks; a block is a header and a chunk at least
+  if ((w & kMixed) && !ZEF_BOUNDS_OK((w & kOffsetMask) + 1u + kChunkWords * max(1u, (w & ~kMixed) >> kChunkShift) <=
+                                         (uint64_t)(reinterpret_cast<const float4 *>(g.words) - g.blocks), a.status, 32))
+    return 0u;
+  return w;
 }
 
 // Both by the whole warp: whether the point is inside; *omega = Omega.
@@ -597,7 +609,9 @@ __device__ double solid64_block(const GridArgs &a, const GridComp &g, float x, f
       if (e < len) {
         o0 = sh.seg[cur][e];
         n = 1;
-        if (o0.y == 0) {
+        if (o0.y == 0 && !ZEF_BOUNDS_OK(o0.x >= 0 && o0.x < a.n_nodes, a.status, 37)) {
+          n = 0;
+        } else if (o0.y == 0) {
           const CapNode nd = a.nodes[o0.x];
           const bool far = nd.hi[0] < px || nd.lo[0] > px || nd.hi[1] < py || nd.lo[1] > py || nd.hi[2] < pz || nd.lo[2] > pz;
           if (!far && nd.left >= 0) {
@@ -652,7 +666,8 @@ __device__ double solid64_block(const GridArgs &a, const GridComp &g, float x, f
       if (sh.first[mid] <= j) lo = mid;
       else hi = mid - 1;
     }
-    part += group64(a.cseg, sh.seg[cur][lo].x + 4 * (j - sh.first[lo]), px, py, pz, &K);
+    const int pos = sh.seg[cur][lo].x + 4 * (j - sh.first[lo]);
+    if (ZEF_BOUNDS_OK(pos >= 0 && (int64_t)pos + 4 <= a.n_cseg, a.status, 38)) part += group64(a.cseg, pos, px, py, pz, &K);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
@@ -822,6 +837,7 @@ __device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, c
         const float4 *t = block + 1 + ti;
         int chunks = (int)((w & ~kMixed) >> kChunkShift);
         if (!chunks) chunks = (int)(((__float_as_uint(h.w) >> 8) + kSub - 1) / kSub);
+        if (!ZEF_BOUNDS_OK(chunks <= kMaxList / kSub, a.status, 33)) chunks = 0;
         const int k0 = (int)(signed char)(__float_as_uint(h.w) & 0xffu);
         const float dx = q.x - h.x, dy = q.y - h.y, dz = q.z - h.z;
         bool open = k0 == kNoK;
@@ -940,8 +956,9 @@ __device__ __forceinline__ typename FieldCell<WIDE>::T field_cell(const GridArgs
     const int cx = min((int)((x - a.field.lo[0]) * a.field.inv[0]), a.field.n[0] - 1),
               cy = min((int)((y - a.field.lo[1]) * a.field.inv[1]), a.field.n[1] - 1),
               cz = min((int)((z - a.field.lo[2]) * a.field.inv[2]), a.field.n[2] - 1);
-    c = __ldg(reinterpret_cast<const typename FieldCell<WIDE>::T *>(a.field.cells) +
-              ((cz * a.field.n[1] + cy) * a.field.n[0] + cx));
+    const int at = (cz * a.field.n[1] + cy) * a.field.n[0] + cx;
+    if (ZEF_BOUNDS_OK(at >= 0 && at < a.field.n[0] * a.field.n[1] * a.field.n[2], a.status, 39))
+      c = __ldg(reinterpret_cast<const typename FieldCell<WIDE>::T *>(a.field.cells) + at);
   }
   return c;
 }
@@ -1048,7 +1065,8 @@ __global__ void __launch_bounds__(kGlThreads, 4) k_grid_label(GridArgs a) {
         p.i = (int32_t)i;
         p.ins = ins;
         p.mix = mix;
-        s_q[wid][queued + __popc(ob & ((1u << lane) - 1u))] = p;
+        const int at = queued + __popc(ob & ((1u << lane) - 1u));
+        if (ZEF_BOUNDS_OK(at < kGlQueue, a.status, 40)) s_q[wid][at] = p;
       }
       queued += __popc(ob);
     }
@@ -1128,7 +1146,8 @@ __global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
         if (!in_box[u] && !(isfinite(x[u]) && isfinite(y[u]) && isfinite(z[u]))) l = -1;
         if (!open && base + 32 * u + lane < count) lab[32 * u] = l;
         const uint32_t ob = __ballot_sync(0xffffffffu, open);
-        if (open) s_q[wid][queued + __popc(ob & ((1u << lane) - 1u))] = (int32_t)(first + base + 32 * u + lane);
+        const int at = queued + __popc(ob & ((1u << lane) - 1u));
+        if (open && ZEF_BOUNDS_OK(at < kGsQueue, a.status, 41)) s_q[wid][at] = (int32_t)(first + base + 32 * u + lane);
         queued += __popc(ob);
       } else {
         const int64_t i = first + base + 32 * u + lane;
@@ -1142,7 +1161,8 @@ __global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
         }
         if (valid) field_store<WIDE>(a, s_id + 1, off, i, ins, mix, fin, open);
         const uint32_t ob = __ballot_sync(0xffffffffu, open);
-        if (open) s_q[wid][queued + __popc(ob & ((1u << lane) - 1u))] = (int32_t)i;
+        const int at = queued + __popc(ob & ((1u << lane) - 1u));
+        if (open && ZEF_BOUNDS_OK(at < kGsQueue, a.status, 42)) s_q[wid][at] = (int32_t)i;
         queued += __popc(ob);
       }
     }
@@ -1151,7 +1171,8 @@ __global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
       unsigned long long at = 0;
       if (lane == 0) at = atomicAdd((unsigned long long *)(a.counters + CNT_PEND), (unsigned long long)queued);
       at = __shfl_sync(0xffffffffu, at, 0);
-      for (int j = lane; j < queued; j += 32) a.pending[at + j] = s_q[wid][j];
+      for (int j = lane; j < queued; j += 32)
+        if (ZEF_BOUNDS_OK(at + j < (unsigned long long)a.pend_cap, a.status, 43)) a.pending[at + j] = s_q[wid][j];
       queued = 0;
       __syncwarp();
     }
@@ -1163,8 +1184,9 @@ __global__ void __launch_bounds__(kGlThreads, 6) k_grid_stream(GridArgs a) {
 template <bool WIDE, bool LIST>
 __device__ __forceinline__ void pending_batch(const GridArgs &a, const GridComp *s_g, const int32_t *s_id, Batch &sb, int wid,
                                               int lane, int64_t off, int64_t j, int64_t m, LaneStats &st) {
-  const bool have = j < m;
+  bool have = j < m;
   const int32_t i = have ? a.pending[j] : 0;
+  have = have && ZEF_BOUNDS_OK(i >= 0 && i < (a.n_host >= 0 ? a.n_host : a.counters[CNT_N]), a.status, 44);
   float x = __int_as_float(0x7fc00000), y = x, z = x;
   if (have) {
     const float *p = a.pts + 3 * (off + i);
@@ -1354,6 +1376,11 @@ zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
   a.comps = ctx->d_comps;
   a.nodes = ctx->d_nodes;
   a.cseg = ctx->d_cseg;
+#ifdef ZEF_DEBUG_BOUNDS
+  a.n_nodes = (int64_t)ctx->h_nodes.size();
+  a.n_cseg = (int64_t)ctx->h_cseg.size();
+  a.pend_cap = ctx->lb.cap_pending;
+#endif
   a.scale = ctx->scale;
   // The list serves calls that fill the GPU; below that one launch is shorter.
   const bool listed = grid_listed(ctx, plan.n_cap);
