@@ -44,3 +44,69 @@ def test_evaluated_pairs_are_those_of_the_cells_triangles(zef, n):
     first = st["pairs_evaluated"] - st["pairs_rescued"]
     assert 0.9 * n < first <= 4 * n
     assert st["pairs_nominal"] == 4 * n
+
+
+def _equal_general(zef, ctx, pts):
+    """Labels, early and full, and solid angles of the default path against the
+    general kernels'."""
+    p = torch.from_numpy(pts).cuda()
+    lab, om, st = ctx.label_points(p, want_omega=True)
+    early, _, _ = ctx.label_points(p, stats=False)
+    opts = zef.make_opts(block_threads=256, points_per_thread=2)
+    glab, gom, gst = ctx.label_points(p, want_omega=True, opts=opts)
+    ctx.synchronize()
+    assert torch.equal(lab, glab) and torch.equal(early, glab)
+    assert torch.equal(om.isnan(), gom.isnan())
+    # a certified value is 4 pi k in float32, an FP64 sum its rounding
+    assert float((om - gom).nan_to_num().abs().max()) <= 1e-6
+    assert st["nonfinite_points"] == gst["nonfinite_points"] and st["points"] == len(pts)
+    return lab.cpu().numpy(), st
+
+
+# a warp of the streaming kernel takes 128 points at a time, lists 256 together
+@pytest.mark.parametrize("n", [LISTED - 1, LISTED, LISTED + 1, LISTED + 127, LISTED + 128, LISTED + 129, LISTED + 32 * 128 + 1])
+def test_calls_around_the_listed_size(zef, n):
+    w = zs.config1(npts_limit=0)
+    ctx = _context(zef, w.surfaces, w.priority)
+    rng = np.random.default_rng(n)
+    v = np.concatenate([s.verts for s in w.surfaces])
+    pts = rng.uniform(v.min(0) * 1.1, v.max(0) * 1.1, (n, 3)).astype(np.float32)
+    # a stretch where every point is open, at the end too, and points not finite
+    near = v[rng.integers(0, len(v), 3000)] + rng.normal(0, 0.3, (3000, 3)).astype(np.float32)
+    pts[1000:3500] = near[:2500]
+    pts[-500:] = near[2500:]
+    bad = np.concatenate([rng.integers(0, n, 300), [0, n - 1]])
+    pts[bad, rng.integers(0, 3, len(bad))] = rng.choice([np.nan, np.inf, -np.inf], len(bad))
+    lab, st = _equal_general(zef, ctx, pts)
+    ctx.close()
+    assert np.array_equal(lab == -1, ~np.isfinite(pts).all(1))
+    assert st["kernel_launches"] == (2 if n < LISTED else 4)
+
+
+def _spheres(count):
+    v, t = zs.geodesic_sphere(6)
+    rng = np.random.default_rng(count)
+    return [zs.Surface(k + 1, "s", (v * rng.uniform(0.4, 1.5) + rng.uniform(-3, 3, 3)).astype(np.float32), t)
+            for k in range(count)]
+
+
+# up to 32 surfaces a cell of the label field is two 32-bit words, then two of 64
+@pytest.mark.parametrize("count", [32, 33, 64])
+@pytest.mark.parametrize("n", [1000, 65_000, LISTED + 77])
+def test_many_surfaces(zef, count, n):
+    surfs = _spheres(count)
+    prio = [s.id for s in surfs[::-1]]
+    ctx = _context(zef, surfs, prio)
+    rng = np.random.default_rng(n)
+    v = np.concatenate([s.verts for s in surfs])
+    pts = rng.uniform(v.min(0), v.max(0), (n, 3)).astype(np.float32)
+    lab, _ = _equal_general(zef, ctx, pts)
+    assert len(np.unique(lab)) > count // 2 or n < 10_000
+    # the four-nodes rule takes every row's bit of every node
+    tets = torch.from_numpy(rng.integers(0, min(n, 500), (4000, 4)).astype(np.int32)).cuda()
+    nodes = torch.from_numpy(pts).cuda()
+    el, _, _ = ctx.label_elements(nodes, tets, stats=False)
+    gel, _, _ = ctx.label_elements(nodes, tets, opts=zef.make_opts(block_threads=256, points_per_thread=2), stats=False)
+    ctx.synchronize()
+    assert torch.equal(el, gel)
+    ctx.close()
