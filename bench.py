@@ -271,10 +271,13 @@ def roofline(st, ms_label, peak, sms, clocks=None, traffic=None):
 HBM_FALLBACK_GBS = 6800.0
 
 
-def grid_roofline(n_points, surface_bytes, ms_label):
+def grid_roofline(n_points, surface_bytes, ms_label, launches):
     """Labels from the cell grids (the default path): every point is read and
     every label written once, the grids' words and products come from L2, so
-    the denominator is the copy bandwidth."""
+    the denominator is the copy bandwidth.  Calls of up to 2^18 points are one
+    kernel (and one that clears the statistics); larger ones stream, decide
+    the open points and take points on a surface to FP64 (the time is that of
+    the first two)."""
     peak, basis = HBM_FALLBACK_GBS, "fallback copy bandwidth (no MEASURED_PEAKS.json)"
     try:
         peak = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"])
@@ -283,13 +286,15 @@ def grid_roofline(n_points, surface_bytes, ms_label):
         pass
     achieved = (16.0 * n_points + surface_bytes) / (ms_label * 1e-3) / 1e9
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-            "traffic": None, "kernel": "k_grid_label", "peak_basis": basis,
+            "traffic": None, "kernel": "k_grid_label" if launches <= 2 else "k_grid_stream + k_grid_pending",
+            "peak_basis": basis,
             "bytes_per_launch": int(16 * n_points + surface_bytes), "ms_per_launch": ms_label}
 
 
-def label_roofline(args_kernel, args_shape, st, w, n_points, ms_label, peak, sms, clocks=None, traffic=None):
-    if args_kernel == 0 and not args_shape and st["kernel_launches"] <= 3:   # the cell grids served the call
-        return grid_roofline(n_points, sum(12 * len(s.verts) + 12 * s.ntris for s in w.surfaces), ms_label)
+def label_roofline(st, w, n_points, ms_label, peak, sms, clocks=None, traffic=None):
+    if st["cell_grids"]:
+        return grid_roofline(n_points, sum(12 * len(s.verts) + 12 * s.ntris for s in w.surfaces), ms_label,
+                             st["kernel_launches"])
     return roofline(st, ms_label, peak, sms, clocks, traffic)
 
 
@@ -332,7 +337,7 @@ def secondary(zef, torch, dev, cfg, flush, stream, barrier, peak, sms, kernel):
            "ms_label_kernel": r["ms_label"], "ms_rescue": r["ms_rescue"],
            "uncertain_pairs_per_step": st["uncertain_pairs"],
            "autotuned_shape": [st["block_threads"], st["points_per_thread"]],
-           "roofline_frac": label_roofline(kernel, "", st, w, w.points.shape[0], r["ms_label"], peak, sms)["frac"],
+           "roofline_frac": label_roofline(st, w, w.points.shape[0], r["ms_label"], peak, sms)["frac"],
            "step_ms": [round(x, 3) for x in r["step_ms"]]}
     ctx.close()
     del pts, labels
@@ -490,7 +495,7 @@ def run_ours(args):
     nominal_job = job_points * tt
     value = nominal_job / (ms_step * 1e-3)
     sms, peak = fp32_peak_tflops(torch, dev)
-    rl = label_roofline(args.kernel, args.shape, st, w, n_local, r["ms_label"], peak, sms, r["clocks"],
+    rl = label_roofline(st, w, n_local, r["ms_label"], peak, sms, r["clocks"],
                         traffic_record(args.config, st, args.kernel) if not sharded else None)
 
     line = {"metric": METRIC, "value": value, "unit": "pairs/s", "n_gpus": ws, "steps": args.steps,

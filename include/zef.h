@@ -158,7 +158,8 @@ typedef struct zef_label_stats {
     float ms_total;            /* device time of the call (CUDA events) */
     float ms_label;            /* device time of the main labeling kernel */
     float ms_rescue;           /* device time of the FP64 re-evaluation */
-    float reserved;
+    int32_t cell_grids;        /* 1: the cell grids served the call, 0: the general
+                                  kernels did */
     int64_t coherent_pairs;    /* (point, compartment) pairs decided by the
                                   representative point of a tile or group,
                                   or by the anchor of their grid cell */

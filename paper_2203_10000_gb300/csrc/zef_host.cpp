@@ -862,7 +862,8 @@ static zef_status read_stats(zef_ctx *ctx, int64_t n, const zef_label_opts &o, c
   stats->work_items = h[CNT_ITEMS];
   // the cell grid's tiles: 64 consecutive points each, as many as the
   // points inside the union box would fill
-  stats->tiles = grid_serves(ctx, o) ? (h[CNT_NIN] + 63) / 64 : h[CNT_TILES];
+  stats->cell_grids = grid_serves(ctx, o);
+  stats->tiles = stats->cell_grids ? (h[CNT_NIN] + 63) / 64 : h[CNT_TILES];
   stats->coherent_pairs = h[CNT_COHERENT];
   stats->representative_pairs = h[CNT_REP_PAIRS];
   stats->lane_walk_items = h[CNT_LANE_TILES];

@@ -65,12 +65,12 @@ class LabelStats(ctypes.Structure):
                 ("work_items", ctypes.c_int64), ("tiles", ctypes.c_int64),
                 ("block_threads", ctypes.c_int32), ("points_per_thread", ctypes.c_int32),
                 ("ms_total", ctypes.c_float), ("ms_label", ctypes.c_float),
-                ("ms_rescue", ctypes.c_float), ("reserved", ctypes.c_float),
+                ("ms_rescue", ctypes.c_float), ("cell_grids", ctypes.c_int32),
                 ("coherent_pairs", ctypes.c_int64), ("representative_pairs", ctypes.c_int64),
                 ("lane_walk_items", ctypes.c_int64), ("kernel_launches", ctypes.c_int64)]
 
     def as_dict(self):
-        return {k: getattr(self, k) for k, _ in self._fields_ if k != "reserved"}
+        return {k: getattr(self, k) for k, _ in self._fields_}
 
 
 class Mesh(ctypes.Structure):

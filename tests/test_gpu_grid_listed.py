@@ -110,3 +110,13 @@ def test_many_surfaces(zef, count, n):
     ctx.synchronize()
     assert torch.equal(el, gel)
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [1000, LISTED])
+def test_statistics_say_which_path_served_the_call(zef, n):
+    w = zs.config0()
+    ctx = _context(zef, w.surfaces)
+    pts = torch.rand((n, 3), device="cuda")
+    assert ctx.label_points(pts)[2]["cell_grids"] == 1
+    assert ctx.label_points(pts, opts=zef.make_opts(block_threads=256, points_per_thread=2))[2]["cell_grids"] == 0
+    ctx.close()
