@@ -96,6 +96,7 @@ constexpr int kMaxAxis = 512;
 // cells, 630 with 2^22, 607 with 2^23; 20.5 M points in 20 small structures:
 // 108, 109 and 111.
 constexpr int64_t kMaxField = 1 << 22;
+constexpr size_t kScratchKept = (size_t)32 << 20;  // bytes of construction scratch kept between registrations
 constexpr int kMaxList = 1024;  // longest triangle list of a usable grid
 
 struct Geom {
@@ -1646,9 +1647,17 @@ zef_status grid_update(zef_ctx *ctx) {
     if (st) return st;
     ctx->grids.push_back(g);
   }
-  // the anchors' work buffers, where they are large: calls that the grids
-  // serve need none
+  // what the construction alone needed is given back where it is large: the
+  // anchors' work buffers (calls that the grids serve need none) and the
+  // scratch (24 bytes a cell and the triangle lists), which small surfaces
+  // registered one after the other reuse
   if (ctx->lb.cap_points > held && ctx->lb.cap_points > (int64_t)1 << 22) label_release(ctx);
+  if (ctx->gr_cap[0] + ctx->gr_cap[1] > kScratchKept)
+    for (int k = 0; k < 2; ++k) {
+      if (ctx->gr_buf[k]) cudaFree(ctx->gr_buf[k]);
+      ctx->gr_buf[k] = nullptr;
+      ctx->gr_cap[k] = 0;
+    }
   if (!ctx->d_grid) CK(cudaMalloc(&ctx->d_grid, ZEF_MAX_COMPARTMENTS * sizeof(GridComp)), "cudaMalloc(cell grids)");
   std::vector<GridComp> &d = ctx->h_grid;  // outlives the copy
   d.assign(C, GridComp{});

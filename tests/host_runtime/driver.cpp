@@ -1,7 +1,10 @@
 // Host code of the library on the runtime of fake_cudart.cpp: one scenario
 // per name; prints what is wrong and exits 1, or exits 0.
+#include <algorithm>
+#include <array>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -29,14 +32,13 @@ struct Surface {
 };
 Surface octahedron(float r, int m) {
   Surface s;
-  std::vector<std::vector<int>> keys;
+  std::map<std::array<int, 3>, int32_t> index;
   auto vertex = [&](int x, int y, int z) {
-    const std::vector<int> k = {x, y, z};
-    for (size_t i = 0; i < keys.size(); ++i)
-      if (keys[i] == k) return (int32_t)i;
-    keys.push_back(k);
-    for (int c : k) s.v.push_back(r * (float)c / (float)m);
-    return (int32_t)(keys.size() - 1);
+    const std::array<int, 3> k = {x, y, z};
+    const auto [it, fresh] = index.emplace(k, (int32_t)index.size());
+    if (fresh)
+      for (int c : k) s.v.push_back(r * (float)c / (float)m);
+    return it->second;
   };
   for (int o = 0; o < 8; ++o) {
     const int sx = o & 1 ? -1 : 1, sy = o & 2 ? -1 : 1, sz = o & 4 ? -1 : 1;
@@ -193,6 +195,25 @@ int anchors_cut_short() {
   return 0;
 }
 
+// What registration needed for itself is given back where it is large.
+int scratch_given_back() {
+  zef_ctx *ctx = nullptr;
+  CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+  size_t largest = 0;
+  for (int m : {4, 60, 120, 8}) {
+    CHECK(add(ctx, m, octahedron(1.f, m)) == ZEF_OK, "surface: %s", zef_last_error(ctx));
+    const CompGrid &g = ctx->grids.back();
+    largest = std::max(largest, (size_t)g.n[0] * g.n[1] * g.n[2] * 24);
+    const size_t held = ctx->gr_cap[0] + ctx->gr_cap[1];
+    CHECK(held <= (size_t)32 << 20, "%zu bytes of scratch held after a surface of %d triangles", held, 8 * m * m);
+    for (int k = 0; k < 2; ++k)
+      CHECK((ctx->gr_buf[k] != nullptr) == (ctx->gr_cap[k] > 0), "buffer %d and its size differ", k);
+  }
+  CHECK(largest > (size_t)32 << 20, "no surface needed more than is kept");
+  zef_destroy(ctx);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -202,6 +223,7 @@ int main(int argc, char **argv) {
   else if (name == "status_once") status_once();
   else if (name == "no_tets") no_tets();
   else if (name == "anchors_cut_short") anchors_cut_short();
+  else if (name == "scratch_given_back") scratch_given_back();
   else return 2;
   return g_bad ? 1 : 0;
 }

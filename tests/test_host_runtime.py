@@ -48,3 +48,7 @@ def test_host_meshes_without_tets_keep_their_nodes(driver):
 
 def test_anchors_cut_short_make_no_grid(driver):
     _run(driver, "anchors_cut_short")
+
+
+def test_large_construction_scratch_is_given_back(driver):
+    _run(driver, "scratch_given_back")
