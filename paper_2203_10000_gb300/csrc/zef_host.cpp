@@ -520,8 +520,8 @@ zef_status zef_compartment_priority(zef_ctx *ctx, const int32_t *ids, int32_t n)
   std::sort(sb.begin(), sb.end());
   if (sa != sb || std::adjacent_find(sa.begin(), sa.end()) != sa.end())
     return fail(ctx, ZEF_ERR_INVALID_ARG, "priority is not a permutation of the registered ids");
+  if (a != ctx->priority) ctx->rows_dirty = true;
   ctx->priority = a;
-  ctx->dirty = true;
   DeviceGuard g(ctx->device);
   return ensure_uploaded(ctx);
 }
@@ -1041,15 +1041,11 @@ UnionBox surface_box(const CompHost &first, int n) {
   return ub;
 }
 
-zef_status ensure_uploaded(zef_ctx *ctx) {
-  if (ctx->device == ZEF_HOST_ONLY) return ZEF_OK;
-  if (!ctx->dirty) return ZEF_OK;
+// The surfaces themselves (entries, triangles, cap trees, hull bounds).  The
+// copies go to the context's stream: one on the legacy stream may still be on
+// its way when it returns, and a non-blocking stream's kernels do not wait.
+static zef_status upload_surfaces(zef_ctx *ctx) {
   const int C = (int)ctx->comps.size();
-  if (C == 0) return ZEF_OK;
-  // Labelings still running read what is overwritten here, and the copies below
-  // go to the context's stream: one on the legacy stream may still be on its
-  // way when it returns, and a non-blocking stream's kernels do not wait for it.
-  CK(cudaStreamSynchronize(ctx->stream), "wait before the upload");
   int64_t ne = (int64_t)ctx->h_entries.size();
   int64_t ntv = (int64_t)ctx->h_tris.size();
   if (ctx->d_entries_cap < ne) {
@@ -1128,6 +1124,38 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
   // range (a point outside it is outside every compartment's box)
   const UnionBox ub = surface_box(ctx->comps[0], C);
   ctx->ubox = ub;
+  // hull bounds in scaled coordinates: h s (exact power-of-two scaling) plus a
+  // margin that covers the float evaluation of d . p for |p| <= 1000 (scaled
+  // units; every surface lies within 64), rounded up to float
+  std::vector<float> dop((size_t)C * kDop);
+  for (int i = 0; i < C; ++i)
+    for (int k = 0; k < kDop; ++k) {
+      const double thr = ctx->comps[i].dop[k] * s + 6.4e-4;
+      float f = (float)thr;
+      if ((double)f < thr) f = std::nextafter(f, std::numeric_limits<float>::infinity());
+      dop[(size_t)i * kDop + k] = f;
+    }
+  CK(cudaMemcpyAsync(ctx->d_dop, dop.data(), dop.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream), "upload dop");
+  CK(cudaMemcpyAsync(ctx->d_entries, es.data(), ne * sizeof(Entry), cudaMemcpyHostToDevice, ctx->stream), "upload entries");
+  CK(cudaMemcpyAsync(ctx->d_tris, ts.data(), ntv * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream), "upload tris");
+  CK(cudaStreamSynchronize(ctx->stream), "upload");  // the copies' host arrays end with this call
+  return ZEF_OK;
+}
+
+// What is not on the device yet: after a registration everything, after a new
+// priority order the compartments' records.
+zef_status ensure_uploaded(zef_ctx *ctx) {
+  if (ctx->device == ZEF_HOST_ONLY) return ZEF_OK;
+  if (!ctx->dirty && !ctx->rows_dirty) return ZEF_OK;
+  const int C = (int)ctx->comps.size();
+  if (C == 0) return ZEF_OK;
+  // labelings still running read what is overwritten here
+  CK(cudaStreamSynchronize(ctx->stream), "wait before the upload");
+  if (ctx->dirty) {
+    const zef_status st = upload_surfaces(ctx);
+    if (st) return st;
+  }
+  const float s = ctx->scale;
   std::vector<DevComp> dc(C);
   std::vector<int32_t> rows(C), lpt(C);
   for (int i = 0; i < C; ++i) {
@@ -1151,28 +1179,14 @@ zef_status ensure_uploaded(zef_ctx *ctx) {
       if (ctx->priority[r] == h.id) d.row = r;
     rows[d.row] = h.id;
   }
-  // hull bounds in scaled coordinates: h s (exact power-of-two scaling) plus a
-  // margin that covers the float evaluation of d . p for |p| <= 1000 (scaled
-  // units; every surface lies within 64), rounded up to float
-  std::vector<float> dop((size_t)C * kDop);
-  for (int i = 0; i < C; ++i)
-    for (int k = 0; k < kDop; ++k) {
-      const double thr = ctx->comps[i].dop[k] * s + 6.4e-4;
-      float f = (float)thr;
-      if ((double)f < thr) f = std::nextafter(f, std::numeric_limits<float>::infinity());
-      dop[(size_t)i * kDop + k] = f;
-    }
   std::iota(lpt.begin(), lpt.end(), 0);
   std::stable_sort(lpt.begin(), lpt.end(),
                    [&](int a, int b) { return ctx->comps[a].nt > ctx->comps[b].nt; });
-  CK(cudaMemcpyAsync(ctx->d_dop, dop.data(), dop.size() * sizeof(float), cudaMemcpyHostToDevice, ctx->stream), "upload dop");
-  CK(cudaMemcpyAsync(ctx->d_entries, es.data(), ne * sizeof(Entry), cudaMemcpyHostToDevice, ctx->stream), "upload entries");
-  CK(cudaMemcpyAsync(ctx->d_tris, ts.data(), ntv * sizeof(float4), cudaMemcpyHostToDevice, ctx->stream), "upload tris");
   CK(cudaMemcpyAsync(ctx->d_comps, dc.data(), C * sizeof(DevComp), cudaMemcpyHostToDevice, ctx->stream), "upload comps");
   CK(cudaMemcpyAsync(ctx->d_row_ids, rows.data(), C * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream), "upload rows");
   CK(cudaMemcpyAsync(ctx->d_lpt, lpt.data(), C * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream), "upload lpt");
   CK(cudaStreamSynchronize(ctx->stream), "upload");  // the copies' host arrays end with this call
-  ctx->dirty = false;
+  ctx->dirty = ctx->rows_dirty = false;
   ++ctx->gen;
   const zef_status st = grid_update(ctx);
   if (st) ctx->dirty = true;

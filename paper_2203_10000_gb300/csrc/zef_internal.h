@@ -300,7 +300,8 @@ struct zef_ctx {
   std::vector<zef::Entry> h_cseg;     // cap-tree strip segments
   std::vector<int32_t> h_ctidx;       // cap-tree leaves' triangles (compartment-local indices), tree order
 
-  bool dirty = true;
+  bool dirty = true;       // surfaces that are not on the device yet
+  bool rows_dirty = false;  // a priority order that is not
   uint64_t gen = 0;   // upload generation: cached graphs keyed on it see every change of the surfaces
   // power of two applied to every coordinate on the device so that the
   // registered surfaces fit in [-64, 64]^3 (exact; solid angles are scale

@@ -86,7 +86,7 @@ extern "C" zef_status zef_label_points_noalloc(zef_ctx *ctx, const float *pts, i
   ctx->err.clear();
   if (ctx->device == ZEF_HOST_ONLY) return fail(ctx, ZEF_ERR_NOT_READY, "host-only context cannot label");
   if (ctx->comps.empty()) return fail(ctx, ZEF_ERR_NOT_READY, "no compartment registered");
-  if (ctx->dirty) return fail(ctx, ZEF_ERR_NOT_READY, "compartments are not uploaded");
+  if (ctx->dirty || ctx->rows_dirty) return fail(ctx, ZEF_ERR_NOT_READY, "compartments are not uploaded");
   if (n < 0 || n > kMaxPoints)
     return fail(ctx, ZEF_ERR_INVALID_ARG,
                 "zef_label_points_noalloc takes at most ZEF_NOALLOC_MAX_POINTS (65536) points");

@@ -214,6 +214,31 @@ int scratch_given_back() {
   return 0;
 }
 
+// A new priority order uploads the rows, not the surfaces; the same one nothing.
+int priority_uploads() {
+  zef_ctx *ctx = nullptr;
+  CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+  CHECK(add(ctx, 1, octahedron(1.f, 20)) == ZEF_OK && add(ctx, 2, octahedron(2.f, 20)) == ZEF_OK, "surfaces: %s",
+        zef_last_error(ctx));
+  const int32_t same[2] = {1, 2}, other[2] = {2, 1};
+  size_t before = fake_uploaded();
+  const uint64_t gen = ctx->gen;
+  CHECK(zef_compartment_priority(ctx, same, 2) == ZEF_OK, "priority: %s", zef_last_error(ctx));
+  CHECK(fake_uploaded() == before && ctx->gen == gen, "the same order uploaded %zu bytes", fake_uploaded() - before);
+  CHECK(zef_compartment_priority(ctx, other, 2) == ZEF_OK, "priority: %s", zef_last_error(ctx));
+  CHECK(fake_uploaded() > before && fake_uploaded() - before <= 4096, "another order uploaded %zu bytes",
+        fake_uploaded() - before);
+  CHECK(ctx->gen != gen && ctx->h_grid[0].comp == 1 && ctx->h_grid[1].comp == 0, "the rows are the old order's");
+  fake_settle();
+  const int32_t *ids = ctx->d_row_ids;
+  CHECK(ids[0] == 2 && ids[1] == 1 && ctx->d_comps[0].row == 1 && ctx->d_comps[1].row == 0, "the old order's records");
+  before = fake_uploaded();
+  CHECK(add(ctx, 3, octahedron(3.f, 20)) == ZEF_OK, "surface: %s", zef_last_error(ctx));
+  CHECK(fake_uploaded() - before > 100000, "a surface uploaded %zu bytes", fake_uploaded() - before);
+  zef_destroy(ctx);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -224,6 +249,7 @@ int main(int argc, char **argv) {
   else if (name == "no_tets") no_tets();
   else if (name == "anchors_cut_short") anchors_cut_short();
   else if (name == "scratch_given_back") scratch_given_back();
+  else if (name == "priority_uploads") priority_uploads();
   else return 2;
   return g_bad ? 1 : 0;
 }

@@ -35,6 +35,7 @@ std::map<const void *, std::string> g_names;
 std::map<const void *, std::vector<unsigned char>> g_vars;
 cudaError_t g_last = cudaSuccess;
 long g_allocs = 0, g_fail_at = -1, g_unordered = 0;
+size_t g_uploaded = 0;
 std::string g_first_unordered, g_hook_name;
 std::function<void()> g_hook;
 struct Config {
@@ -71,6 +72,7 @@ cudaError_t enqueue_copy(Stream *s, void *dst, const void *src, size_t n, cudaMe
     return done(cudaErrorInvalidValue);
   if ((kind == cudaMemcpyDeviceToHost || kind == cudaMemcpyDeviceToDevice) && !inside(g_device, src, n))
     return done(cudaErrorInvalidValue);
+  if (kind == cudaMemcpyHostToDevice) g_uploaded += n;
   if (kind == cudaMemcpyHostToDevice && !inside(g_pinned, src)) {
     std::vector<unsigned char> stage((const unsigned char *)src, (const unsigned char *)src + n);
     s->queue.push_back([dst, stage] { std::memcpy(dst, stage.data(), stage.size()); });
@@ -101,6 +103,7 @@ size_t fake_device_bytes() {
   for (auto &p : g_device) n += p.second;
   return n;
 }
+size_t fake_uploaded() { return g_uploaded; }
 void fake_settle() { drain_all(); }
 
 // ---- the runtime

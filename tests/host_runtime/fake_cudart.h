@@ -12,4 +12,5 @@ long fake_allocs();            // device allocations since fake_fail_alloc
 long fake_unordered(std::string *first);
 void fake_on_launch(const char *name, std::function<void()> f);  // when such a kernel's turn comes
 size_t fake_device_bytes();
+size_t fake_uploaded();        // bytes copied from the host so far
 void fake_settle();            // every queue runs

@@ -52,3 +52,7 @@ def test_anchors_cut_short_make_no_grid(driver):
 
 def test_large_construction_scratch_is_given_back(driver):
     _run(driver, "scratch_given_back")
+
+
+def test_a_priority_order_uploads_its_rows(driver):
+    _run(driver, "priority_uploads")
