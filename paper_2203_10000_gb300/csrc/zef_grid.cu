@@ -184,18 +184,32 @@ __global__ void __launch_bounds__(256) k_gr_refs(const float4 *tris, float to_ra
   }
 }
 
-// words of every cell's block (to be scanned into offsets) and the longest list
+// Words of every cell's block (to be scanned into offsets); the longest list,
+// and the sums of the lists and of the blocks in 64 bits: the scans wrap where
+// these do not fit 32, and such a grid must not be filled.
 __global__ void __launch_bounds__(256) k_gr_sizes(const uint32_t *cnt, int64_t cells, uint32_t *size,
                                                   unsigned long long *longest) {
   uint32_t mx = 0;
+  unsigned long long refs = 0, words = 0;
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < cells; c += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t v = cnt[c];
-    size[c] = v ? 1u + kChunkWords * ((v + kSub - 1) / kSub) : 0u;
+    const uint32_t w = v ? 1u + kChunkWords * ((v + kSub - 1) / kSub) : 0u;
+    size[c] = w;
     mx = max(mx, v);
+    refs += v;
+    words += w;
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0 && mx) atomicMax(longest, (unsigned long long)mx);
+  for (int o = 16; o > 0; o >>= 1) {
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    refs += __shfl_xor_sync(0xffffffffu, refs, o);
+    words += __shfl_xor_sync(0xffffffffu, words, o);
+  }
+  if ((threadIdx.x & 31) == 0 && mx) {
+    atomicMax(longest, (unsigned long long)mx);
+    atomicAdd(longest + 1, refs);
+    atomicAdd(longest + 2, words);
+  }
 }
 
 __device__ __forceinline__ uint32_t hash32(uint32_t x) {
@@ -1519,7 +1533,8 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   const int nt = (int)h.nt;
   cudaStream_t st = ctx->stream;
 
-  // scratch: counts / list ends, block sizes / offsets, scan sums, totals, anchors, their Omega
+  // scratch: counts / list ends, block sizes / offsets, scan sums, totals
+  // (longest list, triangles of all lists, words of all blocks), anchors, their Omega
   const int64_t bs = cells / 2048 + 2;
   const size_t o_flag = (size_t)cells * 4, o_sum = o_flag + (size_t)cells * 4, o_tot = (o_sum + (size_t)bs * 4 + 15) & ~(size_t)15,
                o_anch = o_tot + 32, o_om = o_anch + (size_t)cells * 12, bytes = o_om + (size_t)cells * 4;
@@ -1547,9 +1562,9 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
   const int g_t = grid_blocks(ctx, (int64_t)nt * 32, 256), g_c = grid_blocks(ctx, cells, 256),
             g_w = grid_blocks(ctx, cells * 32, 256);
   k_gr_refs<<<g_t, 256, 0, st>>>(tris, to_raw, nt, g, cnt, nullptr);
-  k_gr_sizes<<<g_c, 256, 0, st>>>(cnt, cells, flag, (unsigned long long *)(tot + 2));
-  zef_status zs = scan_exclusive(ctx, cnt, nullptr, 1, cells, tot, bsum);
-  if (!zs) zs = scan_exclusive(ctx, flag, nullptr, 1, cells, tot + 1, bsum);
+  k_gr_sizes<<<g_c, 256, 0, st>>>(cnt, cells, flag, (unsigned long long *)tot);
+  zef_status zs = scan_exclusive(ctx, cnt, nullptr, 1, cells, nullptr, bsum);
+  if (!zs) zs = scan_exclusive(ctx, flag, nullptr, 1, cells, nullptr, bsum);
   int64_t totals[3] = {0, 0, 0};
   if (!zs) {
     e = cudaMemcpyAsync(totals, tot, sizeof(totals), cudaMemcpyDeviceToHost, st);
@@ -1557,8 +1572,8 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
     if (e != cudaSuccess) zs = cuda_fail(ctx, e, "cell grid");
   }
   if (zs) return zs;
-  const int64_t refs = totals[0], words16 = totals[1];
-  if (totals[2] > kMaxList || refs > 64 * (int64_t)nt + 65536 || words16 > (int64_t)kOffsetMask)
+  const int64_t refs = totals[1], words16 = totals[2];
+  if (totals[0] > kMaxList || refs > (int64_t)UINT32_MAX || refs > 64 * (int64_t)nt + 65536 || words16 > (int64_t)kOffsetMask)
     return ZEF_OK;
   // blocks and words; the triangle lists are scratch
   const size_t p_word = (size_t)words16 * 16, p_end = p_word + (size_t)cells * 4;

@@ -239,6 +239,29 @@ int priority_uploads() {
   return 0;
 }
 
+// Cells that list more triangles than 32 bits count (the scans' totals wrap to
+// small ones) make no grid.
+int sums_beyond_32_bits() {
+  for (const bool refs : {true, false}) {
+    zef_ctx *ctx = nullptr;
+    CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+    const long before = fake_launches("k_gr_finish");
+    fake_on_launch_args("k_gr_sizes", [refs](void **args) {
+      int64_t *sums = *reinterpret_cast<int64_t **>(args[3]) + 1;  // triangles of all lists, words of all blocks
+      return [=] {
+        sums[0] = refs ? ((int64_t)1 << 32) + 100 : 100;
+        sums[1] = refs ? 25 : ((int64_t)1 << 32) + 25;
+      };
+    });
+    CHECK(add(ctx, 1, octahedron(1.f, 8)) == ZEF_OK, "surface: %s", zef_last_error(ctx));
+    fake_on_launch("", [] {});
+    CHECK(ctx->grids.size() == 1 && !ctx->grids[0].usable, "a grid with %s beyond 32 bits", refs ? "lists" : "blocks");
+    CHECK(fake_launches("k_gr_finish") == before, "blocks were written");
+    zef_destroy(ctx);
+  }
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -250,6 +273,7 @@ int main(int argc, char **argv) {
   else if (name == "anchors_cut_short") anchors_cut_short();
   else if (name == "scratch_given_back") scratch_given_back();
   else if (name == "priority_uploads") priority_uploads();
+  else if (name == "sums_beyond_32_bits") sums_beyond_32_bits();
   else return 2;
   return g_bad ? 1 : 0;
 }

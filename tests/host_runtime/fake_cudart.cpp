@@ -37,7 +37,8 @@ cudaError_t g_last = cudaSuccess;
 long g_allocs = 0, g_fail_at = -1, g_unordered = 0;
 size_t g_uploaded = 0;
 std::string g_first_unordered, g_hook_name;
-std::function<void()> g_hook;
+std::function<std::function<void()>(void **)> g_hook;
+std::map<std::string, long> g_launches;
 struct Config {
   dim3 grid, block;
   size_t smem;
@@ -95,8 +96,17 @@ long fake_unordered(std::string *first) {
   return g_unordered;
 }
 void fake_on_launch(const char *name, std::function<void()> f) {
+  fake_on_launch_args(name, [f](void **) { return f; });
+}
+void fake_on_launch_args(const char *name, std::function<std::function<void()>(void **)> f) {
   g_hook_name = name;
   g_hook = std::move(f);
+}
+long fake_launches(const char *name) {
+  long n = 0;
+  for (auto &l : g_launches)
+    if (l.first.find(name) != std::string::npos) n += l.second;
+  return n;
 }
 size_t fake_device_bytes() {
   size_t n = 0;
@@ -248,10 +258,11 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) {
   *k = reinterpret_cast<cudaKernel_t>(const_cast<void *>(f));
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **, size_t, cudaStream_t s) {
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **args, size_t, cudaStream_t s) {
   const std::string &name = g_names[reinterpret_cast<const void *>(k)];
+  ++g_launches[name];
   if (s && !g_legacy.queue.empty() && !g_unordered++) g_first_unordered = name;
-  if (!g_hook_name.empty() && name.find(g_hook_name) != std::string::npos) of(s)->queue.push_back(g_hook);
+  if (!g_hook_name.empty() && name.find(g_hook_name) != std::string::npos) of(s)->queue.push_back(g_hook(args));
   return cudaSuccess;
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args) {

@@ -56,3 +56,7 @@ def test_large_construction_scratch_is_given_back(driver):
 
 def test_a_priority_order_uploads_its_rows(driver):
     _run(driver, "priority_uploads")
+
+
+def test_cell_lists_beyond_32_bits_make_no_grid(driver):
+    _run(driver, "sums_beyond_32_bits")
