@@ -1402,7 +1402,8 @@ zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
   a.pending = ctx->lb.pending;
   a.open = ctx->lb.open;
   if (plan.timed) cudaEventRecord(ctx->ev[0], s);
-  if (a.stats || (listed && ctx->lb.lists_dirty)) {
+  const bool dirty = ctx->lb.lists_dirty;
+  if (a.stats || (listed && dirty)) {
     k_grid_reset<<<1, 32, 0, s>>>(ctx->lb.counters);
     ++ctx->launches;
   }
@@ -1465,7 +1466,8 @@ zef_status grid_enqueue(zef_ctx *ctx, const LabelPlan &plan) {
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "k_grid_label launch");
-  ctx->lb.lists_dirty = false;
+  // enqueued into one of the library's graphs (n_host < 0) nothing has run yet
+  if (listed) ctx->lb.lists_dirty = plan.n_host < 0 && dirty;
   return ZEF_OK;
 }
 

@@ -262,6 +262,43 @@ int sums_beyond_32_bits() {
   return 0;
 }
 
+// A call whose launches failed half-way leaves counts in the lists: the next
+// call clears them first, and enqueueing into a graph (which may never run)
+// does not count as having done so.
+int lists_cleared_after_a_failure() {
+  zef_ctx *ctx = nullptr;
+  CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+  CHECK(add(ctx, 1, octahedron(1.f, 4)) == ZEF_OK, "surface: %s", zef_last_error(ctx));
+  const int64_t n = 1 << 18;
+  const std::vector<float> pts(3 * n, 0.25f);
+  std::vector<int32_t> lab(n);
+  auto call = [&] { return zef_label_points(ctx, pts.data(), n, lab.data(), nullptr, nullptr, nullptr); };
+  CHECK(call() == ZEF_OK, "call: %s", zef_last_error(ctx));
+  const long resets = fake_launches("k_grid_reset");
+  CHECK(call() == ZEF_OK && fake_launches("k_grid_reset") == resets, "a plain call clears lists that are empty");
+  fake_fail_launch("k_grid_pending");
+  CHECK(call() == ZEF_ERR_CUDA, "the failed launch was not reported");
+  fake_fail_launch("");
+  CHECK(zef_label_points(ctx, pts.data(), 100, lab.data(), nullptr, nullptr, nullptr) == ZEF_OK, "a call without lists: %s",
+        zef_last_error(ctx));
+  LabelPlan p;
+  std::memset(&p.opts, 0, sizeof(p.opts));
+  fill_default_opts(&p.opts);
+  p.pts = ctx->lb.pts_tmp;
+  p.labels = ctx->lb.labels_tmp;
+  p.omega = nullptr;
+  p.omega_ld = p.n_cap = n;
+  p.d_n = p.d_off = ctx->lb.counters;
+  p.timed = false;
+  p.counted = false;
+  CHECK(grid_enqueue(ctx, p) == ZEF_OK, "enqueue: %s", zef_last_error(ctx));
+  CHECK(fake_launches("k_grid_reset") == resets + 1, "enqueueing did not clear the lists");
+  CHECK(call() == ZEF_OK && fake_launches("k_grid_reset") == resets + 2, "the call behind a failure did not clear the lists");
+  CHECK(call() == ZEF_OK && fake_launches("k_grid_reset") == resets + 2, "the lists are cleared for good");
+  zef_destroy(ctx);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -274,6 +311,7 @@ int main(int argc, char **argv) {
   else if (name == "scratch_given_back") scratch_given_back();
   else if (name == "priority_uploads") priority_uploads();
   else if (name == "sums_beyond_32_bits") sums_beyond_32_bits();
+  else if (name == "lists_cleared_after_a_failure") lists_cleared_after_a_failure();
   else return 2;
   return g_bad ? 1 : 0;
 }

@@ -36,7 +36,7 @@ std::map<const void *, std::vector<unsigned char>> g_vars;
 cudaError_t g_last = cudaSuccess;
 long g_allocs = 0, g_fail_at = -1, g_unordered = 0;
 size_t g_uploaded = 0;
-std::string g_first_unordered, g_hook_name;
+std::string g_first_unordered, g_hook_name, g_fail_launch;
 std::function<std::function<void()>(void **)> g_hook;
 std::map<std::string, long> g_launches;
 struct Config {
@@ -102,6 +102,7 @@ void fake_on_launch_args(const char *name, std::function<std::function<void()>(v
   g_hook_name = name;
   g_hook = std::move(f);
 }
+void fake_fail_launch(const char *name) { g_fail_launch = name; }
 long fake_launches(const char *name) {
   long n = 0;
   for (auto &l : g_launches)
@@ -260,6 +261,7 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) {
 }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **args, size_t, cudaStream_t s) {
   const std::string &name = g_names[reinterpret_cast<const void *>(k)];
+  if (!g_fail_launch.empty() && name.find(g_fail_launch) != std::string::npos) return done(cudaErrorLaunchOutOfResources);
   ++g_launches[name];
   if (s && !g_legacy.queue.empty() && !g_unordered++) g_first_unordered = name;
   if (!g_hook_name.empty() && name.find(g_hook_name) != std::string::npos) of(s)->queue.push_back(g_hook(args));

@@ -60,3 +60,7 @@ def test_a_priority_order_uploads_its_rows(driver):
 
 def test_cell_lists_beyond_32_bits_make_no_grid(driver):
     _run(driver, "sums_beyond_32_bits")
+
+
+def test_lists_are_cleared_after_a_failed_call(driver):
+    _run(driver, "lists_cleared_after_a_failure")
