@@ -929,6 +929,9 @@ __device__ __forceinline__ void decide(const GridArgs &a, const GridComp *s_g, c
         OpenPoint p;
         p.ins = mask;
         p.open = left;
+        p.x = x;
+        p.y = y;
+        p.z = z;
         p.i = i;
         a.open[at] = p;
       }
@@ -1254,6 +1257,7 @@ __global__ void __launch_bounds__(kOpenThreads) k_grid_open(GridArgs a) {
   static_assert(kOpenThreads == kGlThreads, "the second part's batches");
   asm volatile("griddepcontrol.wait;" ::: "memory");  // for k_grid_pending, where launched beside it
   const int64_t listed = a.counters[CNT_OPEN];
+  OpenPoint p = a.open[min((int)blockIdx.x, kOpenCap - 1)];  // the block's first, if it has one (with the count, not behind it)
   if (listed == 0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) a.counters[CNT_PEND] = 0;
     return;
@@ -1270,10 +1274,9 @@ __global__ void __launch_bounds__(kOpenThreads) k_grid_open(GridArgs a) {
       pending_batch<WIDE, false>(a, sh.again.g, sh.again.id, sh.again.batch, wid, lane, off, run_point(t, tiles, lane), m, st);
   } else {
     for (int64_t e = blockIdx.x; e < listed; e += gridDim.x) {
-      const OpenPoint p = a.open[e];
+      if (e != blockIdx.x) p = a.open[e];
       if (!ZEF_BOUNDS_OK(p.i >= 0 && p.i < n, a.status, 31)) continue;
-      const float *q = a.pts + 3 * (off + p.i);
-      const float x = q[0], y = q[1], z = q[2];
+      const float x = p.x, y = p.y, z = p.z;
       M mask = (M)p.ins, left = (M)p.open;
       while (left) {
         const int r = first_row(left);

@@ -191,8 +191,9 @@ struct CompHost {
 };
 
 // A point that the cell grid leaves to the FP64 solid angles (zef_grid.cu).
-struct OpenPoint {
+struct __align__(16) OpenPoint {
   unsigned long long ins, open;  // rows it is inside of, rows to be decided
+  float x, y, z;
   int32_t i;
 };
 constexpr int kOpenCap = 1 << 15;

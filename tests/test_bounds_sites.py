@@ -21,7 +21,7 @@ GRID = {
     "queue of the streaming kernel": (r"at < kGsQueue, a\.status", r"s_q\[wid\]\[at\] = \(int32_t\)"),
     "list of open points": (r"at \+ j < \(unsigned long long\)a\.pend_cap, a\.status", r"a\.pending\[at \+ j\] ="),
     "listed point": (r"i >= 0 && i < \(a\.n_host >= 0 \? a\.n_host : a\.counters\[CNT_N\]\), a\.status", r"a\.pts \+ 3 \* \(off \+ i\)"),
-    "point on a surface": (r"p\.i < n, a\.status", r"a\.pts \+ 3 \* \(off \+ p\.i\)"),
+    "point on a surface": (r"p\.i < n, a\.status", r"M mask = \(M\)p\.ins"),
 }
 
 
