@@ -151,8 +151,10 @@ typedef struct zef_label_stats {
                                   grid */
     int64_t pairs_rescued;     /* point x triangle pairs re-evaluated in FP64 */
     int64_t uncertain_pairs;   /* (point, compartment) pairs sent to FP64 */
-    int64_t work_items;        /* (compartment, point tile) items after culling */
-    int64_t tiles;             /* point tiles */
+    int64_t work_items;        /* (compartment, point tile) items after culling
+                                  (cell grids: as tiles) */
+    int64_t tiles;             /* point tiles (cell grids: of 64, as many as the
+                                  points in the surfaces' box would fill) */
     int32_t block_threads;     /* launch shape used */
     int32_t points_per_thread;
     float ms_total;            /* device time of the call (CUDA events) */

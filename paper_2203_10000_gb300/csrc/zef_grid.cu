@@ -371,7 +371,7 @@ __device__ __forceinline__ void count_add(const GridArgs &a, int c, unsigned lon
 
 // statistics of the labeling kernel, summed per warp and block before they
 // reach the counters (thousands of warps adding to one word would queue)
-enum GridStat { GS_EVAL = 0, GS_COHERENT, GS_OWN, GS_ITEMS, GS_NONFINITE, GS_NIN, GS_COUNT };
+enum GridStat { GS_EVAL = 0, GS_COHERENT, GS_OWN, GS_NONFINITE, GS_NIN, GS_COUNT };
 
 // FP64 re-evaluation of one (point, compartment) pair by the whole warp: the
 // crossings from the vertices in FP64, each sign taken only beyond its
@@ -991,12 +991,10 @@ __device__ void flush_stats(const GridArgs &a, const LaneStats &st, unsigned lon
   v[GS_EVAL] = st.eval;
   v[GS_COHERENT] = st.coh;
   v[GS_OWN] = lane == 0 ? st.own : 0u;  // counted by the whole warp
-  v[GS_ITEMS] = 0u;
   v[GS_NONFINITE] = st.nonfin;
   v[GS_NIN] = st.nin;
 #pragma unroll
   for (int q = 0; q < GS_COUNT; ++q) v[q] = __reduce_add_sync(0xffffffffu, v[q]);
-  v[GS_ITEMS] = (v[GS_NIN] + 63) / 64;
   if (lane == 0)
 #pragma unroll
     for (int q = 0; q < GS_COUNT; ++q) s_stat[wid][q] = v[q];
@@ -1004,7 +1002,7 @@ __device__ void flush_stats(const GridArgs &a, const LaneStats &st, unsigned lon
   if (threadIdx.x < GS_COUNT) {
     unsigned long long t = 0ull;
     for (int w = 0; w < kGlWarps; ++w) t += s_stat[w][threadIdx.x];
-    constexpr int kCnt[GS_COUNT] = {CNT_PAIRS_EVAL, CNT_COHERENT, CNT_LANE_TILES, CNT_ITEMS, CNT_NONFINITE, CNT_NIN};
+    constexpr int kCnt[GS_COUNT] = {CNT_PAIRS_EVAL, CNT_COHERENT, CNT_LANE_TILES, CNT_NONFINITE, CNT_NIN};
     if (t) count_add(a, kCnt[threadIdx.x], t);
   }
 }

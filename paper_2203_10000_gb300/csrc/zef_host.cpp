@@ -859,11 +859,11 @@ static zef_status read_stats(zef_ctx *ctx, int64_t n, const zef_label_opts &o, c
   stats->pairs_rescued = h[CNT_PAIRS_RESCUE];
   stats->pairs_evaluated = h[CNT_PAIRS_EVAL] + h[CNT_PAIRS_RESCUE];
   stats->uncertain_pairs = h[CNT_UNC];
-  stats->work_items = h[CNT_ITEMS];
-  // the cell grid's tiles: 64 consecutive points each, as many as the
-  // points inside the union box would fill
+  // the cell grid's tiles, and items: of 64 points each, as many as the points
+  // inside the union box would fill
   stats->cell_grids = grid_serves(ctx, o);
   stats->tiles = stats->cell_grids ? (h[CNT_NIN] + 63) / 64 : h[CNT_TILES];
+  stats->work_items = stats->cell_grids ? stats->tiles : h[CNT_ITEMS];
   stats->coherent_pairs = h[CNT_COHERENT];
   stats->representative_pairs = h[CNT_REP_PAIRS];
   stats->lane_walk_items = h[CNT_LANE_TILES];

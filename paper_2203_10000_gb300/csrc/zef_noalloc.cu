@@ -181,9 +181,9 @@ extern "C" zef_status zef_label_points_noalloc(zef_ctx *ctx, const float *pts, i
     stats->pairs_rescued = h[CNT_PAIRS_RESCUE];
     stats->pairs_evaluated = h[CNT_PAIRS_EVAL] + h[CNT_PAIRS_RESCUE];
     stats->uncertain_pairs = h[CNT_UNC];
-    stats->work_items = h[CNT_ITEMS];
     stats->cell_grids = grid;
     stats->tiles = grid ? (h[CNT_NIN] + 63) / 64 : h[CNT_TILES];
+    stats->work_items = grid ? stats->tiles : h[CNT_ITEMS];
     stats->coherent_pairs = h[CNT_COHERENT];
     stats->representative_pairs = h[CNT_REP_PAIRS];
     stats->lane_walk_items = h[CNT_LANE_TILES];

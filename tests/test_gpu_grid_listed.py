@@ -120,3 +120,16 @@ def test_statistics_say_which_path_served_the_call(zef, n):
     assert ctx.label_points(pts)[2]["cell_grids"] == 1
     assert ctx.label_points(pts, opts=zef.make_opts(block_threads=256, points_per_thread=2))[2]["cell_grids"] == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [100, 5000, 100_000, LISTED])
+def test_work_items_do_not_depend_on_the_split(zef, n):
+    """Of 64 points of the surfaces' box each, however few a warp was given."""
+    w = zs.config0()
+    ctx = _context(zef, w.surfaces)
+    v = w.surfaces[0].verts
+    pts = np.random.default_rng(n).uniform(v.min(0) * 1.2, v.max(0) * 1.2, (n, 3)).astype(np.float32)
+    inside = int(((pts >= v.min(0)) & (pts <= v.max(0))).all(1).sum())
+    st = ctx.label_points(torch.from_numpy(pts).cuda())[2]
+    ctx.close()
+    assert st["work_items"] == st["tiles"] == (inside + 63) // 64
