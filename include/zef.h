@@ -83,7 +83,13 @@ typedef enum zef_precision {
 } zef_precision;
 
 typedef struct zef_label_opts {
-    /* |Omega32 - 2 pi| < margin marks a (point, compartment) pair uncertain.
+    /* margin and winding_tol say which FP32 sums the general kernels send to
+       FP64.  The cell grids, which serve a call whose options are at their
+       defaults but for these two (margin below 6), sum no solid angle per
+       point: a pair is uncertain there, and goes to FP64, where a crossing
+       test is not beyond its own error bound, whatever the two values, and
+       every value they report is 4 pi k exactly or an FP64 sum.
+       |Omega32 - 2 pi| < margin marks a (point, compartment) pair uncertain.
        Default 1e-3 (<= 0 selects the default). */
     float margin;
     /* A pair is also uncertain when Omega32 is farther than winding_tol from
@@ -159,7 +165,10 @@ typedef struct zef_label_stats {
     int32_t points_per_thread;
     float ms_total;            /* device time of the call (CUDA events) */
     float ms_label;            /* device time of the main labeling kernel */
-    float ms_rescue;           /* device time of the FP64 re-evaluation */
+    float ms_rescue;           /* device time of the FP64 re-evaluation (cell
+                                  grids: of the pairs that a call of 2^18 points
+                                  or more lists; below that it is part of
+                                  ms_label) */
     int32_t cell_grids;        /* 1: the cell grids served the call, 0: the general
                                   kernels did */
     int64_t coherent_pairs;    /* (point, compartment) pairs decided by the

@@ -6,7 +6,7 @@
 // count of crossings along a segment that does: k(p) = k(q) + (inward -
 // outward crossings of the segment q -> p).  So the solid angle needs to be
 // summed at a few fixed points only.  At registration every compartment's box
-// is cut into cells about two triangle edges wide; each cell lists the
+// is cut into cells one mean triangle edge wide; each cell lists the
 // triangles that meet it, and one anchor point per cell gets its winding
 // number from the solid-angle pipeline (FP32 certified, FP64 where it is not:
 // zef_label.cu).  A point then takes
@@ -28,20 +28,22 @@
 // else -- a point within about 1e-5 cell widths of a triangle's plane inside
 // the triangle, a segment that close to an edge -- is re-evaluated in FP64
 // from the vertices (again with a bound), and what FP64 cannot decide either
-// (a point on the surface) by the FP64 solid angle over the cap tree, as the
-// re-evaluation of zef_label.cu does.
+// (a point on the surface) by the FP64 solid angle over the cap tree, in the
+// order of additions of zef_label.cu's re-evaluation of whole pairs.
 //
 // Why: the general kernels sum about 1,000 strip entries of a tile's walk for
 // every point near a surface (FP32 ALUs, 54 of the 58 ms of 56.2 M points in
-// 24 compartments); here such a point costs about a dozen crossing tests held
-// by the lanes of one warp, and every other point one word per compartment.
-// No sort of the points and no work list: one launch, two for large calls.
-// 56.2 M points in 24 compartments take 0.57 ms (58 ms with the tile kernels,
+// 24 compartments); here such a point costs about a dozen crossing tests by
+// four lanes, and every other point one cell of the label field (below).  No
+// sort of the points: one launch, three for large calls, which list the points
+// that the field leaves open and, of these, those on a surface.
+// 56.2 M points in 24 compartments take 0.51 ms (58 ms with the tile kernels,
 // 2.4 ms when every compartment met by a warp was looked up and its cells
 // taken one after the other), 20.5 M in 20 small structures 0.10 ms (2.8),
-// 36,864 with solid angles 8.3 us (258).  What bounds them now: the streaming
-// kernel is near half the copy bandwidth (12 + 4 bytes a point), the open
-// points' kernel waits on its two dependent L2 reads per point.
+// 36,864 with solid angles 8.2 us (258), 4,096 vertices of a surface 1.06 ms
+// (2.9).  What bounds them now: the streaming kernel is near half the copy
+// bandwidth (12 + 4 bytes a point), the open points' kernel waits on its two
+// dependent L2 reads per point, points on a surface on the FP64 pipe.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -212,6 +214,7 @@ __global__ void __launch_bounds__(256) k_gr_sizes(const uint32_t *cnt, int64_t c
   }
 }
 
+// Scatters the anchors: lowbias32 of C. Wellons' Hash Prospector.
 __device__ __forceinline__ uint32_t hash32(uint32_t x) {
   x ^= x >> 16;
   x *= 0x7feb352du;
@@ -1103,7 +1106,7 @@ __global__ void __launch_bounds__(kGlThreads, 4) k_grid_label(GridArgs a) {
   if (a.stats) flush_stats(a, st, s_stat, wid, lane);
 }
 
-// Two launches (large calls).  Streaming: labels of the points that the field
+// Three launches (large calls).  Streaming: labels of the points that the field
 // decides (12 bytes in, 4 out per point, the field from L2; few registers, so
 // many loads in flight); the indices of the others are listed, a warp's
 // consecutive points in runs of at least kGsFlush.  PLAIN: labels alone, no
@@ -1345,9 +1348,9 @@ bool grid_serves(const zef_ctx *ctx, const zef_label_opts &o) {
 // Calls of at least kListedMin points list the points that the field leaves
 // open and decide them in a second kernel: the streaming part alone needs 40
 // registers instead of 64 and the lists fill every batch (56.2 M points: 958
-// us in one kernel, 657 in two; 5 M: 151 and 97).  Below that the second
-// launch costs more than it saves (scratch: 4 bytes per point, which the allocation-free entry point,
-// at most 65,536 points, never needs).
+// us in one kernel, 657 in two; 5 M: 151 and 97).  Below that the further
+// launches cost more than they save (scratch: 4 bytes per point, which the
+// allocation-free entry point, at most 65,536 points, never needs).
 constexpr int64_t kListedMin = 1 << 18;
 static_assert(kListedMin > ZEF_NOALLOC_MAX_POINTS, "the allocation-free entry point has no list");
 static bool grid_listed(const zef_ctx *ctx, int64_t n_cap) {

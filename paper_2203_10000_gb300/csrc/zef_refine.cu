@@ -4,13 +4,17 @@
 //   k_rf_flag      tets whose four node labels are not all equal (the tissue
 //                  boundary of the labeled mesh) -> flag
 //   scan           rank of every flagged tet, count F
-//   k_rf_check     capacity checks (tets M + 7F, hash table)
-//   k_rf_insert    the six edges of every flagged tet into an open-addressing
-//                  table keyed by the sorted node pair; atomicMin keeps the
-//                  smallest (rank, local edge) code, i.e. the first appearance
+//   k_rf_check     capacity checks (tets M + 7F), size of the level's edge table
+//   k_rf_clear     that much of the table (conforming: the closure has filled
+//                  all of it)
+//   k_rf_list      the flagged tets by rank
+//   k_rf_insert    the six edges of every flagged tet, one thread each, into an
+//                  open-addressing table keyed by the sorted node pair;
+//                  atomicMin keeps the smallest (rank, local edge) code, i.e.
+//                  the first appearance; every edge keeps its slot
 //   k_rf_owner/scan  new node numbers in order of first appearance, count K
 //   k_rf_nodes     the K edge midpoints, rounded once to float32
-//   label pipeline only the K new nodes are labeled (zef_label.cu)
+//   labeling       only the K new nodes (zef_grid.cu, or zef_label.cu)
 //   k_rf_children  1 -> 8 split: the slot of the flagged tet receives child 0,
 //                  children 1..7 are appended; the octahedron is cut along its
 //                  shortest diagonal (float32 squared lengths, ties to the
