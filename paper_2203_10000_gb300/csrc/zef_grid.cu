@@ -98,6 +98,7 @@ constexpr int kMaxAxis = 512;
 // cells, 630 with 2^22, 607 with 2^23; 20.5 M points in 20 small structures:
 // 108, 109 and 111.
 constexpr int64_t kMaxField = 1 << 22;
+constexpr double kBoxCells = 67108864.0;  // cells of the triangles' boxes that any surface may have (a few ms)
 constexpr size_t kScratchKept = (size_t)32 << 20;  // bytes of construction scratch kept between registrations
 constexpr int kMaxList = 1024;  // longest triangle list of a usable grid
 
@@ -1489,6 +1490,24 @@ void grid_free(zef_ctx *ctx) {
   ctx->field.cells = ctx->field_mem = nullptr;
 }
 
+// Cells of the boxes of all triangles of a surface, n cells a side.
+static double box_cells(const zef_ctx *ctx, const CompHost &h, const int (&n)[3]) {
+  const float4 *v = ctx->h_tris.data() + 3 * h.tri_off;
+  float inv[3];
+  for (int k = 0; k < 3; ++k) inv[k] = h.hi[k] > h.lo[k] ? (float)n[k] / (h.hi[k] - h.lo[k]) : 0.f;
+  double sum = 0.0;
+  for (int64_t t = 0; t < h.nt; ++t, v += 3) {
+    const float lo[3] = {std::min(v[0].x, std::min(v[1].x, v[2].x)), std::min(v[0].y, std::min(v[1].y, v[2].y)),
+                         std::min(v[0].z, std::min(v[1].z, v[2].z))};
+    const float hi[3] = {std::max(v[0].x, std::max(v[1].x, v[2].x)), std::max(v[0].y, std::max(v[1].y, v[2].y)),
+                         std::max(v[0].z, std::max(v[1].z, v[2].z))};
+    double box = 1.0;
+    for (int k = 0; k < 3; ++k) box *= (double)((int)((hi[k] - h.lo[k]) * inv[k]) - (int)((lo[k] - h.lo[k]) * inv[k]) + 1);
+    sum += box;
+  }
+  return sum;
+}
+
 // Cell grid of compartment c (uploaded, with its cap tree).  Cells are one
 // mean triangle edge wide (a cell with triangles then lists about seven of
 // them, one chunk; 56.2 M points in 24 compartments: 650 us at 0.8 edges, 657
@@ -1518,13 +1537,20 @@ static zef_status grid_build(zef_ctx *ctx, size_t c, CompGrid *out) {
     finest[k] = std::max(1.0, std::floor((double)ext[k] * 65536.0 / std::max(std::fabs(h.lo[k]), std::fabs(h.hi[k]))));
   Geom g;
   int64_t cells = 0;
-  for (;; w *= 1.1) {
+  for (double grow = 1.1;; w *= grow) {
     cells = 1;
     for (int k = 0; k < 3; ++k) {
       g.n[k] = (int)std::min<double>(std::min<double>(kMaxAxis, finest[k]), std::max(1.0, std::ceil(ext[k] / w)));
       cells *= g.n[k];
     }
-    if (cells <= kMaxCells) break;
+    if (cells > kMaxCells) continue;
+    // k_gr_refs goes through the cells of every triangle's box, a few of them
+    // for triangles as wide as a cell; for long thin ones across the surface's
+    // box nearly all, so their cells are as wide as kBoxCells allows (2,000
+    // needles: 192 ms to register, 27 now)
+    const double most = kBoxCells + 1024.0 * (double)h.nt, boxes = box_cells(ctx, h, g.n);
+    if (boxes <= most) break;
+    grow = std::max(1.1, std::cbrt(boxes / most));
   }
   for (int k = 0; k < 3; ++k) {
     g.lo[k] = h.lo[k];

@@ -2,6 +2,7 @@
 // per name; prints what is wrong and exits 1, or exits 0.
 #include <algorithm>
 #include <array>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -299,6 +300,47 @@ int lists_cleared_after_a_failure() {
   return 0;
 }
 
+// The cells of all triangles' boxes, which registration goes through, stay in
+// proportion to the triangles also where these are long and thin.
+int needles() {
+  Surface s;
+  const int count = 2000;
+  for (int i = 0; i < count; ++i) {  // tetrahedra from corner to corner, side by side
+    const float x = 0.4f * (float)(i % 50), y = 0.4f * (float)(i / 50);
+    const float v[4][3] = {{x, y, 0.f}, {x + 0.01f, y, 0.f}, {x, y + 0.01f, 0.f}, {x + 100.f, y + 100.f, 100.f}};
+    for (auto &p : v) s.v.insert(s.v.end(), p, p + 3);
+    const int32_t b = 4 * i;
+    s.t.insert(s.t.end(), {b, b + 2, b + 1, b, b + 1, b + 3, b + 1, b + 2, b + 3, b + 2, b, b + 3});
+  }
+  zef_ctx *ctx = nullptr;
+  CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+  for (const Surface &q : {s, octahedron(50.f, 40)}) {
+    CHECK(add(ctx, (int)ctx->comps.size() + 1, q) == ZEF_OK, "surface: %s", zef_last_error(ctx));
+    const CompHost &h = ctx->comps.back();
+    const CompGrid &g = ctx->grids.back();
+    double cells = 0.0;
+    for (size_t t = 0; t < q.t.size(); t += 3) {
+      double box = 1.0;
+      for (int k = 0; k < 3; ++k) {
+        float lo = 1e30f, hi = -1e30f;
+        for (int c = 0; c < 3; ++c) {
+          lo = std::min(lo, q.v[3 * q.t[t + c] + k]);
+          hi = std::max(hi, q.v[3 * q.t[t + c] + k]);
+        }
+        box *= std::floor((hi - h.lo[k]) * g.inv[k]) - std::floor((lo - h.lo[k]) * g.inv[k]) + 1.0;
+      }
+      cells += box;
+    }
+    const double nt = (double)q.t.size() / 3.0;
+    CHECK(cells <= 67108864.0 + 1024.0 * nt, "%.3g cells in the boxes of %.0f triangles (grid of %d x %d x %d)", cells, nt,
+          g.n[0], g.n[1], g.n[2]);
+    CHECK(g.usable && g.n[0] >= 8, "no grid, or one of %d cells a side", g.n[0]);
+  }
+  CHECK(ctx->grids[1].n[0] > 50, "the octahedron's cells grew: %d a side", ctx->grids[1].n[0]);
+  zef_destroy(ctx);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -312,6 +354,7 @@ int main(int argc, char **argv) {
   else if (name == "priority_uploads") priority_uploads();
   else if (name == "sums_beyond_32_bits") sums_beyond_32_bits();
   else if (name == "lists_cleared_after_a_failure") lists_cleared_after_a_failure();
+  else if (name == "needles") needles();
   else return 2;
   return g_bad ? 1 : 0;
 }

@@ -64,3 +64,7 @@ def test_cell_lists_beyond_32_bits_make_no_grid(driver):
 
 def test_lists_are_cleared_after_a_failed_call(driver):
     _run(driver, "lists_cleared_after_a_failure")
+
+
+def test_long_thin_triangles_do_not_fill_the_registration(driver):
+    _run(driver, "needles")
