@@ -729,7 +729,7 @@ struct FieldCell<true> {
 
 // A field cell's cells in one surface's grid that its thread looks at alone.
 // One thread for all of them took 17 ms for a surface of 450,000 triangles in
-// one hundred times as wide (50,000 cells in one of the field's).
+// one fifty times as wide (50,000 cells in one of the field's), now 4.
 constexpr int kFieldAlone = 64;
 
 template <bool WIDE>

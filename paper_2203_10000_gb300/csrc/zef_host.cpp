@@ -789,14 +789,17 @@ zef_status label_points_impl(zef_ctx *ctx, const float *pts, int64_t n, int32_t 
   bool dlab = is_device_ptr(labels, ctx->device);
   // Small host calls: the kernel reads the points from, and writes the labels
   // to, pinned host memory, so the call is two host copies, one launch and one
-  // wait.
-  const bool small = !dpts && !dlab && !omega && n <= kPinnedPoints && grid_serves(ctx, o);
+  // wait.  (Without page-locked memory to be had they are staged as others are.)
+  bool small = !dpts && !dlab && !omega && n <= kPinnedPoints && grid_serves(ctx, o);
+  if (small && !ctx->h_stage &&
+      cudaMallocHost(&ctx->h_stage, (size_t)kPinnedPoints * (3 * sizeof(float) + sizeof(int32_t))) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->h_stage = nullptr;
+    small = false;
+  }
   st = reserve_call(ctx, n, o, (!dpts || !dlab) && !small);
   if (st) return st;
   if (small) {
-    if (!ctx->h_stage)
-      CK(cudaMallocHost(&ctx->h_stage, (size_t)kPinnedPoints * (3 * sizeof(float) + sizeof(int32_t))),
-         "cudaMallocHost(staging)");
     float *hp = reinterpret_cast<float *>(ctx->h_stage);
     int32_t *hl = reinterpret_cast<int32_t *>(hp + 3 * kPinnedPoints);
     std::memcpy(hp, pts, (size_t)n * 3 * sizeof(float));

@@ -341,6 +341,26 @@ int needles() {
   return 0;
 }
 
+// A small host call without page-locked memory to be had takes the way of the
+// large ones.
+int no_pinned_memory() {
+  const std::vector<float> pts(300, 0.25f);
+  std::vector<int32_t> lab(100, -7);
+  zef_ctx *ctx = nullptr;
+  CHECK(zef_create(&ctx, 0, nullptr) == ZEF_OK, "create");
+  CHECK(add(ctx, 1, octahedron(1.f, 3)) == ZEF_OK, "surface: %s", zef_last_error(ctx));
+  fake_fail_pinned(true);
+  for (int k = 0; k < 2; ++k)
+    CHECK(zef_label_points(ctx, pts.data(), 100, lab.data(), nullptr, nullptr, nullptr) == ZEF_OK, "call %d: %s", k,
+          zef_last_error(ctx));
+  fake_fail_pinned(false);
+  CHECK(!ctx->h_stage, "page-locked memory from nowhere");
+  CHECK(zef_label_points(ctx, pts.data(), 100, lab.data(), nullptr, nullptr, nullptr) == ZEF_OK && ctx->h_stage,
+        "the next call: %s", zef_last_error(ctx));
+  zef_destroy(ctx);
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
@@ -355,6 +375,7 @@ int main(int argc, char **argv) {
   else if (name == "sums_beyond_32_bits") sums_beyond_32_bits();
   else if (name == "lists_cleared_after_a_failure") lists_cleared_after_a_failure();
   else if (name == "needles") needles();
+  else if (name == "no_pinned_memory") no_pinned_memory();
   else return 2;
   return g_bad ? 1 : 0;
 }

@@ -36,6 +36,7 @@ std::map<const void *, std::vector<unsigned char>> g_vars;
 cudaError_t g_last = cudaSuccess;
 long g_allocs = 0, g_fail_at = -1, g_unordered = 0;
 size_t g_uploaded = 0;
+bool g_fail_pinned = false;
 std::string g_first_unordered, g_hook_name, g_fail_launch;
 std::function<std::function<void()>(void **)> g_hook;
 std::map<std::string, long> g_launches;
@@ -102,6 +103,7 @@ void fake_on_launch_args(const char *name, std::function<std::function<void()>(v
   g_hook_name = name;
   g_hook = std::move(f);
 }
+void fake_fail_pinned(bool fail) { g_fail_pinned = fail; }
 void fake_fail_launch(const char *name) { g_fail_launch = name; }
 long fake_launches(const char *name) {
   long n = 0;
@@ -134,6 +136,7 @@ cudaError_t cudaFree(void *p) {
   return cudaSuccess;
 }
 cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) {
+  if (g_fail_pinned) return done(cudaErrorMemoryAllocation);
   *p = std::calloc(n, 1);
   g_pinned[(uintptr_t)*p] = n;
   return cudaSuccess;

@@ -68,3 +68,7 @@ def test_lists_are_cleared_after_a_failed_call(driver):
 
 def test_long_thin_triangles_do_not_fill_the_registration(driver):
     _run(driver, "needles")
+
+
+def test_small_host_calls_without_page_locked_memory(driver):
+    _run(driver, "no_pinned_memory")
